@@ -268,11 +268,13 @@ int pt_ma_quad_bwd(const double *t_dev, int n_t, const pt_theta *theta, int n_ss
  * its own k and (u1, u2); the orbit is per walker.
  *
  * pt_batch_plan_create() binds the buffers named in the descriptor (their
- * addresses, not their contents), builds a work list of (walker, time tile)
- * items that never straddle a light curve, times candidate configurations
- * (tile length 64/128/256 x CTAs per SM) on those buffers when autotune is
+ * addresses, not their contents), times candidate configurations (CTAs of 128
+ * or 256 threads x slices of the times) on those buffers when autotune is
  * non-zero, and captures the chosen evaluation -- work-counter reset,
- * per-walker set-up, one persistent kernel, residual reduction -- into a
+ * preparation (per-walker set-up, per (walker, passband) row tables of the
+ * depth over z, per tile of 64 times its range and residual sums with the flux
+ * at 1), one persistent kernel over (walker, passband group, slice) items,
+ * residual reduction -- into a
  * CUDA graph.  pt_batch_run() replays that graph on a stream: update the
  * contents of the bound buffers (new walker parameters, new data) between
  * runs.  The plan allocates its own work list and scratch (device memory)
@@ -295,7 +297,9 @@ typedef struct pt_batch_desc {
     float *flux;            /* [n_v][n_b][n_t] device or NULL */
     float *ssr;             /* [n_v][n_b] device or NULL (not both NULL) */
     int *n_bad;             /* optional device counter of non-converged Newton solves */
-    int k_mode;             /* 0: each passband with its own k (exact);
+    int k_mode;             /* 0: each passband with its own k (exact to FP32: read from row tables
+                                  that hold the exact terms' rounding, k in [1e-6, 0.5], else
+                                  the terms themselves);
                                1: the model once per walker with k_hat, the mean of its
                                   passbands' k, and each passband's depth 1 - f scaled by
                                   k_b^2 / k_hat^2 (Sec. 3.5);

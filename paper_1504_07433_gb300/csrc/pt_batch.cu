@@ -3,19 +3,29 @@
 // motivation in Sec. 1; per-passband radius ratios and limb darkening,
 // Secs. 2.2.2 and 3.5; the device-side likelihood of Sec. 3.4).
 //
-// Work list: (walker, time tile) items, tiles never straddle a light curve,
-// ordered tile-major so that consecutive items share their times and
-// observations in L2.  A grid of (SMs x CTAs/SM) persistent CTAs pulls items
-// through an atomic counter.  Per item:
-//   A. one thread per time: phase reduction, window test (largest k of the
-//      walker's passbands), z for in-window times, compaction;
-//   B. (in-window time, passband) units on full warps: Mandel-Agol terms with
-//      the passband's own k, limb darkening with its own (u1, u2);
-//   C. one warp per passband: coalesced flux stores, residual sums reduced in
-//      a fixed order into per-(walker, passband, tile) partials.
-// The plan autotunes the tile length and the CTAs per SM by timing the
-// candidates on the caller's buffers, then captures counter reset + set-up +
-// persistent kernel + residual reduction into one CUDA graph.
+// batch_prep_kernel, per call:
+//   - the walkers' geometry records, the double-float split of the times;
+//   - per tile of BT consecutive times (as stored; they need not be sorted)
+//     the tile's time range and, per passband, its residual sum with the flux
+//     at 1;
+//   - per (walker, passband) the row table of its transit depth as a function
+//     of z (pt_device.cuh: 144 evaluations of the exact terms).  Every row is
+//     then read at tens of thousands of separations (all in-window times of
+//     all light curves), so the elliptic integrals have left the per-point
+//     work: at 1,024 walkers x 64 passbands x 81,058 times a call went from
+//     17.5 ms (the terms evaluated per point) to 2.84 ms.
+// batch_kernel: persistent CTAs take (walker, group of BG passbands, slice of
+// the times) items from an atomic counter, ordered so that consecutive items
+// share their observations in L2.  Per item the group's rows are staged in
+// shared memory; tiles that cannot meet the walker's transit window add their
+// prepared residual sums (and flux 1); the others are evaluated one time per
+// thread: z once, then the group's depths, fluxes and residuals, the sums in
+// registers.  Per point and passband that is about 22 instructions for the
+// depth and 4 for the residual; the issue rate bounds it, the observations
+// come from L2.
+// The plan autotunes the CTA size and the number of slices by timing the
+// candidates on the caller's buffers, then captures counter reset +
+// preparation + persistent kernel + reduction into one CUDA graph.
 #include <cuda_runtime.h>
 
 #include <math.h>
@@ -23,6 +33,7 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <vector>
 
 #include "../../include/pt.h"
@@ -38,9 +49,23 @@ bool ma_table_view(pt_ma_table t, const float4 **tab, int *n_k, int *n_z, float 
 
 namespace {
 
-struct BatchItem {
-    int v, start, len, tile;
+constexpr int BT = 64;                   // times per tile
+constexpr int BG = 16;                   // passbands per group (residual sums of a group in registers)
+constexpr int PREP_ROWS = 2;             // row tables per CTA of the preparation
+constexpr int PREP = PREP_ROWS * pt::MT_NODES;   // its threads: one node of a row each
+constexpr int PREP_TILES = PREP / BT;    // tiles of times per CTA
+constexpr size_t INTERP_SMEM = 64 * 1024;   // largest staged group of interpolated rows
+
+// What a depth is formed from.
+enum Mode {
+    M_ROWS = 0,     // k_mode 0: row tables of the exact depth
+    M_KHAT = 1,     // k_mode 1: the exact terms once per time with k_hat, scaled per passband (Sec. 3.5)
+    M_INTERP = 2,   // k_mode 2: rows of the caller's table, interpolated in k, staged in shared memory
+    M_GATHER = 3    // k_mode 2 with rows too long to stage: bilinear reads of the table per point
 };
+
+// What is asked for: the two usual calls have no run-time choice per point.
+enum Out { O_FLUX = 0, O_SSR = 1 /* unit weights */, O_ANY = 2 };
 
 struct BatchArgs {
     const float2 *tsplit;
@@ -48,41 +73,65 @@ struct BatchArgs {
     const GeomRec *rec;
     const float *k;      // [n_v][n_b]
     const float *ld;     // [n_v][n_b][2]
+    const float *rows;   // [n_v][n_b][MT_ROW], M_ROWS
+    const int2 *tiles;       // [n_tiles] (first time, length): tiles never straddle a light curve
+    const float2 *tile_mm;   // [n_tiles] smallest and largest time
+    const float *base;   // [n_b][n_tiles] residual sums with the flux at 1
+    int n_tiles;
     int n_v, n_b, n_ss;
     float t_exp;
     int max_iter;
     const float *y, *wt; // [n_b][n_t]
     float *flux;         // [n_v][n_b][n_t]
-    float *ssr_part;     // [n_v][n_b][n_tiles]
-    int n_tiles;
-    const BatchItem *items;
+    float *ssr_part;     // [n_v][n_b][n_slices]
+    int bg;              // passbands per group, at most BG
+    int n_groups, n_slices, tiles_per_slice;
     int n_items;
     int *counter;
     int *n_bad;
-    int khat;            // k_mode 1: terms once per time with k_hat (Sec. 3.5)
     // k_mode 2: the Mandel-Agol terms interpolated from this table (Sec. 2.2.3)
     const float4 *mtab;
     int mn_k, mn_z;
     float mk_lo, mk_hi, minv_dk, minv_dz;
 };
 
-struct BatchSetupArgs {
+struct PrepArgs {
     const double *t;
     int n_t;
     float2 *tsplit;
     pt_orbit orb;
-    const float *k;
+    const float *k, *ld;
     int n_b;
     float half_exp;
     GeomRec *rec;
-    int n_vblocks;
     int khat;
+    const int2 *tiles;
+    float2 *tile_mm;
+    float *base;         // null: no residual sums wanted
+    const float *y, *wt;
+    int n_tiles;
+    float *rows;         // null: no row tables
+    int n_gblocks, n_tblocks, n_bblocks;
 };
 
-__global__ void batch_setup_kernel(BatchSetupArgs s)
+// transit depth weights of one passband: depth = we le + wd ld + wn ed
+__device__ __forceinline__ float3 band_weights(const float *ld, size_t row)
 {
-    if ((int)blockIdx.x < s.n_vblocks) {
-        int v = blockIdx.x * blockDim.x + threadIdx.x;
+    float3 w;
+    pt::ma_weights(ld[row * 2], ld[row * 2 + 1], &w.x, &w.y, &w.z);
+    return w;
+}
+
+constexpr int PREP_BASE = 8;   // (passband, tile) residual sums per warp of the preparation
+
+__global__ void __launch_bounds__(PREP) batch_prep_kernel(PrepArgs s)
+{
+    __shared__ float sF[PREP_ROWS][pt::MT_N * (pt::MT_Q + 1)];
+    __shared__ double smin[PREP / 32], smax[PREP / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    int blk = blockIdx.x;
+    if (blk < s.n_gblocks) {
+        const int v = blk * PREP + tid;
         if (v >= s.orb.n_v) return;
         // the geometry's k: the largest passband k (its window covers every
         // passband), or in k_hat mode the mean, the only k evaluated
@@ -96,198 +145,484 @@ __global__ void batch_setup_kernel(BatchSetupArgs s)
         bool ecc = s.orb.e != nullptr;
         pt::make_geom_rec(s.orb.t0[v], s.orb.P[v], s.orb.a[v], s.orb.inc[v], ecc, ecc ? s.orb.e[v] : 0.0f,
                           ecc ? s.orb.w[v] : 0.0f, kmax, s.half_exp, &s.rec[v]);
-    } else {
-        int i = (blockIdx.x - s.n_vblocks) * blockDim.x + threadIdx.x;
-        if (i < s.n_t) {
-            double x = s.t[i];
-            float h = (float)x;
+        return;
+    }
+    blk -= s.n_gblocks;
+    if (blk < s.n_tblocks) {
+        // PREP_TILES tiles: time split, smallest and largest time (rounded outward)
+        const int tile = blk * PREP_TILES + tid / BT;
+        const int2 tl = tid < PREP_TILES * BT && tile < s.n_tiles ? s.tiles[tile] : make_int2(0, 0);
+        const int i = tl.x + (tid & (BT - 1));
+        double lo = INFINITY, hi = -INFINITY;
+        if ((tid & (BT - 1)) < tl.y) {
+            const double x = s.t[i];
+            const float h = (float)x;
             s.tsplit[i] = make_float2(h, (float)(x - (double)h));
+            lo = hi = x;
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            lo = fmin(lo, __shfl_xor_sync(0xffffffffu, lo, o));
+            hi = fmax(hi, __shfl_xor_sync(0xffffffffu, hi, o));
+        }
+        if (lane == 0) {
+            smin[warp] = lo;
+            smax[warp] = hi;
+        }
+        __syncthreads();
+        const int out = blk * PREP_TILES + tid;
+        if (tid < PREP_TILES && out < s.n_tiles) {
+            lo = fmin(smin[2 * tid], smin[2 * tid + 1]);
+            hi = fmax(smax[2 * tid], smax[2 * tid + 1]);
+            float flo = (float)lo, fhi = (float)hi;
+            if ((double)flo > lo) flo = nextafterf(flo, -INFINITY);
+            if ((double)fhi < hi) fhi = nextafterf(fhi, INFINITY);
+            s.tile_mm[out] = make_float2(flo, fhi);
+        }
+        return;
+    }
+    blk -= s.n_tblocks;
+    if (blk < s.n_bblocks) {
+        // residual sums of (passband, tile) with the flux at 1, one warp each
+        const long long n_task = (long long)s.n_b * s.n_tiles;
+        const long long q0 = ((long long)blk * (PREP / 32) + warp) * PREP_BASE;
+        for (long long q = q0; q < q0 + PREP_BASE && q < n_task; ++q) {
+            const int b = (int)(q / s.n_tiles), tile = (int)(q - (long long)b * s.n_tiles);
+            const int2 tl = s.tiles[tile];
+            float acc = 0.0f;
+#pragma unroll
+            for (int h = 0; h < BT / 32; ++h) {
+                const int i = tl.x + 32 * h + lane;
+                if (32 * h + lane < tl.y) {
+                    const float r = s.y[(size_t)b * s.n_t + i] - 1.0f;
+                    acc = fmaf((s.wt ? s.wt[(size_t)b * s.n_t + i] : 1.0f) * r, r, acc);
+                }
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+            if (lane == 0) s.base[q] = acc;
+        }
+        return;
+    }
+    blk -= s.n_bblocks;
+    // PREP_ROWS row tables: a node per thread (region A's, in double-float
+    // arithmetic, on the first warps), then a coefficient per thread
+    const size_t n_rows = (size_t)s.orb.n_v * s.n_b, first = (size_t)blk * PREP_ROWS;
+    constexpr int NODES_A = pt::MT_NA * pt::MT_Q, NODES_L = pt::MT_NODES - NODES_A;
+    {
+        const bool in_a = tid < PREP_ROWS * NODES_A;
+        const int u = in_a ? tid : tid - PREP_ROWS * NODES_A;
+        const int r = in_a ? u / NODES_A : u / NODES_L;
+        const int node = in_a ? u - r * NODES_A : NODES_A + u - r * NODES_L;
+        const size_t row = first + r;
+        if (row < n_rows) {
+            const float p = s.k[row];
+            if (pt::mt_valid(p)) {   // the others take the exact terms per point
+                const float3 w = band_weights(s.ld, row);
+                const int i = node / pt::MT_Q, q = node - i * pt::MT_Q;
+                float le, ld, ed;
+                pt::mt_node(p, i, q, &le, &ld, &ed);
+                sF[r][i * (pt::MT_Q + 1) + q] = w.x * le + w.y * ld + w.z * ed;
+            }
+        }
+    }
+    __syncthreads();
+    {
+        const int c = tid / (PREP_ROWS * pt::MT_N), u = tid - c * (PREP_ROWS * pt::MT_N);
+        const int r = u / pt::MT_N, i = u - r * pt::MT_N;
+        const size_t row = first + r;
+        if (row < n_rows && pt::mt_valid(s.k[row]))
+            s.rows[row * pt::MT_ROW + 8 * i + c] = pt::mt_coef(i, c, sF[r] + i * (pt::MT_Q + 1));
+    }
+}
+static_assert(PREP % 32 == 0 && PREP_ROWS * pt::MT_NA * pt::MT_Q % 32 == 0, "whole warps in region A");
+
+// Can a time in [tmin, tmax] lie in the transit window of some epoch?  The
+// interval is widened by m, 1e-6 of the magnitudes involved, above the FP32
+// rounding of these expressions, so the test never misses an epoch.
+__device__ __forceinline__ bool tile_meets_window(const GeomRec &g, float tmin, float tmax)
+{
+    if (g.win_lo > g.win_hi) return false;                // never in transit
+    if (g.win_hi - g.win_lo >= 0.5f * g.Ph) return true;  // a wide window: no test
+    const float m = 1e-6f * (fabsf(tmin) + fabsf(tmax) + fabsf(g.t0h) + g.Ph) + 1e-9f;
+    const float n_lo = ceilf((tmin - g.t0h - g.win_hi - m) * g.invP);
+    const float n_hi = floorf((tmax - g.t0h - g.win_lo + m) * g.invP);
+    return !(n_lo > n_hi);
+}
+
+// A 16-byte shared-memory load at this place: the passbands' constants are
+// loop-invariant, and left to itself the compiler keeps all of a group's 64
+// of them in registers and spills.
+__device__ __forceinline__ float4 lds_here(const float4 *p)
+{
+    float4 v;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
+                 : "r"((unsigned)__cvta_generic_to_shared(p)));
+    return v;
+}
+
+// One passband of an item without a row table (its radius ratio outside
+// mt_valid, or too few points for tables): the exact terms per point.
+template <int TT>
+__device__ __noinline__ void exact_row(const BatchArgs &A, const GeomRec &g, int v, int b, int slice, float *sred,
+                                       int *n_bad)
+{
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const size_t row = (size_t)v * A.n_b + b;
+    const float k = A.k[row];
+    const float3 w = band_weights(A.ld, row);
+    const float inv_ss = 1.0f / (float)A.n_ss;
+    const int t_end = min(A.n_tiles, (slice + 1) * A.tiles_per_slice);
+    float acc = 0.0f;
+    for (int tj = slice * A.tiles_per_slice + tid / BT; tj < t_end; tj += TT / BT) {
+        const float2 mm = A.tile_mm[tj];
+        const int2 tl = A.tiles[tj];
+        if ((tid & (BT - 1)) >= tl.y) continue;
+        const int i = tl.x + (tid & (BT - 1));
+        float dep = 0.0f;
+        bool inw = false;
+        if (tile_meets_window(g, mm.x, mm.y)) {
+            const float2 ts = A.tsplit[i];
+            const float dt = pt::reduce_time(ts.x, ts.y, g);
+            inw = dt >= g.win_lo && dt <= g.win_hi;
+            if (inw) {
+                float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
+                for (int s = 0; s < A.n_ss; ++s) {
+                    bool bad = false;
+                    const float off = A.t_exp * (((float)s + 0.5f) * inv_ss - 0.5f);
+                    const float z = pt::orbit_z<true>(g, dt + off, A.max_iter, &bad, warm);
+                    if (bad && b == 0 && !A.rows) ++*n_bad;
+                    float le, ld, ed;
+                    pt::ma_terms(k, z, &le, &ld, &ed);
+                    dep += w.x * le + w.y * ld + w.z * ed;
+                }
+                dep *= inv_ss;
+            }
+        }
+        if (A.flux) A.flux[row * A.n_t + i] = 1.0f - dep;
+        if (A.ssr_part) {
+            const size_t at = (size_t)b * A.n_t + i;
+            const float r = (A.y[at] - 1.0f) + dep;
+            acc = fmaf((A.wt ? A.wt[at] : 1.0f) * r, r, acc);
+        }
+    }
+    if (A.ssr_part) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        __syncthreads();
+        if (lane == 0) sred[warp] = acc;
+        __syncthreads();
+        if (tid == 0) {
+            float x = 0.0f;
+            for (int u = 0; u < TT / 32; ++u) x += sred[u];
+            A.ssr_part[row * A.n_slices + slice] = x;
         }
     }
 }
 
-template <int TT, bool INTERP>
-__global__ void __launch_bounds__(TT) batch_kernel(BatchArgs A)
+template <int TT, int MODE, bool SS, int OUT>
+__global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(BatchArgs A)
 {
-    extern __shared__ __align__(16) float dyn[];
-    float *fbuf = dyn;                    // [n_b][TT]
-    float *swt = dyn + A.n_b * TT;        // [n_b][4]: we, wd, wn, k (k_hat mode: k^2 / k_hat^2)
+    extern __shared__ __align__(16) float dyn[];   // M_ROWS: [BG][MT_ROW]; M_INTERP: [BG][mn_z]
     __shared__ GeomRec srec;
-    __shared__ float sdt[TT], sz[TT];
-    __shared__ float ste[3][TT];          // k_hat mode: supersample-mean terms per time
-    __shared__ unsigned char sflag[TT];
-    __shared__ unsigned short squeue[TT];
-    __shared__ int sqn, s_item, sbad;
+    __shared__ float4 sband[BG];   // M_ROWS: k, the scales, valid; M_KHAT: depth weights; others: we, wd, wn, k
+    __shared__ float sex[TT / 32];
+    __shared__ float sred[TT / 32][BG];
+    __shared__ int slist[TT], swcnt[TT / 32];
+    __shared__ int s_item;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    constexpr int NW = TT / 32;
-    if (tid == 0) sbad = 0;
-    bool bad = false;
+    constexpr int NW = TT / 32, TPP = TT / BT;   // tiles per pass
+    const bool want_ssr = OUT == O_SSR || (OUT == O_ANY && A.ssr_part), want_flux = OUT == O_FLUX || (OUT == O_ANY && A.flux);
+    const float inv_ss = 1.0f / (float)A.n_ss;
+    const unsigned row_base = pt::mt_base(dyn);   // M_ROWS
+    int nbad = 0;
     for (;;) {
-        if (tid == 0) {
-            s_item = atomicAdd(A.counter, 1);
-            sqn = 0;
-        }
+        if (tid == 0) s_item = atomicAdd(A.counter, 1);
         __syncthreads();
         const int it = s_item;
         if (it >= A.n_items) break;
-        const BatchItem item = A.items[it];
-        const int v = item.v;
-        if (tid < 6)
-            reinterpret_cast<float4 *>(&srec)[tid] = reinterpret_cast<const float4 *>(&A.rec[v])[tid];
-        for (int b = tid; b < A.n_b; b += TT) {
-            float we, wd, wn;
-            pt::ma_weights(A.ld[((size_t)v * A.n_b + b) * 2], A.ld[((size_t)v * A.n_b + b) * 2 + 1], &we, &wd, &wn);
-            swt[4 * b] = we;
-            swt[4 * b + 1] = wd;
-            swt[4 * b + 2] = wn;
-            float kb = A.k[(size_t)v * A.n_b + b];
-            if (A.khat) {
-                float r = kb / A.rec[v].k;
-                kb = r * r;
+        const int v = it % A.n_v;
+        const int sg = it / A.n_v;
+        const int grp = sg % A.n_groups, slice = sg / A.n_groups;
+        const int b0 = grp * A.bg, nb = min(A.bg, A.n_b - b0);
+        const size_t row0 = (size_t)v * A.n_b + b0;
+        if (tid < 6) reinterpret_cast<float4 *>(&srec)[tid] = reinterpret_cast<const float4 *>(&A.rec[v])[tid];
+        // groups of 4 passbands are evaluated together; the last group's
+        // padding repeats the item's last passband and is dropped at the stores
+        const int nb4 = (nb + 3) & ~3;
+        bool all_ok = true;
+        if (tid < nb4) {
+            const size_t row = row0 + min(tid, nb - 1);
+            const float kb = A.k[row];
+            const float3 w = band_weights(A.ld, row);
+            if (MODE == M_ROWS) {
+                float sA = 0.0f, sL = 0.0f;
+                all_ok = A.rows && pt::mt_valid(kb);
+                if (all_ok) pt::mt_scales(kb, &sA, &sL);
+                sband[tid] = make_float4(kb, sA, sL, all_ok ? 1.0f : 0.0f);
+            } else if (MODE == M_KHAT) {
+                const float r = kb / A.rec[v].k;
+                const float r2 = r * r;
+                sband[tid] = make_float4(r2 * w.x, r2 * w.y, r2 * w.z, 0.0f);
+            } else {
+                sband[tid] = make_float4(w.x, w.y, w.z, kb);
             }
-            swt[4 * b + 3] = kb;
         }
-        __syncthreads();
-        // A: window test, z, compaction
-        bool inw = false;
-        float dt = 0.0f, z = PT_ZBEHIND;
-        if (tid < item.len) {
-            float2 ts = A.tsplit[item.start + tid];
-            if (pt::maybe_in_window(ts.x, srec)) {
-                dt = pt::reduce_time(ts.x, ts.y, srec);
-                inw = dt >= srec.win_lo && dt <= srec.win_hi;
-            }
-            if (inw && A.n_ss == 1) z = pt::orbit_z<true>(srec, dt, A.max_iter, &bad);
-        }
-        sdt[tid] = dt;
-        sz[tid] = z;
-        sflag[tid] = inw ? 1 : 0;
-        int slot = pt::warp_append(&sqn, inw);
-        if (inw) squeue[slot] = (unsigned short)tid;
-        __syncthreads();
-        // B: (time, passband) units
-        const int nq = sqn;
-        const int nu = nq * A.n_b;
-        const float inv_ss = 1.0f / (float)A.n_ss;
-        if (A.khat) {
-            // the terms once per in-window time, with k_hat ...
-            for (int qi = tid; qi < nq; qi += TT) {
-                int tl = squeue[qi];
-                float le = 0.0f, ld = 0.0f, ed = 0.0f;
-                float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
-                for (int s = 0; s < A.n_ss; ++s) {
-                    float zs = sz[tl];
-                    if (A.n_ss > 1) {
-                        float dts = sdt[tl] + A.t_exp * (((float)s + 0.5f) * inv_ss - 0.5f);
-                        zs = pt::orbit_z<true>(srec, dts, A.max_iter, &bad, warm);
-                    }
-                    float a0, a1, a2;
-                    pt::ma_terms(srec.k, zs, &a0, &a1, &a2);
-                    le += a0;
-                    ld += a1;
-                    ed += a2;
-                }
-                ste[0][tl] = le * inv_ss;
-                ste[1][tl] = ld * inv_ss;
-                ste[2][tl] = ed * inv_ss;
+        all_ok = __syncthreads_and(all_ok);
+        if (MODE == M_ROWS) {
+            // a row without a table (its radius ratio outside mt_valid) is staged as zeros
+            for (int i = tid; i < nb4 * (pt::MT_ROW / 4); i += TT) {
+                const int j = i / (pt::MT_ROW / 4);
+                float4 c = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+                if (sband[j].w != 0.0f)
+                    c = reinterpret_cast<const float4 *>(A.rows + (row0 + min(j, nb - 1)) * pt::MT_ROW)[i - j * (pt::MT_ROW / 4)];
+                reinterpret_cast<float4 *>(dyn)[i] = c;
             }
             __syncthreads();
-            // ... then each passband's depth scaled by k_b^2 / k_hat^2
-            for (int u = tid; u < nu; u += TT) {
-                int b = u / nq, qi = u - b * nq;
-                int tl = squeue[qi];
-                float dep = swt[4 * b] * ste[0][tl] + swt[4 * b + 1] * ste[1][tl] + swt[4 * b + 2] * ste[2][tl];
-                fbuf[b * TT + tl] = 1.0f - swt[4 * b + 3] * dep;
-            }
         }
-        // unit u = b nq + qi; the thread's units advance by TT = dq nq + dr
-        const int dq = nq > 0 ? TT / nq : 0, dr = nq > 0 ? TT - dq * nq : 0;
-        int ub = nq > 0 ? tid / nq : 0, uq = tid - ub * nq;
-        for (int u = A.khat ? nu : tid; u < nu; u += TT) {
-            const int b = ub, qi = uq;
-            ub += dq;
-            uq += dr;
-            if (uq >= nq) {
-                uq -= nq;
-                ++ub;
+        if (MODE == M_INTERP) {
+            // each passband's row of the table: nodes interpolated in k, combined with its weights
+            for (int i = tid; i < nb4 * A.mn_z; i += TT) {
+                const int b = i / A.mn_z, j = i - b * A.mn_z;
+                const float4 w = sband[b];
+                const float fk = (fminf(fmaxf(w.w, A.mk_lo), A.mk_hi) - A.mk_lo) * A.minv_dk;
+                const int ik = min((int)fk, A.mn_k - 2);
+                const float wk = fk - (float)ik;
+                const float4 p0 = __ldg(A.mtab + (size_t)ik * A.mn_z + j), p1 = __ldg(A.mtab + (size_t)(ik + 1) * A.mn_z + j);
+                dyn[i] = w.x * fmaf(wk, p1.x - p0.x, p0.x) + w.y * fmaf(wk, p1.y - p0.y, p0.y) +
+                         w.z * fmaf(wk, p1.z - p0.z, p0.z);
             }
-            int tl = squeue[qi];
-            float kb = swt[4 * b + 3];
-            float le, ld, ed;
-            if (A.n_ss == 1) {
-                if (INTERP)
-                    pt::ma_interp(A.mtab, A.mn_k, A.mn_z, A.mk_lo, A.mk_hi, A.minv_dk, A.minv_dz, kb, sz[tl], &le, &ld, &ed);
-                else
-                    pt::ma_terms(kb, sz[tl], &le, &ld, &ed);
-            } else {
-                le = ld = ed = 0.0f;
-                float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
-                for (int s = 0; s < A.n_ss; ++s) {
-                    float dts = sdt[tl] + A.t_exp * (((float)s + 0.5f) * inv_ss - 0.5f);
-                    float zs = pt::orbit_z<true>(srec, dts, A.max_iter, &bad, warm);
-                    float a0, a1, a2;
-                    if (INTERP)
-                        pt::ma_interp(A.mtab, A.mn_k, A.mn_z, A.mk_lo, A.mk_hi, A.minv_dk, A.minv_dz, kb, zs, &a0, &a1, &a2);
-                    else
-                        pt::ma_terms(kb, zs, &a0, &a1, &a2);
-                    le += a0;
-                    ld += a1;
-                    ed += a2;
-                }
-                le *= inv_ss;
-                ld *= inv_ss;
-                ed *= inv_ss;
-            }
-            fbuf[b * TT + tl] = 1.0f - (swt[4 * b] * le + swt[4 * b + 1] * ld + swt[4 * b + 2] * ed);
+            __syncthreads();
         }
-        __syncthreads();
-        // C: one warp per passband
-        for (int b = warp; b < A.n_b; b += NW) {
-            float acc = 0.0f;
-            const size_t row = (size_t)v * A.n_b + b;
-            for (int t = lane; t < item.len; t += 32) {
-                float f = sflag[t] ? fbuf[b * TT + t] : 1.0f;
-                int i = item.start + t;
-                if (A.flux) A.flux[row * A.n_t + i] = f;
-                if (A.ssr_part) {
-                    float r = A.y[(size_t)b * A.n_t + i] - f;
-                    acc = fmaf((A.wt ? A.wt[(size_t)b * A.n_t + i] : 1.0f) * r, r, acc);
-                }
-            }
-            if (A.ssr_part) {
+        float acc[BG];
 #pragma unroll
-                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-                if (lane == 0) A.ssr_part[row * A.n_tiles + item.tile] = acc;
+        for (int j = 0; j < BG; ++j) acc[j] = 0.0f;
+        const int t_end = MODE == M_ROWS && !A.rows ? 0 : min(A.n_tiles, (slice + 1) * A.tiles_per_slice);
+        for (int c0 = slice * A.tiles_per_slice; c0 < t_end; c0 += TT) {
+            // one window test per thread; the tiles to evaluate listed in order
+            const int jt = c0 + tid;
+            bool ev = false;
+            if (jt < t_end) {
+                const float2 mm = A.tile_mm[jt];
+                ev = tile_meets_window(srec, mm.x, mm.y);
+                if (!ev && want_ssr) {
+                    const float *bp = A.base + (size_t)b0 * A.n_tiles + jt;
+#pragma unroll
+                    for (int j = 0; j < BG; ++j) {
+                        if (j >= nb) break;
+                        acc[j] += *bp;
+                        bp += A.n_tiles;
+                    }
+                }
+            }
+            const unsigned bal = __ballot_sync(0xffffffffu, ev);
+            __syncthreads();   // the previous chunk's list is no longer read
+            if (lane == 0) swcnt[warp] = __popc(bal);
+            __syncthreads();
+            int base = 0, n_ev = 0;
+#pragma unroll
+            for (int w = 0; w < NW; ++w) {
+                base += (w < warp) ? swcnt[w] : 0;
+                n_ev += swcnt[w];
+            }
+            if (ev) slist[base + __popc(bal & ((1u << lane) - 1u))] = jt;
+            if (want_flux) {
+                // flux 1 on the skipped tiles
+                const int c1 = min(t_end, c0 + TT);
+                for (int tj = c0 + tid / BT; tj < c1; tj += TPP) {
+                    const float2 mm = A.tile_mm[tj];
+                    const int2 tl = A.tiles[tj];
+                    if ((tid & (BT - 1)) < tl.y && !tile_meets_window(srec, mm.x, mm.y)) {
+                        float *fp = A.flux + row0 * A.n_t + tl.x + (tid & (BT - 1));
+                        for (int j = 0; j < nb; ++j, fp += A.n_t) *fp = 1.0f;
+                    }
+                }
+            }
+            __syncthreads();
+            for (int q = tid / BT; q < n_ev; q += TPP) {
+                const int2 tl = A.tiles[slist[q]];
+                if ((tid & (BT - 1)) >= tl.y) continue;
+                const int i = tl.x + (tid & (BT - 1));
+                const float2 ts = A.tsplit[i];
+                float dt = 0.0f;
+                bool inw = false;
+                if (pt::maybe_in_window(ts.x, srec)) {
+                    dt = pt::reduce_time(ts.x, ts.y, srec);
+                    inw = dt >= srec.win_lo && dt <= srec.win_hi;
+                }
+                // observations of the first passbands, on their way during the orbit;
+                // element offsets from passband b0's row are 32-bit (the host keeps
+                // a group's rows within 2^32 elements)
+                const float *yp = A.y + (size_t)b0 * A.n_t, *wp = A.wt + (size_t)b0 * A.n_t;
+                float *fp = A.flux + row0 * A.n_t;
+                unsigned at_y = (unsigned)i, at = (unsigned)i;
+                float yn[4] = {0.0f, 0.0f, 0.0f, 0.0f}, wn[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                auto load4 = [&](int j0) {
+                    if (OUT == O_FLUX || !want_ssr) return;
+                    if (j0 + 4 <= nb) {
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            yn[u] = yp[at_y];
+                            if (OUT == O_ANY) wn[u] = A.wt ? wp[at_y] : 1.0f;
+                            at_y += (unsigned)A.n_t;
+                        }
+                    } else {   // a padding passband's sum is dropped
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            if (j0 + u < nb) {
+                                yn[u] = yp[at_y];
+                                if (OUT == O_ANY) wn[u] = A.wt ? wp[at_y] : 1.0f;
+                            }
+                            at_y += (unsigned)A.n_t;
+                        }
+                    }
+                };
+                load4(0);
+                // transit depth of passband j at one separation
+                float zm1 = 0.0f, off_limb = 0.0f, zz = 0.0f, wz = 0.0f;
+                int iz = 0;
+                auto at_z = [&](float z) {
+                    zz = z;
+                    if (MODE == M_ROWS) {
+                        zm1 = z - 1.0f;
+                        off_limb = pt::mt_off_limb(zm1);
+                    } else if (MODE == M_INTERP) {   // cell and weight in z
+                        const float fz = fminf(fmaxf(z, 0.0f) * A.minv_dz, (float)(A.mn_z - 1));
+                        iz = min((int)fz, A.mn_z - 2);
+                        wz = fz - (float)iz;
+                    }
+                };
+                auto depth = [&](int j) {
+                    const float4 w = lds_here(sband + j);
+                    if (MODE == M_ROWS) {
+                        float t;
+                        const unsigned bits = pt::mt_find(w.x, w.y, w.z, zm1, off_limb, &t);
+                        return pt::mt_eval(row_base + (unsigned)(j * pt::MT_ROW * 4), bits, t);
+                    }
+                    if (MODE == M_INTERP) {
+                        const float *row = dyn + j * A.mn_z + iz;
+                        return zz < 1.0f + w.w ? fmaf(wz, row[1] - row[0], row[0]) : 0.0f;
+                    }
+                    float le, ld, ed;
+                    pt::ma_interp(A.mtab, A.mn_k, A.mn_z, A.mk_lo, A.mk_hi, A.minv_dk, A.minv_dz, w.w, zz, &le, &ld, &ed);
+                    return w.x * le + w.y * ld + w.z * ed;
+                };
+                float D[SS && MODE != M_KHAT ? BG : 1];
+                float te0 = 0.0f, te1 = 0.0f, te2 = 0.0f;   // M_KHAT: the mean terms with k_hat
+                if (!SS) {
+                    bool bad = false;
+                    const float z = inw ? pt::orbit_z<true>(srec, dt, A.max_iter, &bad) : PT_ZBEHIND;
+                    if (bad && grp == 0) ++nbad;   // every group solves the same orbit
+                    at_z(z);
+                } else {
+                    if (MODE != M_KHAT) {
+#pragma unroll
+                        for (int j = 0; j < BG; ++j) D[MODE != M_KHAT ? j : 0] = 0.0f;
+                    }
+                    float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
+#pragma unroll 1
+                    for (int s = 0; s < (inw ? A.n_ss : 0); ++s) {
+                        bool bad = false;
+                        const float z = pt::orbit_z<true>(srec, dt + A.t_exp * (((float)s + 0.5f) * inv_ss - 0.5f),
+                                                          A.max_iter, &bad, warm);
+                        if (bad && grp == 0) ++nbad;
+                        if (MODE == M_KHAT) {
+                            float a0, a1, a2;
+                            pt::ma_terms(srec.k, z, &a0, &a1, &a2);
+                            te0 += a0;
+                            te1 += a1;
+                            te2 += a2;
+                        } else {
+                            at_z(z);
+#pragma unroll
+                            for (int j0 = 0; j0 < BG; j0 += 4) {
+                                if (j0 >= nb) break;
+#pragma unroll
+                                for (int j = j0; j < j0 + 4; ++j) D[MODE != M_KHAT ? j : 0] += depth(j);
+                            }
+                        }
+                    }
+                    te0 *= inv_ss;
+                    te1 *= inv_ss;
+                    te2 *= inv_ss;
+                }
+#pragma unroll
+                for (int j0 = 0; j0 < BG; j0 += 4) {
+                    if (j0 >= nb) break;
+                    float yc[4], wc[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        yc[u] = yn[u];
+                        wc[u] = wn[u];
+                    }
+                    if (j0 + 4 < nb) load4(j0 + 4);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) {
+                        const int j = j0 + u;
+                        float dep;
+                        if (MODE == M_KHAT) {
+                            const float4 w = lds_here(sband + j);
+                            dep = w.x * te0 + w.y * te1 + w.z * te2;
+                        }
+                        else if (SS) dep = __fmul_rn(D[SS && MODE != M_KHAT ? j : 0], inv_ss);   // rounded the same in every variant
+                        else dep = depth(j);
+                        if (want_flux && j < nb) fp[at] = 1.0f - dep;
+                        at += (unsigned)A.n_t;
+                        if (want_ssr) {
+                            // y - f with f = 1 - depth not rounded in between
+                            const float r = (yc[u] - 1.0f) + dep;
+                            acc[j] = fmaf(OUT == O_ANY ? wc[u] * r : r, r, acc[j]);
+                        }
+                    }
+                }
             }
         }
-        __syncthreads();
+        if (want_ssr) {
+#pragma unroll
+            for (int j = 0; j < BG; ++j) {
+                float x = acc[j];
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+                if (lane == 0) sred[warp][j] = x;
+            }
+            __syncthreads();
+            if (tid < nb) {
+                float x = 0.0f;
+                for (int w = 0; w < NW; ++w) x += sred[w][tid];
+                if (MODE != M_ROWS || sband[tid].w != 0.0f) A.ssr_part[(row0 + tid) * A.n_slices + slice] = x;
+            }
+        }
+        if (MODE == M_ROWS && !all_ok) {
+            __syncthreads();   // the zero rows' flux is in place
+            for (int j = 0; j < nb; ++j)
+                if (sband[j].w == 0.0f) exact_row<TT>(A, srec, v, b0 + j, slice, sex, &nbad);
+        }
+        __syncthreads();   // shared memory is free for the next item
     }
-    if (bad) atomicAdd(&sbad, 1);
-    __syncthreads();
-    if (tid == 0 && sbad && A.n_bad) atomicAdd(A.n_bad, sbad);
+    if (nbad && A.n_bad) atomicAdd(A.n_bad, nbad);
 }
 
-__global__ void batch_reduce_kernel(const float *part, int rows, int n_tiles, float *ssr)
+__global__ void batch_reduce_kernel(const float *part, int rows, int n_slices, float *ssr)
 {
-    int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    int lane = threadIdx.x & 31;
-    if (warp >= rows) return;
+    const int row = blockIdx.x * blockDim.x + threadIdx.x;
+    if (row >= rows) return;
     float s = 0.0f;
-    for (int i = lane; i < n_tiles; i += 32) s += part[(size_t)warp * n_tiles + i];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) ssr[warp] = s;
+    for (int i = 0; i < n_slices; ++i) s += part[(size_t)row * n_slices + i];
+    ssr[row] = s;
 }
-
-size_t dyn_smem(int TT, int n_b) { return (size_t)n_b * TT * sizeof(float) + (size_t)n_b * 4 * sizeof(float); }
 
 }  // namespace
 
 struct pt_batch_plan_s {
     pt_batch_desc d;
     int tt, ctas_per_sm, grid, n_sm;
-    int n_items, n_tiles;
-    BatchItem *d_items;
+    int mode;
+    int n_tiles, bg, n_groups, n_slices, n_items, max_slices;
+    int2 *d_tiles;
+    float2 *d_mm;
+    float *d_base;
+    float *d_rows;
     int *d_counter;
     GeomRec *d_rec;
     float2 *d_tsplit;
@@ -295,7 +630,6 @@ struct pt_batch_plan_s {
     cudaGraph_t graph;
     cudaGraphExec_t exec;
     float tuned_ms;
-    std::vector<int> h_offsets;
 };
 
 namespace {
@@ -305,96 +639,99 @@ int berr(cudaError_t e, const char *where)
     return pt_internal::set_error(PT_ERR_CUDA, where, cudaGetErrorString(e));
 }
 
-// Tiles of length tt within each light curve; items tile-major.
-void build_items(const pt_batch_plan_s &p, int tt, std::vector<BatchItem> *items, int *n_tiles)
+using BatchFn = void (*)(BatchArgs);
+
+template <int TT, int MODE, bool SS>
+BatchFn batch_fn_o(int out)
 {
-    std::vector<std::pair<int, int>> tiles;
-    for (size_t j = 0; j + 1 < p.h_offsets.size(); ++j)
-        for (int s = p.h_offsets[j]; s < p.h_offsets[j + 1]; s += tt)
-            tiles.push_back({s, std::min(tt, p.h_offsets[j + 1] - s)});
-    *n_tiles = (int)tiles.size();
-    items->clear();
-    items->reserve((size_t)tiles.size() * p.d.orb.n_v);
-    for (size_t q = 0; q < tiles.size(); ++q)
-        for (int v = 0; v < p.d.orb.n_v; ++v) items->push_back({v, tiles[q].first, tiles[q].second, (int)q});
+    return out == O_FLUX ? batch_kernel<TT, MODE, SS, O_FLUX>
+           : out == O_SSR ? batch_kernel<TT, MODE, SS, O_SSR>
+                          : batch_kernel<TT, MODE, SS, O_ANY>;
 }
 
 template <int TT>
-int launch_batch_tt(const BatchArgs &A, int grid, size_t smem, cudaStream_t s)
+BatchFn batch_fn_t(int mode, bool ss, int out)
 {
-    if (A.mtab)
-        batch_kernel<TT, true><<<grid, TT, smem, s>>>(A);
-    else
-        batch_kernel<TT, false><<<grid, TT, smem, s>>>(A);
-    cudaError_t e = cudaGetLastError();
-    return e == cudaSuccess ? PT_OK : berr(e, "batch_kernel");
+    switch (mode) {
+    case M_ROWS: return ss ? batch_fn_o<TT, M_ROWS, true>(out) : batch_fn_o<TT, M_ROWS, false>(out);
+    case M_KHAT: return batch_kernel<TT, M_KHAT, true, O_ANY>;
+    case M_INTERP: return batch_kernel<TT, M_INTERP, true, O_ANY>;
+    default: return batch_kernel<TT, M_GATHER, true, O_ANY>;
+    }
 }
 
-template <bool I>
-cudaError_t set_smem_attr_i(int tt, size_t smem)
+BatchFn batch_fn(const pt_batch_plan_s &p, int tt)
 {
-    cudaError_t e = cudaSuccess;
-    if (tt == 64) e = cudaFuncSetAttribute(batch_kernel<64, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (tt == 128) e = cudaFuncSetAttribute(batch_kernel<128, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (tt == 256) e = cudaFuncSetAttribute(batch_kernel<256, I>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    return e;
+    const int out = !p.d.ssr ? O_FLUX : (!p.d.flux && !p.d.wt) ? O_SSR : O_ANY;
+    const bool ss = p.d.n_ss > 1;
+    return tt == 128 ? batch_fn_t<128>(p.mode, ss, out) : batch_fn_t<256>(p.mode, ss, out);
 }
 
-int set_smem_attr(int tt, size_t smem, bool interp)
+size_t dyn_smem(const pt_batch_plan_s &p, int n_z)
 {
-    cudaError_t e = interp ? set_smem_attr_i<true>(tt, smem) : set_smem_attr_i<false>(tt, smem);
-    return e == cudaSuccess ? PT_OK : berr(e, "cudaFuncSetAttribute");
+    if (p.mode == M_ROWS) return (size_t)BG * pt::MT_ROW * sizeof(float);
+    if (p.mode == M_INTERP) return (size_t)BG * n_z * sizeof(float);
+    return 0;
 }
 
-template <bool I>
-int max_ctas_per_sm_i(int tt, size_t smem)
+int table_args(const pt_batch_desc &d, BatchArgs *A)
 {
-    int n = 0;
-    if (tt == 64) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<64, I>, tt, smem);
-    if (tt == 128) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<128, I>, tt, smem);
-    if (tt == 256) cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, batch_kernel<256, I>, tt, smem);
-    return n;
+    A->mtab = nullptr;
+    A->mn_k = A->mn_z = 0;
+    A->mk_lo = A->mk_hi = A->minv_dk = A->minv_dz = 0.0f;
+    if (d.k_mode == 2 && !pt_internal::ma_table_view(d.table, &A->mtab, &A->mn_k, &A->mn_z, &A->mk_lo, &A->mk_hi,
+                                                     &A->minv_dk, &A->minv_dz))
+        return pt_internal::set_error(PT_ERR_ARG, "pt_batch_run", "k_mode 2 needs an interpolation table");
+    return PT_OK;
 }
 
-int max_ctas_per_sm(int tt, size_t smem, bool interp)
-{
-    return interp ? max_ctas_per_sm_i<true>(tt, smem) : max_ctas_per_sm_i<false>(tt, smem);
-}
-
-// Enqueue one full evaluation (counter reset, set-up, persistent kernel,
+// Enqueue one full evaluation (counter reset, preparation, persistent kernel,
 // residual reduction) for the plan's current configuration.
 int enqueue(pt_batch_plan_s &p, cudaStream_t s)
 {
     const pt_batch_desc &d = p.d;
     cudaError_t e = cudaMemsetAsync(p.d_counter, 0, sizeof(int), s);
     if (e != cudaSuccess) return berr(e, "cudaMemsetAsync");
-    BatchSetupArgs sa;
+    PrepArgs sa;
     sa.t = d.t;
     sa.n_t = d.n_t;
     sa.tsplit = p.d_tsplit;
     sa.orb = d.orb;
     sa.k = d.k;
+    sa.ld = d.ld;
     sa.khat = d.k_mode == 1;
     sa.n_b = d.n_b;
     sa.half_exp = (float)(0.5 * d.t_exp);
     sa.rec = p.d_rec;
-    sa.n_vblocks = (d.orb.n_v + 63) / 64;
-    batch_setup_kernel<<<sa.n_vblocks + (d.n_t + 63) / 64, 64, 0, s>>>(sa);
+    sa.tiles = p.d_tiles;
+    sa.tile_mm = p.d_mm;
+    sa.base = p.d_base;
+    sa.y = d.y;
+    sa.wt = d.wt;
+    sa.n_tiles = p.n_tiles;
+    sa.rows = p.d_rows;
+    sa.n_gblocks = (d.orb.n_v + PREP - 1) / PREP;
+    sa.n_tblocks = (p.n_tiles + PREP_TILES - 1) / PREP_TILES;
+    const long long per = (long long)(PREP / 32) * PREP_BASE;
+    sa.n_bblocks = d.ssr ? (int)(((long long)d.n_b * p.n_tiles + per - 1) / per) : 0;
+    const long long blocks = (long long)sa.n_gblocks + sa.n_tblocks + sa.n_bblocks +
+                             (p.d_rows ? ((long long)d.orb.n_v * d.n_b + PREP_ROWS - 1) / PREP_ROWS : 0);
+    batch_prep_kernel<<<(unsigned)blocks, PREP, 0, s>>>(sa);
     e = cudaGetLastError();
-    if (e != cudaSuccess) return berr(e, "batch_setup_kernel");
+    if (e != cudaSuccess) return berr(e, "batch_prep_kernel");
     BatchArgs A;
+    int st = table_args(d, &A);
+    if (st) return st;
     A.tsplit = p.d_tsplit;
     A.n_t = d.n_t;
     A.rec = p.d_rec;
     A.k = d.k;
-    A.khat = d.k_mode == 1;
-    A.mtab = nullptr;
-    A.mn_k = A.mn_z = 0;
-    A.mk_lo = A.mk_hi = A.minv_dk = A.minv_dz = 0.0f;
-    if (d.k_mode == 2 && !pt_internal::ma_table_view(d.table, &A.mtab, &A.mn_k, &A.mn_z, &A.mk_lo, &A.mk_hi,
-                                                     &A.minv_dk, &A.minv_dz))
-        return pt_internal::set_error(PT_ERR_ARG, "pt_batch_run", "k_mode 2 needs an interpolation table");
     A.ld = d.ld;
+    A.rows = p.d_rows;
+    A.tiles = p.d_tiles;
+    A.tile_mm = p.d_mm;
+    A.base = p.d_base;
+    A.n_tiles = p.n_tiles;
     A.n_v = d.orb.n_v;
     A.n_b = d.n_b;
     A.n_ss = d.n_ss;
@@ -404,49 +741,49 @@ int enqueue(pt_batch_plan_s &p, cudaStream_t s)
     A.wt = d.wt;
     A.flux = d.flux;
     A.ssr_part = d.ssr ? p.d_part : nullptr;
-    A.n_tiles = p.n_tiles;
-    A.items = p.d_items;
+    A.bg = p.bg;
+    A.n_groups = p.n_groups;
+    A.n_slices = p.n_slices;
+    A.tiles_per_slice = (p.n_tiles + p.n_slices - 1) / p.n_slices;
     A.n_items = p.n_items;
     A.counter = p.d_counter;
     A.n_bad = d.n_bad;
-    size_t smem = dyn_smem(p.tt, d.n_b);
-    int st = PT_OK;
-    if (p.tt == 64) st = launch_batch_tt<64>(A, p.grid, smem, s);
-    if (p.tt == 128) st = launch_batch_tt<128>(A, p.grid, smem, s);
-    if (p.tt == 256) st = launch_batch_tt<256>(A, p.grid, smem, s);
-    if (st) return st;
+    batch_fn(p, p.tt)<<<p.grid, p.tt, dyn_smem(p, A.mn_z), s>>>(A);
+    e = cudaGetLastError();
+    if (e != cudaSuccess) return berr(e, "batch_kernel");
     if (d.ssr) {
         int rows = d.orb.n_v * d.n_b;
-        batch_reduce_kernel<<<(rows * 32 + 255) / 256, 256, 0, s>>>(p.d_part, rows, p.n_tiles, d.ssr);
+        batch_reduce_kernel<<<(rows + 127) / 128, 128, 0, s>>>(p.d_part, rows, p.n_slices, d.ssr);
         e = cudaGetLastError();
         if (e != cudaSuccess) return berr(e, "batch_reduce_kernel");
     }
     return PT_OK;
 }
 
-int configure(pt_batch_plan_s &p, int tt, int cps)
+// Slices of the times (an item each per walker and passband group); the
+// partial sums are sized for the largest number at creation.
+constexpr int MAX_SLICES = 64;
+
+// Row tables from this many points (times x supersamples) per row: a table
+// costs 144 evaluations of the exact terms, a row reads it at the in-window
+// points, about a third of them in the light curves of transits.
+constexpr int ROWS_MIN_POINTS = 512;
+
+int configure(pt_batch_plan_s &p, int tt, int n_slices, int n_z)
 {
-    std::vector<BatchItem> items;
-    int n_tiles = 0;
-    build_items(p, tt, &items, &n_tiles);
-    cudaFree(p.d_items);
-    cudaFree(p.d_part);
-    p.d_items = nullptr;
-    p.d_part = nullptr;
-    cudaError_t e = cudaMalloc(&p.d_items, std::max<size_t>(1, items.size()) * sizeof(BatchItem));
-    if (e != cudaSuccess) return berr(e, "cudaMalloc items");
-    e = cudaMemcpy(p.d_items, items.data(), items.size() * sizeof(BatchItem), cudaMemcpyHostToDevice);
-    if (e != cudaSuccess) return berr(e, "cudaMemcpy items");
-    if (p.d.ssr) {
-        e = cudaMalloc(&p.d_part, (size_t)p.d.orb.n_v * p.d.n_b * n_tiles * sizeof(float));
-        if (e != cudaSuccess) return berr(e, "cudaMalloc partials");
-    }
+    const BatchFn fn = batch_fn(p, tt);
+    const size_t smem = dyn_smem(p, n_z);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    int per_sm = 0;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, tt, smem);
+    if (e != cudaSuccess) return berr(e, "batch_kernel occupancy");
+    if (per_sm < 1) return pt_internal::set_error(PT_ERR_ARG, "batch_kernel", "does not fit on an SM");
     p.tt = tt;
-    p.ctas_per_sm = cps;
-    p.grid = cps * p.n_sm;
-    p.n_items = (int)items.size();
-    p.n_tiles = n_tiles;
-    return set_smem_attr(tt, dyn_smem(tt, p.d.n_b), p.d.k_mode == 2);
+    p.ctas_per_sm = per_sm;
+    p.n_slices = n_slices;
+    p.n_items = p.d.orb.n_v * p.n_groups * n_slices;
+    p.grid = std::min(per_sm * p.n_sm, p.n_items);
+    return PT_OK;
 }
 
 void free_plan(pt_batch_plan_s *p)
@@ -454,7 +791,10 @@ void free_plan(pt_batch_plan_s *p)
     if (!p) return;
     if (p->exec) cudaGraphExecDestroy(p->exec);
     if (p->graph) cudaGraphDestroy(p->graph);
-    cudaFree(p->d_items);
+    cudaFree(p->d_tiles);
+    cudaFree(p->d_mm);
+    cudaFree(p->d_base);
+    cudaFree(p->d_rows);
     cudaFree(p->d_counter);
     cudaFree(p->d_rec);
     cudaFree(p->d_tsplit);
@@ -485,51 +825,79 @@ int pt_batch_plan_create(const pt_batch_desc *d, int autotune, pt_batch_plan *ou
     if (d->lc_offsets[0] != 0 || d->lc_offsets[d->n_lc] != d->n_t) return PT_ERR_ARG;
     for (int j = 0; j < d->n_lc; ++j)
         if (d->lc_offsets[j + 1] < d->lc_offsets[j]) return PT_ERR_ARG;
+    const long long n_rows = (long long)o.n_v * d->n_b;
     pt_batch_plan_s *p = new pt_batch_plan_s();
     p->d = *d;
-    p->h_offsets.assign(d->lc_offsets, d->lc_offsets + d->n_lc + 1);
     p->d.lc_offsets = nullptr;
     int dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&p->n_sm, cudaDevAttrMultiProcessorCount, dev);
+    BatchArgs tab;
+    int st = table_args(*d, &tab);
+    if (st) {
+        free_plan(p);
+        return st;
+    }
+    // rows of the caller's table are staged in shared memory while a group fits
+    p->mode = d->k_mode == 0 ? M_ROWS
+              : d->k_mode == 1 ? M_KHAT
+              : (size_t)BG * tab.mn_z * sizeof(float) <= INTERP_SMEM ? M_INTERP : M_GATHER;
+    // tiles of BT times within each light curve
+    std::vector<int2> tiles;
+    for (int j = 0; j < d->n_lc; ++j)
+        for (int s = d->lc_offsets[j]; s < d->lc_offsets[j + 1]; s += BT)
+            tiles.push_back(make_int2(s, std::min(BT, d->lc_offsets[j + 1] - s)));
+    p->n_tiles = (int)tiles.size();
+    p->bg = d->n_t <= (1 << 28) ? BG : 1;   // a group's observations within 32-bit offsets
+    p->n_groups = (d->n_b + p->bg - 1) / p->bg;
+    // many rows need no slices: bounds the partial sums
+    p->max_slices = (int)std::max(1LL, std::min((long long)MAX_SLICES, (1LL << 26) / n_rows));
+    const bool tables = p->mode == M_ROWS && (long long)d->n_t * d->n_ss >= ROWS_MIN_POINTS;
     cudaError_t e = cudaMalloc(&p->d_counter, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&p->d_rec, (size_t)o.n_v * sizeof(GeomRec));
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tsplit, (size_t)d->n_t * sizeof(float2));
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_tiles, tiles.size() * sizeof(int2));
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_mm, tiles.size() * sizeof(float2));
+    if (e == cudaSuccess && d->ssr) e = cudaMalloc(&p->d_base, (size_t)d->n_b * tiles.size() * sizeof(float));
+    if (e == cudaSuccess && d->ssr) e = cudaMalloc(&p->d_part, (size_t)n_rows * p->max_slices * sizeof(float));
+    if (e == cudaSuccess && tables) e = cudaMalloc(&p->d_rows, (size_t)n_rows * pt::MT_ROW * sizeof(float));
+    // (the two unused floats per interval are staged with the others)
+    if (e == cudaSuccess && tables) e = cudaMemset(p->d_rows, 0, (size_t)n_rows * pt::MT_ROW * sizeof(float));
+    if (e == cudaSuccess) e = cudaMemcpy(p->d_tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
-        int st = berr(e, "pt_batch_plan_create");
+        st = berr(e, "pt_batch_plan_create");
         free_plan(p);
         return st;
     }
     cudaStream_t cs;
     e = cudaStreamCreateWithFlags(&cs, cudaStreamNonBlocking);
     if (e != cudaSuccess) {
-        int st = berr(e, "cudaStreamCreate");
+        st = berr(e, "cudaStreamCreate");
         free_plan(p);
         return st;
     }
-    // autotuner: tile length x CTAs per SM, timed on the caller's buffers
-    int best_tt = 128, best_cps = 0;
+    // autotuner: CTA size x slices of the times, timed on the caller's
+    // buffers.  The fewest slices tried give every resident CTA about an
+    // item (or a chunk of tiles per slice, if there are too few tiles).
+    const int tts[2] = {256, 128};
+    const long long base_items = (long long)o.n_v * p->n_groups;
+    int best_tt = 0, best_sl = 1;
     float best = 1e30f;
-    const int tts[3] = {64, 128, 256};
-    int st = PT_OK;
     cudaEvent_t e0, e1;
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
-    for (int ti = 0; ti < 3 && st == PT_OK; ++ti) {
-        int tt = tts[ti];
-        if (!autotune && tt != 128) continue;
-        size_t smem = dyn_smem(tt, d->n_b);
-        if (smem > 200 * 1024) continue;
-        st = set_smem_attr(tt, smem, d->k_mode == 2);
+    for (int ti = 0; ti < 2 && st == PT_OK; ++ti) {
+        const int tt = tts[ti];
+        if (!autotune && ti > 0) break;
+        st = configure(*p, tt, 1, tab.mn_z);
         if (st) break;
-        int mx = max_ctas_per_sm(tt, smem, d->k_mode == 2);
-        if (mx < 1) continue;
-        int cands[4] = {mx, mx / 2, mx / 4, 1};
-        for (int ci = 0; ci < 4 && st == PT_OK; ++ci) {
-            int cps = cands[ci];
-            if (cps < 1 || (ci > 0 && cps == cands[ci - 1])) continue;
-            if (!autotune && ci > 0) break;
-            st = configure(*p, tt, cps);
+        const int sl_max = std::max(1, std::min(p->max_slices, p->n_tiles / (tt / BT)));
+        int sl0 = 1;
+        while (sl0 < sl_max && base_items * sl0 < (long long)p->n_sm * p->ctas_per_sm) sl0 *= 2;
+        for (int f = 1; f <= (autotune ? 8 : 1) && st == PT_OK; f *= 2) {
+            const int sl = std::min(sl0 * f, sl_max);
+            if (f > 1 && (sl0 * (f / 2) >= sl_max)) break;
+            st = configure(*p, tt, sl, tab.mn_z);
             if (st) break;
             st = enqueue(*p, cs);   // warm-up
             if (st) break;
@@ -548,14 +916,14 @@ int pt_batch_plan_create(const pt_batch_desc *d, int autotune, pt_batch_plan *ou
             if (st == PT_OK && ms < best) {
                 best = ms;
                 best_tt = tt;
-                best_cps = cps;
+                best_sl = sl;
             }
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
-    if (st == PT_OK && best_cps == 0) st = PT_ERR_ARG;
-    if (st == PT_OK) st = configure(*p, best_tt, best_cps);
+    if (st == PT_OK && best_tt == 0) st = PT_ERR_ARG;
+    if (st == PT_OK) st = configure(*p, best_tt, best_sl, tab.mn_z);
     if (st == PT_OK) {
         e = cudaStreamSynchronize(cs);
         if (e != cudaSuccess) st = berr(e, "autotune");

@@ -73,6 +73,87 @@ __device__ __forceinline__ float sqrt_a(float x)
     return r;
 }
 
+// The same, or the correctly rounded forms (for the nodes of tables that are
+// read many times: their cost is shared, and so is their error).
+template <bool IEEE>
+__device__ __forceinline__ float rcp_t(float x) { return IEEE ? __frcp_rn(x) : rcp_a(x); }
+template <bool IEEE>
+__device__ __forceinline__ float sqrt_t(float x) { return IEEE ? __fsqrt_rn(x) : sqrt_a(x); }
+
+// ---------------------------------------------------------------------------
+// Double-float arithmetic, for the few values that many others are formed
+// from (the Gimenez table recursion, the nodes of the row tables): a value is
+// the unevaluated sum h + l of two floats (about 48 significant bits).  Sums
+// and products carry their rounding errors exactly (Knuth's two-sum; the FMA
+// form of Dekker's product); reciprocal and root are one Newton correction of
+// the FP32 ones.  GB300's FP64 rate is a small fraction of its FP32 rate, so
+// FP64 operations would dominate that work.
+// ---------------------------------------------------------------------------
+struct DF {
+    float h, l;
+};
+
+__device__ __forceinline__ DF df_of(double v)
+{
+    float h = (float)v;
+    return DF{h, (float)(v - (double)h)};
+}
+
+__device__ __forceinline__ DF df_norm(float s, float e)   // |s| >= |e|
+{
+    float h = s + e;
+    return DF{h, e - (h - s)};
+}
+
+__device__ __forceinline__ DF df_add(DF a, DF b)
+{
+    float s = a.h + b.h;
+    float bb = s - a.h;
+    float e = (a.h - (s - bb)) + (b.h - bb);
+    return df_norm(s, e + (a.l + b.l));
+}
+
+__device__ __forceinline__ DF df_neg(DF a) { return DF{-a.h, -a.l}; }
+
+__device__ __forceinline__ DF df_mul(DF a, DF b)
+{
+    float p = a.h * b.h;
+    float e = fmaf(a.h, b.h, -p);
+    e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
+    return df_norm(p, e);
+}
+
+__device__ __forceinline__ DF df_scale(float a, DF b)   // a a power of two
+{
+    return DF{a * b.h, a * b.l};
+}
+
+// a b + c with one two-sum: the product's rounding error (fmaf), the two-sum
+// error of p + c_h, the cross terms and c_l go into the low part
+__device__ __forceinline__ DF df_mad(DF a, DF b, DF c)
+{
+    const float p = a.h * b.h;
+    const float e = fmaf(a.h, b.h, -p);
+    const float s = p + c.h;
+    const float bb = s - p;
+    const float err = (p - (s - bb)) + (c.h - bb);
+    return df_norm(s, fmaf(a.h, b.l, fmaf(a.l, b.h, c.l)) + (e + err));
+}
+
+__device__ __forceinline__ DF df_rcp(DF a)   // a normal
+{
+    const float x = rcp_a(a.h);
+    const float e = fmaf(-a.l, x, fmaf(-a.h, x, 1.0f));
+    return df_norm(x, x * e);
+}
+
+__device__ __forceinline__ DF df_sqrt(DF a)   // a > 0, normal
+{
+    const float r = sqrt_a(a.h);
+    const float e = fmaf(-r, r, a.h) + a.l;
+    return df_norm(r, 0.5f * e * rcp_a(r));
+}
+
 // atan2(y, x) for y >= 0 (an angle in [0, pi]), for the lens angles of the
 // Mandel-Agol terms.  r = min(y, |x|) / max(y, |x|) lies in [0, 1] and
 // atan(r) = r P(r^2) with P of degree 8, fitted to atan(r)/r on [0, 1] by
@@ -272,6 +353,7 @@ __device__ __forceinline__ unsigned long long f2_add(unsigned long long a, unsig
     return d;
 }
 
+template <bool IEEE = false>
 __device__ __forceinline__ void cel2(float kc, float a1, float b1, float srho, float a2, float *r1,
                                      float *r2)
 {
@@ -282,7 +364,7 @@ __device__ __forceinline__ void cel2(float kc, float a1, float b1, float srho, f
     float m = 1.0f, e = kc;
 #pragma unroll 1
     for (int it = 0; it < 10; ++it) {
-        const unsigned long long ip = f2_pack(rcp_a(f2_lo(P)), rcp_a(f2_hi(P)));
+        const unsigned long long ip = f2_pack(rcp_t<IEEE>(f2_lo(P)), rcp_t<IEEE>(f2_hi(P)));
         const unsigned long long F = A;
         A = f2_fma(B, ip, A);
         const unsigned long long G = f2_mul(f2_pack(e, e), ip);
@@ -292,11 +374,11 @@ __device__ __forceinline__ void cel2(float kc, float a1, float b1, float srho, f
         float g = m;
         m = kc + m;
         if (fabsf(g - kc) <= g * 3e-4f) break;
-        kc = 2.0f * sqrt_a(e);
+        kc = 2.0f * sqrt_t<IEEE>(e);
         e = kc * m;
     }
-    *r1 = (0.5f * PT_PI_F) * fmaf(f2_lo(A), m, f2_lo(B)) * rcp_a(m * (m + f2_lo(P)));
-    *r2 = (0.5f * PT_PI_F) * fmaf(f2_hi(A), m, f2_hi(B)) * rcp_a(m * (m + f2_hi(P)));
+    *r1 = (0.5f * PT_PI_F) * fmaf(f2_lo(A), m, f2_lo(B)) * rcp_t<IEEE>(m * (m + f2_lo(P)));
+    *r2 = (0.5f * PT_PI_F) * fmaf(f2_hi(A), m, f2_hi(B)) * rcp_t<IEEE>(m * (m + f2_hi(P)));
 }
 
 // cel2's loop carrying K = cel(kc, 1, 1, 1) and E = cel(kc, 1, 1, kc^2) in place
@@ -374,25 +456,17 @@ __device__ __forceinline__ void cel3(float kc, float srho, float a2, float *K, f
 // With KE, K and E of the general cases' modulus (cases 2, 3, 8, 9: the
 // partial and inside overlaps) come back too, *have_ke = true; other cases
 // leave *have_ke false.
-template <bool KE = false>
-__device__ __forceinline__ void ma_terms(float p, float z, float *le, float *ld, float *ed, float *Kout = nullptr,
-                                         float *Eout = nullptr, bool *have_ke = nullptr)
+// ma_terms_core takes d = z + p - 1 and e1 = 1 - z + p beside p and z, for
+// callers that know the distances to the contacts better than the rounded z
+// does (the nodes of the row tables below); it is for points in transit
+// (e1 > 0, p > 0) that do not cover the star.
+template <bool KE = false, bool IEEE = false>
+__device__ __forceinline__ void ma_terms_core(float p, float z, float d, float e1, float *le, float *ld, float *ed,
+                                              float *Kout = nullptr, float *Eout = nullptr, bool *have_ke = nullptr)
 {
-    if (KE) *have_ke = false;
-    *le = 0.0f;
-    *ld = 0.0f;
-    *ed = 0.0f;
-    if (!(z < 1.0f + p) || !(p > 0.0f)) return;    // out of transit (also PT_ZBEHIND, NaN)
-    if (p >= 1.0f && z <= p - 1.0f) {               // case 11: star covered
-        *le = 1.0f;
-        *ld = 2.0f / 3.0f;
-        *ed = 0.5f;
-        return;
-    }
     const float pi = PT_PI_F;
     float p2 = p * p, z2 = z * z;
-    float d = (z - 1.0f) + p;
-    float oma = (1.0f - z + p) * (1.0f + z - p);
+    float oma = e1 * (1.0f + z - p);
     float bm1 = d * (1.0f + z + p);
     float zmp = z - p;
     float eta2 = 0.5f * p2 * (p2 + 2.0f * z2);
@@ -401,7 +475,7 @@ __device__ __forceinline__ void ma_terms(float p, float z, float *le, float *ld,
     // lens geometry: only the partial (and contact) cases need it
     float le_part = p2, eta1 = eta2;
     if (!inside) {
-        float fa = sqrt_a(oma * bm1);                    // 4 x triangle area (oma, bm1 >= 0)
+        float fa = sqrt_t<IEEE>(oma * bm1);                    // 4 x triangle area (oma, bm1 >= 0)
         float k1 = atan2_pos(fa, 1.0f - p2 + z2);
         float k0 = atan2_pos(fa, p2 + z2 - 1.0f);
         le_part = (p2 * k0 + k1 - 0.5f * fa) * (1.0f / pi);
@@ -441,19 +515,19 @@ __device__ __forceinline__ void ma_terms(float p, float z, float *le, float *ld,
             e_out = eta1;
         }
     } else if (inside) {                             // cases 3, 9: lambda_2
-        kc = sqrt_a(-bm1 * rcp_a(oma));
-        cKp = bm1 * (p2 * p - p2 * z - p * z2 + 2.0f * p + z2 * z - 4.0f * z) * rcp_a(p + z);
+        kc = sqrt_t<IEEE>(-bm1 * rcp_t<IEEE>(oma));
+        cKp = bm1 * (p2 * p - p2 * z - p * z2 + 2.0f * p + z2 * z - 4.0f * z) * rcp_t<IEEE>(p + z);
         cE = oma * (z2 + 7.0f * p2 - 4.0f);
-        srho = (p + z) * rcp_a(fabsf(zmp));
-        cR = (12.0f * z * p) * rcp_a(zmp * (z + p));
-        pref = 2.0f * rcp_a(9.0f * pi * sqrt_a(oma));
+        srho = (p + z) * rcp_t<IEEE>(fabsf(zmp));
+        cR = (12.0f * z * p) * rcp_t<IEEE>(zmp * (z + p));
+        pref = 2.0f * rcp_t<IEEE>(9.0f * pi * sqrt_t<IEEE>(oma));
     } else {                                         // cases 2, 8: lambda_1
-        kc = sqrt_a(bm1 * rcp_a(4.0f * z * p));
+        kc = sqrt_t<IEEE>(bm1 * rcp_t<IEEE>(4.0f * z * p));
         cKp = -bm1 * (6.0f * p2 + 2.0f * p * z - 3.0f);
         cE = 4.0f * p * z * (z2 + 7.0f * p2 - 4.0f);
-        srho = rcp_a(fabsf(zmp));
-        cR = (3.0f * (p + z) * oma) * rcp_a(zmp);
-        pref = rcp_a(9.0f * pi * sqrt_a(p * z));
+        srho = rcp_t<IEEE>(fabsf(zmp));
+        cR = (3.0f * (p + z) * oma) * rcp_t<IEEE>(zmp);
+        pref = rcp_t<IEEE>(9.0f * pi * sqrt_t<IEEE>(p * z));
     }
     float lam = cst;
     if (need_cel) {
@@ -466,7 +540,7 @@ __device__ __forceinline__ void ma_terms(float p, float z, float *le, float *ld,
             *Eout = E;
             *have_ke = true;
         } else {
-            cel2(kc, cKp + cE, fmaf(cE, kc * kc, cKp), srho, cR, &r1, &r2);
+            cel2<IEEE>(kc, cKp + cE, fmaf(cE, kc * kc, cKp), srho, cR, &r1, &r2);
         }
         lam = fmaf(pref, r1 + r2, cst);
     }
@@ -474,6 +548,234 @@ __device__ __forceinline__ void ma_terms(float p, float z, float *le, float *ld,
     *le = inside ? p2 : le_part;
     *ld = lam;
     *ed = e_out;
+}
+
+template <bool KE = false>
+__device__ __forceinline__ void ma_terms(float p, float z, float *le, float *ld, float *ed, float *Kout = nullptr,
+                                         float *Eout = nullptr, bool *have_ke = nullptr)
+{
+    if (KE) *have_ke = false;
+    *le = 0.0f;
+    *ld = 0.0f;
+    *ed = 0.0f;
+    if (!(z < 1.0f + p) || !(p > 0.0f)) return;    // out of transit (also PT_ZBEHIND, NaN)
+    if (p >= 1.0f && z <= p - 1.0f) {               // case 11: star covered
+        *le = 1.0f;
+        *ld = 2.0f / 3.0f;
+        *ed = 0.5f;
+        return;
+    }
+    ma_terms_core<KE>(p, z, (z - 1.0f) + p, 1.0f - z + p, le, ld, ed, Kout, Eout, have_ke);
+}
+
+// ---------------------------------------------------------------------------
+// Row tables: a Mandel-Agol quantity of one radius ratio p as a function of z,
+// as piecewise polynomials good to the rounding of the FP32 terms themselves.
+//
+// Where a kernel evaluates one radius ratio at thousands of separations, the
+// elliptic integrals need not be summed for each of them: between the
+// contacts z = 1 - p and z = 1 + p the terms are analytic in z, and at the
+// contacts they are analytic in the square root of the distance up to
+// w^4 log w terms.  So with
+//   region A, planet inside the disk:  w^2 = (1 - p) - z,
+//   region B, limb, z < 1:             w^2 = z - (1 - p),
+//   region C, limb, z >= 1:            w^2 = (1 + p) - z,
+// and MT_NA, MT_NL, MT_NL equal intervals in w, a degree-5 polynomial per
+// interval is within 1e-9 of the terms (measured in 64 bits over p = 0.001 ..
+// 0.5: 4e-10 at p = 0.05, 7e-10 at 0.3, 8e-10 at 0.5), below the ~1e-8 to
+// 1e-7 of the FP32 evaluation.  A table is 144 evaluations of the exact terms
+// at Chebyshev nodes; a look-up is about 22 instructions against 170 (inside)
+// to 230 (limb) of the terms.
+// With u = w s, interval i covers u in [i - 1/2, i + 1/2] (the first of a
+// region only its upper half), t = u - i, so one FMA with a large constant
+// rounds to the interval and one more gives t.  The scales s keep u below the
+// region's last interval's end by 2e-6, more than the rounding of w.
+// Radius ratios outside [MT_PMIN, MT_PMAX] (where another contact's
+// singularity comes within an interval's width) take the exact terms.
+// Layout of a row: 8 floats per interval, c0..c5 and two unused, so that one
+// address serves a 16-byte and an 8-byte load.  c0 of
+// region C's first interval is set to 0, so a separation at or beyond 1 + p
+// reads exactly 0.
+// ---------------------------------------------------------------------------
+constexpr int MT_NA = 8, MT_NL = 8, MT_N = MT_NA + 2 * MT_NL, MT_Q = 6, MT_NODES = MT_N * MT_Q;
+constexpr int MT_ROW = 8 * MT_N;                    // floats per row
+constexpr float MT_PMIN = 1e-6f, MT_PMAX = 0.5f;
+constexpr float MT_MAGIC = 12582912.0f;             // 1.5 2^23: adding it rounds to an integer
+
+// values at the interval's Chebyshev nodes -> monomial coefficients in t, for
+// a region's first interval (nodes t = (1 + x) / 4) and the others (t = x / 2)
+struct MtMat {
+    float m[2][MT_Q][MT_Q];   // [first ? 0 : 1][coefficient][node]
+};
+constexpr MtMat make_mt()
+{
+    const double x[MT_Q] = {0.96592582628906828675, 0.70710678118654752440,  0.25881904510252076235,
+                            -0.25881904510252076235, -0.70710678118654752440, -0.96592582628906828675};
+    MtMat r{};
+    for (int kind = 0; kind < 2; ++kind) {
+        // T_k(y), y = al t + be, as polynomials in t
+        const double al = kind == 0 ? 4.0 : 2.0, be = kind == 0 ? -1.0 : 0.0;
+        double T[MT_Q][MT_Q] = {};
+        T[0][0] = 1.0;
+        T[1][0] = be;
+        T[1][1] = al;
+        for (int k = 2; k < MT_Q; ++k)
+            for (int c = 0; c < MT_Q; ++c)
+                T[k][c] = 2.0 * be * T[k - 1][c] + (c > 0 ? 2.0 * al * T[k - 1][c - 1] : 0.0) - T[k - 2][c];
+        for (int q = 0; q < MT_Q; ++q) {
+            double tk[MT_Q] = {1.0, x[q]};
+            for (int k = 2; k < MT_Q; ++k) tk[k] = 2.0 * x[q] * tk[k - 1] - tk[k - 2];
+            for (int c = 0; c < MT_Q; ++c) {
+                double v = 0.0;
+                for (int k = 0; k < MT_Q; ++k) v += (k == 0 ? 1.0 : 2.0) / MT_Q * tk[k] * T[k][c];
+                r.m[kind][c][q] = (float)v;
+            }
+        }
+    }
+    return r;
+}
+static __constant__ MtMat c_mt = make_mt();
+
+__device__ __forceinline__ bool mt_valid(float p) { return p >= MT_PMIN && p <= MT_PMAX; }
+
+// scales of regions A and B, C
+__device__ __forceinline__ void mt_scales(float p, float *sA, float *sL)
+{
+    *sA = ((float)MT_NA - 0.5f) * (1.0f - 2e-6f) / sqrtf(1.0f - p);
+    *sL = ((float)MT_NL - 0.5f) * (1.0f - 2e-6f) / sqrtf(p);
+}
+
+// Coefficient c of interval i from the interval's node values f.  The rows of
+// the matrix alternate in sign and reach 10^3, so they are applied to the
+// differences from one node (the constant goes to c0 alone): applied to the
+// values, their FP32 rounding would show (3e-6 at p = 0.5).
+__device__ __forceinline__ float mt_coef(int i, int c, const float *f)
+{
+    const int kind = (i == 0 || i == MT_NA || i == MT_NA + MT_NL) ? 0 : 1;   // a region's first interval
+    float a = 0.0f;
+#pragma unroll
+    for (int q = 0; q < MT_Q; ++q) a = fmaf(c_mt.m[kind][c][q], f[q] - f[2], a);
+    if (c != 0) return a;
+    return i == MT_NA + MT_NL ? 0.0f : a + f[2];
+}
+
+// lambda_2 + 2/3 Theta(p - z) with the planet wholly inside the disk, at
+// z = 1 - p - w^2, in double-float arithmetic.  The brace's two integrals are
+// of order one and cancel to the order of p^2: in FP32 that leaves 2e-8 to
+// 4e-8, which averages out over the rounding of many separations but would be
+// frozen into the rows of a table.  Formulas as in ma_terms_core (cases 3, 9)
+// with a = (z - p)^2 and the distances as polynomials in p and w^2.
+__device__ __forceinline__ float mt_lambda_inside(float p, float w)
+{
+    const float w2h = w * w;
+    const DF W = DF{w2h, fmaf(w, w, -w2h)};                 // w^2
+    const DF one = DF{1.0f, 0.0f}, P = DF{p, 0.0f};
+    const DF zpp = df_add(one, df_neg(W));                  // z + p = 1 - w^2
+    const DF z = df_add(zpp, DF{-p, 0.0f});
+    const DF zmp = df_add(z, DF{-p, 0.0f});
+    const DF oma = df_mul(df_add(DF{2.0f * p, 0.0f}, W), df_add(one, zmp));   // (1 - z + p)(1 + z - p)
+    const DF bm1 = df_neg(df_mul(W, df_add(one, zpp)));     // (z + p - 1)(z + p + 1)
+    const DF izpp = df_rcp(zpp), izmp = df_rcp(zmp), ioma = df_rcp(oma);
+    const DF kc2 = df_neg(df_mul(bm1, ioma));
+    DF kc = df_sqrt(kc2);
+    // cK' = (b - 1) (a + (2p - 4z)/(z + p)), cE = (1 - a)(z^2 + 7 p^2 - 4)
+    const DF cK = df_mul(bm1, df_mad(df_add(DF{2.0f * p, 0.0f}, df_scale(-4.0f, z)), izpp, df_mul(zmp, zmp)));
+    const DF p2 = df_mul(P, P);
+    const DF cE = df_mul(oma, df_add(df_mad(z, z, df_mul(DF{7.0f, 0.0f}, p2)), DF{-4.0f, 0.0f}));
+    const float sg = zmp.h < 0.0f ? -1.0f : 1.0f;
+    DF A1 = df_add(cK, cE), B1 = df_mad(cE, kc2, cK), P1 = one;
+    DF A2 = df_mul(df_mul(DF{12.0f, 0.0f}, df_mul(z, P)), df_mul(izmp, izpp)), B2 = DF{0.0f, 0.0f};
+    DF P2 = df_mul(zpp, df_scale(sg, izmp));
+    DF m = one, e = kc;
+#pragma unroll 1
+    for (int it = 0; it < 10; ++it) {
+        DF ip = df_rcp(P1);
+        DF f = A1, g = df_mul(e, ip);
+        A1 = df_mad(B1, ip, A1);
+        B1 = df_scale(2.0f, df_mad(f, g, B1));
+        P1 = df_add(P1, g);
+        ip = df_rcp(P2);
+        f = A2;
+        g = df_mul(e, ip);
+        A2 = df_mad(B2, ip, A2);
+        B2 = df_scale(2.0f, df_mad(f, g, B2));
+        P2 = df_add(P2, g);
+        const float mh = m.h;
+        m = df_add(kc, m);
+        if (fabsf(mh - kc.h) <= mh * 1e-4f) break;   // quadratic convergence leaves ~1e-9
+        kc = df_scale(2.0f, df_sqrt(e));
+        e = df_mul(kc, m);
+    }
+    const DF r1 = df_mul(df_mad(A1, m, B1), df_rcp(df_mul(m, df_add(m, P1))));
+    const DF r2 = df_mul(df_mad(A2, m, B2), df_rcp(df_mul(m, df_add(m, P2))));
+    // pref (pi/2) = 1 / (9 sqrt(1 - a))
+    const DF lam = df_mul(df_add(r1, r2), df_rcp(df_mul(DF{9.0f, 0.0f}, df_sqrt(oma))));
+    return zmp.h < 0.0f ? df_add(lam, DF{0.666666687f, -1.98682151e-08f}).h : lam.h;
+}
+
+// The exact terms at node q of interval i, with the distances to the contacts
+// formed from w (not from the rounded z).
+__device__ __forceinline__ void mt_node(float p, int i, int q, float *le, float *ld, float *ed)
+{
+    const int q3 = q < 3 ? q : 5 - q;
+    const float xa = q3 == 0 ? 0.96592582629f : (q3 == 1 ? 0.70710678119f : 0.25881904510f);
+    const float x = q < 3 ? xa : -xa;
+    float sA, sL;
+    mt_scales(p, &sA, &sL);
+    const int reg = i < MT_NA ? 0 : (i < MT_NA + MT_NL ? 1 : 2);
+    const int il = i - (reg == 0 ? 0 : (reg == 1 ? MT_NA : MT_NA + MT_NL));
+    const float u = il == 0 ? 0.25f * (1.0f + x) : (float)il + 0.5f * x;
+    const float w = u / (reg == 0 ? sA : sL);
+    const float w2 = w * w;
+    const float d = reg == 0 ? -w2 : (reg == 1 ? w2 : 2.0f * p - w2);
+    const float e1 = reg == 0 ? 2.0f * p + w2 : (reg == 1 ? 2.0f * p - w2 : w2);
+    const float z = reg == 2 ? (1.0f + p) - w2 : (1.0f - p) + d;
+    ma_terms_core<false, true>(p, z, d, e1, le, ld, ed);
+    // (z = p, where the second integral's parameters are infinite, keeps the separate case)
+    if (reg == 0 && fabsf(z - p) > 1e-5f) *ld = mt_lambda_inside(p, w);
+}
+
+// Interval and offset of separation z.  zm1 = z - 1; off_limb is the constant
+// of region B (z < 1) or C (z >= 1, or NaN), which depends on z alone.
+// |z - (1 - p)| and (1 + p) - z: the smaller one is w^2 in every region
+// (p <= 1/2).  z >= 1 + p gives w = 0 of region C, where the polynomial is 0.
+__device__ __forceinline__ float mt_off_limb(float zm1)
+{
+    return zm1 < 0.0f ? MT_MAGIC + (float)MT_NA : MT_MAGIC + (float)(MT_NA + MT_NL);
+}
+
+// The bits of the rounded w s: MT_BITS0 plus the interval.  (1 + p) - z
+// saturated to [0, 1] costs nothing; where it saturates at 1, |z - (1 - p)| is
+// below 1 and the smaller.
+constexpr unsigned MT_BITS0 = 0x4B400000u;
+
+__device__ __forceinline__ unsigned mt_find(float p, float sA, float sL, float zm1, float off_limb, float *t)
+{
+    const float d = zm1 + p;
+    const float w = sqrt_a(fminf(fabsf(d), __saturatef(p - zm1)));
+    const bool in_a = d < 0.0f;
+    const float s = in_a ? sA : sL;
+    const float off = in_a ? MT_MAGIC : off_limb;
+    const float b = fmaf(w, s, off);
+    *t = fmaf(w, s, off - b);
+    return __float_as_uint(b);
+}
+
+// The polynomial of the row at shared-memory address row (bytes) - 32 MT_BITS0
+// (mt_base of the row): the interval's bits, shifted, are added as they are.
+__device__ __forceinline__ unsigned mt_base(const float *row)
+{
+    return (unsigned)__cvta_generic_to_shared(row) - 32u * MT_BITS0;
+}
+
+__device__ __forceinline__ float mt_eval(unsigned base, unsigned bits, float t)
+{
+    const unsigned at = base + 32u * bits;
+    float4 c;
+    float2 g;
+    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c.x), "=f"(c.y), "=f"(c.z), "=f"(c.w) : "r"(at));
+    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(g.x), "=f"(g.y) : "r"(at + 16u));
+    return fmaf(fmaf(fmaf(fmaf(fmaf(g.y, t, g.x), t, c.w), t, c.z), t, c.y), t, c.x);
 }
 
 // Bilinear interpolation of the tabulated Mandel-Agol terms (Sec. 2.2.3):

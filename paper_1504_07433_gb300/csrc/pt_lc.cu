@@ -32,7 +32,12 @@
 #include "../../include/pt.h"
 #include "pt_device.cuh"
 
+using pt::DF;
 using pt::GeomRec;
+using pt::df_add;
+using pt::df_mad;
+using pt::df_mul;
+using pt::df_of;
 
 namespace {
 
@@ -343,55 +348,6 @@ struct GimArgs {
     int ppi;              // pairs per work item (GS_THREADS or MA_PPI)
     int *n_bad;
 };
-
-// Double-float arithmetic for the table recursion: a value is the unevaluated
-// sum h + l of two floats (about 48 significant bits).  Sums and products
-// carry their rounding errors exactly (Knuth's two-sum; the FMA form of
-// Dekker's product).  GB300's FP64 rate is a small fraction of its FP32
-// rate, so a chain of FP64 operations would dominate the table work.
-struct DF {
-    float h, l;
-};
-
-__device__ __forceinline__ DF df_of(double v)
-{
-    float h = (float)v;
-    return DF{h, (float)(v - (double)h)};
-}
-
-__device__ __forceinline__ DF df_norm(float s, float e)   // |s| >= |e|
-{
-    float h = s + e;
-    return DF{h, e - (h - s)};
-}
-
-__device__ __forceinline__ DF df_add(DF a, DF b)
-{
-    float s = a.h + b.h;
-    float bb = s - a.h;
-    float e = (a.h - (s - bb)) + (b.h - bb);
-    return df_norm(s, e + (a.l + b.l));
-}
-
-__device__ __forceinline__ DF df_mul(DF a, DF b)
-{
-    float p = a.h * b.h;
-    float e = fmaf(a.h, b.h, -p);
-    e = fmaf(a.h, b.l, fmaf(a.l, b.h, e));
-    return df_norm(p, e);
-}
-
-// a b + c with one two-sum: the product's rounding error (fmaf), the two-sum
-// error of p + c_h, the cross terms and c_l go into the low part
-__device__ __forceinline__ DF df_mad(DF a, DF b, DF c)
-{
-    const float p = a.h * b.h;
-    const float e = fmaf(a.h, b.h, -p);
-    const float s = p + c.h;
-    const float bb = s - p;
-    const float err = (p - (s - bb)) + (c.h - bb);
-    return df_norm(s, fmaf(a.h, b.l, fmaf(a.l, b.h, c.l)) + (e + err));
-}
 
 // Gimenez per-geometry table for Clenshaw's summation: entry (n, j) packs the
 // z-recursion coefficients r1_j, r2_j, r3_{j+1} of G_j(nu+2, 1; x) with
