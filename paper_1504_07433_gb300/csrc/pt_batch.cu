@@ -131,8 +131,9 @@ __global__ void __launch_bounds__(PREP) batch_prep_kernel(PrepArgs s)
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     int blk = blockIdx.x;
     if (blk < s.n_gblocks) {
-        const int v = blk * PREP + tid;
-        if (v >= s.orb.n_v) return;
+        // one warp per CTA: the records' FP64 operations share one slow pipe per SM
+        const int v = blk * 32 + tid;
+        if (tid >= 32 || v >= s.orb.n_v) return;
         // the geometry's k: the largest passband k (its window covers every
         // passband), or in k_hat mode the mean, the only k evaluated
         float kmax = 0.0f, ksum = 0.0f;
@@ -287,7 +288,7 @@ __device__ __noinline__ void exact_row(const BatchArgs &A, const GeomRec &g, int
             const float dt = pt::reduce_time(ts.x, ts.y, g);
             inw = dt >= g.win_lo && dt <= g.win_hi;
             if (inw) {
-                float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
+                float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
                 for (int s = 0; s < A.n_ss; ++s) {
                     bool bad = false;
                     const float off = A.t_exp * (((float)s + 0.5f) * inv_ss - 0.5f);
@@ -520,7 +521,7 @@ __global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(BatchArgs A)
 #pragma unroll
                         for (int j = 0; j < BG; ++j) D[MODE != M_KHAT ? j : 0] = 0.0f;
                     }
-                    float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
+                    float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
 #pragma unroll 1
                     for (int s = 0; s < (inw ? A.n_ss : 0); ++s) {
                         bool bad = false;
@@ -710,7 +711,7 @@ int enqueue(pt_batch_plan_s &p, cudaStream_t s)
     sa.wt = d.wt;
     sa.n_tiles = p.n_tiles;
     sa.rows = p.d_rows;
-    sa.n_gblocks = (d.orb.n_v + PREP - 1) / PREP;
+    sa.n_gblocks = (d.orb.n_v + 31) / 32;
     sa.n_tblocks = (p.n_tiles + PREP_TILES - 1) / PREP_TILES;
     const long long per = (long long)(PREP / 32) * PREP_BASE;
     sa.n_bblocks = d.ssr ? (int)(((long long)d.n_b * p.n_tiles + per - 1) / per) : 0;

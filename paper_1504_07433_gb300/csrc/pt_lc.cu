@@ -27,10 +27,12 @@
 #include <stdio.h>
 #include <string.h>
 
+#include <algorithm>
 #include <mutex>
 
 #include "../../include/pt.h"
 #include "pt_device.cuh"
+#include "pt_rows.cuh"
 
 using pt::DF;
 using pt::GeomRec;
@@ -114,6 +116,117 @@ __global__ void setup_kernel(SetupArgs s)
             double t = s.t[i];
             float h = (float)t;
             s.tsplit[i] = make_float2(h, (float)(t - (double)h));
+        }
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Preparation of a light-curve call from row tables (pt_rows.cuh): the
+// geometry records, the time split and the Mandel-Agol rows, in one launch
+// (the records' FP64 latency and the tables' elliptic integrals run side by
+// side).  Row CTAs take ROW_GEOM geometries: one node of a geometry's table
+// per thread (the region inside the disk, in double-float arithmetic, on the
+// first warps), then per row one coefficient per thread.
+// ---------------------------------------------------------------------------
+constexpr int ROW_GEOM = 2;
+constexpr int ROW_THREADS = ROW_GEOM * pt::MT_NODES;
+
+struct RowPrep {
+    SetupArgs s;
+    int n_tblocks;
+    float *rows;      // [n_geom][nr][row_len]
+    int row_len, nr, terms, n_bpg;
+    const float *ld;
+    // R_INTERP: the caller's table
+    const float4 *mtab;
+    int mn_k, mn_z;
+    float mk_lo, mk_hi, minv_dk;
+};
+
+// weights of row r of a geometry: a passband's depth, or one of the terms
+__device__ __forceinline__ float3 row_weights(const RowPrep &P, int g, int r)
+{
+    if (P.terms) return make_float3(r == 0 ? 1.0f : 0.0f, r == 1 ? 1.0f : 0.0f, r == 2 ? 1.0f : 0.0f);
+    float3 w;
+    const float *ld = P.ld + 2 * ((size_t)g * P.n_bpg + r);
+    pt::ma_weights(ld[0], ld[1], &w.x, &w.y, &w.z);
+    return w;
+}
+
+template <int MODEL>
+__global__ void __launch_bounds__(ROW_THREADS) row_prep_kernel(RowPrep P)
+{
+    __shared__ float3 sF[ROW_GEOM][pt::MT_N * pt::MT_Q];
+    const int tid = threadIdx.x;
+    const SetupArgs &s = P.s;
+    int blk = blockIdx.x;
+    if (blk < s.n_gblocks) {
+        // one warp per CTA: the records' FP64 operations share one slow pipe per SM
+        const int g = blk * 32 + tid;
+        if (tid < 32 && g < s.n_geom) make_geom(s, g, &s.rec[g]);
+        return;
+    }
+    blk -= s.n_gblocks;
+    if (blk < P.n_tblocks) {
+        const int i = blk * ROW_THREADS + tid;
+        if (i < s.n_t) {
+            const double t = s.t[i];
+            const float h = (float)t;
+            s.tsplit[i] = make_float2(h, (float)(t - (double)h));
+        }
+        return;
+    }
+    blk -= P.n_tblocks;
+    if (MODEL == rows::R_INTERP) {
+        // each row: the table's nodes at the geometry's k, combined
+        const long long at = (long long)blk * ROW_THREADS + tid;
+        const long long row = at / P.row_len;
+        const int j = (int)(at - row * P.row_len);
+        if (row >= (long long)s.n_geom * P.nr) return;
+        const int g = (int)(row / P.nr), r = (int)(row - (long long)g * P.nr);
+        float v = 0.0f;
+        if (j < P.mn_z) {
+            const float fk = (fminf(fmaxf(s.k[g], P.mk_lo), P.mk_hi) - P.mk_lo) * P.minv_dk;
+            const int ik = min((int)fk, P.mn_k - 2);
+            const float wk = fk - (float)ik;
+            const float4 a = __ldg(P.mtab + (size_t)ik * P.mn_z + j), b = __ldg(P.mtab + (size_t)(ik + 1) * P.mn_z + j);
+            const float3 w = row_weights(P, g, r);
+            v = w.x * fmaf(wk, b.x - a.x, a.x) + w.y * fmaf(wk, b.y - a.y, a.y) + w.z * fmaf(wk, b.z - a.z, a.z);
+        }
+        P.rows[at] = v;
+        return;
+    }
+    const int first = blk * ROW_GEOM;
+    constexpr int NODES_A = pt::MT_NA * pt::MT_Q, NODES_L = pt::MT_NODES - NODES_A;
+    {
+        const bool in_a = tid < ROW_GEOM * NODES_A;
+        const int u = in_a ? tid : tid - ROW_GEOM * NODES_A;
+        const int gl = in_a ? u / NODES_A : u / NODES_L;
+        const int node = in_a ? u - gl * NODES_A : NODES_A + u - gl * NODES_L;
+        if (first + gl < s.n_geom) {
+            const float p = s.k[first + gl];
+            if (pt::mt_valid(p)) {   // the others take the exact terms per point
+                float3 f;
+                pt::mt_node(p, node / pt::MT_Q, node % pt::MT_Q, &f.x, &f.y, &f.z);
+                sF[gl][node] = f;
+            }
+        }
+    }
+    __syncthreads();
+    {
+        const int c = tid / (ROW_GEOM * pt::MT_N), u = tid - c * (ROW_GEOM * pt::MT_N);
+        const int gl = u / pt::MT_N, i = u - gl * pt::MT_N, g = first + gl;
+        if (g < s.n_geom && pt::mt_valid(s.k[g])) {
+            for (int r = 0; r < P.nr; ++r) {
+                const float3 w = row_weights(P, g, r);
+                float f[pt::MT_Q];
+#pragma unroll
+                for (int q = 0; q < pt::MT_Q; ++q) {
+                    const float3 v = sF[gl][i * pt::MT_Q + q];
+                    f[q] = w.x * v.x + w.y * v.y + w.z * v.z;
+                }
+                P.rows[((size_t)g * P.nr + r) * P.row_len + 8 * i + c] = pt::mt_coef(i, c, f);
+            }
         }
     }
 }
@@ -1037,7 +1150,7 @@ __global__ void __launch_bounds__(GS_THREADS, 5) gim_cheb_kernel(GimArgs A, cons
         float al[NP1];   // alpha sums over the supersamples
 #pragma unroll
         for (int n = 0; n < NP1; ++n) al[n] = 0.0f;
-        float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
+        float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
 #pragma unroll 1
         for (int sb0 = 0; sb0 < nss; sb0 += ssb) {
             // 1. in-transit supersamples of this pair, in order
@@ -1278,7 +1391,7 @@ __global__ void __launch_bounds__(GS_THREADS) gim_zi_kernel(GimArgs A, const flo
             float dt = pt::reduce_time(ts.x, ts.y, srec);
             const float kk = srec.k;
             const ZiGrid G = zi_grid(kk, n_in, n_edge);
-            float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
+            float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
 #pragma unroll 1
             for (int s = 0; s < nss; ++s) {
                 bool bad = false;
@@ -1327,177 +1440,6 @@ __global__ void __launch_bounds__(GS_THREADS) gim_zi_kernel(GimArgs A, const flo
 }
 
 size_t gim_zi_smem(int N, int nz) { return (size_t)(N + 1) * (nz + GS_THREADS) * sizeof(float); }
-
-// ---------------------------------------------------------------------------
-// Mandel-Agol over the window kernel's pair lists: persistent CTAs take work
-// items of MA_PPI listed (time, geometry) pairs.  An item runs in batches of
-// up to MA_SSB supersamples:
-//  1. each thread (one pair) computes z at the batch's supersamples and keeps
-//     the in-transit ones (z < 1 + k) in order; a scan over the CTA places
-//     every pair's z in one dense list, the supersamples with the planet
-//     wholly inside the stellar disk (z <= 1 - k) first and those on the limb
-//     after them, and records where each of its entries went;
-//  2. each thread evaluates lambda_e, lambda_d + 2/3 Theta and eta_d at
-//     entries tid, tid + MA_PPI, ... of the list, whatever pairs they belong
-//     to: no lane idles on an out-of-transit supersample, and a warp mostly
-//     takes one branch of the case table (the limb cases add the lens
-//     geometry).  The terms go to shared memory;
-//  3. each thread adds its own pair's terms in supersample order (the others
-//     are zero), so the sums do not depend on where the terms were computed.
-// Then the passband fluxes (Eq. ma_model).
-// ---------------------------------------------------------------------------
-constexpr int MA_PPI = 128;   // pairs per work item (= threads per CTA)
-constexpr int MA_SSB = 16;    // supersamples per batch
-
-__global__ void __launch_bounds__(MA_PPI, 8) ma_pairs_kernel(GimArgs A)
-{
-    __shared__ GeomRec srec;
-    __shared__ int sitem, sgeom, sfirst, scount, sbad;
-    __shared__ int swarp[MA_PPI / 32];
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int nss = A.n_ss;
-    const int ssb = min(nss, MA_SSB);
-    extern __shared__ __align__(16) unsigned char msm[];
-    float *sT = reinterpret_cast<float *>(msm);                     // [3][ssb MA_PPI] terms of the list
-    float *sz = sT + 3 * ssb * MA_PPI;                              // [ssb MA_PPI] the dense list of z
-    float *szp = sz + ssb * MA_PPI;                                 // [ssb][MA_PPI] each pair's z, in order
-    unsigned short *spos = reinterpret_cast<unsigned short *>(szp + ssb * MA_PPI);   // [ssb][MA_PPI] list slots
-    const int total = A.pref[A.n_geom];
-    const float inv_nss = 1.0f / (float)nss;
-    int nbad = 0;
-    int staged = -1;
-    if (tid == 0) sbad = 0;
-#pragma unroll 1
-    for (;;) {
-        if (warp == 0) {
-            int it = 0;
-            if (lane == 0) it = atomicAdd(A.ctr, 1);
-            it = __shfl_sync(0xffffffffu, it, 0);
-            if (it < total) {
-                const int pos = item_geometry(A.pref, A.n_geom, it, lane);
-                if (lane == 0) {
-                    const int g = A.gord[pos];
-                    sgeom = g;
-                    sfirst = A.pref[pos];
-                    scount = A.cnt[g];
-                }
-            }
-            if (lane == 0) sitem = it;
-        }
-        __syncthreads();
-        const int it = sitem;
-        const int g = sgeom;
-        if (it >= total) break;   // uniform over the CTA
-        if (g != staged) {
-            if (tid < 6) reinterpret_cast<float4 *>(&srec)[tid] = reinterpret_cast<const float4 *>(&A.rec[g])[tid];
-            staged = g;
-        }
-        __syncthreads();
-        const int i = (it - sfirst) * MA_PPI + tid;
-        const bool own = i < scount;
-        const int t = own ? A.list[(size_t)g * A.n_t + i] : 0;
-        float dt = 0.0f;
-        if (own) {
-            const float2 ts = A.tsplit[t];
-            dt = pt::reduce_time(ts.x, ts.y, srec);
-        }
-        const float kk = srec.k;
-        float le = 0.0f, ld = 0.0f, ed = 0.0f;
-        float warm[3] = {__int_as_float(0x7fffffff), 0.0f, 0.0f};   // Kepler warm start (none yet)
-#pragma unroll 1
-        for (int sb0 = 0; sb0 < nss; sb0 += ssb) {
-            // 1. in-transit supersamples of this pair, in order (the terms of
-            //    the others are zero: ma_terms returns zeros there), and which
-            //    of them have the planet wholly inside the disk
-            int c = 0, n_in = 0;
-            unsigned limb = 0u;
-            if (own) {
-                const int s1 = min(nss, sb0 + ssb);
-#pragma unroll 1
-                for (int s = sb0; s < s1; ++s) {
-                    bool bad = false;
-                    const float z = pt::orbit_z<true, true>(srec, dt + ss_offset(A.t_exp, s, inv_nss), A.max_iter, &bad, warm);
-                    if (bad) ++nbad;
-                    if (z < 1.0f + kk && kk > 0.0f) {
-                        szp[c * MA_PPI + tid] = z;
-                        if ((z - 1.0f) + kk > 0.0f) limb |= 1u << c;
-                        else ++n_in;
-                        ++c;
-                    }
-                }
-            }
-            // both classes' counts in one scan: inside in the low 16 bits,
-            // limb in the high ones (at most MA_SSB MA_PPI = 2048 each)
-            const int v = n_in | ((c - n_in) << 16);
-            int incl = v;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int y = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += y;
-            }
-            if (lane == 31) swarp[warp] = incl;
-            __syncthreads();
-            int base = 0, all = 0;
-#pragma unroll
-            for (int w = 0; w < MA_PPI / 32; ++w) {
-                base += (w < warp) ? swarp[w] : 0;
-                all += swarp[w];
-            }
-            const int excl = base + incl - v;
-            const int n_inside = all & 0xffff;
-            int p_in = excl & 0xffff, p_limb = n_inside + (excl >> 16);
-            for (int j = 0; j < c; ++j) {
-                const int pos = ((limb >> j) & 1u) ? p_limb++ : p_in++;
-                sz[pos] = szp[j * MA_PPI + tid];
-                spos[j * MA_PPI + tid] = (unsigned short)pos;
-            }
-            const int n_e = n_inside + (all >> 16);
-            __syncthreads();
-            // 2. the terms of every entry of the list
-            const int stride = ssb * MA_PPI;
-#pragma unroll 1
-            for (int e = tid; e < n_e; e += MA_PPI) {
-                float a0, a1, a2;
-                pt::ma_terms(kk, sz[e], &a0, &a1, &a2);
-                sT[e] = a0;
-                sT[stride + e] = a1;
-                sT[2 * stride + e] = a2;
-            }
-            __syncthreads();
-            // 3. this pair's terms, in supersample order
-            for (int j = 0; j < c; ++j) {
-                const int pos = spos[j * MA_PPI + tid];
-                le += sT[pos];
-                ld += sT[stride + pos];
-                ed += sT[2 * stride + pos];
-            }
-            __syncthreads();
-        }
-        if (own) {
-            le *= inv_nss;
-            ld *= inv_nss;
-            ed *= inv_nss;
-#pragma unroll 1
-            for (int bb = 0; bb < A.n_bpg; ++bb) {
-                size_t row = (size_t)g * A.n_bpg + bb;
-                float we, wd, wn;
-                pt::ma_weights(A.ld[row * 2], A.ld[row * 2 + 1], &we, &wd, &wn);
-                A.flux[row * A.n_t + t] = 1.0f - (we * le + wd * ld + wn * ed);
-            }
-        }
-    }
-    if (nbad) atomicAdd(&sbad, nbad);
-    __syncthreads();
-    if (tid == 0 && sbad && A.n_bad) atomicAdd(A.n_bad, sbad);
-}
-
-// the list's terms, the list, each pair's z and the list slots
-size_t ma_pairs_smem(int n_ss)
-{
-    const size_t n = (size_t)(n_ss < MA_SSB ? n_ss : MA_SSB) * MA_PPI;
-    return n * (5 * sizeof(float) + sizeof(unsigned short));
-}
 
 __global__ void ssr_reduce_kernel(const float *part, int rows, int n_tiles, float *ssr)
 {
@@ -1772,25 +1714,118 @@ WorkLayout work_layout(int n_t, int n_v, int n_b, int k_per_band, int NP1, int n
     return L;
 }
 
-// pt_ma_quad runs over the window kernel's pair lists (the list layout: no
-// Gimenez tables), except for a few geometries: there the tile kernel's two
-// launches (set-up, evaluation) beat the list path's four (one light curve
-// of 1,000 points: 12.3 against 16.4 us per CUDA-graph replay; the list path
-// wins from about 16 geometries).  The tile kernel also serves the
-// interpolated and the allocation-free variants.
-constexpr bool MA_LIST = true;
-constexpr int MA_TILE_MAX_GEOM = 4;
+// Light curves from row tables: records, time split, rows, residual partials
+// and, when many passbands share a geometry and only residuals are wanted, a
+// flux scratch.
+struct RowLayout {
+    size_t rec, tsplit, rows, part, fscr, total;
+};
 
-bool ma_small(const pt_orbit *orb, int n_b, int k_per_band)
+// rows of a geometry: one per passband, or the model's terms when more
+// passbands share it
+bool row_terms(int n_bpg) { return n_bpg > rows::MAX_BAND_ROWS; }
+int rows_per_geom(int n_bpg, int n_terms) { return row_terms(n_bpg) ? n_terms : n_bpg; }
+
+RowLayout row_layout(int n_t, int n_v, int n_b, int k_per_band, int n_terms, size_t row_len)
 {
-    if (!orb || orb->n_v < 0 || n_b < 1) return false;
-    const long long n_geom = k_per_band ? (long long)orb->n_v * n_b : orb->n_v;
-    return n_geom <= MA_TILE_MAX_GEOM;
+    const size_t n_geom = k_per_band ? (size_t)n_v * n_b : (size_t)n_v;
+    const int n_bpg = k_per_band ? 1 : n_b;
+    const size_t n_tiles = ((size_t)n_t + TT - 1) / TT;
+    RowLayout L;
+    size_t off = 0;
+    L.rec = off;
+    off += align256(n_geom * sizeof(GeomRec));
+    L.tsplit = off;
+    off += align256((size_t)n_t * sizeof(float2));
+    L.rows = off;
+    off += align256(n_geom * rows_per_geom(n_bpg, n_terms) * row_len * sizeof(float));
+    L.part = off;   // per tile, or per chunk of a flux row
+    off += align256((size_t)n_v * n_b * n_tiles * sizeof(float));
+    L.fscr = off;
+    if (row_terms(n_bpg)) off += align256((size_t)n_v * n_b * n_t * sizeof(float));
+    L.total = off;
+    return L;
 }
 
-size_t ma_list_work_bytes(int n_t, int n_v, int n_b, int k_per_band)
+// Tables pay from this many points (times x supersamples) per geometry: a
+// Mandel-Agol row costs 144 evaluations of the terms, and only the in-window
+// points read it.
+constexpr long long ROWS_MIN_POINTS = 512;
+
+// Tile of the row kernel: geometries x blocks of 256 times.  As many
+// geometries as 48 KB of rows hold (so that four CTAs fit an SM), the rest of
+// the 32 bits in blocks of times (which spreads the staging of the rows over
+// more pairs); then smaller tiles until there are four CTAs per SM.
+int launch_rows(int model, rows::Args &A, int n_sm, cudaStream_t s)
 {
-    return work_layout(n_t, n_v, n_b, k_per_band, 1, 0).total;
+    const size_t row_bytes = (size_t)A.nr * A.row_len * sizeof(float);
+    const bool staged = row_bytes <= 96 * 1024;
+    // residuals keep a value per pair and passband: fewer pairs per tile then
+    const int bits = A.ssr_part ? (A.nr <= 2 ? 16 : A.nr <= 4 ? 8 : 4) : rows::MAX_BITS;
+    int vt = 1, log_kt = 0;
+    while (vt < bits && vt < A.n_geom && (!staged || 2 * vt * row_bytes <= 48 * 1024)) vt *= 2;
+    while ((vt << log_kt) < bits && (rows::TB << log_kt) < A.n_t) ++log_kt;
+    auto ctas = [&](int v, int lk) {
+        return ((long long)A.n_t + (rows::TB << lk) - 1) / (rows::TB << lk) * ((A.n_geom + v - 1) / v);
+    };
+    while (log_kt > 0 && ctas(vt, log_kt) < 4LL * n_sm) --log_kt;
+    while (vt > 1 && ctas(vt, log_kt) < 4LL * n_sm) vt /= 2;
+    A.log_vt = 0;
+    while ((1 << A.log_vt) < vt) ++A.log_vt;
+    A.log_kt = log_kt;
+    A.flux_vec = A.flux && A.n_t % 4 == 0 && ((uintptr_t)A.flux & 15u) == 0;
+    A.n_tiles = (A.n_t + (rows::TB << log_kt) - 1) / (rows::TB << log_kt);
+    const int smem = rows::smem_layout(vt, log_kt, A.nr, A.row_len, staged, A.ssr_part ? A.nr : 0).total;
+    const bool one = A.nr == 1;
+    void (*fn)(rows::Args) = nullptr;
+#define PT_ROWS_FN(M)                                                                                               \
+    fn = staged ? (one ? rows::lc_rows_kernel<M, 1, true> : rows::lc_rows_kernel<M, 4, true>)                       \
+                : rows::lc_rows_kernel<M, 4, false>
+    if (model == rows::R_MA) fn = one ? rows::lc_rows_kernel<rows::R_MA, 1, true> : rows::lc_rows_kernel<rows::R_MA, 4, true>;
+    else PT_ROWS_FN(rows::R_INTERP);
+#undef PT_ROWS_FN
+    if (smem > 40 * 1024) {   // beyond the default limit less the static arrays
+        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+        if (e != cudaSuccess) return set_cuda_error(e, "lc_rows_kernel smem attribute");
+    }
+    // geometries along x, time tiles along y, in as many launches as y takes
+    for (A.tile0 = 0; A.tile0 < A.n_tiles; A.tile0 += 65535) {
+        const dim3 grid((unsigned)((A.n_geom + vt - 1) / vt), (unsigned)std::min(65535, A.n_tiles - A.tile0));
+        fn<<<grid, rows::TB, smem, s>>>(A);
+        const int st = check_launch("lc_rows_kernel");
+        if (st) return st;
+    }
+    return PT_OK;
+}
+
+int sm_count(int *n_sm)
+{
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(n_sm, cudaDevAttrMultiProcessorCount, dev);
+    return e == cudaSuccess ? PT_OK : set_cuda_error(e, "SM count");
+}
+
+// pt_ma_quad and pt_ma_quad_interp run from row tables, except for a few
+// geometries (there the tile kernel's two launches, without tables, are as
+// fast) and for too few points per geometry.  The tile kernel also serves the
+// allocation-free variant, whose scratch must stay small.
+constexpr int MA_TILE_MAX_GEOM = 4;
+
+bool ma_use_rows(int n_t, int n_v, int n_b, int k_per_band, int n_ss)
+{
+    const long long n_geom = k_per_band ? (long long)n_v * n_b : n_v;
+    return n_geom > MA_TILE_MAX_GEOM && (long long)n_t * n_ss >= ROWS_MIN_POINTS;
+}
+
+// Rows of a caller's table: staged whole, so short ones only, and no longer
+// than a light curve (a row is built node by node).
+constexpr int INTERP_ROW_MAX = 2048;
+size_t interp_row_len(int n_z) { return ((size_t)n_z + 3) & ~(size_t)3; }
+size_t row_len_max(int n_t)
+{
+    const size_t m = interp_row_len(n_t < INTERP_ROW_MAX ? n_t : INTERP_ROW_MAX);
+    return m > (size_t)pt::MT_ROW ? m : (size_t)pt::MT_ROW;
 }
 
 }  // namespace
@@ -2131,8 +2166,33 @@ static int lc_common_check(const double *t, int n_t, const pt_orbit *orb, const 
 size_t pt_ma_quad_work_bytes(int n_t, int n_v, int n_b, int k_per_band)
 {
     if (n_t < 0 || n_v < 0 || n_b < 1) return 0;
-    size_t tile = work_layout(n_t, n_v, n_b, k_per_band, 0, 0).total;
-    return MA_LIST ? ma_list_work_bytes(n_t, n_v, n_b, k_per_band) : tile;
+    // the tile kernel, the exact rows, or a table's rows (of any length that takes them)
+    size_t need = work_layout(n_t, n_v, n_b, k_per_band, 0, 0).total;
+    const size_t r = row_layout(n_t, n_v, n_b, k_per_band, 3, row_len_max(n_t)).total;
+    return r > need ? r : need;
+}
+
+static void fill_setup(SetupArgs *sa, const double *t, int n_t, const pt_orbit *orb, const float *k, int k_per_band,
+                       int n_b, double t_exp, GeomRec *rec, float2 *tsplit)
+{
+    sa->t = t;
+    sa->n_t = n_t;
+    sa->tsplit = tsplit;
+    sa->t0 = orb->t0;
+    sa->P = orb->P;
+    sa->a = orb->a;
+    sa->inc = orb->inc;
+    sa->e = orb->e;
+    sa->w = orb->w;
+    sa->k = k;
+    sa->n_v = orb->n_v;
+    sa->n_b = n_b;
+    sa->k_per_band = k_per_band;
+    sa->n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
+    sa->rec = rec;
+    sa->cnt = nullptr;
+    sa->half_exp = (float)(0.5 * t_exp);
+    sa->n_gblocks = 0;
 }
 
 static int launch_setup(const double *t, int n_t, const pt_orbit *orb, const float *k, int k_per_band, int n_b,
@@ -2165,73 +2225,86 @@ static int launch_setup(const double *t, int n_t, const pt_orbit *orb, const flo
 
 }  // extern "C"
 
-// pt_ma_quad over the pair lists (window kernel, scan, ma_pairs_kernel).
-static int ma_quad_list(const double *t, int n_t, const pt_orbit *orb, const float *k, int k_per_band,
-                        const float *ld, int n_b, int n_ss, double t_exp, int max_iter, const float *y,
-                        const float *wt, float *flux, float *ssr, void *work, size_t work_bytes, int *n_bad,
-                        pt_stream_t stream)
+// pt_ma_quad and pt_ma_quad_interp from row tables: preparation, row kernel
+// (and the sum of the residual partials).
+static int ma_quad_rows(const pt_ma_table_s *tab, const double *t, int n_t, const pt_orbit *orb, const float *k,
+                        int k_per_band, const float *ld, int n_b, int n_ss, double t_exp, int max_iter,
+                        const float *y, const float *wt, float *flux, float *ssr, void *work, size_t work_bytes,
+                        int *n_bad, pt_stream_t stream)
 {
-    int st = lc_common_check(t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, flux, ssr, work);
-    if (st) return st;
-    if (n_t == 0 || orb->n_v == 0) return PT_OK;
-    WorkLayout L = work_layout(n_t, orb->n_v, n_b, k_per_band, 1, 0);
+    const size_t row_len = tab ? interp_row_len(tab->n_z) : (size_t)pt::MT_ROW;
+    const RowLayout L = row_layout(n_t, orb->n_v, n_b, k_per_band, 3, row_len);
     if (work_bytes < L.total) return PT_ERR_WORKSPACE;
     const int n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
-    const int n_tiles = (n_t + TT - 1) / TT;
-    const int gy = (n_geom + GW_VT - 1) / GW_VT;
-    if (gy > 65535) return PT_ERR_ARG;
+    const int n_bpg = k_per_band ? 1 : n_b;
+    if ((n_geom + 31) / 32 > 65535) return PT_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     char *wb = (char *)work;
-    GeomRec *rec = (GeomRec *)(wb + L.rec);
-    float2 *tsplit = (float2 *)(wb + L.tsplit);
-    int *cnt = (int *)(wb + L.cnt);
-    st = launch_setup(t, n_t, orb, k, k_per_band, n_b, t_exp, rec, tsplit, cnt, s);
+    int n_sm = 0;
+    int st = sm_count(&n_sm);
     if (st) return st;
-    GimArgs A;
+    RowPrep P;
+    memset(&P, 0, sizeof(P));
+    fill_setup(&P.s, t, n_t, orb, k, k_per_band, n_b, t_exp, (GeomRec *)(wb + L.rec), (float2 *)(wb + L.tsplit));
+    P.s.n_gblocks = (n_geom + 31) / 32;
+    P.n_tblocks = (n_t + ROW_THREADS - 1) / ROW_THREADS;
+    P.rows = (float *)(wb + L.rows);
+    P.row_len = (int)row_len;
+    P.nr = rows_per_geom(n_bpg, 3);
+    P.terms = row_terms(n_bpg);
+    P.n_bpg = n_bpg;
+    P.ld = ld;
+    if (tab) {
+        P.mtab = tab->d_tab;
+        P.mn_k = tab->n_k;
+        P.mn_z = tab->n_z;
+        P.mk_lo = tab->k_lo;
+        P.mk_hi = tab->k_hi;
+        P.minv_dk = tab->inv_dk;
+    }
+    const long long rblocks = tab ? ((long long)n_geom * P.nr * P.row_len + ROW_THREADS - 1) / ROW_THREADS
+                                  : (n_geom + ROW_GEOM - 1) / ROW_GEOM;
+    const long long blocks = (long long)P.s.n_gblocks + P.n_tblocks + rblocks;
+    if (blocks > 0x7fffffffLL) return PT_ERR_ARG;
+    if (tab) row_prep_kernel<rows::R_INTERP><<<(unsigned)blocks, ROW_THREADS, 0, s>>>(P);
+    else row_prep_kernel<rows::R_MA><<<(unsigned)blocks, ROW_THREADS, 0, s>>>(P);
+    st = check_launch("row_prep_kernel");
+    if (st) return st;
+    rows::Args A;
     memset(&A, 0, sizeof(A));
-    A.tsplit = tsplit;
+    A.tsplit = P.s.tsplit;
     A.n_t = n_t;
-    A.rec = rec;
+    A.rec = P.s.rec;
     A.n_geom = n_geom;
+    A.rows = P.rows;
+    A.row_len = P.row_len;
+    A.nr = P.nr;
+    A.terms = P.terms;
+    A.n_bpg = n_bpg;
+    A.n_b = n_b;
+    A.k_per_band = k_per_band;
     A.ld = ld;
     A.N = 2;
-    A.n_bpg = k_per_band ? 1 : n_b;
     A.n_ss = n_ss;
     A.t_exp = (float)t_exp;
     A.max_iter = max_iter;
-    A.flux = flux ? flux : (float *)(wb + L.fscr);
-    A.cnt = cnt;
-    A.pref = (int *)(wb + L.pref);
-    A.gord = A.pref + n_geom + 1;
-    A.ctr = cnt + n_geom;
-    A.list = (int *)(wb + L.list);
-    A.ppi = MA_PPI;
+    const bool fused_ssr = ssr && !P.terms;
+    float *part = (float *)(wb + L.part);
+    A.flux = flux ? flux : (P.terms ? (float *)(wb + L.fscr) : nullptr);
+    A.ssr_part = fused_ssr ? part : nullptr;
+    A.y = y;
+    A.wt = wt;
     A.n_bad = n_bad;
-    TableJob J;
-    memset(&J, 0, sizeof(J));
-    const size_t n_cta = (size_t)n_tiles * gy;
-    if (n_cta > 0x7fffffffULL) return PT_ERR_ARG;
-    gim_window_kernel<<<(unsigned)n_cta, TT, 0, s>>>(A, J, n_tiles);
-    st = check_launch("gim_window_kernel");
-    if (st) return st;
-    gim_scan_kernel<<<1, 1024, 0, s>>>(cnt, A.rec, A.t_exp, n_geom, MA_PPI, false, A.pref, A.gord, A.ctr);
-    st = check_launch("gim_scan_kernel");
-    if (st) return st;
-    const size_t msm = ma_pairs_smem(n_ss);   // at most 44 KB: no opt-in needed
-    int dev = 0, n_sm = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, ma_pairs_kernel, MA_PPI, msm);
-    if (e != cudaSuccess) return set_cuda_error(e, "ma_pairs_kernel occupancy");
-    size_t grid = (size_t)n_sm * (per_sm > 0 ? per_sm : 1);
-    const size_t max_items = (size_t)n_geom * ((n_t + MA_PPI - 1) / MA_PPI);
-    if (grid > max_items) grid = max_items;
-    if (grid < 1) grid = 1;
-    ma_pairs_kernel<<<(unsigned)grid, MA_PPI, msm, s>>>(A);
-    st = check_launch("ma_pairs_kernel");
-    if (st) return st;
-    if (ssr) st = launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)orb->n_v * n_b, (float *)(wb + L.part), ssr, s);
-    return st;
+    if (tab) {
+        A.inv_dz = tab->inv_dz;
+        A.n_z = tab->n_z;
+    }
+    st = launch_rows(tab ? rows::R_INTERP : rows::R_MA, A, n_sm, s);
+    if (st || !ssr) return st;
+    const int n_rows = orb->n_v * n_b;
+    if (!fused_ssr) return launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)n_rows, part, ssr, s);
+    ssr_reduce_kernel<<<(unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s>>>(part, n_rows, A.n_tiles, ssr);
+    return check_launch("ssr_reduce_kernel");
 }
 
 // pt_ma_quad and pt_ma_quad_interp: exact terms when tab is null, else the
@@ -2239,11 +2312,14 @@ static int ma_quad_list(const double *t, int n_t, const pt_orbit *orb, const flo
 static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, const pt_orbit *orb, const float *k,
                         int k_per_band, const float *ld, int n_b, int n_ss, double t_exp, int max_iter,
                         const float *y, const float *wt, float *flux, float *ssr, void *work, size_t work_bytes,
-                        int *n_bad, pt_stream_t stream)
+                        int *n_bad, pt_stream_t stream, bool use_rows = true)
 {
     int st = lc_common_check(t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, flux, ssr, work);
     if (st) return st;
     if (n_t == 0 || orb->n_v == 0) return PT_OK;
+    if (use_rows && ma_use_rows(n_t, orb->n_v, n_b, k_per_band, n_ss) && (!tab || interp_row_len(tab->n_z) <= row_len_max(n_t)))
+        return ma_quad_rows(tab, t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, wt, flux, ssr, work,
+                            work_bytes, n_bad, stream);
     WorkLayout L = work_layout(n_t, orb->n_v, n_b, k_per_band, 0, 0);
     if (work_bytes < L.total) return PT_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
@@ -2304,9 +2380,6 @@ int pt_ma_quad(const double *t, int n_t, const pt_orbit *orb, const float *k, in
                int n_b, int n_ss, double t_exp, int max_iter, const float *y, const float *wt, float *flux,
                float *ssr, void *work, size_t work_bytes, int *n_bad, pt_stream_t stream)
 {
-    if (MA_LIST && !ma_small(orb, n_b, k_per_band))
-        return ma_quad_list(t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, wt, flux, ssr, work,
-                            work_bytes, n_bad, stream);
     return ma_quad_impl(nullptr, t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, wt, flux, ssr,
                         work, work_bytes, n_bad, stream);
 }
@@ -2688,5 +2761,5 @@ extern "C" int pt_ma_quad_noalloc(const double *t, int n_t, const pt_orbit *orb,
     // Every scratch byte the kernels read is written earlier in the same call
     // (geometry records, time split, residual partials), so nothing is cleared.
     return ma_quad_impl(nullptr, t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, wt, flux, ssr,
-                        scratch, (size_t)PT_MA_NOALLOC_SCRATCH_BYTES, n_bad, stream);
+                        scratch, (size_t)PT_MA_NOALLOC_SCRATCH_BYTES, n_bad, stream, false);
 }

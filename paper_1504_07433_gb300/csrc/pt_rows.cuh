@@ -1,0 +1,506 @@
+// pt_rows.cuh -- light curves from row tables: one kernel for every model.
+//
+// A light-curve call evaluates each geometry (orbit and radius ratio) at
+// thousands of separations, so a preparation kernel first tabulates, per
+// geometry and passband, the transit depth as a function of the separation
+// (a "row"), and lc_rows_kernel does the rest in one pass:
+//   - a CTA covers VT geometries x KT blocks of 256 times (VT KT <= 32, one
+//     bit per (geometry, block) of a thread); it stages the geometries'
+//     records and rows in shared memory;
+//   - window test of every pair in plain FP32 with a margin; the pairs that
+//     pass go to one list per geometry in shared memory; every flux is set
+//     to 1;
+//   - each lane takes a listed pair (the lists end to end, so that lanes stay
+//     full), reduces its time in double-float (a pair beyond the exact window
+//     keeps depth 0), solves the orbit at its supersamples and reads the
+//     pair's rows there; mean, flux, residual;
+//   - residual sums: each thread adds up its own times, in order.
+// The place of a pair in its list is not determined, but no value depends on
+// it, so results are reproducible bit by bit.
+// The rows and what a look-up does are the model's:
+//   R_MA      piecewise polynomials in the distance to the contacts
+//             (pt_device.cuh); the exact terms where a geometry has none;
+//   R_GIM     piecewise polynomials of the Gimenez series;
+//   R_ZI      Gimenez on z nodes (Sec. 3.3), linear;
+//   R_INTERP  the Mandel-Agol table at the geometry's k (Sec. 2.2.3), linear.
+// Before, the path was a set-up, a window kernel writing pair lists to memory,
+// a scan, and an evaluation kernel per model that solved Kepler's equation for
+// every supersample, packed the in-transit ones and evaluated the terms for
+// each.  50,000 times x 256 eccentric vectors x 10 supersamples: Mandel-Agol
+// 85.7 -> 50.0 us a call, from the caller's table 110 -> 46.7 us; 3,001 times x
+// 800 circular geometries x 3, residual sums: 75.8 -> 45 us.  What bounds it:
+// issue (about 65 %), two thirds of the instructions in the window test, the
+// lists and the stores of a survey's mostly empty pairs.
+#pragma once
+
+#include "pt_device.cuh"
+
+namespace rows {
+
+using pt::GeomRec;
+
+enum Model { R_MA = 0, R_GIM = 1, R_ZI = 2, R_INTERP = 3 };
+
+constexpr int TB = 256;          // times per block of a tile, threads per CTA
+constexpr int NW = TB / 32;
+constexpr int MAX_BITS = 32;     // VT KT
+constexpr int MAX_BAND_ROWS = 8; // passbands of a geometry with a row each; more share the rows of the terms
+
+struct Args {
+    const float2 *tsplit;
+    int n_t;
+    const GeomRec *rec;
+    int n_geom;
+    const float *rows;      // [n_geom][nr][row_len]
+    int row_len;            // floats, a multiple of 4
+    int nr;                 // rows per geometry
+    int terms;              // rows hold the model's terms, combined per passband with its weights
+    int n_bpg, n_b, k_per_band;
+    const float *ld;
+    int N;                  // coefficients per passband (2, or the general law's)
+    int n_ss;
+    float t_exp;
+    int max_iter;
+    float *flux;            // [n_geom n_bpg][n_t] or null
+    float *ssr_part;        // [n_geom n_bpg][n_tiles] or null (needs !terms)
+    int n_tiles, tile0;
+    const float *y, *wt;
+    int *n_bad;
+    int log_vt, log_kt;
+    int flux_vec;           // 16-byte stores of whole rows are aligned
+    float scale;            // R_GIM
+    int n_in, n_edge;       // R_ZI
+    float inv_dz;           // R_INTERP
+    int n_z;
+};
+
+// The exact Mandel-Agol terms of a geometry without a table.
+__device__ __noinline__ float3 exact_terms(float k, float z)
+{
+    float3 t;
+    pt::ma_terms(k, z, &t.x, &t.y, &t.z);
+    return t;
+}
+
+// A look-up: the place in the row and the offset from it.
+template <int MODEL>
+__device__ __forceinline__ unsigned find(const Args &A, const float4 &q, float z, float *t)
+{
+    if (MODEL == R_MA) {
+        const float zm1 = z - 1.0f;
+        return pt::mt_find(q.x, q.y, q.z, zm1, pt::mt_off_limb(zm1), t);
+    }
+    if (MODEL == R_GIM) {
+        // u = sqrt(1 - z / (1 + k)), 0 at and beyond the contact
+        const float u = pt::sqrt_a(__saturatef((q.x - (z - 1.0f)) * q.y));
+        const float b = fmaf(u, A.scale, pt::MT_MAGIC);
+        *t = fmaf(u, A.scale, pt::MT_MAGIC - b);
+        return __float_as_uint(b);
+    }
+    if (MODEL == R_ZI) {   // q: k, zb, 1 / h1 (0: the first region is z = 0), 1 / h2
+        if (z <= q.y) {
+            const float f = z * q.z;
+            const int i = q.z > 0.0f ? min((int)f, A.n_in - 2) : 0;
+            *t = q.z > 0.0f ? f - (float)i : 0.0f;
+            return (unsigned)i;
+        }
+        const float f = fminf((z - q.y) * q.w, 1e9f);
+        const int c = min((int)f, A.n_edge - 1);
+        *t = f - (float)c;
+        return (unsigned)(A.n_in - 1 + c);
+    }
+    const float f = fminf(fmaxf(z, 0.0f) * A.inv_dz, (float)(A.n_z - 1));
+    const int i = min((int)f, A.n_z - 2);
+    *t = f - (float)i;
+    return (unsigned)i;
+}
+
+constexpr int GIM_DEG = 12;   // coefficients per interval of a Gimenez row
+
+// base: byte address in shared memory (SMEM) of the row, less the place's
+// constant bits; or the row in global memory
+template <int MODEL, bool SMEM>
+__device__ __forceinline__ float eval(unsigned base, const float *row, const float4 &q, float z, unsigned pos, float t)
+{
+    if (MODEL == R_MA && SMEM) return pt::mt_eval(base, pos, t);
+    if (MODEL == R_GIM || MODEL == R_MA) {
+        constexpr int L = MODEL == R_GIM ? GIM_DEG : 8;   // floats per interval
+        float4 c[3];
+        if (SMEM) {
+            const unsigned at = base + (unsigned)(4 * L) * pos;
+#pragma unroll
+            for (int i = 0; i < 3; ++i)
+                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                             : "=f"(c[i].x), "=f"(c[i].y), "=f"(c[i].z), "=f"(c[i].w)
+                             : "r"(at + 16u * i));
+        } else {
+            const float4 *p = reinterpret_cast<const float4 *>(row + (size_t)(pos - pt::MT_BITS0) * L);
+            c[0] = __ldg(p);
+            c[1] = __ldg(p + 1);
+            if (MODEL == R_GIM) c[2] = __ldg(p + 2);
+        }
+        if (MODEL == R_MA)
+            return fmaf(fmaf(fmaf(fmaf(fmaf(c[1].y, t, c[1].x), t, c[0].w), t, c[0].z), t, c[0].y), t, c[0].x);
+        float v = fmaf(c[2].w, t, c[2].z);
+        v = fmaf(v, t, c[2].y);
+        v = fmaf(v, t, c[2].x);
+        v = fmaf(v, t, c[1].w);
+        v = fmaf(v, t, c[1].z);
+        v = fmaf(v, t, c[1].y);
+        v = fmaf(v, t, c[1].x);
+        v = fmaf(v, t, c[0].w);
+        v = fmaf(v, t, c[0].z);
+        v = fmaf(v, t, c[0].y);
+        return fmaf(v, t, c[0].x);
+    }
+    float a, b;
+    if (SMEM) {
+        const unsigned at = base + 4u * pos;
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(at));
+        asm volatile("ld.shared.f32 %0, [%1];" : "=f"(b) : "r"(at + 4u));
+    } else {
+        a = __ldg(row + pos);
+        b = __ldg(row + pos + 1);
+    }
+    return z < 1.0f + q.x ? fmaf(t, b - a, a) : 0.0f;
+}
+
+// constants of a geometry's look-ups
+template <int MODEL>
+__device__ __forceinline__ float4 look_up_constants(const Args &A, float k)
+{
+    float4 q = make_float4(k, 0.0f, 0.0f, 1.0f);
+    if (MODEL == R_MA) {
+        if (pt::mt_valid(k)) pt::mt_scales(k, &q.y, &q.z);
+        else q.w = 0.0f;
+    } else if (MODEL == R_GIM) {
+        q.y = 1.0f / (1.0f + k);
+    } else if (MODEL == R_ZI) {
+        q.y = fmaxf(1.0f - k, 0.0f);
+        q.z = q.y > 0.0f ? 1.0f / (q.y / (float)(A.n_in - 1)) : 0.0f;
+        q.w = 1.0f / ((1.0f + k - q.y) / (float)A.n_edge);
+    }
+    return q;
+}
+
+struct Smem {   // byte offsets in dynamic shared memory
+    int list, rows, sval, sred, total;
+};
+
+__host__ __device__ inline Smem smem_layout(int vt, int log_kt, int nr, int row_len, bool staged, int n_ssr)
+{
+    Smem s;
+    const int pairs = vt * (TB << log_kt);
+    int off = 0;
+    s.list = off;
+    off += pairs * 2;
+    s.rows = off;
+    if (staged) off += vt * nr * row_len * 4;
+    s.sval = off;
+    off += n_ssr * pairs * 4;
+    s.sred = off;
+    off += NW * vt * n_ssr * 4;
+    s.total = off;
+    return s;
+}
+
+template <int MODEL, int NRT, bool SMEM>
+__global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
+{
+    extern __shared__ __align__(16) unsigned char dsm[];
+    __shared__ GeomRec srec[MAX_BITS];
+    __shared__ float4 stest[MAX_BITS];   // 1/P, -(t0 + window centre)/P, half width + margin (periods)
+    __shared__ float4 sgeo[MAX_BITS];    // constants of the look-ups
+    __shared__ int sband[MAX_BITS];      // passband of each geometry's data
+    __shared__ int scnt[MAX_BITS];       // pairs of each geometry
+    __shared__ int soff[MAX_BITS + 1];   // ... before each geometry, lists end to end
+    __shared__ float swmax[NW];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int log_vt = A.log_vt, vt = 1 << log_vt, log_kt = A.log_kt, kt = 1 << log_kt;
+    const int tile = A.tile0 + blockIdx.y;
+    const int g0 = blockIdx.x << log_vt;
+    const int ng = min(vt, A.n_geom - g0);
+    const int tb = tile * (TB << log_kt);
+    const int n_ssr = A.ssr_part ? A.nr : 0;
+    const Smem L = smem_layout(vt, log_kt, A.nr, A.row_len, SMEM, n_ssr);
+    const int cap = TB << log_kt;        // entries of a geometry's list
+    unsigned short *list = reinterpret_cast<unsigned short *>(dsm + L.list);   // [vt][cap]: k TB + thread
+    for (int i = tid; i < ng * 6; i += TB) {
+        const int vl = i / 6, c = i - 6 * vl;
+        reinterpret_cast<float4 *>(&srec[vl])[c] = reinterpret_cast<const float4 *>(&A.rec[g0 + vl])[c];
+    }
+    if (SMEM) {
+        const float4 *src = reinterpret_cast<const float4 *>(A.rows + (size_t)g0 * A.nr * A.row_len);
+        const unsigned dst = (unsigned)__cvta_generic_to_shared(dsm + L.rows);
+        const int n4 = ng * A.nr * A.row_len / 4;
+        for (int i = tid; i < n4; i += TB)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst + 16u * i), "l"(src + i) : "memory");
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    if (tid < MAX_BITS) scnt[tid] = 0;
+    // the tile's largest |t_h| (non-negative floats order like their bits)
+    float am = 0.0f;
+    for (int k = 0; k < kt; ++k) {
+        const int t = tb + k * TB + tid;
+        if (t < A.n_t) am = fmaxf(am, fabsf(A.tsplit[t].x));
+    }
+    am = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(am)));
+    if (lane == 0) swmax[warp] = am;
+    __syncthreads();
+    if (tid < MAX_BITS) stest[tid] = make_float4(0.0f, 0.0f, -1.0f, 0.0f);   // beyond the last geometry: never
+    if (tid < ng) {
+        float tmax = swmax[0];
+        for (int w = 1; w < NW; ++w) tmax = fmaxf(tmax, swmax[w]);
+        const GeomRec &r = srec[tid];
+        // The test is in periods from the window's centre, one FMA: off by less
+        // than 5 roundings of the magnitudes involved (the products with the
+        // rounded 1/P, the low parts of t, t0 and P, the sum).  Where that is
+        // no small part of a period, every pair is listed.
+        const float mid = 0.5f * (r.win_lo + r.win_hi);
+        const float m = 3.0e-7f * (tmax + fabsf(r.t0h) + fabsf(mid) + r.Ph) * r.invP + 1e-7f;
+        float half = 0.5f * (r.win_hi - r.win_lo) * r.invP * 1.000001f + m;
+        if (r.win_lo > r.win_hi) half = -1.0f;
+        else if (!(m < 0.25f)) half = INFINITY;
+        stest[tid] = make_float4(r.invP, -(r.t0h + mid) * r.invP, half, 0.0f);
+        sgeo[tid] = look_up_constants<MODEL>(A, r.k);
+        sband[tid] = A.k_per_band ? (g0 + tid) % A.n_b : 0;
+    }
+    // every flux of the tile is 1 until its pair is evaluated
+    if (A.flux) {
+        const int n_row = ng * A.n_bpg, n_tt = min(cap, A.n_t - tb);
+        float *fp = A.flux + (size_t)g0 * A.n_bpg * A.n_t + tb;
+        if (A.flux_vec) {   // rows and the array start on 16 bytes
+            const float4 one = make_float4(1.0f, 1.0f, 1.0f, 1.0f);
+            const int n4 = n_tt / 4;   // (n_t, and so n_tt, a multiple of 4)
+            for (int r = tid >> 6; r < n_row; r += TB / 64)
+                for (int i = tid & 63; i < n4; i += 64) reinterpret_cast<float4 *>(fp + (size_t)r * A.n_t)[i] = one;
+        } else {
+            for (int r = 0; r < n_row; ++r, fp += A.n_t)
+                for (int i = tid; i < n_tt; i += TB) fp[i] = 1.0f;
+        }
+    }
+    __syncthreads();
+    unsigned bits = 0u;   // bit k vt + vl: the time of block k may be in geometry vl's window
+    for (int k = 0; k < kt; ++k) {
+        const int t = tb + k * TB + tid;
+        const float th = t < A.n_t ? A.tsplit[t].x : __int_as_float(0x7fffffff);   // NaN: in no window
+        unsigned cand = 0u;
+        for (int v0 = 0; v0 < vt; v0 += 4) {
+            unsigned c4 = 0u;
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {   // (vt < 4: the entries beyond never pass)
+                const float4 q = stest[v0 + u];
+                const float ph = fmaf(th, q.x, q.y);
+                const float fr = ph - ((ph + pt::MT_MAGIC) - pt::MT_MAGIC);
+                c4 |= fabsf(fr) <= q.z ? (1u << u) : 0u;
+            }
+            cand |= c4 << v0;
+        }
+        bits |= cand << (k << log_vt);
+    }
+    {
+        // append to the lists: one atomic per warp and geometry where the
+        // warp's lanes share geometries (exposures around one planet's
+        // transits), one per pair where they do not (survey cadence)
+        const unsigned wbits = __reduce_or_sync(0xffffffffu, bits);
+        const int wpairs = __reduce_add_sync(0xffffffffu, __popc(bits));
+        if (wpairs > 4 * __popc(wbits)) {
+            for (unsigned rest = wbits; rest; rest &= rest - 1u) {
+                const int p = __ffs(rest) - 1, vl = p & (vt - 1), k = p >> log_vt;
+                const bool in = (bits >> p) & 1u;
+                const unsigned mb = __ballot_sync(0xffffffffu, in);
+                int base = 0;
+                if (lane == 0) base = atomicAdd(&scnt[vl], __popc(mb));
+                base = __shfl_sync(0xffffffffu, base, 0);
+                if (in) list[vl * cap + base + __popc(mb & ((1u << lane) - 1u))] = (unsigned short)(k * TB + tid);
+            }
+        } else {
+            for (unsigned rest = bits; rest; rest &= rest - 1u) {
+                const int p = __ffs(rest) - 1, vl = p & (vt - 1), k = p >> log_vt;
+                list[vl * cap + atomicAdd(&scnt[vl], 1)] = (unsigned short)(k * TB + tid);
+            }
+        }
+    }
+    if (SMEM) asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    if (warp == 0) {
+        const int v = lane < vt ? scnt[lane] : 0;
+        int x = v;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int u = __shfl_up_sync(0xffffffffu, x, o);
+            if (lane >= o) x += u;
+        }
+        if (lane < vt) soff[lane] = x - v;
+        if (lane == 31) soff[vt] = x;
+    }
+    __syncthreads();
+    const int nq = soff[vt];
+    // the lists end to end, 32 pairs per warp and turn
+    const float inv_nss = 1.0f / (float)A.n_ss;
+    const unsigned sbase = (unsigned)__cvta_generic_to_shared(dsm + L.rows) -
+                           (MODEL == R_MA ? 32u * pt::MT_BITS0 : MODEL == R_GIM ? 4u * GIM_DEG * pt::MT_BITS0 : 0u);
+    float *sval = reinterpret_cast<float *>(dsm + L.sval);   // [n_ssr][kt vt][TB]
+    int nbad = 0;
+    for (int e = tid; e < nq; e += TB) {
+        int vl = 0;   // the last geometry with soff <= e
+        for (int o = vt >> 1; o > 0; o >>= 1)
+            if (soff[vl + o] <= e) vl += o;
+        const int code = list[vl * cap + (e - soff[vl])];
+        const int t = tb + code;
+        const GeomRec &r = srec[vl];
+        const float4 q = sgeo[vl];
+        const float2 ts = A.tsplit[t];
+        const float dt = pt::reduce_time(ts.x, ts.y, r);
+        const int n_ss = dt >= r.win_lo && dt <= r.win_hi ? A.n_ss : 0;
+        const size_t row0 = (size_t)(g0 + vl) * A.n_bpg;
+        // Kepler's equation once, at mid-exposure; the supersamples from the
+        // f and g series at offsets x0 + s dx of mean anomaly
+        pt::OrbitState o;
+        bool bad0 = false;
+        pt::orbit_state(r, dt, A.max_iter, &bad0, &o);
+        const float cosi = r.cosi, dx = A.n_ss > 1 ? r.nang * A.t_exp * inv_nss : 0.0f;
+        const float x0 = -0.5f * (float)(A.n_ss - 1) * dx;
+        const bool series = pt::fg_valid(r, o.E1, x0);
+        const pt::FgSeries fg = pt::fg_series(o.E1, o.esin);
+        if (series && bad0) nbad += n_ss;
+        float mean[NRT];
+#pragma unroll 1
+        for (int r0 = 0; r0 < A.nr; r0 += NRT) {
+#pragma unroll
+            for (int u = 0; u < NRT; ++u) mean[u] = 0.0f;
+            const unsigned lbase = sbase + (unsigned)((vl * A.nr + r0) * A.row_len) * 4u;
+            const float *grow = A.rows + ((size_t)(g0 + vl) * A.nr + r0) * A.row_len;
+            // one supersample's depth (or terms)
+            auto add = [&](float z) {
+                if (MODEL == R_MA && q.w == 0.0f) {
+                    const float3 te = exact_terms(q.x, z);
+#pragma unroll
+                    for (int u = 0; u < NRT; ++u) {
+                        if (r0 + u >= A.nr) break;
+                        if (A.terms) {
+                            mean[u] += u == 0 ? te.x : (u == 1 ? te.y : te.z);   // (three rows: r0 = 0)
+                        } else {
+                            float we, wd, wn;
+                            const float *ld = A.ld + 2 * (row0 + r0 + u);
+                            pt::ma_weights(ld[0], ld[1], &we, &wd, &wn);
+                            mean[u] += we * te.x + wd * te.y + wn * te.z;
+                        }
+                    }
+                } else {
+                    float off_t;
+                    const unsigned pos = find<MODEL>(A, q, z, &off_t);
+#pragma unroll
+                    for (int u = 0; u < NRT; ++u) {
+                        if (r0 + u >= A.nr) break;
+                        mean[u] += eval<MODEL, SMEM>(lbase + (unsigned)(u * A.row_len) * 4u, grow + u * A.row_len, q, z,
+                                                     pos, off_t);
+                    }
+                }
+            };
+            if (series) {
+#pragma unroll 1
+                for (int s = 0; s < n_ss; ++s)
+                    add(pt::fg_z(o, fg, cosi, x0 + (float)s * dx));
+            } else {
+                // (exposures too long a part of the period for the series)
+                float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
+#pragma unroll 1
+                for (int s = 0; s < n_ss; ++s) {
+                    bool bad = false;
+                    const float off = A.t_exp * (((float)s + 0.5f) * inv_nss - 0.5f);
+                    const float z = pt::orbit_z<true, true>(r, dt + off, A.max_iter, &bad, warm);
+                    if (bad && r0 == 0) ++nbad;
+                    add(z);
+                }
+            }
+            if (A.terms) {
+                // the terms' share of every passband's depth; the flux holds the
+                // depth so far (this lane's alone) until the last rows
+                for (int bb = 0; bb < A.n_bpg; ++bb) {
+                    const float *ld = A.ld + (row0 + bb) * A.N;
+                    float w[NRT];
+                    if (MODEL == R_MA || MODEL == R_INTERP) {
+                        float we, wd, wn;
+                        pt::ma_weights(ld[0], ld[1], &we, &wd, &wn);
+#pragma unroll
+                        for (int u = 0; u < NRT; ++u) w[u] = u == 0 ? we : (u == 1 ? wd : (u == 2 ? wn : 0.0f));
+                    } else {   // C_0 = (1 - sum u)/D, C_n = u_n/D, D = 1 - sum n u_n/(n+2)   (Sec. 2.1.3)
+                        float su = 0.0f, sd = 0.0f;
+                        for (int n = 1; n <= A.N; ++n) {
+                            su += ld[n - 1];
+                            sd += (float)n * ld[n - 1] / (float)(n + 2);
+                        }
+#pragma unroll
+                        for (int u = 0; u < NRT; ++u)
+                            w[u] = r0 + u > A.N ? 0.0f : (r0 + u == 0 ? 1.0f - su : ld[max(r0 + u - 1, 0)]) / (1.0f - sd);
+                    }
+                    float *fp = A.flux + (row0 + bb) * A.n_t + t;
+                    float dep = r0 == 0 ? 0.0f : *fp;
+#pragma unroll
+                    for (int u = 0; u < NRT; ++u)
+                        if (r0 + u < A.nr) dep += w[u] * (mean[u] * inv_nss);
+                    *fp = r0 + NRT >= A.nr ? 1.0f - dep : dep;
+                }
+                continue;
+            }
+#pragma unroll
+            for (int u = 0; u < NRT; ++u) {
+                if (r0 + u >= A.nr) break;
+                const float dep = __fmul_rn(mean[u], inv_nss);
+                if (A.flux) A.flux[(row0 + r0 + u) * A.n_t + t] = 1.0f - dep;
+                if (n_ssr) {
+                    const int band = sband[vl] + (A.k_per_band ? 0 : r0 + u);
+                    // y - f with f = 1 - depth not rounded in between
+                    const float res = (A.y[(size_t)band * A.n_t + t] - 1.0f) + dep;
+                    const int p = ((code >> 8) << log_vt) + vl;
+                    sval[(((r0 + u) << (log_vt + log_kt)) + p) * TB + (code & (TB - 1))] =
+                        (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * res * res;
+                }
+            }
+        }
+    }
+    if (nbad && A.n_bad) atomicAdd(A.n_bad, nbad);
+    if (!n_ssr) return;
+    __syncthreads();
+    // residual sums per geometry and passband: every thread's own times, from
+    // the evaluated pairs or with the flux at 1
+    float *sred = reinterpret_cast<float *>(dsm + L.sred);     // [NW][vt][n_ssr]
+    for (int bb = 0; bb < n_ssr; ++bb) {
+        float r1 = 0.0f;
+        int band_of = -1;
+        for (int vl = 0; vl < ng; ++vl) {
+            const int band = sband[vl] + (A.k_per_band ? 0 : bb);
+            float x = 0.0f;
+            for (int k = 0; k < kt; ++k) {
+                const int p = (k << log_vt) + vl;
+                if ((bits >> p) & 1u) {
+                    x += sval[((bb << (log_vt + log_kt)) + p) * TB + tid];
+                    continue;
+                }
+                const int t = tb + k * TB + tid;
+                if (kt > 1 || band != band_of) {
+                    r1 = 0.0f;
+                    if (t < A.n_t) {
+                        const float r = A.y[(size_t)band * A.n_t + t] - 1.0f;
+                        r1 = (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * r * r;
+                    }
+                    band_of = band;
+                }
+                x += r1;
+            }
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+            if (lane == 0) sred[(warp * vt + vl) * n_ssr + bb] = x;
+        }
+    }
+    __syncthreads();
+    for (int i = tid; i < ng * n_ssr; i += TB) {
+        const int vl = i / n_ssr, bb = i - vl * n_ssr;
+        float x = 0.0f;
+        for (int w = 0; w < NW; ++w) x += sred[(w * vt + vl) * n_ssr + bb];
+        A.ssr_part[((size_t)(g0 + vl) * A.n_bpg + bb) * A.n_tiles + tile] = x;
+    }
+}
+
+}  // namespace rows
