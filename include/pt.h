@@ -434,18 +434,13 @@ int pt_ma_quad_noalloc(const double *t_dev, int n_t, const pt_orbit *orb, const 
  *
  * A plan holds the tables of Sec. 2.1.4 for a given number of general-law
  * coefficients N (Eq. ld_general; alpha_0..alpha_N are evaluated) and series
- * depth n_j: the recursion coefficients of G_j(nu+2, 1; x) and the A_{n,j}
- * of Eq. (gimemez_a), in device memory allocated by pt_gim_plan_create and
- * released by pt_gim_plan_destroy.  1 <= N <= 16, 2 <= n_j <= 512.
- * A plan may be used from any stream; its tables are read-only after
- * creation.  The plan also owns a CUDA stream (the device's highest priority)
- * and two events: pt_gimenez forks the per-geometry table recursion and the
- * series coefficients, which depend on k alone, onto that stream at the start
- * of the call (after all earlier work of the call's stream) and joins it
- * before the evaluation kernel, so that they run beside the set-up and window
- * kernels.  Calls from several host threads or streams may share a plan:
- * their forked work runs in the order the calls were made.  Stream capture of
- * a call captures the fork and the join.
+ * depth n_j: the recursion coefficients of G_j(nu+2, 1; x), the A_{n,j} of
+ * Eq. (gimemez_a), and the series' functions of z as piecewise polynomials
+ * (4 (N+1) n_j 8 n_int bytes, n_int about (2 n_j + N)/3.75: 5.9 MB at N = 8,
+ * n_j = 192), in device memory allocated by pt_gim_plan_create and released by
+ * pt_gim_plan_destroy.  1 <= N <= 16, 2 <= n_j <= 512.
+ * A plan may be used from any stream and from several host threads: its
+ * tables are read-only after creation, and a call runs on its own stream only.
  * ---------------------------------------------------------------------- */
 typedef struct pt_gim_plan_s *pt_gim_plan;
 
@@ -454,7 +449,8 @@ int pt_gim_plan_destroy(pt_gim_plan plan);
 
 /* Profiling hook: ev_start and ev_end (cudaEvent_t handles, owned by the
  * caller, which keeps them alive while calls use them) are recorded on the
- * call's stream right before and right after the series-evaluation kernel
+ * call's stream right before and right after the light-curve kernel (window
+ * test, orbits, look-ups in the rows formed from the series)
  * of every later pt_gimenez call with this plan, so that the caller can time
  * that kernel alone; NULL, NULL stops it.  This is the one setting that
  * changes a plan: a plan with events set must not be used by two host

@@ -32,14 +32,10 @@
 
 #include "../../include/pt.h"
 #include "pt_device.cuh"
+#include "pt_gim.cuh"
 #include "pt_rows.cuh"
 
-using pt::DF;
 using pt::GeomRec;
-using pt::df_add;
-using pt::df_mad;
-using pt::df_mul;
-using pt::df_of;
 
 namespace {
 
@@ -141,6 +137,8 @@ struct RowPrep {
     const float4 *mtab;
     int mn_k, mn_z;
     float mk_lo, mk_hi, minv_dk;
+    // R_GIM: the weighted T_{n,j} (pt_gim.cuh)
+    gim::Table gim;
 };
 
 // weights of row r of a geometry: a passband's depth, or one of the terms
@@ -194,6 +192,10 @@ __global__ void __launch_bounds__(ROW_THREADS) row_prep_kernel(RowPrep P)
             v = w.x * fmaf(wk, b.x - a.x, a.x) + w.y * fmaf(wk, b.y - a.y, a.y) + w.z * fmaf(wk, b.z - a.z, a.z);
         }
         P.rows[at] = v;
+        return;
+    }
+    if (MODEL == rows::R_GIM) {
+        gim::table_cta(P.gim, s.k, s.n_geom, P.nr, P.terms, P.n_bpg, P.ld, blk % P.gim.NP1, blk / P.gim.NP1);
         return;
     }
     const int first = blk * ROW_GEOM;
@@ -413,1033 +415,6 @@ __global__ void __launch_bounds__(TT) ma_lc_kernel(LcArgs A)
     }
     if (tl == 0 && sbad && A.n_bad) atomicAdd(A.n_bad, sbad);
 }
-
-// ---------------------------------------------------------------------------
-// Gimenez light curves
-//
-// Per geometry the table pass stores T_{n,j} = A_{n,j} G_j(nu+2, nu+1; 1-b)^2
-// (Sec. 2.1.4: the z-independent factors).  Per (time, geometry) pair the
-// evaluation accumulates, for n = 0..N,
-//   alpha_n = b^2 (1 - c^2)^{nu+1} sum_j T_{n,j} G_j(nu+2, 1; c^2),
-// with only summations and multiplications in the z-dependent part
-// (Sec. 2.1.4).  Kernels:
-//   gim_window_kernel  the tables (leading CTAs); then every pair: window
-//                      test; pairs in the window go to a per-geometry list,
-//                      the others get flux 1;
-//   gim_scan_kernel    work items per geometry (ppi listed pairs each) and
-//                      their exclusive prefix;
-//   gim_cheb_coef_kernel / gim_cheb_kernel  the series in a Chebyshev basis
-//                      shared by the orders (below): coefficients per
-//                      geometry, then persistent CTAs that take work items
-//                      from an atomic counter, evaluate the items' in-transit
-//                      supersamples as a dense list and sum each pair's
-//                      terms on the pair's own thread.
-// Every pair's sums are taken in the same order whatever thread evaluated
-// its terms and whatever CTA took its item, so the result is deterministic.
-// ---------------------------------------------------------------------------
-constexpr int GW_VT = 32;         // geometries per CTA of the window kernel (<= 32: one bit each)
-constexpr int GS_THREADS = 128;   // threads per CTA of the evaluation kernels (one owned pair each)
-
-struct GimArgs {
-    const float2 *tsplit;
-    int n_t;
-    const GeomRec *rec;
-    int n_geom;
-    const float4 *gtab;   // [n_geom][N+1][n_j]: (r1_j, r2_j, r3_{j+1}, T_j)
-    int N, n_j;
-    const float *ld;      // [rows][N]
-    int n_bpg;            // band rows per geometry
-    int n_ss;
-    float t_exp;
-    int max_iter;
-    float *flux;          // [rows][n_t]
-    int *cnt;             // [n_geom] listed pairs per geometry
-    int *pref;            // [n_geom + 1] work items before each position of the geometry order
-    int *gord;            // [n_geom] geometry at each position of the order
-    int *ctr;             // next work item of the evaluation kernel
-    int *list;            // [n_geom][n_t] time indices of listed pairs
-    int ppi;              // pairs per work item (GS_THREADS or MA_PPI)
-    int *n_bad;
-};
-
-// Gimenez per-geometry table for Clenshaw's summation: entry (n, j) packs the
-// z-recursion coefficients r1_j, r2_j, r3_{j+1} of G_j(nu+2, 1; x) with
-// T_{n,j} = A_{n,j} G_j(nu+2, nu+1; 1-b)^2, the z-independent factor of
-// Sec. 2.1.4 (recursion in double-float arithmetic, stored FP32).
-// A table CTA covers one order n and TABLE_GPC geometries (one thread each;
-// the CTA's other threads only help stage row n of the plan's coefficients
-// in shared memory as double-float pairs).  The recursion is a chain of n_j
-// dependent steps per thread, so the chains are spread thinly over many SMs,
-// and the table CTAs run inside the window kernel's launch, in the shadow of
-// its wide grid.
-constexpr int TABLE_GPC = 64;
-struct TableJob {
-    const float *k;           // [n_geom] radius ratio of each geometry (the call's k)
-    int n_geom, NP1, n_j;
-    const double *A, *recb;   // the plan's A_{n,j} and recursion of G_j(nu+2, nu+1; x), FP64
-    const float4 *coef;       // the plan's recursion of G_j(nu+2, 1; x), FP32
-    float4 *tab;              // [n_geom][NP1][n_j]
-    int n_blocks;             // table CTAs (0: none)
-};
-
-__device__ __forceinline__ void table_cta(const TableJob &J, int n, int gb)
-{
-    extern __shared__ __align__(16) unsigned char tsm[];
-    const int n_j = J.n_j;
-    float4 *scf = reinterpret_cast<float4 *>(tsm);   // [n_j]
-    DF *sA = reinterpret_cast<DF *>(scf + n_j);      // [n_j]
-    DF *srb = sA + n_j;                              // [n_j][3]
-    for (int i = threadIdx.x; i < n_j; i += blockDim.x) {
-        scf[i] = J.coef[(size_t)n * n_j + i];
-        sA[i] = df_of(J.A[(size_t)n * n_j + i]);
-    }
-    for (int i = threadIdx.x; i < 3 * n_j; i += blockDim.x) srb[i] = df_of(J.recb[(size_t)n * n_j * 3 + i]);
-    __syncthreads();
-    const int g = gb * TABLE_GPC + threadIdx.x;
-    if (threadIdx.x >= TABLE_GPC || g >= J.n_geom) return;
-    const double k = J.k[g];
-    const DF x = df_of(1.0 - k / (1.0 + k));
-    float4 *out = J.tab + ((size_t)g * J.NP1 + n) * n_j;
-    DF gp = DF{0.0f, 0.0f}, gc = DF{1.0f, 0.0f};
-    for (int j = 0; j < n_j; ++j) {
-        float4 c = scf[j];
-        float r3n = (j + 1 < n_j) ? scf[j + 1].z : 0.0f;
-        DF t = df_mul(df_mul(sA[j], gc), gc);
-        out[j] = make_float4(c.x, c.y, r3n, t.h + t.l);
-        DF al = df_add(srb[3 * j], df_mul(srb[3 * j + 1], x));
-        DF gn = df_add(df_mul(al, gc), df_mul(srb[3 * j + 2], gp));
-        gp = gc;
-        gc = gn;
-    }
-}
-
-size_t gim_table_smem(int n_j) { return (size_t)n_j * (sizeof(float4) + 4 * sizeof(DF)); }
-
-// The same table from the standalone launch (the Chebyshev path's side
-// stream), with the chain threads doing only the recurrence: a chain runs
-// alone on its scheduler, so its time is the length of its instruction
-// stream.  Per CTA: order n, TABLE_GPC2 geometries.  All threads first form
-// r1_j + r2_j x of every geometry and step, the chain threads (one per
-// geometry) then run G_{j+1} = (r1 + r2 x) G_j + r3 G_{j-1} and keep each
-// G_j, and all threads finally form T_{n,j} = A_{n,j} G_j^2 and store the
-// packed rows.  The double-float operations are those of table_cta, so the
-// table is bitwise the same.
-constexpr int TABLE_GPC2 = 16;
-
-size_t gim_table2_smem(int n_j)
-{
-    return (size_t)n_j * (sizeof(float4) + 4 * sizeof(DF)) + 2 * (size_t)TABLE_GPC2 * (n_j + 1) * sizeof(DF) +
-           TABLE_GPC2 * sizeof(DF);
-}
-
-__device__ __forceinline__ void table_cta2(const TableJob &J, int n, int gb)
-{
-    extern __shared__ __align__(16) unsigned char tsm[];
-    const int n_j = J.n_j;
-    float4 *scf = reinterpret_cast<float4 *>(tsm);   // [n_j]
-    DF *sA = reinterpret_cast<DF *>(scf + n_j);      // [n_j]
-    DF *srb = sA + n_j;                              // [n_j][3]
-    // rows of n_j + 1: the chain lanes, one geometry each, read and write
-    // their rows at the same step without bank conflicts
-    const int rs = n_j + 1;
-    DF *sal = srb + 3 * n_j;                         // [TABLE_GPC2][n_j + 1]: r1_j + r2_j x
-    DF *sG = sal + TABLE_GPC2 * rs;                  // [TABLE_GPC2][n_j + 1]: G_j
-    DF *sx = sG + TABLE_GPC2 * rs;                   // [TABLE_GPC2]: x = 1 - b
-    const int tid = threadIdx.x;
-    const int g0 = gb * TABLE_GPC2;
-    const int ng = min(TABLE_GPC2, J.n_geom - g0);
-    for (int i = tid; i < n_j; i += blockDim.x) {
-        scf[i] = J.coef[(size_t)n * n_j + i];
-        sA[i] = df_of(J.A[(size_t)n * n_j + i]);
-    }
-    for (int i = tid; i < 3 * n_j; i += blockDim.x) srb[i] = df_of(J.recb[(size_t)n * n_j * 3 + i]);
-    if (tid < ng) {
-        const double k = J.k[g0 + tid];
-        sx[tid] = df_of(1.0 - k / (1.0 + k));
-    }
-    __syncthreads();
-    for (int j = tid; j < n_j; j += blockDim.x)
-        for (int gl = 0; gl < ng; ++gl) sal[gl * rs + j] = df_add(srb[3 * j], df_mul(srb[3 * j + 1], sx[gl]));
-    __syncthreads();
-    if (tid < ng) {
-        const DF *al = sal + tid * rs;
-        DF *G = sG + tid * rs;
-        // G_{j+1} = al_j G_j + r3_j G_{j-1}; q = r3_j G_{j-1} is formed one
-        // step ahead, so each step's dependent path is one df_mad
-        DF gc = DF{1.0f, 0.0f}, q = DF{0.0f, 0.0f};
-        for (int j = 0; j < n_j; ++j) {
-            G[j] = gc;
-            const DF gn = df_mad(al[j], gc, q);
-            if (j + 1 < n_j) q = df_mul(srb[3 * (j + 1) + 2], gc);
-            gc = gn;
-        }
-    }
-    __syncthreads();
-    for (int j = tid; j < n_j; j += blockDim.x) {
-        const float4 c = scf[j];
-        const float r3n = (j + 1 < n_j) ? scf[j + 1].z : 0.0f;
-        for (int gl = 0; gl < ng; ++gl) {
-            const DF gc = sG[gl * rs + j];
-            const DF t = df_mul(df_mul(sA[j], gc), gc);
-            J.tab[((size_t)(g0 + gl) * J.NP1 + n) * n_j + j] = make_float4(c.x, c.y, r3n, t.h + t.l);
-        }
-    }
-}
-
-// One CTA covers TT times x GW_VT geometries.  The first pass of the window
-// test (as pt::maybe_in_window, but with its margin bounded once per tile and
-// geometry from the tile's largest |t_h|) costs a subtraction, a product, a
-// rounding, an FMA and two comparisons per pair against constants staged in
-// shared memory; candidates then take the exact double-float test.  Appends
-// in two passes over a per-thread bit mask: ballots count each warp's pairs
-// per geometry, one global atomic per geometry reserves the CTA's stretch of
-// its list, and the same ballots place every pair (warp order, then lane
-// order) inside that stretch.  Every other pair gets flux 1.
-__device__ __forceinline__ void window_cta(const GimArgs &A, int bx, int by)
-{
-    constexpr int NW = TT / 32;
-    __shared__ GeomRec srec[GW_VT];
-    __shared__ float4 stest[GW_VT];   // t0_h, 1/P, P_h, win_lo - m
-    __shared__ float shi[GW_VT];      // win_hi + m
-    __shared__ int swc[NW][GW_VT];    // pairs per (warp, geometry), then the warp's offset
-    __shared__ int sbase[GW_VT];
-    __shared__ float swmax[NW];
-    const int tl = threadIdx.x, lane = tl & 31, warp = tl >> 5;
-    const int g0 = by * GW_VT;
-    const int ng = min(GW_VT, A.n_geom - g0);
-    for (int i = tl; i < ng * 6; i += TT) {
-        int vl = i / 6, c = i % 6;
-        reinterpret_cast<float4 *>(&srec[vl])[c] = reinterpret_cast<const float4 *>(&A.rec[g0 + vl])[c];
-    }
-    const int t = bx * TT + tl;
-    const bool tv = t < A.n_t;
-    const float2 ts = tv ? A.tsplit[t] : make_float2(0.0f, 0.0f);
-    // the tile's largest |t_h| (non-negative floats order like their bits)
-    float am = __int_as_float(__reduce_max_sync(0xffffffffu, __float_as_int(fabsf(ts.x))));
-    if (lane == 0) swmax[warp] = am;
-    __syncthreads();
-    if (tl < ng) {
-        float tmax = swmax[0];
-        for (int w = 1; w < NW; ++w) tmax = fmaxf(tmax, swmax[w]);
-        const GeomRec &r = srec[tl];
-        // the margin of pt::maybe_in_window with |s| <= |t_h| + |t0_h|,
-        // |n| P_h <= |s| + P_h / 2 and |d| <= P_h / 2
-        float m = 1.2e-7f * (3.0f * tmax + 3.0f * fabsf(r.t0h) + r.Ph) + 1e-9f;
-        stest[tl] = make_float4(r.t0h, r.invP, r.Ph, r.win_lo - m);
-        shi[tl] = r.win_hi + m;
-    }
-    __syncthreads();
-    unsigned bits = 0u;
-    if (tv) {
-        const float th = ts.x;
-        // first pass without branches: a mask of the candidates ...
-        unsigned cand = 0u;
-#pragma unroll 8
-        for (int vl = 0; vl < ng; ++vl) {
-            const float4 q = stest[vl];
-            const float sv = th - q.x;
-            const float d = fmaf(-rintf(sv * q.y), q.z, sv);
-            cand |= ((d >= q.w) & (d <= shi[vl])) ? (1u << vl) : 0u;
-        }
-        // ... then the exact test for those only
-        for (unsigned rest = cand; rest; rest &= rest - 1u) {
-            const int vl = __ffs(rest) - 1;
-            const float dt = pt::reduce_time(th, ts.y, srec[vl]);
-            if ((dt >= srec[vl].win_lo) && (dt <= srec[vl].win_hi)) bits |= 1u << vl;
-        }
-    }
-    // geometries with a pair in this warp (the ballots below visit only those)
-    const unsigned wbits = __reduce_or_sync(0xffffffffu, bits);
-    if (lane < GW_VT) swc[warp][lane] = 0;
-    __syncwarp();
-    for (unsigned rest = wbits; rest; rest &= rest - 1u) {
-        const int vl = __ffs(rest) - 1;
-        unsigned mb = __ballot_sync(0xffffffffu, (bits >> vl) & 1u);
-        if (lane == 0) swc[warp][vl] = __popc(mb);
-    }
-    __syncthreads();
-    if (tl < ng) {   // per geometry: warp offsets, then one reservation
-        int run = 0;
-        for (int w = 0; w < NW; ++w) {
-            int c = swc[w][tl];
-            swc[w][tl] = run;
-            run += c;
-        }
-        sbase[tl] = run > 0 ? atomicAdd(A.cnt + g0 + tl, run) : 0;
-    }
-    __syncthreads();
-    {
-        const unsigned lt = (1u << lane) - 1u;
-        for (unsigned rest = wbits; rest; rest &= rest - 1u) {
-            const int vl = __ffs(rest) - 1;
-            const bool in = (bits >> vl) & 1u;
-            unsigned mb = __ballot_sync(0xffffffffu, in);
-            if (in) A.list[(size_t)(g0 + vl) * A.n_t + sbase[vl] + swc[warp][vl] + __popc(mb & lt)] = t;
-        }
-    }
-    if (tv) {
-        const size_t row_stride = (size_t)A.n_t;
-        float *fp = A.flux + (size_t)g0 * A.n_bpg * row_stride + t;
-        if (A.n_bpg == 1) {
-#pragma unroll 8
-            for (int vl = 0; vl < ng; ++vl, fp += row_stride)
-                if (!((bits >> vl) & 1u)) *fp = 1.0f;
-        } else {
-            for (int vl = 0; vl < ng; ++vl)
-                for (int bb = 0; bb < A.n_bpg; ++bb, fp += row_stride)
-                    if (!((bits >> vl) & 1u)) *fp = 1.0f;
-        }
-    }
-}
-
-// One launch: J.n_blocks table CTAs first (they start first and run in the
-// shadow of the window CTAs), then n_tiles x ceil(n_geom / GW_VT) window CTAs.
-__global__ void __launch_bounds__(TT) gim_window_kernel(GimArgs A, TableJob J, int n_tiles)
-{
-    int id = blockIdx.x;
-    if (id < J.n_blocks) {
-        table_cta(J, id % J.NP1, id / J.NP1);
-        return;
-    }
-    id -= J.n_blocks;
-    window_cta(A, id % n_tiles, id / n_tiles);
-}
-
-// The table alone (table_cta2): the Chebyshev path launches it on the plan's
-// side stream at the start of the call (it needs only k), beside the set-up
-// and window kernels.
-__global__ void __launch_bounds__(TT) gim_table_kernel(TableJob J)
-{
-    table_cta2(J, blockIdx.x % J.NP1, blockIdx.x / J.NP1);
-}
-
-// pref[g] = sum over g' < g of ceil(cnt[g'] / ppi); pref[n_geom] = total.
-// One CTA of 1024 threads; also rewinds the evaluation kernels' item counter.
-// Work items in a cost order: geometries sorted by an estimate of the
-// in-transit supersamples per listed pair, largest first, so that the items
-// handed out last are the cheap ones and the persistent CTAs finish close
-// together.  The window of a geometry is its transit plus half an exposure on
-// each side (and margins), so a listed pair is in transit for about a
-// fraction (W - t_exp) / W of its exposure, W = win_hi - win_lo.  Ties (and
-// every geometry when there is no exposure time) keep their index order.
-// gord[p] is the geometry at position p; pref[p] the items before position p.
-// Up to 1,024 geometries each thread counts the geometries before its own
-// (no barriers), up to SCAN_SORT_MAX a bitonic sort in shared memory, above
-// that the order is the index order.  The Mandel-Agol pairs kernel (order =
-// false: items of a few microseconds, and measured slower with the cost
-// order) takes the index order.
-constexpr int SCAN_SORT_MAX = 4096;
-
-__device__ __forceinline__ float scan_key(const int *cnt, const GeomRec *rec, float t_exp, int g)
-{
-    const float w = rec[g].win_hi - rec[g].win_lo;
-    return (cnt[g] > 0 && w > 0.0f) ? fmaxf(w - t_exp, 0.0f) / w : -1.0f;
-}
-
-__global__ void __launch_bounds__(1024) gim_scan_kernel(const int *cnt, const GeomRec *rec, float t_exp, int n_geom,
-                                                        int ppi, bool order, int *pref, int *gord, int *ctr)
-{
-    __shared__ int swarp[32];
-    __shared__ int scarry;
-    __shared__ float skey[SCAN_SORT_MAX];
-    __shared__ int sidx[SCAN_SORT_MAX];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nwarp = blockDim.x >> 5;
-    const bool sorted = order && n_geom <= SCAN_SORT_MAX;
-    if (threadIdx.x == 0) {
-        scarry = 0;
-        *ctr = 0;
-    }
-    if (sorted && n_geom <= (int)blockDim.x) {
-        // one thread per geometry: its position is the number of geometries
-        // before it in the order
-        const int i = threadIdx.x;
-        if (i < n_geom) skey[i] = scan_key(cnt, rec, t_exp, i);
-        __syncthreads();
-        if (i < n_geom) {
-            const float ki = skey[i];
-            int r = 0;
-            for (int j = 0; j < n_geom; ++j) {
-                const float kj = skey[j];
-                r += (kj > ki || (kj == ki && j < i)) ? 1 : 0;
-            }
-            sidx[r] = i;
-        }
-        __syncthreads();
-    } else if (sorted) {
-        int n2 = 1;
-        while (n2 < n_geom) n2 <<= 1;
-        for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-            skey[i] = i < n_geom ? scan_key(cnt, rec, t_exp, i) : -2.0f;   // padding sorts last
-            sidx[i] = i;
-        }
-        __syncthreads();
-        // bitonic sort: key descending, index ascending among equal keys
-        for (int kk = 2; kk <= n2; kk <<= 1) {
-            for (int j = kk >> 1; j > 0; j >>= 1) {
-                for (int i = threadIdx.x; i < n2; i += blockDim.x) {
-                    const int l = i ^ j;
-                    if (l > i) {
-                        const float ki = skey[i], kl = skey[l];
-                        const int ii = sidx[i], il = sidx[l];
-                        const bool i_first = ki > kl || (ki == kl && ii < il);
-                        const bool up = (i & kk) == 0;   // this block in the final order
-                        if (up != i_first) {
-                            skey[i] = kl;
-                            skey[l] = ki;
-                            sidx[i] = il;
-                            sidx[l] = ii;
-                        }
-                    }
-                }
-                __syncthreads();
-            }
-        }
-    }
-    for (int p = threadIdx.x; p < n_geom; p += blockDim.x) gord[p] = sorted ? sidx[p] : p;
-    __syncthreads();
-    for (int base = 0; base < n_geom; base += blockDim.x) {
-        int p = base + threadIdx.x;
-        int v = (p < n_geom) ? (cnt[sorted ? sidx[p] : p] + ppi - 1) / ppi : 0;
-        int x = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            int y = __shfl_up_sync(0xffffffffu, x, o);
-            if (lane >= o) x += y;
-        }
-        if (lane == 31) swarp[warp] = x;
-        __syncthreads();
-        if (warp == 0) {
-            int w = (lane < nwarp) ? swarp[lane] : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                int y = __shfl_up_sync(0xffffffffu, w, o);
-                if (lane >= o) w += y;
-            }
-            swarp[lane] = w;
-        }
-        __syncthreads();
-        int incl = scarry + (warp > 0 ? swarp[warp - 1] : 0) + x;
-        if (p < n_geom) pref[p] = incl - v;
-        __syncthreads();
-        if (threadIdx.x == blockDim.x - 1) scarry = incl;
-        __syncthreads();
-    }
-    if (threadIdx.x == 0) pref[n_geom] = scarry;
-}
-
-// ---------------------------------------------------------------------------
-// Chebyshev form of the series.  For one geometry and order n,
-//   S_n(x) = sum_{j < n_j} T_{n,j} G_j(nu+2, 1; x)
-// is a polynomial of degree n_j - 1 in x, so it has an exact expansion
-//   S_n(x) = sum_{m < n_j} d_{n,m} T_m(y),   y = 2x - 1.
-// The Chebyshev basis does not depend on n, so one recurrence
-// T_{m+1} = 2y T_m - T_{m-1} per supersample serves all N + 1 orders:
-// N + 2 FMAs per term instead of 3 (N + 1).
-// gim_cheb_coef_kernel forms the d_{n,m} by Clenshaw's backward summation of
-// the Jacobi series (the recursion of Sec. 2.1.4, the table's r1_j, r2_j,
-// r3_{j+1}, T_{n,j}),
-//   b_j = T_j + (r1_j + r2_j x) b_{j+1} + r3_{j+1} b_{j+2},   S_n = b_0,
-// carried out on Chebyshev coefficient vectors instead of values: with
-// x = (1 + y)/2, multiplying by x is (1/2)(b + y b), and y T_m =
-// (T_{m+1} + T_{m-1})/2 (y T_0 = T_1), so (y b)_m = (b_{m-1} + b_{m+1})/2,
-// (y b)_0 = b_1 / 2, (y b)_1 = b_0 + b_2 / 2.  Each step touches every
-// coefficient once (about n_j^2 / 2 x 3 FMAs per order in all); in FP32 the
-// alpha_n it leads to stay within ~1e-7 of the FP64 series (emulated at
-// n_j = 192 over k = 0.05 .. 0.2), the level of the FP32 evaluation.
-// One warp per (geometry, order): lane l holds coefficients l S .. l S + S - 1
-// in registers, so a step needs the two neighbours across lanes only (two
-// shuffles); the table row sits in the warp's shared memory, read by
-// broadcast.  Warps for the row padding (orders N + 1 .. DS - 1) write zeros.
-// ---------------------------------------------------------------------------
-constexpr int CW_WARPS = 1;   // warps per CTA of the coefficient kernel (one: the scheduler spreads the chains evenly)
-
-template <int S>
-__global__ void __launch_bounds__(32 * CW_WARPS) gim_cheb_coef_kernel(const float4 *gtab, int NP1, int n_j, int DS,
-                                                                     float *dtab)
-{
-    extern __shared__ __align__(16) float4 ctab_sm[];   // [CW_WARPS][n_j]
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = blockIdx.x;
-    const int n = blockIdx.y * CW_WARPS + warp;
-    if (n >= DS) return;   // a whole warp; the kernel has no CTA-wide barrier
-    float *out = dtab + (size_t)g * n_j * DS + n;   // d_{n,m} at out[m DS]
-    if (n >= NP1) {
-        for (int m = lane; m < n_j; m += 32) out[(size_t)m * DS] = 0.0f;
-        return;
-    }
-    float4 *tab = ctab_sm + warp * n_j;
-    const float4 *src = gtab + ((size_t)g * NP1 + n) * n_j;
-    for (int j = lane; j < n_j; j += 32) tab[j] = src[j];
-    __syncwarp();
-    float b1[S], b2[S];
-    float wl[S];   // weight of the lower neighbour in (y b)_m: 1/2, 1 at m = 1, 0 at m = 0
-    const int m0 = lane * S;
-#pragma unroll
-    for (int s = 0; s < S; ++s) {
-        b1[s] = b2[s] = 0.0f;
-        wl[s] = (m0 + s == 0) ? 0.0f : (m0 + s == 1 ? 1.0f : 0.5f);
-    }
-    // one step: from (bn = b_{j+1}, bo = b_{j+2}) to b_j, written over bo
-    auto step = [&](int j, float (&bn)[S], float (&bo)[S]) {
-        const float4 c = tab[j];
-        const float a = fmaf(0.5f, c.y, c.x);   // the part of r1 + r2 x without y
-        const float h = 0.5f * c.y;             // the coefficient of y b
-        const float left = __shfl_up_sync(0xffffffffu, bn[S - 1], 1);   // b_{m0 - 1}
-        const float right = __shfl_down_sync(0xffffffffu, bn[0], 1);   // b_{m0 + S}
-#pragma unroll
-        for (int s = 0; s < S; ++s) {
-            const float bl = (s == 0) ? left : bn[s - 1];
-            const float br = (s == S - 1) ? (lane == 31 ? 0.0f : right) : bn[s + 1];
-            const float yb = fmaf(wl[s], bl, 0.5f * br);
-            bo[s] = fmaf(a, bn[s], fmaf(h, yb, c.z * bo[s]));
-        }
-        if (lane == 0) bo[0] += c.w;             // + T_j (degree 0)
-    };
-    int j = n_j - 1;
-#pragma unroll 1
-    for (; j >= 1; j -= 2) {
-        step(j, b1, b2);       // b_j into b2
-        step(j - 1, b2, b1);   // b_{j-1} into b1
-    }
-    if (j == 0) {
-        step(0, b1, b2);
-#pragma unroll
-        for (int s = 0; s < S; ++s) b1[s] = b2[s];
-    }
-#pragma unroll
-    for (int s = 0; s < S; ++s)
-        if (m0 + s < n_j) out[(size_t)(m0 + s) * DS] = b1[s];
-}
-
-// coefficients per lane of the coefficient kernel for a series depth
-int gim_cheb_coef_s(int n_j) { return (n_j + 31) / 32; }
-
-// Evaluation over the pair lists.  Persistent CTAs take items of GS_THREADS
-// listed pairs of one geometry and stage its coefficient rows once per item.
-// An item runs in batches of up to GS_SSB supersamples:
-//  1. each thread (one pair) computes z at the batch's supersamples and keeps
-//     the in-transit ones, (y = 2x - 1, q = sqrt(1 - x)) with x = c^2, in
-//     order; a scan over the CTA places every pair's entries in one dense
-//     list (pair-major, supersample-minor);
-//  2. the list is cut into rounds; in a round each thread evaluates G
-//     consecutive entries, whatever pairs they belong to, so that no lane
-//     idles on an out-of-transit supersample: one Chebyshev recurrence per
-//     entry, T_{m+1} = 2y T_m - T_{m-1}, and one FMA per order n and m for
-//     d_{n,m} T_m, two orders per two-lane FMA instruction (fma.rn.f32x2:
-//     a third fewer instructions than scalar FMAs, and measured on this
-//     part 0.68 of the FP32 peak in series multiply-adds against 0.52 for
-//     the scalar form of the same loop).  Rounds of GS_GMAX = 4 entries per
-//     thread while at least 4 GS_THREADS entries are left, then one round of
-//     the fewest entries per thread (1 to 3) that holds the rest (each
-//     coefficient load serves the thread's entries).  The S_n go to shared
-//     memory;
-//  3. each thread adds its own pair's b^2 q^(n+4) S_n to alpha_n in
-//     supersample order, so the sums do not depend on the rounds.
-// After the last batch, the passband combination of Sec. 2.1.3.
-constexpr int GS_SSB = 16;    // supersamples per batch of the Chebyshev kernel
-constexpr int GS_GMAX = 4;    // entries per thread in the largest round
-constexpr int GS_WROWS = 8;   // passbands whose combination weights are staged per geometry
-
-// The geometry of work item it: the largest g with pref[g] <= it (pref is
-// non-decreasing, pref[0] = 0 <= it), found by one warp: each round splits
-// [lo, hi] into 32 strides and loads their first entries in parallel, the
-// lanes whose entry is <= it form a prefix, and its last lane brackets the
-// answer.  Two rounds (two dependent loads) up to 1,024 geometries.
-__device__ __forceinline__ int item_geometry(const int *pref, int n_geom, int it, int lane)
-{
-    int lo = 0, hi = n_geom - 1;
-    for (;;) {
-        const int step = (hi - lo + 32) / 32;   // ceil((hi - lo + 1) / 32)
-        const int idx = lo + lane * step;
-        const bool ok = idx <= hi && pref[idx] <= it;
-        const unsigned m = __ballot_sync(0xffffffffu, ok);
-        lo += (31 - __clz(m)) * step;
-        if (step == 1) return lo;
-        hi = min(hi, lo + step - 1);
-    }
-}
-
-// (a0, a1) += (d0, d1) w as one two-lane FMA (sm_100 and later).  Each lane
-// is a fused multiply-add rounded once, so the result is that of two fmaf.
-__device__ __forceinline__ void fma2_pair(float d0, float d1, float w, float &a0, float &a1)
-{
-    float2 a = make_float2(a0, a1);
-    const float2 d = make_float2(d0, d1);
-    const float2 ww = make_float2(w, w);
-    asm("fma.rn.f32x2 %0, %1, %2, %0;"
-        : "+l"(*reinterpret_cast<unsigned long long *>(&a))
-        : "l"(*reinterpret_cast<const unsigned long long *>(&d)), "l"(*reinterpret_cast<const unsigned long long *>(&ww)));
-    a0 = a.x;
-    a1 = a.y;
-}
-
-template <int NP1, int G>
-__device__ __forceinline__ void cheb_eval(const float *sd, int nj, const float (&y)[G], float (&acc)[G][NP1])
-{
-    constexpr int DS = (NP1 + 3) & ~3;
-    float wa[G], wb[G], a2[G];
-#pragma unroll
-    for (int e = 0; e < G; ++e) {
-        a2[e] = y[e] + y[e];
-        wa[e] = 1.0f;
-        wb[e] = y[e];
-#pragma unroll
-        for (int n = 0; n < NP1; ++n) acc[e][n] = fmaf(sd[DS + n], wb[e], sd[n]);
-    }
-    // one step: T_m = 2y T_{m-1} - T_{m-2} in place of T_{m-2} (wa for even m,
-    // wb for odd m, so the loop carries no register copies)
-    auto step = [&](int m, float (&wn)[G], const float (&wp)[G]) {
-        float dm[DS];
-        const float4 *row = reinterpret_cast<const float4 *>(sd + m * DS);
-#pragma unroll
-        for (int n = 0; n < DS; n += 4) {
-            const float4 v = row[n / 4];
-            dm[n] = v.x;
-            dm[n + 1] = v.y;
-            dm[n + 2] = v.z;
-            dm[n + 3] = v.w;
-        }
-#pragma unroll
-        for (int e = 0; e < G; ++e) {
-            wn[e] = fmaf(a2[e], wp[e], -wn[e]);
-            // orders in pairs through the two-lane FMA (each lane one FMA,
-            // rounded once: the same result as two fmaf), the odd last order
-            // scalar
-#pragma unroll
-            for (int n = 0; n + 1 < NP1; n += 2) fma2_pair(dm[n], dm[n + 1], wn[e], acc[e][n], acc[e][n + 1]);
-            if (NP1 & 1) acc[e][NP1 - 1] = fmaf(dm[NP1 - 1], wn[e], acc[e][NP1 - 1]);
-        }
-    };
-    int m = 2;
-#pragma unroll 2
-    for (; m + 1 < nj; m += 2) {
-        step(m, wa, wb);
-        step(m + 1, wb, wa);
-    }
-    if (m < nj) step(m, wa, wb);
-}
-
-// One round: entries [r0, r0 + G GS_THREADS) of the dense list (those below
-// n_e), G consecutive ones per thread; S_n to sS[n][slot].
-template <int NP1, int G>
-__device__ __forceinline__ void cheb_round(const float *sd, int nj, const float2 *syq, const int *sst, float *sS,
-                                           int r0, int n_e)
-{
-    constexpr int CH = GS_GMAX * GS_THREADS;
-    const int tid = threadIdx.x;
-    const int e0 = r0 + G * tid;
-    if (e0 >= n_e) return;
-    float y[G];
-    int p = 0;
-    {
-        int lo = 0, hi = GS_THREADS - 1;   // the last pair with sst[p] <= e0
-        while (lo < hi) {
-            const int mid = (lo + hi + 1) >> 1;
-            if (sst[mid] <= e0) lo = mid;
-            else hi = mid - 1;
-        }
-        p = lo;
-    }
-#pragma unroll
-    for (int u = 0; u < G; ++u) {
-        const int e = e0 + u;
-        y[u] = 0.0f;
-        if (e < n_e) {
-            while (sst[p + 1] <= e) ++p;
-            y[u] = syq[(e - sst[p]) * GS_THREADS + p].x;
-        }
-    }
-    float acc[G][NP1];
-    cheb_eval<NP1, G>(sd, nj, y, acc);
-#pragma unroll
-    for (int n = 0; n < NP1; ++n) {
-        float *dst = sS + n * CH + G * tid;
-        if (G % 4 == 0) {
-#pragma unroll
-            for (int u = 0; u < G; u += 4)
-                *reinterpret_cast<float4 *>(dst + u) = make_float4(acc[u][n], acc[u + 1][n], acc[u + 2][n], acc[u + 3][n]);
-        } else if (G % 2 == 0) {
-#pragma unroll
-            for (int u = 0; u < G; u += 2) *reinterpret_cast<float2 *>(dst + u) = make_float2(acc[u][n], acc[u + 1][n]);
-        } else {
-#pragma unroll
-            for (int u = 0; u < G; ++u) dst[u] = acc[u][n];
-        }
-    }
-}
-
-template <int NP1>
-__global__ void __launch_bounds__(GS_THREADS, 5) gim_cheb_kernel(GimArgs A, const float *dtab)
-{
-    constexpr int DS = (NP1 + 3) & ~3;        // floats per coefficient row
-    constexpr int CH = GS_GMAX * GS_THREADS;  // entries of the largest round
-    const int nj = A.n_j;
-    const int nss = A.n_ss;
-    const int ssb = min(nss, GS_SSB);
-    extern __shared__ __align__(16) unsigned char dsm[];
-    float *sd = reinterpret_cast<float *>(dsm);                  // [n_j][DS] coefficient rows
-    float *sS = sd + nj * DS;                                    // [NP1][CH] series values of a round
-    float2 *syq = reinterpret_cast<float2 *>(sS + NP1 * CH);     // [ssb][GS_THREADS] (y, q) per pair
-    __shared__ GeomRec srec;
-    __shared__ int sitem, sgeom, sfirst, scount, sbad;
-    __shared__ float swt[GS_WROWS][NP1 + 1];   // per passband: 1 - sum u, u_1..u_N, D
-    __shared__ int sst[GS_THREADS + 1];   // first dense entry of each pair; sst[GS_THREADS] = entries
-    __shared__ int swarp[GS_THREADS / 32];
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int total = A.pref[A.n_geom];
-    const float inv_nss = 1.0f / (float)nss;
-    int nbad = 0;
-    int staged = -1;
-    if (tid == 0) sbad = 0;
-#pragma unroll 1
-    for (;;) {
-        if (warp == 0) {
-            int it = 0;
-            if (lane == 0) it = atomicAdd(A.ctr, 1);
-            it = __shfl_sync(0xffffffffu, it, 0);
-            if (it < total) {
-                const int pos = item_geometry(A.pref, A.n_geom, it, lane);
-                if (lane == 0) {
-                    const int g = A.gord[pos];
-                    sgeom = g;
-                    sfirst = A.pref[pos];
-                    scount = A.cnt[g];
-                }
-            }
-            if (lane == 0) sitem = it;
-        }
-        __syncthreads();
-        const int it = sitem;
-        const int g = sgeom;
-        if (it >= total) break;   // uniform over the CTA
-        if (g != staged) {
-            const float4 *src = reinterpret_cast<const float4 *>(dtab + (size_t)g * nj * DS);
-            float4 *dst = reinterpret_cast<float4 *>(sd);
-            for (int i = tid; i < nj * DS / 4; i += GS_THREADS) dst[i] = src[i];
-            if (tid < 6) reinterpret_cast<float4 *>(&srec)[tid] = reinterpret_cast<const float4 *>(&A.rec[g])[tid];
-            if (tid < A.n_bpg && tid < GS_WROWS) {
-                // C_0 D = 1 - sum u, C_n D = u_n, D = 1 - sum n u_n/(n+2)   (Sec. 2.1.3)
-                const float *u = A.ld + ((size_t)g * A.n_bpg + tid) * A.N;
-                float su = 0.0f, sdn = 0.0f;
-#pragma unroll
-                for (int n = 1; n < NP1; ++n) {
-                    const float un = u[n - 1];
-                    su += un;
-                    sdn += (float)n * un / (float)(n + 2);
-                    swt[tid][n] = un;
-                }
-                swt[tid][0] = 1.0f - su;
-                swt[tid][NP1] = 1.0f - sdn;
-            }
-            staged = g;
-        }
-        __syncthreads();
-        const int i = (it - sfirst) * GS_THREADS + tid;
-        const bool own = i < scount;
-        const int t = own ? A.list[(size_t)g * A.n_t + i] : 0;
-        float dt = 0.0f;
-        if (own) {
-            const float2 ts = A.tsplit[t];
-            dt = pt::reduce_time(ts.x, ts.y, srec);
-        }
-        const float kk = srec.k;
-        const float bk = kk / (1.0f + kk);
-        const float b2 = bk * bk;
-        float al[NP1];   // alpha sums over the supersamples
-#pragma unroll
-        for (int n = 0; n < NP1; ++n) al[n] = 0.0f;
-        float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
-#pragma unroll 1
-        for (int sb0 = 0; sb0 < nss; sb0 += ssb) {
-            // 1. in-transit supersamples of this pair, in order
-            int c = 0;
-            if (own) {
-                const int s1 = min(nss, sb0 + ssb);
-#pragma unroll 1
-                for (int s = sb0; s < s1; ++s) {
-                    bool bad = false;
-                    const float z = pt::orbit_z<true, true>(srec, dt + ss_offset(A.t_exp, s, inv_nss), A.max_iter, &bad, warm);
-                    if (bad) ++nbad;
-                    if (z < 1.0f + kk) {
-                        // z < 1 + k; the rounded reciprocal may put cz an ulp above 1
-                        const float cz = fminf(z * pt::rcp_a(1.0f + kk), 1.0f);
-                        const float x = cz * cz;
-                        // (1 - cz)(1 + cz) is 0 or at least ~2^-24: a normal argument
-                        syq[c * GS_THREADS + tid] = make_float2(fmaf(2.0f, x, -1.0f), pt::sqrt_a((1.0f - cz) * (1.0f + cz)));
-                        ++c;
-                    }
-                }
-            }
-            // exclusive scan of the counts over the CTA
-            int incl = c;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            if (lane == 31) swarp[warp] = incl;
-            __syncthreads();
-            int base = 0;
-#pragma unroll
-            for (int w = 0; w < GS_THREADS / 32; ++w) base += (w < warp) ? swarp[w] : 0;
-            sst[tid] = base + incl - c;
-            if (tid == GS_THREADS - 1) sst[GS_THREADS] = base + incl;
-            __syncthreads();
-            const int n_e = sst[GS_THREADS];
-            const int my0 = sst[tid];
-            int r0 = 0;
-#pragma unroll 1
-            while (r0 < n_e) {
-                // 2. a round of series values; its size from what is left
-                const int rem = n_e - r0;
-                int size;
-                const int gfit = (rem + GS_THREADS - 1) / GS_THREADS;   // the last round fits what is left
-                if (gfit >= GS_GMAX) {
-                    cheb_round<NP1, GS_GMAX>(sd, nj, syq, sst, sS, r0, n_e);
-                    size = GS_GMAX * GS_THREADS;
-                } else if (gfit == 3) {
-                    cheb_round<NP1, 3>(sd, nj, syq, sst, sS, r0, n_e);
-                    size = 3 * GS_THREADS;
-                } else if (gfit == 2) {
-                    cheb_round<NP1, 2>(sd, nj, syq, sst, sS, r0, n_e);
-                    size = 2 * GS_THREADS;
-                } else {
-                    cheb_round<NP1, 1>(sd, nj, syq, sst, sS, r0, n_e);
-                    size = GS_THREADS;
-                }
-                __syncthreads();
-                // 3. this pair's entries of the round, in supersample order:
-                //    alpha_n += b^2 q^(n+4) S_n
-                const int ea = max(my0, r0), eb = min(my0 + c, r0 + size);
-#pragma unroll 1
-                for (int e = ea; e < eb; ++e) {
-                    const float qu = syq[(e - my0) * GS_THREADS + tid].y;
-                    const float qq = qu * qu;
-                    float w = b2 * qq * qq;
-#pragma unroll
-                    for (int n = 0; n < NP1; n += 2) {
-                        al[n] = fmaf(sS[n * CH + (e - r0)], w, al[n]);
-                        if (n + 1 < NP1) al[n + 1] = fmaf(sS[(n + 1) * CH + (e - r0)], w * qu, al[n + 1]);
-                        w *= qq;
-                    }
-                }
-                __syncthreads();
-                r0 += size;
-            }
-        }
-        if (own) {
-#pragma unroll 1
-            for (int bb = 0; bb < A.n_bpg; ++bb) {
-                size_t row = (size_t)g * A.n_bpg + bb;
-                // C_0 = (1 - sum u)/D, C_n = u_n/D, D = 1 - sum n u_n/(n+2)   (Sec. 2.1.3);
-                // the first GS_WROWS passbands' (1 - sum u, u_n, D) were staged
-                // with the geometry, the others are formed here the same way
-                float wt[NP1 + 1];
-                if (bb < GS_WROWS) {
-#pragma unroll
-                    for (int n = 0; n <= NP1; ++n) wt[n] = swt[bb][n];
-                } else {
-                    const float *u = A.ld + row * A.N;
-                    float su = 0.0f, sdn = 0.0f;
-#pragma unroll
-                    for (int n = 1; n < NP1; ++n) {
-                        const float un = u[n - 1];
-                        su += un;
-                        sdn += (float)n * un / (float)(n + 2);
-                        wt[n] = un;
-                    }
-                    wt[0] = 1.0f - su;
-                    wt[NP1] = 1.0f - sdn;
-                }
-                float acc_f = wt[0] * al[0];
-#pragma unroll
-                for (int n = 1; n < NP1; ++n) acc_f = fmaf(wt[n], al[n], acc_f);
-                A.flux[row * A.n_t + t] = 1.0f - acc_f / wt[NP1] * inv_nss;
-            }
-        }
-    }
-    if (nbad) atomicAdd(&sbad, nbad);
-    __syncthreads();
-    if (tid == 0 && sbad && A.n_bad) atomicAdd(A.n_bad, sbad);
-}
-
-// floats per coefficient row: the N + 1 orders, padded to 16 bytes
-int gim_cheb_ds(int N) { return (N + 4) & ~3; }
-// coefficient rows, a round of series values and a batch of (y, q) entries
-size_t gim_cheb_smem(int n_j, int N, int n_ss)
-{
-    return ((size_t)n_j * gim_cheb_ds(N) + (size_t)(N + 1) * GS_GMAX * GS_THREADS) * sizeof(float) +
-           (size_t)GS_THREADS * (n_ss < GS_SSB ? n_ss : GS_SSB) * sizeof(float2);
-}
-
-// ---------------------------------------------------------------------------
-// Gimenez model interpolated in z (Sec. 3.3).  gim_zi_table_kernel evaluates
-// alpha_0..alpha_N of every geometry on its z nodes (n_in over [0, zb],
-// zb = max(1 - k, 0), then n_edge over (zb, 1 + k]) with the same Clenshaw
-// summation as the coefficient kernel's node values; gim_zi_kernel reads
-// them by linear interpolation for every listed (time, geometry) pair (one
-// thread per pair), with the same work items and passband combination as
-// the series evaluation.
-// ---------------------------------------------------------------------------
-constexpr int ZI_MAX_VALUES = 16384;   // (n_in + n_edge)(N + 1) per geometry
-
-struct ZiGrid {
-    float zb, h1, h2, inv_h1, inv_h2;
-};
-
-__device__ __forceinline__ ZiGrid zi_grid(float k, int n_in, int n_edge)
-{
-    ZiGrid q;
-    q.zb = fmaxf(1.0f - k, 0.0f);
-    q.h1 = q.zb / (float)(n_in - 1);
-    q.h2 = (1.0f + k - q.zb) / (float)n_edge;
-    q.inv_h1 = (q.zb > 0.0f) ? 1.0f / q.h1 : 0.0f;
-    q.inv_h2 = 1.0f / q.h2;
-    return q;
-}
-
-__global__ void __launch_bounds__(128) gim_zi_table_kernel(const GeomRec *rec, const float4 *gtab, int NP1, int n_j,
-                                                          int n_in, int n_edge, float *atab)
-{
-    const int g = blockIdx.x;
-    const int nz = n_in + n_edge;
-    const float kk = rec[g].k;
-    const ZiGrid G = zi_grid(kk, n_in, n_edge);
-    const float4 *tab = gtab + (size_t)g * NP1 * n_j;
-    const float bk = kk / (1.0f + kk);
-    const float b2 = bk * bk;
-    for (int i = threadIdx.x; i < nz; i += blockDim.x) {
-        float z = (i < n_in) ? (float)i * G.h1 : G.zb + (float)(i - n_in + 1) * G.h2;
-        float x = 0.0f, q = 0.0f;
-        if (z < 1.0f + kk) {
-            float c = z / (1.0f + kk);
-            x = c * c;
-            q = sqrtf((1.0f - c) * (1.0f + c));
-        }
-        float *out = atab + ((size_t)g * nz + i) * NP1;
-        for (int n = 0; n < NP1; ++n) {
-            const float4 *tn = tab + (size_t)n * n_j;
-            float c1 = 0.0f, c2 = 0.0f;
-            for (int j = n_j - 1; j >= 0; --j) {
-                float4 c = tn[j];
-                float bj = fmaf(fmaf(c.y, x, c.x), c1, fmaf(c.z, c2, c.w));
-                c2 = c1;
-                c1 = bj;
-            }
-            float qq = q * q;
-            float pw = qq * qq;
-            for (int m = 0; m < n; ++m) pw *= q;
-            out[n] = (b2 * pw) * c1;
-        }
-    }
-}
-
-__global__ void __launch_bounds__(GS_THREADS) gim_zi_kernel(GimArgs A, const float *atab, int n_in, int n_edge)
-{
-    extern __shared__ __align__(16) unsigned char dsm[];
-    const int NP1 = A.N + 1;
-    const int nz = n_in + n_edge;
-    float *stab = reinterpret_cast<float *>(dsm);   // [nz][N+1]
-    float *salpha = stab + nz * NP1;                // [N+1][GS_THREADS]
-    __shared__ GeomRec srec;
-    __shared__ int sitem, sgeom, sfirst, scount, sbad;
-
-    const int nss = A.n_ss;
-    const int tid = threadIdx.x;
-    const int lane = tid & 31, warp = tid >> 5;
-    const int total = A.pref[A.n_geom];
-    const float inv_nss = 1.0f / (float)nss;
-    int nbad = 0;
-    int staged = -1;
-    if (tid == 0) sbad = 0;
-
-#pragma unroll 1
-    for (;;) {
-        if (warp == 0) {
-            int it = 0;
-            if (lane == 0) it = atomicAdd(A.ctr, 1);
-            it = __shfl_sync(0xffffffffu, it, 0);
-            if (it < total) {
-                const int pos = item_geometry(A.pref, A.n_geom, it, lane);
-                if (lane == 0) {
-                    const int g = A.gord[pos];
-                    sgeom = g;
-                    sfirst = A.pref[pos];
-                    scount = A.cnt[g];
-                }
-            }
-            if (lane == 0) sitem = it;
-        }
-        __syncthreads();
-        const int it = sitem;
-        const int g = sgeom;
-        if (it >= total) break;   // uniform over the CTA
-        if (g != staged) {
-            const float *src = atab + (size_t)g * nz * NP1;
-            for (int i = tid; i < nz * NP1; i += GS_THREADS) stab[i] = src[i];
-            if (tid < 6) reinterpret_cast<float4 *>(&srec)[tid] = reinterpret_cast<const float4 *>(&A.rec[g])[tid];
-            staged = g;
-        }
-        for (int n = 0; n < NP1; ++n) salpha[n * GS_THREADS + tid] = 0.0f;
-        __syncthreads();
-        const int i = (it - sfirst) * GS_THREADS + tid;
-        if (i < scount) {
-            const int t = A.list[(size_t)g * A.n_t + i];
-            float2 ts = A.tsplit[t];
-            float dt = pt::reduce_time(ts.x, ts.y, srec);
-            const float kk = srec.k;
-            const ZiGrid G = zi_grid(kk, n_in, n_edge);
-            float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
-#pragma unroll 1
-            for (int s = 0; s < nss; ++s) {
-                bool bad = false;
-                float z = pt::orbit_z<true>(srec, dt + ss_offset(A.t_exp, s, inv_nss), A.max_iter, &bad, warm);
-                if (bad) ++nbad;
-                if (!(z < 1.0f + kk)) continue;   // out of transit: alpha = 0
-                int i0;
-                float w;
-                if (z <= G.zb && G.zb > 0.0f) {
-                    float f = z * G.inv_h1;
-                    i0 = min((int)f, n_in - 2);
-                    w = f - (float)i0;
-                } else if (z <= G.zb) {            // k >= 1: the first region is z = 0
-                    i0 = 0;
-                    w = 0.0f;
-                } else {
-                    float f = (z - G.zb) * G.inv_h2;
-                    int c = min((int)f, n_edge - 1);
-                    i0 = n_in - 1 + c;
-                    w = f - (float)c;
-                }
-                const float *a0 = stab + i0 * NP1;
-                for (int n = 0; n < NP1; ++n)
-                    salpha[n * GS_THREADS + tid] += fmaf(w, a0[NP1 + n] - a0[n], a0[n]);
-            }
-#pragma unroll 1
-            for (int bb = 0; bb < A.n_bpg; ++bb) {
-                size_t row = (size_t)g * A.n_bpg + bb;
-                const float *u = A.ld + row * A.N;
-                // C_0 = (1 - sum u)/D, C_n = u_n/D, D = 1 - sum n u_n/(n+2)   (Sec. 2.1.3)
-                float su = 0.0f, sd = 0.0f;
-                for (int n = 1; n <= A.N; ++n) {
-                    float un = u[n - 1];
-                    su += un;
-                    sd += (float)n * un / (float)(n + 2);
-                }
-                float al = (1.0f - su) * salpha[tid];
-                for (int n = 1; n <= A.N; ++n) al = fmaf(u[n - 1], salpha[n * GS_THREADS + tid], al);
-                A.flux[row * A.n_t + t] = 1.0f - al / (1.0f - sd) * inv_nss;
-            }
-        }
-    }
-    if (nbad) atomicAdd(&sbad, nbad);
-    __syncthreads();
-    if (tid == 0 && sbad && A.n_bad) atomicAdd(A.n_bad, sbad);
-}
-
-size_t gim_zi_smem(int N, int nz) { return (size_t)(N + 1) * (nz + GS_THREADS) * sizeof(float); }
 
 __global__ void ssr_reduce_kernel(const float *part, int rows, int n_tiles, float *ssr)
 {
@@ -1669,16 +644,12 @@ int check_orbit(const pt_orbit *orb, bool need_ecc)
     return PT_OK;
 }
 
-// Mandel-Agol (NP1 == 0): records, time split, per-tile residual partials.
-// Gimenez: records, time split, per-geometry tables, list counters (+ the
-// work-item counter), work-item prefix, pair lists and a flux scratch used
-// when only residuals are asked for.
+// The tile kernel: records, time split, per-tile residual partials.
 struct WorkLayout {
-    size_t rec, tsplit, T, part, cnt, pref, list, fscr, atab, dtab, total;
+    size_t rec, tsplit, part, total;
 };
 
-// n_zi > 0 adds the z tables of the interpolated Gimenez model.
-WorkLayout work_layout(int n_t, int n_v, int n_b, int k_per_band, int NP1, int n_j, int n_zi = 0)
+WorkLayout work_layout(int n_t, int n_v, int n_b, int k_per_band)
 {
     int n_geom = k_per_band ? n_v * n_b : n_v;
     int n_tiles = (n_t + TT - 1) / TT;
@@ -1688,28 +659,8 @@ WorkLayout work_layout(int n_t, int n_v, int n_b, int k_per_band, int NP1, int n
     off += align256((size_t)n_geom * sizeof(GeomRec));
     L.tsplit = off;
     off += align256((size_t)n_t * sizeof(float2));
-    L.T = L.part = L.cnt = L.pref = L.list = L.fscr = L.atab = L.dtab = off;
-    if (NP1 == 0) {
-        L.part = off;
-        off += align256((size_t)n_v * n_b * n_tiles * sizeof(float));
-    } else {
-        L.T = off;
-        off += align256((size_t)n_geom * NP1 * n_j * sizeof(float4));
-        L.cnt = off;
-        off += align256((size_t)(n_geom + 1) * sizeof(int));
-        L.pref = off;   // the item prefix [n_geom + 1], then the geometry order [n_geom]
-        off += align256((size_t)(2 * n_geom + 1) * sizeof(int));
-        L.list = off;
-        off += align256((size_t)n_geom * n_t * sizeof(int));
-        L.fscr = off;
-        off += align256((size_t)n_v * n_b * n_t * sizeof(float));
-        L.part = off;   // residual chunk sums
-        off += align256((size_t)n_v * n_b * ssr_chunks(n_t) * sizeof(float));
-        L.atab = off;
-        off += align256((size_t)n_geom * n_zi * NP1 * sizeof(float));
-        L.dtab = off;   // Chebyshev coefficient rows, padded to 16 bytes
-        off += align256((size_t)n_geom * n_j * ((NP1 + 3) & ~3) * sizeof(float));
-    }
+    L.part = off;
+    off += align256((size_t)n_v * n_b * n_tiles * sizeof(float));
     L.total = off;
     return L;
 }
@@ -1781,8 +732,12 @@ int launch_rows(int model, rows::Args &A, int n_sm, cudaStream_t s)
 #define PT_ROWS_FN(M)                                                                                               \
     fn = staged ? (one ? rows::lc_rows_kernel<M, 1, true> : rows::lc_rows_kernel<M, 4, true>)                       \
                 : rows::lc_rows_kernel<M, 4, false>
-    if (model == rows::R_MA) fn = one ? rows::lc_rows_kernel<rows::R_MA, 1, true> : rows::lc_rows_kernel<rows::R_MA, 4, true>;
-    else PT_ROWS_FN(rows::R_INTERP);
+    switch (model) {
+    case rows::R_MA: PT_ROWS_FN(rows::R_MA); break;
+    case rows::R_GIM: PT_ROWS_FN(rows::R_GIM); break;
+    case rows::R_ZI: PT_ROWS_FN(rows::R_ZI); break;
+    default: PT_ROWS_FN(rows::R_INTERP); break;
+    }
 #undef PT_ROWS_FN
     if (smem > 40 * 1024) {   // beyond the default limit less the static arrays
         cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
@@ -1858,15 +813,11 @@ struct pt_gim_plan_s {
     float4 *d_coef;   // [N+1][n_j]: recursion of G_j(nu+2, 1; x), FP32
     double *d_A;      // [N+1][n_j]: A_{n,j}, FP64
     double *d_recb;   // [N+1][n_j][3]: recursion of G_j(nu+2, nu+1; x), FP64
-    cudaEvent_t ev0, ev1;   // recorded around the series evaluation kernel when set (profiling)
-    // The table recursion and the Chebyshev coefficients depend on k alone:
-    // they run on this plan-owned stream (highest priority) beside the
-    // set-up, window and scan kernels of the call's stream, forked and joined
-    // by the two events; the mutex keeps a fork's record and wait together
-    // when host threads share the plan.
-    cudaStream_t side;
-    cudaEvent_t ev_fork, ev_join;
-    std::mutex fork_mu;
+    float2 *d_dA;     // the same A_{n,j} and recursion as double-float pairs
+    float2 *d_drb;
+    float *d_B;       // [(N+1) n_j][8 n_int]: piecewise polynomials of the series' functions (pt_gim.cuh)
+    int n_int;
+    cudaEvent_t ev0, ev1;   // recorded around the evaluation kernel when set (profiling)
 };
 
 namespace {
@@ -1900,119 +851,28 @@ void jacobi_rec(double p, double q, int j, double *r)
 }  // namespace
 
 namespace {
-int launch_zi(const GimArgs &A, const float *atab, int n_in, int n_edge, size_t smem, size_t max_items,
-              cudaStream_t s)
-{
-    static thread_local size_t configured = 0;
-    if (smem > 48 * 1024 && smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(gim_zi_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-        if (e != cudaSuccess) return set_cuda_error(e, "gim_zi_kernel smem attribute");
-        configured = smem;
-    }
-    int dev = 0, n_sm = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gim_zi_kernel, GS_THREADS, smem);
-    if (e != cudaSuccess) return set_cuda_error(e, "gim_zi_kernel occupancy");
-    if (per_sm < 1) return pt_internal::set_error(PT_ERR_ARG, "gim_zi_kernel", "does not fit on an SM");
-    size_t grid = (size_t)n_sm * per_sm;
-    if (grid > max_items) grid = max_items;
-    if (grid < 1) grid = 1;
-    gim_zi_kernel<<<(unsigned)grid, GS_THREADS, smem, s>>>(A, atab, n_in, n_edge);
-    return check_launch("gim_zi_kernel");
-}
 
-// Chebyshev path, coefficient kernel for N + 1 orders.
-template <int NP1>
-int launch_cheb_coef_t(const GimArgs &A, const float4 *T, float *dtab, cudaStream_t s)
-{
-    // coefficients: one warp per (geometry, order), rows padded to DS
-    // floats (the warps past order N write the padding zeros)
-    constexpr int DS = (NP1 + 3) & ~3;
-    const size_t csm = (size_t)CW_WARPS * A.n_j * sizeof(float4);
-    const dim3 cgrid(A.n_geom, (DS + CW_WARPS - 1) / CW_WARPS);
-    const int S = gim_cheb_coef_s(A.n_j);
-#define PT_COEF_LAUNCH(SV)                                                                                          \
-    gim_cheb_coef_kernel<SV><<<cgrid, 32 * CW_WARPS, csm, s>>>(T, A.N + 1, A.n_j, DS, dtab)
-    if (S <= 2) PT_COEF_LAUNCH(2);
-    else if (S <= 4) PT_COEF_LAUNCH(4);
-    else if (S <= 6) PT_COEF_LAUNCH(6);
-    else if (S <= 8) PT_COEF_LAUNCH(8);
-    else if (S <= 12) PT_COEF_LAUNCH(12);
-    else PT_COEF_LAUNCH(16);
-#undef PT_COEF_LAUNCH
-    return check_launch("gim_cheb_coef_kernel");
-}
+constexpr int ZI_MAX_VALUES = 16384;   // (n_in + n_edge)(N + 1) per geometry
 
-// Chebyshev path, evaluation kernel (persistent) for N + 1 orders.
-template <int NP1>
-int launch_cheb_eval_t(const GimArgs &A, float *dtab, size_t max_items, cudaEvent_t ev0, cudaEvent_t ev1,
-                       cudaStream_t s)
-{
-    int st = PT_OK;
-    // evaluation: persistent
-    const size_t smem = gim_cheb_smem(A.n_j, A.N, A.n_ss);
-    static thread_local size_t configured = 0;
-    if (smem > 48 * 1024 && smem > configured) {
-        cudaError_t e = cudaFuncSetAttribute(gim_cheb_kernel<NP1>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
-        if (e != cudaSuccess) return set_cuda_error(e, "gim_cheb_kernel smem attribute");
-        configured = smem;
-    }
-    int dev = 0, n_sm = 0, per_sm = 0;
-    cudaError_t e = cudaGetDevice(&dev);
-    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    if (e == cudaSuccess)
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gim_cheb_kernel<NP1>, GS_THREADS, smem);
-    if (e != cudaSuccess) return set_cuda_error(e, "gim_cheb_kernel occupancy");
-    if (per_sm < 1) return pt_internal::set_error(PT_ERR_ARG, "gim_cheb_kernel", "does not fit on an SM");
-    size_t grid = (size_t)n_sm * per_sm;
-    if (grid > max_items) grid = max_items;
-    if (grid < 1) grid = 1;
-    if (ev0 && (e = cudaEventRecord(ev0, s)) != cudaSuccess) return set_cuda_error(e, "pt_gimenez timing event");
-    gim_cheb_kernel<NP1><<<(unsigned)grid, GS_THREADS, smem, s>>>(A, dtab);
-    st = check_launch("gim_cheb_kernel");
-    if (st) return st;
-    if (ev1 && (e = cudaEventRecord(ev1, s)) != cudaSuccess) return set_cuda_error(e, "pt_gimenez timing event");
-    return PT_OK;
-}
+// The row layout, then the weighted T and (interpolated in z) the node rows.
+struct GimLayout {
+    RowLayout row;
+    size_t At, zi, total;
+};
 
-// Chebyshev path dispatch over N + 1 = 2 .. 17 orders.
-#define PT_NP1_DISPATCH(CALL)                                                                                       \
-    switch (A.N + 1) {                                                                                              \
-    case 2: return CALL(2);                                                                                         \
-    case 3: return CALL(3);                                                                                         \
-    case 4: return CALL(4);                                                                                         \
-    case 5: return CALL(5);                                                                                         \
-    case 6: return CALL(6);                                                                                         \
-    case 7: return CALL(7);                                                                                         \
-    case 8: return CALL(8);                                                                                         \
-    case 9: return CALL(9);                                                                                         \
-    case 10: return CALL(10);                                                                                       \
-    case 11: return CALL(11);                                                                                       \
-    case 12: return CALL(12);                                                                                       \
-    case 13: return CALL(13);                                                                                       \
-    case 14: return CALL(14);                                                                                       \
-    case 15: return CALL(15);                                                                                       \
-    case 16: return CALL(16);                                                                                       \
-    default: return CALL(17);                                                                                       \
-    }
-
-int launch_cheb_coef(const GimArgs &A, const float4 *T, float *dtab, cudaStream_t s)
+GimLayout gim_layout(const pt_gim_plan_s *p, int n_t, int n_v, int n_b, int k_per_band, int n_zi)
 {
-#define PT_CALL(V) launch_cheb_coef_t<V>(A, T, dtab, s)
-    PT_NP1_DISPATCH(PT_CALL)
-#undef PT_CALL
+    GimLayout L;
+    L.row = row_layout(n_t, n_v, n_b, k_per_band, p->N + 1, (size_t)gim::Q * p->n_int);
+    const size_t R = (k_per_band ? (size_t)n_v * n_b : (size_t)n_v) * rows_per_geom(k_per_band ? 1 : n_b, p->N + 1);
+    size_t off = L.row.total;
+    L.At = off;
+    off += align256((R + 31) / 32 * 32 * (size_t)(p->N + 1) * p->n_j * sizeof(float));
+    L.zi = off;
+    off += align256(R * (((size_t)n_zi + 3) & ~(size_t)3) * sizeof(float));
+    L.total = off;
+    return L;
 }
-
-int launch_cheb_eval(const GimArgs &A, float *dtab, size_t max_items, cudaEvent_t ev0, cudaEvent_t ev1,
-                     cudaStream_t s)
-{
-#define PT_CALL(V) launch_cheb_eval_t<V>(A, dtab, max_items, ev0, ev1, s)
-    PT_NP1_DISPATCH(PT_CALL)
-#undef PT_CALL
-}
-#undef PT_NP1_DISPATCH
 
 }  // namespace
 
@@ -2167,7 +1027,7 @@ size_t pt_ma_quad_work_bytes(int n_t, int n_v, int n_b, int k_per_band)
 {
     if (n_t < 0 || n_v < 0 || n_b < 1) return 0;
     // the tile kernel, the exact rows, or a table's rows (of any length that takes them)
-    size_t need = work_layout(n_t, n_v, n_b, k_per_band, 0, 0).total;
+    size_t need = work_layout(n_t, n_v, n_b, k_per_band).total;
     const size_t r = row_layout(n_t, n_v, n_b, k_per_band, 3, row_len_max(n_t)).total;
     return r > need ? r : need;
 }
@@ -2320,7 +1180,7 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     if (use_rows && ma_use_rows(n_t, orb->n_v, n_b, k_per_band, n_ss) && (!tab || interp_row_len(tab->n_z) <= row_len_max(n_t)))
         return ma_quad_rows(tab, t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, wt, flux, ssr, work,
                             work_bytes, n_bad, stream);
-    WorkLayout L = work_layout(n_t, orb->n_v, n_b, k_per_band, 0, 0);
+    WorkLayout L = work_layout(n_t, orb->n_v, n_b, k_per_band);
     if (work_bytes < L.total) return PT_ERR_WORKSPACE;
     cudaStream_t s = (cudaStream_t)stream;
     char *wb = (char *)work;
@@ -2453,19 +1313,47 @@ int pt_gim_plan_create(int N, int n_j, pt_gim_plan *out)
     float4 *hcoef = new float4[cnt];
     double *hA = new double[cnt];
     double *hrb = new double[cnt * 3];
+    double *hrc = new double[cnt * 3];
+    float2 *hdA = new float2[cnt];
+    float2 *hdrb = new float2[cnt * 3];
+    auto df = [](double v) {
+        const float h = (float)v;
+        return make_float2(h, (float)(v - (double)h));
+    };
     for (int n = 0; n < NP1; ++n) {
         double nu = 0.5 * (n + 2);
         // A_{n,j} = (-1)^j (2j+nu+2)/nu * prod_{i=1..j} (nu+i)/(i+1)   (Eq. gimemez_a)
         double prod = 1.0;
         for (int j = 0; j < n_j; ++j) {
+            const size_t at = (size_t)n * n_j + j;
             if (j > 0) prod *= (nu + j) / (j + 1.0);
-            hA[(size_t)n * n_j + j] = ((j & 1) ? -1.0 : 1.0) * (2.0 * j + nu + 2.0) / nu * prod;
-            double r[3];
-            jacobi_rec(nu + 2.0, 1.0, j, r);
-            hcoef[(size_t)n * n_j + j] = make_float4((float)r[0], (float)r[1], (float)r[2], 0.0f);
-            jacobi_rec(nu + 2.0, nu + 1.0, j, r);
-            for (int c = 0; c < 3; ++c) hrb[((size_t)n * n_j + j) * 3 + c] = r[c];
+            hA[at] = ((j & 1) ? -1.0 : 1.0) * (2.0 * j + nu + 2.0) / nu * prod;
+            hdA[at] = df(hA[at]);
+            jacobi_rec(nu + 2.0, 1.0, j, hrc + 3 * at);
+            hcoef[at] = make_float4((float)hrc[3 * at], (float)hrc[3 * at + 1], (float)hrc[3 * at + 2], 0.0f);
+            jacobi_rec(nu + 2.0, nu + 1.0, j, hrb + 3 * at);
+            for (int c = 0; c < 3; ++c) hdrb[3 * at + c] = df(hrb[3 * at + c]);
         }
+    }
+    // node values -> monomials on an interval, by Chebyshev coefficients: the
+    // first interval (t in [0, 1/2]) and the others (t in [-1/2, 1/2])
+    constexpr int Q = gim::Q;
+    double mat[2][Q][Q];
+    for (int kind = 0; kind < 2; ++kind) {
+        const double al = kind == 0 ? 4.0 : 2.0, be = kind == 0 ? -1.0 : 0.0;
+        double T[Q][Q] = {};   // T_k(al t + be) by powers of t
+        T[0][0] = 1.0;
+        T[1][0] = be;
+        T[1][1] = al;
+        for (int k = 2; k < Q; ++k)
+            for (int c = 0; c < Q; ++c)
+                T[k][c] = 2.0 * be * T[k - 1][c] + (c > 0 ? 2.0 * al * T[k - 1][c - 1] : 0.0) - T[k - 2][c];
+        for (int q = 0; q < Q; ++q)
+            for (int c = 0; c < Q; ++c) {
+                double v = 0.0;
+                for (int k = 0; k < Q; ++k) v += (k == 0 ? 1.0 : 2.0) / Q * cos(k * (q + 0.5) * PI_D / Q) * T[k][c];
+                mat[kind][c][q] = v;
+            }
     }
     pt_gim_plan p = new pt_gim_plan_s;
     p->N = N;
@@ -2473,31 +1361,47 @@ int pt_gim_plan_create(int N, int n_j, pt_gim_plan *out)
     p->d_coef = nullptr;
     p->d_A = nullptr;
     p->d_recb = nullptr;
+    p->d_dA = p->d_drb = nullptr;
+    p->d_B = nullptr;
+    p->n_int = gim::intervals(N, n_j);
     p->ev0 = p->ev1 = nullptr;
-    p->side = nullptr;
-    p->ev_fork = p->ev_join = nullptr;
-    int prio_lo = 0, prio_hi = 0;
-    cudaError_t e = cudaDeviceGetStreamPriorityRange(&prio_lo, &prio_hi);
-    if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&p->side, cudaStreamNonBlocking, prio_hi);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_fork, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaEventCreateWithFlags(&p->ev_join, cudaEventDisableTiming);
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_coef, cnt * sizeof(float4));
+    const int n_node = Q * p->n_int;
+    double *d_rc = nullptr, *d_mat = nullptr, *d_V = nullptr;   // while the basis is built
+    cudaError_t e = cudaMalloc(&p->d_coef, cnt * sizeof(float4));
     if (e == cudaSuccess) e = cudaMalloc(&p->d_A, cnt * sizeof(double));
     if (e == cudaSuccess) e = cudaMalloc(&p->d_recb, cnt * 3 * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_dA, cnt * sizeof(float2));
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_drb, cnt * 3 * sizeof(float2));
+    if (e == cudaSuccess) e = cudaMalloc(&p->d_B, cnt * n_node * sizeof(float));
+    if (e == cudaSuccess) e = cudaMalloc(&d_rc, cnt * 3 * sizeof(double));
+    if (e == cudaSuccess) e = cudaMalloc(&d_mat, sizeof(mat));
+    if (e == cudaSuccess) e = cudaMalloc(&d_V, cnt * n_node * sizeof(double));
     if (e == cudaSuccess) e = cudaMemcpy(p->d_coef, hcoef, cnt * sizeof(float4), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_A, hA, cnt * sizeof(double), cudaMemcpyHostToDevice);
     if (e == cudaSuccess) e = cudaMemcpy(p->d_recb, hrb, cnt * 3 * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(p->d_dA, hdA, cnt * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(p->d_drb, hdrb, cnt * 3 * sizeof(float2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_rc, hrc, cnt * 3 * sizeof(double), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMemcpy(d_mat, mat, sizeof(mat), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        const int n1 = NP1 * n_node;
+        const long long n2 = (long long)cnt * p->n_int;
+        gim::basis_nodes_kernel<<<(n1 + 63) / 64, 64>>>(d_rc, NP1, n_j, p->n_int, (double)gim::row_scale(p->n_int), d_V);
+        gim::basis_coef_kernel<<<(unsigned)((n2 + 127) / 128), 128>>>(d_V, d_mat, (int)cnt, p->n_int, p->d_B);
+        e = cudaGetLastError();
+    }
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    cudaFree(d_rc);
+    cudaFree(d_mat);
+    cudaFree(d_V);
     delete[] hcoef;
     delete[] hA;
     delete[] hrb;
+    delete[] hrc;
+    delete[] hdA;
+    delete[] hdrb;
     if (e != cudaSuccess) {
-        cudaFree(p->d_coef);
-        cudaFree(p->d_A);
-        cudaFree(p->d_recb);
-        if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-        if (p->ev_join) cudaEventDestroy(p->ev_join);
-        if (p->side) cudaStreamDestroy(p->side);
-        delete p;
+        pt_gim_plan_destroy(p);
         return set_cuda_error(e, "pt_gim_plan_create");
     }
     *out = p;
@@ -2518,9 +1422,9 @@ int pt_gim_plan_destroy(pt_gim_plan p)
     cudaFree(p->d_coef);
     cudaFree(p->d_A);
     cudaFree(p->d_recb);
-    if (p->ev_fork) cudaEventDestroy(p->ev_fork);
-    if (p->ev_join) cudaEventDestroy(p->ev_join);
-    if (p->side) cudaStreamDestroy(p->side);
+    cudaFree(p->d_dA);
+    cudaFree(p->d_drb);
+    cudaFree(p->d_B);
     delete p;
     return PT_OK;
 }
@@ -2542,13 +1446,14 @@ int pt_gimenez_alpha(pt_gim_plan plan, const float *k, const float *z, size_t n,
 size_t pt_gimenez_work_bytes(pt_gim_plan plan, int n_t, int n_v, int n_b, int k_per_band)
 {
     if (!plan || n_t < 0 || n_v < 0 || n_b < 1) return 0;
-    return work_layout(n_t, n_v, n_b, k_per_band, plan->N + 1, plan->n_j).total;
+    return gim_layout(plan, n_t, n_v, n_b, k_per_band, 0).total;
 }
 
 }  // extern "C"
 
-// pt_gimenez (n_in == 0: the series for every pair) and pt_gimenez_zi (the
-// series on z nodes, read back by interpolation).
+// pt_gimenez (n_in == 0: the series' rows) and pt_gimenez_zi (the rows on z
+// nodes): preparation with the weighted T_{n,j}, the product that forms the
+// rows, (the nodes,) the row kernel.
 static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t, int n_t, const pt_orbit *orb,
                         const float *k, int k_per_band, const float *ld, int n_b, int n_ss, double t_exp,
                         int max_iter, const float *y, const float *wt, float *flux, float *ssr, void *work,
@@ -2561,110 +1466,109 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     int st = lc_common_check(t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, flux, ssr, work);
     if (st) return st;
     if (n_t == 0 || orb->n_v == 0) return PT_OK;
-    const int NP1 = plan->N + 1;
-    WorkLayout L = work_layout(n_t, orb->n_v, n_b, k_per_band, NP1, plan->n_j, zi ? n_in + n_edge : 0);
+    const int NP1 = plan->N + 1, K = NP1 * plan->n_j, Nc = gim::Q * plan->n_int;
+    const GimLayout L = gim_layout(plan, n_t, orb->n_v, n_b, k_per_band, zi ? n_in + n_edge : 0);
     if (work_bytes < L.total) return PT_ERR_WORKSPACE;
-    const size_t smem = zi ? gim_zi_smem(plan->N, n_in + n_edge) : gim_cheb_smem(plan->n_j, plan->N, n_ss);
-    if (smem > 200 * 1024) return PT_ERR_ARG;
     const int n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
-    const int n_tiles = (n_t + TT - 1) / TT;
-    const int gy = (n_geom + GW_VT - 1) / GW_VT;
-    if (gy > 65535) return PT_ERR_ARG;
+    const int n_bpg = k_per_band ? 1 : n_b;
+    if ((n_geom + 31) / 32 > 65535) return PT_ERR_ARG;
     cudaStream_t s = (cudaStream_t)stream;
     char *wb = (char *)work;
-    GeomRec *rec = (GeomRec *)(wb + L.rec);
-    float2 *tsplit = (float2 *)(wb + L.tsplit);
-    float4 *T = (float4 *)(wb + L.T);
-    int *cnt = (int *)(wb + L.cnt);
-    float *atab = (float *)(wb + L.atab);
-    float *dtab = (float *)(wb + L.dtab);
-    GimArgs A;
+    int n_sm = 0;
+    st = sm_count(&n_sm);
+    if (st) return st;
+    RowPrep P;
+    memset(&P, 0, sizeof(P));
+    fill_setup(&P.s, t, n_t, orb, k, k_per_band, n_b, t_exp, (GeomRec *)(wb + L.row.rec), (float2 *)(wb + L.row.tsplit));
+    P.s.n_gblocks = (n_geom + 31) / 32;
+    P.n_tblocks = (n_t + ROW_THREADS - 1) / ROW_THREADS;
+    P.rows = (float *)(wb + L.row.rows);
+    P.row_len = Nc;
+    P.nr = rows_per_geom(n_bpg, NP1);
+    P.terms = row_terms(n_bpg);
+    P.n_bpg = n_bpg;
+    P.ld = ld;
+    const size_t R = (size_t)n_geom * P.nr;
+    P.gim.dA = plan->d_dA;
+    P.gim.drb = plan->d_drb;
+    P.gim.NP1 = NP1;
+    P.gim.n_j = plan->n_j;
+    P.gim.At = (float *)(wb + L.At);
+    P.gim.Rp = (int)((R + 31) / 32 * 32);
+    const long long blocks = (long long)P.s.n_gblocks + P.n_tblocks + (long long)NP1 * ((n_geom + gim::GPC - 1) / gim::GPC);
+    if (blocks > 0x7fffffffLL || R > 0x7fffffffULL - 32) return PT_ERR_ARG;
+    const size_t tsm = gim::table_smem(plan->n_j, P.nr);
+    cudaError_t e = cudaSuccess;
+    if (tsm > 40 * 1024)
+        e = cudaFuncSetAttribute(row_prep_kernel<rows::R_GIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm);
+    if (e != cudaSuccess) return set_cuda_error(e, "row_prep_kernel smem attribute");
+    row_prep_kernel<rows::R_GIM><<<(unsigned)blocks, ROW_THREADS, tsm, s>>>(P);
+    st = check_launch("row_prep_kernel");
+    if (st) return st;
+    // the product: tall tiles when they fill half the chip
+    const size_t gx = ((size_t)Nc + gim::CT - 1) / gim::CT;
+    const size_t r32 = (R + 31) / 32, r8 = (R + 7) / 8;
+    if (r32 * gx > 0x7fffffffULL) return PT_ERR_ARG;
+    if (r32 * gx >= (size_t)n_sm / 2) {
+        e = cudaFuncSetAttribute(gim::product_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gim::Split<32>::SMEM);
+        if (e == cudaSuccess)
+            gim::product_kernel<32><<<(unsigned)(r32 * gx), 32 * gim::Split<32>::WARPS, gim::Split<32>::SMEM, s>>>(
+                P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
+    } else {
+        gim::product_kernel<8><<<(unsigned)(r8 * gx), 32 * gim::Split<8>::WARPS, gim::Split<8>::SMEM, s>>>(
+            P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
+    }
+    if (e != cudaSuccess) return set_cuda_error(e, "product_kernel smem attribute");
+    st = check_launch("product_kernel");
+    if (st) return st;
+    rows::Args A;
     memset(&A, 0, sizeof(A));
-    A.tsplit = tsplit;
+    A.tsplit = P.s.tsplit;
     A.n_t = n_t;
-    A.rec = rec;
+    A.rec = P.s.rec;
     A.n_geom = n_geom;
-    A.gtab = T;
-    A.N = plan->N;
-    A.n_j = plan->n_j;
+    A.rows = P.rows;
+    A.row_len = P.row_len;
+    A.nr = P.nr;
+    A.terms = P.terms;
+    A.n_bpg = n_bpg;
+    A.n_b = n_b;
+    A.k_per_band = k_per_band;
     A.ld = ld;
-    A.n_bpg = k_per_band ? 1 : n_b;
+    A.N = plan->N;
     A.n_ss = n_ss;
     A.t_exp = (float)t_exp;
     A.max_iter = max_iter;
-    A.flux = flux ? flux : (float *)(wb + L.fscr);
-    A.cnt = cnt;
-    A.pref = (int *)(wb + L.pref);
-    A.gord = A.pref + n_geom + 1;
-    A.ctr = cnt + n_geom;
-    A.list = (int *)(wb + L.list);
-    A.ppi = GS_THREADS;   // work items of GS_THREADS listed pairs
+    A.scale = gim::row_scale(plan->n_int);
+    const bool fused_ssr = ssr && !P.terms;
+    float *part = (float *)(wb + L.row.part);
+    A.flux = flux ? flux : (P.terms ? (float *)(wb + L.row.fscr) : nullptr);
+    A.ssr_part = fused_ssr ? part : nullptr;
+    A.y = y;
+    A.wt = wt;
     A.n_bad = n_bad;
-    TableJob J;
-    J.k = k;
-    J.n_geom = n_geom;
-    J.NP1 = NP1;
-    J.n_j = plan->n_j;
-    J.A = plan->d_A;
-    J.recb = plan->d_recb;
-    J.coef = plan->d_coef;
-    J.tab = T;
-    J.n_blocks = NP1 * ((n_geom + TABLE_GPC - 1) / TABLE_GPC);
-    const size_t tsm = gim_table_smem(plan->n_j);   // at most 24 KB (n_j <= 512): no opt-in needed
-    if (!zi) {
-        // the table recursion and the Chebyshev coefficients depend on k
-        // alone: forked onto the plan's side stream (after all earlier work
-        // of the call's stream), joined before the evaluation kernel
-        cudaError_t e;
-        {
-            std::lock_guard<std::mutex> lk(plan->fork_mu);
-            e = cudaEventRecord(plan->ev_fork, s);
-            if (e == cudaSuccess) e = cudaStreamWaitEvent(plan->side, plan->ev_fork, 0);
-        }
-        if (e != cudaSuccess) return set_cuda_error(e, "pt_gimenez fork");
-        const size_t tsm2 = gim_table2_smem(plan->n_j);
-        static thread_local size_t tsm2_configured = 0;
-        if (tsm2 > 48 * 1024 && tsm2 > tsm2_configured) {
-            e = cudaFuncSetAttribute(gim_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm2);
-            if (e != cudaSuccess) return set_cuda_error(e, "gim_table_kernel smem attribute");
-            tsm2_configured = tsm2;
-        }
-        const int n_tb = NP1 * ((n_geom + TABLE_GPC2 - 1) / TABLE_GPC2);
-        gim_table_kernel<<<(unsigned)n_tb, TT, tsm2, plan->side>>>(J);
-        st = check_launch("gim_table_kernel");
-        if (st) return st;
-        st = launch_cheb_coef(A, T, dtab, plan->side);
-        if (st) return st;
-        e = cudaEventRecord(plan->ev_join, plan->side);
-        if (e != cudaSuccess) return set_cuda_error(e, "pt_gimenez join");
-        J.n_blocks = 0;   // the window launch without table CTAs
-    }
-    st = launch_setup(t, n_t, orb, k, k_per_band, n_b, t_exp, rec, tsplit, cnt, s);
-    if (st) return st;
-    const size_t n_cta = (size_t)J.n_blocks + (size_t)n_tiles * gy;
-    if (n_cta > 0x7fffffffULL) return PT_ERR_ARG;
-    gim_window_kernel<<<(unsigned)n_cta, TT, J.n_blocks ? tsm : 0, s>>>(A, J, n_tiles);
-    st = check_launch("gim_window_kernel");
-    if (st) return st;
     if (zi) {
-        gim_zi_table_kernel<<<n_geom, 128, 0, s>>>(rec, T, NP1, plan->n_j, n_in, n_edge, atab);
-        st = check_launch("gim_zi_table_kernel");
+        A.n_in = n_in;
+        A.n_edge = n_edge;
+        const int zi_len = (n_in + n_edge + 3) & ~3;
+        float *zrows = (float *)(wb + L.zi);
+        const long long n = (long long)R * zi_len;
+        if ((n + 127) / 128 > 0x7fffffffLL) return PT_ERR_ARG;
+        gim::zi_rows_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(A, k, (int)R, zi_len, zrows);
+        st = check_launch("zi_rows_kernel");
         if (st) return st;
+        A.rows = zrows;
+        A.row_len = zi_len;
     }
-    gim_scan_kernel<<<1, 1024, 0, s>>>(cnt, A.rec, A.t_exp, n_geom, A.ppi, true, A.pref, A.gord, A.ctr);
-    st = check_launch("gim_scan_kernel");
+    if (plan->ev0 && (e = cudaEventRecord(plan->ev0, s)) != cudaSuccess) return set_cuda_error(e, "pt_gimenez timing event");
+    st = launch_rows(zi ? rows::R_ZI : rows::R_GIM, A, n_sm, s);
     if (st) return st;
-    const size_t max_items = (size_t)n_geom * ((n_t + GS_THREADS - 1) / GS_THREADS);
-    if (zi) {
-        st = launch_zi(A, atab, n_in, n_edge, smem, max_items, s);
-    } else {
-        cudaError_t e = cudaStreamWaitEvent(s, plan->ev_join, 0);
-        if (e != cudaSuccess) return set_cuda_error(e, "pt_gimenez join");
-        st = launch_cheb_eval(A, dtab, max_items, plan->ev0, plan->ev1, s);
-    }
-    if (st) return st;
-    if (ssr) st = launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)orb->n_v * n_b, (float *)(wb + L.part), ssr, s);
-    return st;
+    if (plan->ev1 && (e = cudaEventRecord(plan->ev1, s)) != cudaSuccess) return set_cuda_error(e, "pt_gimenez timing event");
+    if (!ssr) return PT_OK;
+    const int n_rows = orb->n_v * n_b;
+    if (!fused_ssr) return launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)n_rows, part, ssr, s);
+    ssr_reduce_kernel<<<(unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s>>>(part, n_rows, A.n_tiles, ssr);
+    return check_launch("ssr_reduce_kernel");
 }
 
 extern "C" {
@@ -2680,7 +1584,7 @@ int pt_gimenez(pt_gim_plan plan, const double *t, int n_t, const pt_orbit *orb, 
 size_t pt_gimenez_zi_work_bytes(pt_gim_plan plan, int n_in, int n_edge, int n_t, int n_v, int n_b, int k_per_band)
 {
     if (!plan || n_t < 0 || n_v < 0 || n_b < 1 || n_in < 2 || n_edge < 1) return 0;
-    return work_layout(n_t, n_v, n_b, k_per_band, plan->N + 1, plan->n_j, n_in + n_edge).total;
+    return gim_layout(plan, n_t, n_v, n_b, k_per_band, n_in + n_edge).total;
 }
 
 int pt_gimenez_zi(pt_gim_plan plan, int n_in, int n_edge, const double *t, int n_t, const pt_orbit *orb,
@@ -2748,7 +1652,7 @@ extern "C" int pt_ma_quad_noalloc(const double *t, int n_t, const pt_orbit *orb,
 {
     if (!orb || n_t < 0 || orb->n_v < 0 || n_b < 1) return PT_ERR_ARG;
     // the tile kernel: its scratch is small (records, time split, partials)
-    size_t need = work_layout(n_t, orb->n_v, n_b, k_per_band, 0, 0).total;
+    size_t need = work_layout(n_t, orb->n_v, n_b, k_per_band).total;
     if (need > (size_t)PT_MA_NOALLOC_SCRATCH_BYTES) {
         snprintf(g_last_error, sizeof(g_last_error),
                  "pt_ma_quad_noalloc: this problem needs %zu bytes of scratch, the static scratch holds %zu; "

@@ -115,7 +115,7 @@ __device__ __forceinline__ unsigned find(const Args &A, const float4 &q, float z
     return (unsigned)i;
 }
 
-constexpr int GIM_DEG = 12;   // coefficients per interval of a Gimenez row
+constexpr int GIM_DEG = 8;   // coefficients per interval of a Gimenez row
 
 // base: byte address in shared memory (SMEM) of the row, less the place's
 // constant bits; or the row in global memory
@@ -124,34 +124,23 @@ __device__ __forceinline__ float eval(unsigned base, const float *row, const flo
 {
     if (MODEL == R_MA && SMEM) return pt::mt_eval(base, pos, t);
     if (MODEL == R_GIM || MODEL == R_MA) {
-        constexpr int L = MODEL == R_GIM ? GIM_DEG : 8;   // floats per interval
-        float4 c[3];
+        // (8 floats per interval in both)
+        float4 c, d;
         if (SMEM) {
-            const unsigned at = base + (unsigned)(4 * L) * pos;
-#pragma unroll
-            for (int i = 0; i < 3; ++i)
-                asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
-                             : "=f"(c[i].x), "=f"(c[i].y), "=f"(c[i].z), "=f"(c[i].w)
-                             : "r"(at + 16u * i));
+            const unsigned at = base + 32u * pos;
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(c.x), "=f"(c.y), "=f"(c.z), "=f"(c.w) : "r"(at));
+            asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(d.x), "=f"(d.y), "=f"(d.z), "=f"(d.w) : "r"(at + 16u));
         } else {
-            const float4 *p = reinterpret_cast<const float4 *>(row + (size_t)(pos - pt::MT_BITS0) * L);
-            c[0] = __ldg(p);
-            c[1] = __ldg(p + 1);
-            if (MODEL == R_GIM) c[2] = __ldg(p + 2);
+            const float4 *p = reinterpret_cast<const float4 *>(row + (size_t)(pos - pt::MT_BITS0) * 8);
+            c = __ldg(p);
+            d = __ldg(p + 1);
         }
-        if (MODEL == R_MA)
-            return fmaf(fmaf(fmaf(fmaf(fmaf(c[1].y, t, c[1].x), t, c[0].w), t, c[0].z), t, c[0].y), t, c[0].x);
-        float v = fmaf(c[2].w, t, c[2].z);
-        v = fmaf(v, t, c[2].y);
-        v = fmaf(v, t, c[2].x);
-        v = fmaf(v, t, c[1].w);
-        v = fmaf(v, t, c[1].z);
-        v = fmaf(v, t, c[1].y);
-        v = fmaf(v, t, c[1].x);
-        v = fmaf(v, t, c[0].w);
-        v = fmaf(v, t, c[0].z);
-        v = fmaf(v, t, c[0].y);
-        return fmaf(v, t, c[0].x);
+        float v = MODEL == R_GIM ? fmaf(fmaf(d.w, t, d.z), t, d.y) : d.y;
+        v = fmaf(v, t, d.x);
+        v = fmaf(v, t, c.w);
+        v = fmaf(v, t, c.z);
+        v = fmaf(v, t, c.y);
+        return fmaf(v, t, c.x);
     }
     float a, b;
     if (SMEM) {
@@ -339,7 +328,7 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
     // the lists end to end, 32 pairs per warp and turn
     const float inv_nss = 1.0f / (float)A.n_ss;
     const unsigned sbase = (unsigned)__cvta_generic_to_shared(dsm + L.rows) -
-                           (MODEL == R_MA ? 32u * pt::MT_BITS0 : MODEL == R_GIM ? 4u * GIM_DEG * pt::MT_BITS0 : 0u);
+                           (MODEL == R_MA || MODEL == R_GIM ? 32u * pt::MT_BITS0 : 0u);
     float *sval = reinterpret_cast<float *>(dsm + L.sval);   // [n_ssr][kt vt][TB]
     int nbad = 0;
     for (int e = tid; e < nq; e += TB) {
