@@ -3,8 +3,10 @@
 // (the network is not in the paper; its analogue there is the
 // interpolation tables of Sec. 2.2.3).
 //
-// One persistent CTA of 128 threads per tile of 128 points (several tiles
-// per CTA):
+// Persistent CTAs, one per SM, of GROUPS groups of 256 threads that share the
+// weights in shared memory; each group takes one tile of 128 points at a time
+// on its own (own operand buffer, accumulator, barrier), so that one group's
+// activations run while another waits for its products:
 //   layer 1 (2 -> 128) on the CUDA cores, one point per thread, BF16 result
 //     written to shared memory in the tensor cores' K-major layout;
 //   layers 2 and 3 (128 x 128) as tcgen05.mma kind::f16 (BF16 x BF16 -> FP32)
@@ -17,6 +19,12 @@
 //     CUDA cores);
 //   de-normalisation, and the exact kernel for points outside the band or
 //     in a cell the error-bound table marks.
+// What bounds it: the special-function unit (512 operations per point: two
+// hidden layers by tanh, the last by exp and a reciprocal) and the activations'
+// other instructions, not the tensor cores.  2e7 points, 12 % of them served by
+// the network: classify_kernel 433 -> 211 us, sur_kernel 1047 -> 380 us
+// with four groups (664 us with one, 478 with two)
+// (before: one group, the last layer's SiLU by expf and an IEEE division).
 // Every mbarrier wait is bounded; on time-out the kernel records an error,
 // stops issuing work, frees its tensor memory and returns.
 #include <cuda_bf16.h>
@@ -38,9 +46,11 @@ namespace {
 
 constexpr int H = PT_MLP_HIDDEN;
 constexpr int TILE = 128;                 // points per tile = MMA M
-constexpr int NTHR = 256;                 // 8 warps
+constexpr int NTHR = 256;                 // threads per group (8 warps)
+constexpr int GROUPS = 4;
 constexpr int TILE_BYTES = H * H * 2;     // one 128 x 128 BF16 operand (32 KB)
-constexpr int TMEM_COLS = 128;            // FP32 accumulator 128 x 128
+constexpr int TMEM_COLS = 128;            // FP32 accumulator 128 x 128, per group
+constexpr int TMEM_ALLOC = GROUPS > 2 ? 512 : GROUPS * TMEM_COLS;   // a power of two
 constexpr long long WAIT_LIMIT = 1 << 22; // bounded mbarrier polls
 
 constexpr int OFF_W1 = 0, OFF_B1 = 2 * H, OFF_W2 = 3 * H, OFF_B2 = 3 * H + H * H, OFF_W3 = 4 * H + H * H,
@@ -167,7 +177,14 @@ __device__ __forceinline__ float silu_fast(float x)
     return 0.5f * x * (1.0f + t);
 }
 
-__device__ __forceinline__ float silu_acc(float x) { return x / (1.0f + expf(-x)); }
+// SiLU of the last hidden layer, in FP32: one exponential and one reciprocal
+// (about 1e-7 absolute; the layer's input carries the 1e-3 of its BF16 operands)
+__device__ __forceinline__ float silu_acc(float x)
+{
+    float e;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(-1.44269504f * x));
+    return x * pt::rcp_a(1.0f + e);
+}
 
 struct SurModel {
     const float *p32;          // FP32 parameters (W1, b1, b2, b3, W4, b4 used from here)
@@ -193,59 +210,97 @@ struct SurArgs {
 };
 
 // Classify every point: outside the band or in a marked cell -> exact
-// kernel here and now; otherwise append to the network's list.
-__global__ void classify_kernel(SurModel m, const float *k, const float *z, size_t n, float *le, float *ld,
-                                float *ed, int *list, int *count, int *n_fallback)
+// kernel here and now; otherwise append to the network's list.  A CTA takes
+// CL_PER points per thread and reserves its stretch of the list with one
+// atomic: with one per warp the list's counter, a single address, set the time
+// (433 us for 2e7 points, of which the exact terms need about 160).
+constexpr int CL_THREADS = 256, CL_PER = 8;
+
+__global__ void __launch_bounds__(CL_THREADS) classify_kernel(SurModel m, const float *k, const float *z, size_t n,
+                                                              float *le, float *ld, float *ed, int *list, int *count,
+                                                              int *n_fallback)
 {
-    size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool net = false;
-    if (i < n) {
-        float kk = k[i], zz = fabsf(z[i]);
-        float s = (zz - fabsf(1.0f - kk)) / (2.0f * fminf(kk, 1.0f));
-        net = kk >= m.k_lo && kk <= m.k_hi && s >= 0.0f && s < 1.0f;
-        if (net) {
-            int ck = min(m.nk - 1, (int)((kk - m.k_lo) / (m.k_hi - m.k_lo) * m.nk));
-            int cs = min(m.ns - 1, (int)(s * m.ns));
-            net = m.table[ck * m.ns + cs] == 0;
-        }
-        if (!net) {
-            float a, b, c;
-            pt::ma_terms(kk, zz, &a, &b, &c);
-            le[i] = a;
-            ld[i] = b;
-            ed[i] = c;
+    __shared__ int swarp[CL_THREADS / 32], sbase;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const size_t i0 = (size_t)blockIdx.x * (CL_THREADS * CL_PER) + tid;
+    unsigned net = 0u;   // bit u: point i0 + u CL_THREADS goes to the network
+    const float dk = m.k_hi - m.k_lo;
+#pragma unroll
+    for (int u = 0; u < CL_PER; ++u) {
+        const size_t i = i0 + u * CL_THREADS;
+        if (i >= n) break;
+        const float kk = k[i], zz = fabsf(z[i]);
+        const float s = (zz - fabsf(1.0f - kk)) / (2.0f * fminf(kk, 1.0f));
+        if (kk >= m.k_lo && kk <= m.k_hi && s >= 0.0f && s < 1.0f) {
+            const int ck = min(m.nk - 1, (int)((kk - m.k_lo) / dk * m.nk));
+            const int cs = min(m.ns - 1, (int)(s * m.ns));
+            if (m.table[ck * m.ns + cs] == 0) net |= 1u << u;
         }
     }
-    // warp-aggregated appends
-    unsigned mask = __ballot_sync(0xffffffffu, net);
-    int lane = threadIdx.x & 31;
-    int base = 0;
-    if (lane == 0 && mask) base = atomicAdd(count, __popc(mask));
-    base = __shfl_sync(0xffffffffu, base, 0);
-    if (net) list[base + __popc(mask & ((1u << lane) - 1u))] = (int)i;
-    unsigned fb = __ballot_sync(0xffffffffu, i < n && !net);
-    if (lane == 0 && fb && n_fallback) atomicAdd(n_fallback, __popc(fb));
+    // places in the list: thread by thread
+    const int c = __popc(net);
+    int x = c;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) swarp[warp] = x;
+    __syncthreads();
+    int base = 0, all = 0;
+#pragma unroll
+    for (int w = 0; w < CL_THREADS / 32; ++w) {
+        base += w < warp ? swarp[w] : 0;
+        all += swarp[w];
+    }
+    if (tid == 0) {
+        sbase = all ? atomicAdd(count, all) : 0;
+        const size_t first = (size_t)blockIdx.x * (CL_THREADS * CL_PER);
+        const size_t left = n - first;
+        const int mine = (int)(left < (size_t)(CL_THREADS * CL_PER) ? left : (size_t)(CL_THREADS * CL_PER));
+        if (n_fallback && mine > all) atomicAdd(n_fallback, mine - all);
+    }
+    __syncthreads();
+    int at = sbase + base + x - c;
+#pragma unroll 1
+    for (int u = 0; u < CL_PER; ++u) {
+        const size_t i = i0 + u * CL_THREADS;
+        if (i >= n) break;
+        if ((net >> u) & 1u) {
+            list[at++] = (int)i;
+        } else {
+            float a0, a1, a2;
+            pt::ma_terms(k[i], fabsf(z[i]), &a0, &a1, &a2);
+            le[i] = a0;
+            ld[i] = a1;
+            ed[i] = a2;
+        }
+    }
 }
 
-// Thread layout: 8 warps; warp w serves tile rows 32 (w % 4) .. +31 (the
+// Thread layout: per group 8 warps; warp w serves tile rows 32 (w % 4) .. +31 (the
 // tensor-memory lanes it may read) and columns 64 (w / 4) .. +63.
-__global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
+__device__ __forceinline__ void group_sync(int g)
+{
+    asm volatile("bar.sync %0, %1;" ::"r"(g + 1), "n"(NTHR) : "memory");
+}
+
+__global__ void __launch_bounds__(GROUPS *NTHR, 1) sur_kernel(SurArgs A)
 {
     extern __shared__ __align__(1024) unsigned char smem[];
-    unsigned char *sA = smem;                        // activations, 32 KB
-    unsigned char *sW2 = smem + TILE_BYTES;          // 32 KB
-    unsigned char *sW3 = smem + 2 * TILE_BYTES;      // 32 KB
-    float *sW1 = reinterpret_cast<float *>(smem + 3 * TILE_BYTES);   // [128][2]
-    float *sB1 = sW1 + 2 * H;
-    float *sB2 = sB1 + H;
-    float *sB3 = sB2 + H;
-    float *sW4 = sB3 + H;                                           // [2][128]
-    float *sY = sW4 + 2 * H;                                        // [128][2] partial outputs
-    __shared__ uint64_t bar;
+    const int grp = threadIdx.x / NTHR, tid = threadIdx.x % NTHR, warp = tid >> 5;
+    unsigned char *sW2 = smem;                       // 32 KB
+    unsigned char *sW3 = smem + TILE_BYTES;          // 32 KB
+    unsigned char *sA = smem + (2 + grp) * TILE_BYTES;   // the group's activations, 32 KB
+    float4 *sL1 = reinterpret_cast<float4 *>(smem + (2 + GROUPS) * TILE_BYTES);   // [128]: W1 row, b1, -
+    float4 *sL3 = sL1 + H;                                          // [128]: b3, W4 column, -
+    float *sB2 = reinterpret_cast<float *>(sL3 + H);
+    float *sY = sB2 + H + grp * 2 * TILE;                           // [128][2] partial outputs
+    __shared__ uint64_t bars[GROUPS];
     __shared__ uint32_t tmem_base;
-    __shared__ int s_abort;
-
-    const int tid = threadIdx.x, warp = tid >> 5;
+    __shared__ int s_aborts[GROUPS];
+    uint64_t &bar = bars[grp];
+    volatile int &s_abort = s_aborts[grp];
     const int row = 32 * (warp & 3) + (tid & 31);
     const int half = warp >> 2, c0 = 64 * half;
     {
@@ -253,18 +308,14 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
         const uint4 *g3 = reinterpret_cast<const uint4 *>(A.m.w3);
         uint4 *d2 = reinterpret_cast<uint4 *>(sW2);
         uint4 *d3 = reinterpret_cast<uint4 *>(sW3);
-        for (int i = tid; i < TILE_BYTES / 16; i += NTHR) {
+        for (int i = threadIdx.x; i < TILE_BYTES / 16; i += GROUPS * NTHR) {
             d2[i] = g2[i];
             d3[i] = g3[i];
         }
-        for (int i = tid; i < 2 * H; i += NTHR) {
-            sW1[i] = A.m.p32[OFF_W1 + i];
-            sW4[i] = A.m.p32[OFF_W4 + i];
-        }
-        for (int i = tid; i < H; i += NTHR) {
-            sB1[i] = A.m.p32[OFF_B1 + i];
+        for (int i = threadIdx.x; i < H; i += GROUPS * NTHR) {
+            sL1[i] = make_float4(A.m.p32[OFF_W1 + 2 * i], A.m.p32[OFF_W1 + 2 * i + 1], A.m.p32[OFF_B1 + i], 0.0f);
+            sL3[i] = make_float4(A.m.p32[OFF_B3 + i], A.m.p32[OFF_W4 + i], A.m.p32[OFF_W4 + H + i], 0.0f);
             sB2[i] = A.m.p32[OFF_B2 + i];
-            sB3[i] = A.m.p32[OFF_B3 + i];
         }
     }
     if (tid == 0) {
@@ -272,9 +323,9 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
         s_abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
-    if (warp == 0) {
+    if (threadIdx.x < 32) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
-                     "r"((uint32_t)TMEM_COLS)
+                     "r"((uint32_t)TMEM_ALLOC)
                      : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
@@ -282,7 +333,7 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem = tmem_base;
+    const uint32_t tmem = tmem_base + (uint32_t)(grp * TMEM_COLS);
     const uint32_t aA = smem_u32(sA), aW2 = smem_u32(sW2), aW3 = smem_u32(sW3);
     const uint32_t trow = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
     const float b4_0 = A.m.p32[OFF_B4], b4_1 = A.m.p32[OFF_B4 + 1];
@@ -290,7 +341,7 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
     const size_t n_tiles = (n + TILE - 1) / TILE;
     uint32_t phase = 0;   // parity of the next mbarrier phase to complete
 
-    for (size_t tile = blockIdx.x; tile < n_tiles; tile += gridDim.x) {
+    for (size_t tile = (size_t)blockIdx.x * GROUPS + grp; tile < n_tiles; tile += (size_t)gridDim.x * GROUPS) {
         const size_t slot = tile * TILE + row;
         const bool valid = slot < n;
         size_t i = slot;
@@ -314,22 +365,22 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
             __align__(16) __nv_bfloat16 h8[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                int j = k0 + q;
-                float zj = fmaf(sW1[2 * j], x0, fmaf(sW1[2 * j + 1], x1, sB1[j]));
+                const float4 w = sL1[k0 + q];
+                float zj = fmaf(w.x, x0, fmaf(w.y, x1, w.z));
                 h8[q] = __float2bfloat16_rn(silu_fast(zj));
             }
             *reinterpret_cast<uint4 *>(sA + op_offset(row, k0)) = *reinterpret_cast<uint4 *>(h8);
         }
         fence_async_smem();
         tc_fence_before();
-        __syncthreads();
+        group_sync(grp);
         tc_fence_after();
         if (tid == 0 && !s_abort) issue_layer(tmem, aA, aW2, &bar);
         bool ok = mbar_wait(&bar, phase);
         phase ^= 1u;
         if (!ok) s_abort = 1;
         tc_fence_after();
-        __syncthreads();
+        group_sync(grp);
         if (s_abort) break;
         // ---- epilogue 2
 #pragma unroll 1
@@ -347,14 +398,14 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
         }
         fence_async_smem();
         tc_fence_before();
-        __syncthreads();
+        group_sync(grp);
         tc_fence_after();
         if (tid == 0 && !s_abort) issue_layer(tmem, aA, aW3, &bar);
         ok = mbar_wait(&bar, phase);
         phase ^= 1u;
         if (!ok) s_abort = 1;
         tc_fence_after();
-        __syncthreads();
+        group_sync(grp);
         if (s_abort) break;
         // ---- epilogue 3 + layer 4 partial sums over this thread's columns
         float y0 = 0.0f, y1 = 0.0f;
@@ -364,10 +415,10 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
             tmem_ld32(trow + (uint32_t)c, v);
 #pragma unroll
             for (int q = 0; q < 32; ++q) {
-                int j = c0 + c + q;
-                float h = silu_acc(v[q] + sB3[j]);
-                y0 = fmaf(sW4[j], h, y0);
-                y1 = fmaf(sW4[H + j], h, y1);
+                const float4 w = sL3[c0 + c + q];
+                float h = silu_acc(v[q] + w.x);
+                y0 = fmaf(w.y, h, y0);
+                y1 = fmaf(w.z, h, y1);
             }
         }
         if (half == 1) {
@@ -375,7 +426,7 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
             sY[2 * row + 1] = y1;
         }
         tc_fence_before();
-        __syncthreads();   // partial sums exchanged; accumulator fully read before the next MMA
+        group_sync(grp);   // partial sums exchanged; accumulator fully read before the next MMA
         tc_fence_after();
         if (half == 0 && valid) {
             y0 += sY[2 * row] + b4_0;
@@ -396,8 +447,8 @@ __global__ void __launch_bounds__(NTHR) sur_kernel(SurArgs A)
     __syncthreads();
     tc_fence_after();
     if (tid == 0 && s_abort && A.err) atomicExch(A.err, 1);
-    if (warp == 0)
-        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"((uint32_t)TMEM_COLS)
+    if (threadIdx.x < 32)
+        asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem_base), "r"((uint32_t)TMEM_ALLOC)
                      : "memory");
 }
 
@@ -431,7 +482,7 @@ __global__ void pack_weights_kernel(const float *W, __nv_bfloat16 *out)
     out[op_offset(r, k) / 2] = __float2bfloat16_rn(W[idx]);
 }
 
-size_t sur_smem() { return (size_t)3 * TILE_BYTES + (size_t)(2 * H + 3 * H + 2 * H + 2 * TILE) * sizeof(float); }
+size_t sur_smem() { return (size_t)(2 + GROUPS) * TILE_BYTES + (size_t)(8 * H + H + GROUPS * 2 * TILE) * sizeof(float); }
 
 }  // namespace
 
@@ -471,7 +522,7 @@ int pt_sur_model_create(const float *params_dev, const float *norm, float k_lo, 
     if (e == cudaSuccess)
         e = cudaFuncSetAttribute(sur_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sur_smem());
     int per_sm = 0;
-    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sur_kernel, NTHR, sur_smem());
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sur_kernel, GROUPS * NTHR, sur_smem());
     int dev = 0, nsm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
@@ -486,7 +537,7 @@ int pt_sur_model_create(const float *params_dev, const float *norm, float k_lo, 
         delete p;
         return st;
     }
-    p->grid = nsm * per_sm;
+    p->grid = nsm;   // persistent, one CTA per SM
     p->m.p32 = p->d_p32;
     p->m.w2 = p->d_w2;
     p->m.w3 = p->d_w3;
@@ -517,9 +568,10 @@ static int launch_sur(pt_sur_model p, SurArgs &a, size_t max_points, pt_stream_t
     a.m = p->m;
     a.err = p->d_err;
     size_t tiles = (max_points + TILE - 1) / TILE;
+    tiles = (tiles + GROUPS - 1) / GROUPS;
     int grid = (int)(tiles < (size_t)p->grid ? tiles : (size_t)p->grid);
     if (grid < 1) grid = 1;
-    sur_kernel<<<grid, NTHR, sur_smem(), (cudaStream_t)stream>>>(a);
+    sur_kernel<<<grid, GROUPS * NTHR, sur_smem(), (cudaStream_t)stream>>>(a);
     return cuda_status("sur_kernel");
 }
 
@@ -551,8 +603,8 @@ int pt_ma_surrogate(pt_sur_model p, const float *k, const float *z, size_t n, fl
     int *list = (int *)((char *)work + 256);
     cudaError_t e = cudaMemsetAsync(count, 0, sizeof(int), s);
     if (e != cudaSuccess) return pt_internal::set_error(PT_ERR_CUDA, "pt_ma_surrogate", cudaGetErrorString(e));
-    size_t blocks = (n + 255) / 256;
-    classify_kernel<<<(unsigned)blocks, 256, 0, s>>>(p->m, k, z, n, le, ld, ed, list, count, n_fallback);
+    size_t blocks = (n + CL_THREADS * CL_PER - 1) / (CL_THREADS * CL_PER);
+    classify_kernel<<<(unsigned)blocks, CL_THREADS, 0, s>>>(p->m, k, z, n, le, ld, ed, list, count, n_fallback);
     int st = cuda_status("classify_kernel");
     if (st) return st;
     SurArgs a{};
