@@ -826,9 +826,9 @@ __device__ __forceinline__ float mt_lambda_inside(float p, float w)
     return zmp.h < 0.0f ? df_add(lam, DF{0.666666687f, -1.98682151e-08f}).h : lam.h;
 }
 
-// The exact terms at node q of interval i, with the distances to the contacts
-// formed from w (not from the rounded z).
-__device__ __forceinline__ void mt_node(float p, int i, int q, float *le, float *ld, float *ed)
+// Node q of interval i: its offset t, the separation and the distances
+// d = z - (1 - p) and e1 = (1 + p) - z, formed from w; returns w.
+__device__ __forceinline__ float mt_node_at(float p, int i, int q, float *z, float *d, float *e1, float *t)
 {
     const int q3 = q < 3 ? q : 5 - q;
     const float xa = q3 == 0 ? 0.96592582629f : (q3 == 1 ? 0.70710678119f : 0.25881904510f);
@@ -837,15 +837,31 @@ __device__ __forceinline__ void mt_node(float p, int i, int q, float *le, float 
     mt_scales(p, &sA, &sL);
     const int reg = i < MT_NA ? 0 : (i < MT_NA + MT_NL ? 1 : 2);
     const int il = i - (reg == 0 ? 0 : (reg == 1 ? MT_NA : MT_NA + MT_NL));
+    *t = il == 0 ? 0.25f * (1.0f + x) : 0.5f * x;
     const float u = il == 0 ? 0.25f * (1.0f + x) : (float)il + 0.5f * x;
     const float w = u / (reg == 0 ? sA : sL);
     const float w2 = w * w;
-    const float d = reg == 0 ? -w2 : (reg == 1 ? w2 : 2.0f * p - w2);
-    const float e1 = reg == 0 ? 2.0f * p + w2 : (reg == 1 ? 2.0f * p - w2 : w2);
-    const float z = reg == 2 ? (1.0f + p) - w2 : (1.0f - p) + d;
-    ma_terms_core<false, true>(p, z, d, e1, le, ld, ed);
-    // (z = p, where the second integral's parameters are infinite, keeps the separate case)
-    if (reg == 0 && fabsf(z - p) > 1e-5f) *ld = mt_lambda_inside(p, w);
+    *d = reg == 0 ? -w2 : (reg == 1 ? w2 : 2.0f * p - w2);
+    *e1 = reg == 0 ? 2.0f * p + w2 : (reg == 1 ? 2.0f * p - w2 : w2);
+    *z = reg == 2 ? (1.0f + p) - w2 : (1.0f - p) + *d;
+    return w;
+}
+
+// The exact terms at that node, with the distances to the contacts formed
+// from w (not from the rounded z).
+__device__ __forceinline__ void mt_node(float p, int i, int q, float *le, float *ld, float *ed)
+{
+    float z, d, e1, t;
+    const float w = mt_node_at(p, i, q, &z, &d, &e1, &t);
+    // (z = p, where the second integral's parameters are infinite, keeps the FP32 terms and their separate case)
+    if (i < MT_NA && fabsf(z - p) > 1e-5f) {
+        const float p2 = p * p;
+        *le = p2;
+        *ed = 0.5f * p2 * (p2 + 2.0f * z * z);
+        *ld = mt_lambda_inside(p, w);
+    } else {
+        ma_terms_core<false, true>(p, z, d, e1, le, ld, ed);
+    }
 }
 
 // Interval and offset of separation z.  zm1 = z - 1; off_limb is the constant
