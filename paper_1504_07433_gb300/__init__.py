@@ -113,25 +113,50 @@ def _check(status, what):
                                               lib.pt_last_error_string().decode()))
 
 
+_TORCH = None
+_RAW_STREAM = None   # (current device index, its current stream's handle) without building a Stream object
+
+
 def _torch():
-    import torch
-    return torch
+    global _TORCH, _RAW_STREAM
+    if _TORCH is None:
+        import torch
+        c = torch._C
+        if hasattr(c, "_cuda_getDevice") and hasattr(c, "_cuda_getCurrentRawStream"):
+            _RAW_STREAM = (c._cuda_getDevice, c._cuda_getCurrentRawStream)
+        _TORCH = torch
+    return _TORCH
+
+
+# A light curve of a few hundred points takes the GPU about 12 us, and the
+# marshalling around it set the time of a call (29 us): a Stream object, an
+# import statement and a c_void_p per argument.  The calls below pass addresses as
+# plain integers (every function's argument types are declared) and read the
+# stream's handle directly.
+def _stream_addr():
+    torch = _torch()
+    if _RAW_STREAM is not None and torch.cuda.is_initialized():
+        return _RAW_STREAM[1](_RAW_STREAM[0]())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _stream():
-    torch = _torch()
-    return _c_void_p(torch.cuda.current_stream().cuda_stream)
+    return _c_void_p(_stream_addr())
 
 
-def _ptr(x):
+def _addr(x):
+    """Device address of a contiguous CUDA tensor (None stays None)."""
     if x is None:
         return None
-    torch = _torch()
-    if not isinstance(x, torch.Tensor) or not x.is_cuda:
+    if not isinstance(x, _torch().Tensor) or not x.is_cuda:
         raise PTError("expected a CUDA tensor")
     if not x.is_contiguous():
         raise PTError("expected a contiguous tensor")
-    return _c_void_p(x.data_ptr())
+    return x.data_ptr()
+
+
+def _ptr(x):
+    return None if x is None else _c_void_p(_addr(x))
 
 
 def _dev(x, dtype, device):
@@ -157,9 +182,16 @@ def orbit_to_device(orbit, device="cuda"):
 
 
 def _orbit_struct(orb):
-    n_v = int(orb["t0"].numel())
-    return Orbit(_ptr(orb["t0"]), _ptr(orb["P"]), _ptr(orb["a"]), _ptr(orb["inc"]),
-                 _ptr(orb.get("e")), _ptr(orb.get("w")), n_v), n_v
+    t0 = orb["t0"]
+    n_v = t0.numel()
+    return Orbit(_addr(t0), _addr(orb["P"]), _addr(orb["a"]), _addr(orb["inc"]),
+                 _addr(orb.get("e")), _addr(orb.get("w")), n_v), n_v
+
+
+def _work(work, need, device):
+    if work is None or work.numel() < need:
+        work = _torch().empty(max(need, 256), dtype=_TORCH.uint8, device=device)
+    return work
 
 
 def z_circ(t, orb, n_ss=1, t_exp=0.0):
@@ -242,19 +274,17 @@ def ma_quad(t, orb, k, ld, n_ss=1, t_exp=0.0, max_iter=16, y=None, wt=None, want
     t [n_t] float64; orb from orbit_to_device; k [n_v] or [n_v, n_b] float32;
     ld [n_v, n_b, 2] float32 (u1, u2).  Returns (flux [n_v, n_b, n_t] or None,
     ssr [n_v, n_b] or None)."""
-    torch = _torch()
     lib = load_library()
     o, n_v = _orbit_struct(orb)
     n_b = int(ld.shape[1])
     kpb = 1 if k.dim() == 2 else 0
     n_t = t.numel()
     fl, ss = _lc_outputs(n_v, n_b, n_t, want_flux, want_ssr, t.device, flux, ssr)
-    need = int(lib.pt_ma_quad_work_bytes(n_t, n_v, n_b, kpb))
-    if work is None or work.numel() < need:
-        work = torch.empty(max(need, 256), dtype=torch.uint8, device=t.device)
-    _check(lib.pt_ma_quad(_ptr(t), n_t, ctypes.byref(o), _ptr(k), kpb, _ptr(ld), n_b, int(n_ss), float(t_exp),
-                          int(max_iter), _ptr(y), _ptr(wt), _ptr(fl), _ptr(ss), _ptr(work), work.numel(),
-                          _ptr(n_bad), _stream()), "pt_ma_quad")
+    need = lib.pt_ma_quad_work_bytes(n_t, n_v, n_b, kpb)
+    work = _work(work, need, t.device)
+    _check(lib.pt_ma_quad(_addr(t), n_t, ctypes.byref(o), _addr(k), kpb, _addr(ld), n_b, int(n_ss), float(t_exp),
+                          int(max_iter), _addr(y), _addr(wt), _addr(fl), _addr(ss), _addr(work), work.numel(),
+                          _addr(n_bad), _stream_addr()), "pt_ma_quad")
     return fl, ss
 
 
@@ -301,19 +331,17 @@ def ma_terms_interp(table, k, z):
 def ma_quad_interp(table, t, orb, k, ld, n_ss=1, t_exp=0.0, max_iter=16, y=None, wt=None, want_flux=True,
                    want_ssr=False, work=None, flux=None, ssr=None, n_bad=None):
     """ma_quad with the terms read from an MATable (pt_ma_quad_interp)."""
-    torch = _torch()
     lib = load_library()
     o, n_v = _orbit_struct(orb)
     n_b = int(ld.shape[1])
     kpb = 1 if k.dim() == 2 else 0
     n_t = t.numel()
     fl, ss = _lc_outputs(n_v, n_b, n_t, want_flux, want_ssr, t.device, flux, ssr)
-    need = int(lib.pt_ma_quad_work_bytes(n_t, n_v, n_b, kpb))
-    if work is None or work.numel() < need:
-        work = torch.empty(max(need, 256), dtype=torch.uint8, device=t.device)
-    _check(lib.pt_ma_quad_interp(table.handle, _ptr(t), n_t, ctypes.byref(o), _ptr(k), kpb, _ptr(ld), n_b,
-                                 int(n_ss), float(t_exp), int(max_iter), _ptr(y), _ptr(wt), _ptr(fl), _ptr(ss),
-                                 _ptr(work), work.numel(), _ptr(n_bad), _stream()), "pt_ma_quad_interp")
+    need = lib.pt_ma_quad_work_bytes(n_t, n_v, n_b, kpb)
+    work = _work(work, need, t.device)
+    _check(lib.pt_ma_quad_interp(table.handle, _addr(t), n_t, ctypes.byref(o), _addr(k), kpb, _addr(ld), n_b,
+                                 int(n_ss), float(t_exp), int(max_iter), _addr(y), _addr(wt), _addr(fl), _addr(ss),
+                                 _addr(work), work.numel(), _addr(n_bad), _stream_addr()), "pt_ma_quad_interp")
     return fl, ss
 
 
@@ -374,7 +402,6 @@ def gimenez_alpha(plan, k, z):
 def gimenez(plan, t, orb, k, ld, n_ss=1, t_exp=0.0, max_iter=16, y=None, wt=None, want_flux=True,
             want_ssr=False, work=None, flux=None, ssr=None, n_bad=None):
     """Gimenez light curves (pt_gimenez); ld [n_v, n_b, N] holds u_1..u_N."""
-    torch = _torch()
     lib = load_library()
     o, n_v = _orbit_struct(orb)
     n_b = int(ld.shape[1])
@@ -383,12 +410,11 @@ def gimenez(plan, t, orb, k, ld, n_ss=1, t_exp=0.0, max_iter=16, y=None, wt=None
     kpb = 1 if k.dim() == 2 else 0
     n_t = t.numel()
     fl, ss = _lc_outputs(n_v, n_b, n_t, want_flux, want_ssr, t.device, flux, ssr)
-    need = plan.work_bytes(n_t, n_v, n_b, kpb)
-    if work is None or work.numel() < need:
-        work = torch.empty(max(need, 256), dtype=torch.uint8, device=t.device)
-    _check(lib.pt_gimenez(plan.handle, _ptr(t), n_t, ctypes.byref(o), _ptr(k), kpb, _ptr(ld), n_b, int(n_ss),
-                          float(t_exp), int(max_iter), _ptr(y), _ptr(wt), _ptr(fl), _ptr(ss), _ptr(work),
-                          work.numel(), _ptr(n_bad), _stream()), "pt_gimenez")
+    need = lib.pt_gimenez_work_bytes(plan.handle, n_t, n_v, n_b, kpb)
+    work = _work(work, need, t.device)
+    _check(lib.pt_gimenez(plan.handle, _addr(t), n_t, ctypes.byref(o), _addr(k), kpb, _addr(ld), n_b, int(n_ss),
+                          float(t_exp), int(max_iter), _addr(y), _addr(wt), _addr(fl), _addr(ss), _addr(work),
+                          work.numel(), _addr(n_bad), _stream_addr()), "pt_gimenez")
     return fl, ss
 
 
@@ -396,7 +422,6 @@ def gimenez_zi(plan, t, orb, k, ld, n_in=64, n_edge=64, n_ss=1, t_exp=0.0, max_i
                want_flux=True, want_ssr=False, work=None, flux=None, ssr=None, n_bad=None):
     """Gimenez light curves interpolated in z (pt_gimenez_zi, Sec. 3.3):
     alpha_n on n_in nodes over [0, 1 - k] and n_edge over (1 - k, 1 + k]."""
-    torch = _torch()
     lib = load_library()
     o, n_v = _orbit_struct(orb)
     n_b = int(ld.shape[1])
@@ -405,12 +430,11 @@ def gimenez_zi(plan, t, orb, k, ld, n_in=64, n_edge=64, n_ss=1, t_exp=0.0, max_i
     kpb = 1 if k.dim() == 2 else 0
     n_t = t.numel()
     fl, ss = _lc_outputs(n_v, n_b, n_t, want_flux, want_ssr, t.device, flux, ssr)
-    need = int(lib.pt_gimenez_zi_work_bytes(plan.handle, int(n_in), int(n_edge), n_t, n_v, n_b, kpb))
-    if work is None or work.numel() < need:
-        work = torch.empty(max(need, 256), dtype=torch.uint8, device=t.device)
-    _check(lib.pt_gimenez_zi(plan.handle, int(n_in), int(n_edge), _ptr(t), n_t, ctypes.byref(o), _ptr(k), kpb,
-                             _ptr(ld), n_b, int(n_ss), float(t_exp), int(max_iter), _ptr(y), _ptr(wt), _ptr(fl),
-                             _ptr(ss), _ptr(work), work.numel(), _ptr(n_bad), _stream()), "pt_gimenez_zi")
+    need = lib.pt_gimenez_zi_work_bytes(plan.handle, int(n_in), int(n_edge), n_t, n_v, n_b, kpb)
+    work = _work(work, need, t.device)
+    _check(lib.pt_gimenez_zi(plan.handle, int(n_in), int(n_edge), _addr(t), n_t, ctypes.byref(o), _addr(k), kpb,
+                             _addr(ld), n_b, int(n_ss), float(t_exp), int(max_iter), _addr(y), _addr(wt), _addr(fl),
+                             _addr(ss), _addr(work), work.numel(), _addr(n_bad), _stream_addr()), "pt_gimenez_zi")
     return fl, ss
 
 
@@ -456,17 +480,16 @@ def ma_quad_bwd(t, theta, y, wt=None, n_ss=1, t_exp=0.0, max_iter=16, want_flux=
     torch = _torch()
     lib = load_library()
     n_v = int(theta["t0"].numel())
-    th = Theta(*(_ptr(theta.get(nm)) for nm in THETA_NAMES), n_v)
+    th = Theta(*(_addr(theta.get(nm)) for nm in THETA_NAMES), n_v)
     n_t = t.numel()
     grad = torch.empty((n_v, 9), dtype=torch.float32, device=t.device)
     ssr = torch.empty(n_v, dtype=torch.float32, device=t.device)
     flux = torch.empty((n_v, n_t), dtype=torch.float32, device=t.device) if want_flux else None
-    need = int(lib.pt_ma_quad_bwd_work_bytes(n_t))
-    if work is None or work.numel() < need:
-        work = torch.empty(max(need, 256), dtype=torch.uint8, device=t.device)
-    _check(lib.pt_ma_quad_bwd(_ptr(t), n_t, ctypes.byref(th), int(n_ss), float(t_exp), int(max_iter), _ptr(y),
-                              _ptr(wt), _ptr(grad), _ptr(ssr), _ptr(flux), _ptr(work), work.numel(), _ptr(n_bad),
-                              _stream()), "pt_ma_quad_bwd")
+    need = lib.pt_ma_quad_bwd_work_bytes(n_t)
+    work = _work(work, need, t.device)
+    _check(lib.pt_ma_quad_bwd(_addr(t), n_t, ctypes.byref(th), int(n_ss), float(t_exp), int(max_iter), _addr(y),
+                              _addr(wt), _addr(grad), _addr(ssr), _addr(flux), _addr(work), work.numel(), _addr(n_bad),
+                              _stream_addr()), "pt_ma_quad_bwd")
     return ssr, grad, flux
 
 
