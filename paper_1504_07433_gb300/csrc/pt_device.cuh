@@ -1017,24 +1017,31 @@ __device__ __forceinline__ void make_geom_rec(double t0, double P, float a_f, fl
     // FP32 suffices: the anchor's sine and cosine only scale the small
     // differential terms of orbit_z (relative error ~1e-7 there), and the
     // sky position at conjunction is zero by construction, not computed.
-    float ef = (float)e, wf = (float)w;
-    float ftrf = 0.5f * PT_PI_F - wf;
-    float Etrf = 2.0f * atan2f(sqrtf(1.0f - ef) * sinf(0.5f * ftrf), sqrtf(1.0f + ef) * cosf(0.5f * ftrf));
-    float sEf, cEf, swf, cwf;
-    sincosf(Etrf, &sEf, &cEf);
-    sincosf(wf, &swf, &cwf);
-    float sef = sqrtf((1.0f - ef) * (1.0f + ef)), af = (float)a;
-    double ftr = 0.5 * PT_PI_D - w;
-    double Etr = Etrf, sE = sEf;
-    r.ecE = ef * cEf;
-    r.esE = ef * sEf;
-    r.cE = cEf;
-    r.sE = sEf;
-    r.Uc = af * cwf;
-    r.Us = af * sef * swf;
-    r.Vs = af * swf;
-    r.Vc = af * sef * cwf;
-    r.Vtr = af * (1.0f - ef * cEf);
+    // A circular orbit uses none of it (orbit_z, orbit_state).
+    double ftr = 0.0, Etr = 0.0, sE = 0.0;
+    r.ecE = r.esE = r.sE = r.Uc = r.Us = r.Vs = r.Vc = r.Vtr = 0.0f;
+    r.cE = 1.0f;
+    if (ecc) {
+        float ef = (float)e, wf = (float)w;
+        float ftrf = 0.5f * PT_PI_F - wf;
+        float Etrf = 2.0f * atan2f(sqrtf(1.0f - ef) * sinf(0.5f * ftrf), sqrtf(1.0f + ef) * cosf(0.5f * ftrf));
+        float sEf, cEf, swf, cwf;
+        sincosf(Etrf, &sEf, &cEf);
+        sincosf(wf, &swf, &cwf);
+        float sef = sqrtf((1.0f - ef) * (1.0f + ef)), af = (float)a;
+        ftr = 0.5 * PT_PI_D - w;
+        Etr = Etrf;
+        sE = sEf;
+        r.ecE = ef * cEf;
+        r.esE = ef * sEf;
+        r.cE = cEf;
+        r.sE = sEf;
+        r.Uc = af * cwf;
+        r.Us = af * sef * swf;
+        r.Vs = af * swf;
+        r.Vc = af * sef * cwf;
+        r.Vtr = af * (1.0f - ef * cEf);
+    }
     r.nq = ecc ? (float)(e / (1.0 - e)) : 0.0f;
     r.pad1 = r.pad2 = 0.0f;
     // Conservative window.  z^2 >= r_min^2 (sin^2(th) sin^2 i + cos^2 i) with
