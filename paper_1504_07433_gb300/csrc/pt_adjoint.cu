@@ -533,6 +533,7 @@ __device__ bool rows_pay(float a, float P, float k, float n, const float2 *tile_
 __global__ void __launch_bounds__(TT) tile_kernel(const double *t, const float *y, const float *wt, int n,
                                                   float2 *tsplit, float2 *tile_mm, double *tile_ssr)
 {
+    pt::chain_next();
     __shared__ double smin[TT / 32], smax[TT / 32], ssum[TT / 32];
     const int i = blockIdx.x * TT + threadIdx.x;
     double lo = INFINITY, hi = -INFINITY, r2 = 0.0;
@@ -732,6 +733,7 @@ __device__ __forceinline__ void vector_sums(const BwdArgs &A, const VecConst &sc
 template <int TB, bool SS1>
 __global__ void __launch_bounds__(TB, 896 / TB) ma_bwd_kernel(BwdArgs A)
 {
+    pt::chain_next();
     constexpr int NW = TB / 32;
     __shared__ VecConst sc;
     __shared__ __align__(16) float srow[GR_ROW];
@@ -751,6 +753,8 @@ __global__ void __launch_bounds__(TB, 896 / TB) ma_bwd_kernel(BwdArgs A)
     // those across the limb.
     if (warp == 0) make_const(A.th, v, 0.5f * A.t_exp, &sc);
     if (threadIdx.x == 0) sbad = 0;
+    // the inputs were there before tile_kernel was launched; its results are waited for here
+    pt::chain_wait();
     if (warp > 0) {
         const bool r = k >= GR_PMIN && k <= pt::MT_PMAX &&
                        rows_pay(A.th.a[v], (float)A.th.P[v], k, (float)A.n_t * (float)A.n_ss, A.tile_mm,
@@ -876,9 +880,9 @@ int pt_ma_quad_bwd(const double *t, int n_t, const pt_theta *th, int n_ss, doubl
     A.flux = flux;
     A.n_bad = n_bad;
     if (th->n_v >= WIDE_MAX_VECTORS)
-        (n_ss == 1 ? ma_bwd_kernel<128, true> : ma_bwd_kernel<128, false>)<<<th->n_v, 128, 0, s>>>(A);
+        pt::launch_chained(n_ss == 1 ? ma_bwd_kernel<128, true> : ma_bwd_kernel<128, false>, th->n_v, 128, 0, s, A);
     else
-        (n_ss == 1 ? ma_bwd_kernel<384, true> : ma_bwd_kernel<384, false>)<<<th->n_v, 384, 0, s>>>(A);
+        pt::launch_chained(n_ss == 1 ? ma_bwd_kernel<384, true> : ma_bwd_kernel<384, false>, th->n_v, 384, 0, s, A);
     e = cudaGetLastError();
     return e == cudaSuccess ? PT_OK : pt_internal::set_error(PT_ERR_CUDA, "ma_bwd_kernel", cudaGetErrorString(e));
 }

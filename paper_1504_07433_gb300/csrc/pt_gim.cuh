@@ -196,6 +196,7 @@ template <int RT>
 __global__ void __launch_bounds__(32 * Split<RT>::WARPS, 1) product_kernel(const float *At, int Rp, const float *B, int K,
                                                                            int Nc, int R, float *out)
 {
+    pt::chain_begin();
     constexpr int WARPS = Split<RT>::WARPS, C = Split<RT>::COLS;
     extern __shared__ __align__(16) float psm[];   // [PARTS][RT][CT]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -216,8 +217,8 @@ __global__ void __launch_bounds__(32 * Split<RT>::WARPS, 1) product_kernel(const
             for (int j = 0; j < C; ++j) acc[i][j] = 0.0f;
 #pragma unroll(RT == 32 ? 3 : 12)
         for (int k = k0; k < k1; ++k) {
-            const float4 a0 = __ldg(reinterpret_cast<const float4 *>(pa + (size_t)k * Rp));
-            const float4 a1 = __ldg(reinterpret_cast<const float4 *>(pa + (size_t)k * Rp + 4));
+            const float4 a0 = *reinterpret_cast<const float4 *>(pa + (size_t)k * Rp);   // this call's: not by __ldg
+            const float4 a1 = *reinterpret_cast<const float4 *>(pa + (size_t)k * Rp + 4);
             const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
             float b[C];
             if (C == 8) {
@@ -253,6 +254,7 @@ __global__ void __launch_bounds__(32 * Split<RT>::WARPS, 1) product_kernel(const
 // Rows on z nodes (Sec. 3.3) read from the series' rows: node i of a row.
 __global__ void zi_rows_kernel(rows::Args A, const float *k, int n_row, int zi_len, float *out)
 {
+    pt::chain_begin();
     const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     const long long row = id / zi_len;
     if (row >= n_row) return;

@@ -100,6 +100,7 @@ __device__ void make_geom(const SetupArgs &s, int g, GeomRec *out)
 
 __global__ void setup_kernel(SetupArgs s)
 {
+    pt::chain_begin();
     if ((int)blockIdx.x < s.n_gblocks) {
         int g = blockIdx.x * blockDim.x + threadIdx.x;
         if (g < s.n_geom) {
@@ -154,6 +155,7 @@ __device__ __forceinline__ float3 row_weights(const RowPrep &P, int g, int r)
 template <int MODEL>
 __global__ void __launch_bounds__(ROW_THREADS) row_prep_kernel(RowPrep P)
 {
+    pt::chain_begin();
     __shared__ float3 sF[ROW_GEOM][pt::MT_N * pt::MT_Q];
     const int tid = threadIdx.x;
     const SetupArgs &s = P.s;
@@ -334,6 +336,7 @@ __device__ __forceinline__ float ss_offset(float t_exp, int s, float inv_nss)
 template <bool INTERP, bool OWN>
 __global__ void __launch_bounds__(TT) ma_lc_kernel(LcArgs A)
 {
+    pt::chain_begin();
     __shared__ GeomRec srec[VT_MA];
     __shared__ float sdt[VT_MA][TT];
     __shared__ unsigned char sflag[VT_MA][TT];
@@ -430,6 +433,7 @@ __global__ void __launch_bounds__(TT) ma_lc_kernel(LcArgs A)
 
 __global__ void ssr_reduce_kernel(const float *part, int rows, int n_tiles, float *ssr)
 {
+    pt::chain_begin();
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (warp >= rows) return;
@@ -454,6 +458,7 @@ int ssr_chunks(int n_t) { return (n_t + SSR_CHUNK - 1) / SSR_CHUNK; }
 __global__ void __launch_bounds__(256) ssr_part_kernel(const float *flux, const float *y, const float *wt, int n_t,
                                                       int n_b, float *part)
 {
+    pt::chain_begin();
     __shared__ float sred[8];
     const size_t row = blockIdx.x;
     const int band = (int)(row % n_b);
@@ -484,10 +489,10 @@ int launch_ssr_rows(const float *flux, const float *y, const float *wt, int n_t,
                     float *ssr, cudaStream_t s)
 {
     const int nc = ssr_chunks(n_t);
-    ssr_part_kernel<<<dim3((unsigned)rows, (unsigned)nc), 256, 0, s>>>(flux, y, wt, n_t, n_b, part);
+    pt::launch_chained(ssr_part_kernel, dim3((unsigned)rows, (unsigned)nc), 256, 0, s, flux, y, wt, n_t, n_b, part);
     int st = check_launch("ssr_part_kernel");
     if (st) return st;
-    ssr_reduce_kernel<<<(unsigned)((rows * 32 + 255) / 256), 256, 0, s>>>(part, (int)rows, nc, ssr);
+    pt::launch_chained(ssr_reduce_kernel, (unsigned)((rows * 32 + 255) / 256), 256, 0, s, part, (int)rows, nc, ssr);
     return check_launch("ssr_reduce_kernel");
 }
 
@@ -758,7 +763,7 @@ int launch_rows(int model, rows::Args &A, int n_sm, cudaStream_t s)
     // geometries along x, time tiles along y, in as many launches as y takes
     for (A.tile0 = 0; A.tile0 < A.n_tiles; A.tile0 += 65535) {
         const dim3 grid((unsigned)((A.n_geom + vt - 1) / vt), (unsigned)std::min(65535, A.n_tiles - A.tile0));
-        fn<<<grid, rows::TB, smem, s>>>(A);
+        pt::launch_chained(fn, grid, rows::TB, (size_t)smem, s, A);
         const int st = check_launch("lc_rows_kernel");
         if (st) return st;
     }
@@ -1181,7 +1186,8 @@ static int ma_quad_rows(const pt_ma_table_s *tab, const double *t, int n_t, cons
     if (st || !ssr) return st;
     const int n_rows = orb->n_v * n_b;
     if (!fused_ssr) return launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)n_rows, part, ssr, s);
-    ssr_reduce_kernel<<<(unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s>>>(part, n_rows, A.n_tiles, ssr);
+    pt::launch_chained(ssr_reduce_kernel, (unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s, part, n_rows, A.n_tiles,
+                       ssr);
     return check_launch("ssr_reduce_kernel");
 }
 
@@ -1236,6 +1242,7 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     A.n_tiles = n_tiles;
     A.n_bad = n_bad;
     dim3 grid(A.n_tiles, gy);
+    void (*fn)(LcArgs);
     if (tab) {
         A.mtab = tab->d_tab;
         A.mn_k = tab->n_k;
@@ -1244,15 +1251,19 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
         A.mk_hi = tab->k_hi;
         A.minv_dk = tab->inv_dk;
         A.minv_dz = tab->inv_dz;
-        (own ? ma_lc_kernel<true, true> : ma_lc_kernel<true, false>)<<<grid, TT, 0, s>>>(A);
+        fn = own ? ma_lc_kernel<true, true> : ma_lc_kernel<true, false>;
     } else {
-        (own ? ma_lc_kernel<false, true> : ma_lc_kernel<false, false>)<<<grid, TT, 0, s>>>(A);
+        fn = own ? ma_lc_kernel<false, true> : ma_lc_kernel<false, false>;
     }
+    if (own)
+        fn<<<grid, TT, 0, s>>>(A);
+    else
+        pt::launch_chained(fn, grid, TT, 0, s, A);
     st = check_launch("ma_lc_kernel");
     if (st) return st;
     if (ssr) {
         int rows = orb->n_v * n_b;
-        ssr_reduce_kernel<<<(rows * 32 + 255) / 256, 256, 0, s>>>(part, rows, A.n_tiles, ssr);
+        pt::launch_chained(ssr_reduce_kernel, (rows * 32 + 255) / 256, 256, 0, s, part, rows, A.n_tiles, ssr);
         st = check_launch("ssr_reduce_kernel");
     }
     return st;
@@ -1536,11 +1547,11 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     if (r32 * gx >= (size_t)n_sm / 2) {
         e = cudaFuncSetAttribute(gim::product_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gim::Split<32>::SMEM);
         if (e == cudaSuccess)
-            gim::product_kernel<32><<<(unsigned)(r32 * gx), 32 * gim::Split<32>::WARPS, gim::Split<32>::SMEM, s>>>(
-                P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
+            pt::launch_chained(gim::product_kernel<32>, (unsigned)(r32 * gx), 32 * gim::Split<32>::WARPS,
+                               (size_t)gim::Split<32>::SMEM, s, P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
     } else {
-        gim::product_kernel<8><<<(unsigned)(r8 * gx), 32 * gim::Split<8>::WARPS, gim::Split<8>::SMEM, s>>>(
-            P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
+        pt::launch_chained(gim::product_kernel<8>, (unsigned)(r8 * gx), 32 * gim::Split<8>::WARPS,
+                           (size_t)gim::Split<8>::SMEM, s, P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
     }
     if (e != cudaSuccess) return set_cuda_error(e, "product_kernel smem attribute");
     st = check_launch("product_kernel");
@@ -1578,7 +1589,7 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
         float *zrows = (float *)(wb + L.zi);
         const long long n = (long long)R * zi_len;
         if ((n + 127) / 128 > 0x7fffffffLL) return PT_ERR_ARG;
-        gim::zi_rows_kernel<<<(unsigned)((n + 127) / 128), 128, 0, s>>>(A, k, (int)R, zi_len, zrows);
+        pt::launch_chained(gim::zi_rows_kernel, (unsigned)((n + 127) / 128), 128, 0, s, A, k, (int)R, zi_len, zrows);
         st = check_launch("zi_rows_kernel");
         if (st) return st;
         A.rows = zrows;
@@ -1591,7 +1602,8 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     if (!ssr) return PT_OK;
     const int n_rows = orb->n_v * n_b;
     if (!fused_ssr) return launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)n_rows, part, ssr, s);
-    ssr_reduce_kernel<<<(unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s>>>(part, n_rows, A.n_tiles, ssr);
+    pt::launch_chained(ssr_reduce_kernel, (unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s, part, n_rows, A.n_tiles,
+                       ssr);
     return check_launch("ssr_reduce_kernel");
 }
 

@@ -257,6 +257,7 @@ __device__ __forceinline__ void put_sums(float *sRed, int what, int tx, const fl
 template <int RM>
 __global__ void __launch_bounds__(256, 1) mlp_tile_kernel(TileArgs A)
 {
+    pt::chain_begin();
     constexpr int M = 16 * RM;
     extern __shared__ __align__(16) float tsm[];
     float *sW = tsm;                       // [H][H]
@@ -480,6 +481,7 @@ __device__ __forceinline__ void cp16(float *dst, const float *src, bool ok)
 __global__ void __launch_bounds__(256, 2) wgrad_kernel(const float *dZ2, const float *dZ3, const float *H1, const float *H2,
                                                        int n, int chunk, float *pw)
 {
+    pt::chain_begin();
     __shared__ __align__(16) float sb[WG_STAGES][2][WG_ROWS * H];
     const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int layer = blockIdx.y;   // 0: W2, 1: W3
@@ -540,6 +542,7 @@ constexpr int RG_GRP = 8, RG_OUT = 32;
 __global__ void __launch_bounds__(RG_GRP *RG_OUT) reduce_grad_kernel(const float *pw, int n_chunk, const float *psmall,
                                                                      int n_tile, int n, float *grad, float *loss)
 {
+    pt::chain_begin();
     __shared__ float4 s4[RG_GRP][RG_OUT];
     const int o = threadIdx.x % RG_OUT, g = threadIdx.x / RG_OUT;
     constexpr int N_W = 2 * H * H / 4 / RG_OUT;   // CTAs of the weight gradients
@@ -734,11 +737,11 @@ int pt_mlp_loss_grad(const float *params, const float *X, const float *T, int n,
     int st = launch_tile(A, &n_tile, s);
     if (st) return st;
     const int chunk = wgrad_chunk(n), n_chunk = (n + chunk - 1) / chunk;
-    wgrad_kernel<<<dim3(n_chunk, 2), 256, 0, s>>>(w.dZ2, w.dZ3, w.H1, w.H2, n, chunk, w.pw);
+    pt::launch_chained(wgrad_kernel, dim3(n_chunk, 2), 256, 0, s, w.dZ2, w.dZ3, w.H1, w.H2, n, chunk, w.pw);
     st = cuda_status("wgrad_kernel");
     if (st) return st;
-    reduce_grad_kernel<<<2 * H * H / 4 / RG_OUT + (N_RED * H + 3 + RG_OUT - 1) / RG_OUT, RG_GRP * RG_OUT, 0, s>>>(
-        w.pw, n_chunk, w.psmall, n_tile, n, grad, loss);
+    pt::launch_chained(reduce_grad_kernel, 2 * H * H / 4 / RG_OUT + (N_RED * H + 3 + RG_OUT - 1) / RG_OUT,
+                       RG_GRP * RG_OUT, 0, s, w.pw, n_chunk, w.psmall, n_tile, n, grad, loss);
     return cuda_status("reduce_grad_kernel");
 }
 

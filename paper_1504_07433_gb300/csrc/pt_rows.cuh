@@ -132,8 +132,8 @@ __device__ __forceinline__ float eval(unsigned base, const float *row, const flo
             asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];" : "=f"(d.x), "=f"(d.y), "=f"(d.z), "=f"(d.w) : "r"(at + 16u));
         } else {
             const float4 *p = reinterpret_cast<const float4 *>(row + (size_t)(pos - pt::MT_BITS0) * 8);
-            c = __ldg(p);
-            d = __ldg(p + 1);
+            c = *p;
+            d = p[1];
         }
         float v = MODEL == R_GIM ? fmaf(fmaf(d.w, t, d.z), t, d.y) : d.y;
         v = fmaf(v, t, d.x);
@@ -148,8 +148,8 @@ __device__ __forceinline__ float eval(unsigned base, const float *row, const flo
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(a) : "r"(at));
         asm volatile("ld.shared.f32 %0, [%1];" : "=f"(b) : "r"(at + 4u));
     } else {
-        a = __ldg(row + pos);
-        b = __ldg(row + pos + 1);
+        a = row[pos];
+        b = row[pos + 1];
     }
     return z < 1.0f + q.x ? fmaf(t, b - a, a) : 0.0f;
 }
@@ -196,6 +196,7 @@ __host__ __device__ inline Smem smem_layout(int vt, int log_kt, int nr, int row_
 template <int MODEL, int NRT, bool SMEM>
 __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
 {
+    pt::chain_begin();
     extern __shared__ __align__(16) unsigned char dsm[];
     __shared__ GeomRec srec[MAX_BITS];
     __shared__ float4 stest[MAX_BITS];   // 1/P, -(t0 + window centre)/P, half width + margin (periods)
