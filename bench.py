@@ -112,10 +112,15 @@ class ClockSampler:
                 "samples": len(sm)}
 
 
-# DRAM traffic of one gim_cheb_kernel launch (dram__bytes_read.sum +
-# dram__bytes_write.sum) from its ncu capture, per vector of the long-cadence
-# workload, and the build it was taken on (null for any other depth)
-TRAFFIC = {"per_vector_bytes": (2.398208e6 + 7.424e3) / 128.0, "n_j": 192}
+# DRAM traffic of one lc_rows_kernel launch of the Gimenez call
+# (dram__bytes_read.sum + dram__bytes_write.sum) from its ncu capture at the
+# long-cadence workload (50,000 times x 256 vectors x 10 supersamples; null
+# for any other sizes; the 51 MB of fluxes were still in L2 at its end)
+TRAFFIC = {"bytes": 1.56e6, "n_t": 50000, "n_v": 256, "n_ss": 10}
+# FP32 operations of one in-transit supersample in that kernel: the f and g
+# series (18), the position and its separation (11), the interval and offset
+# of the look-up (10) and a degree-7 polynomial (14)
+FLOPS_PER_EVAL = 53
 
 
 def whole_job_rate(ms_local, pts_per_rank, ws, device="cpu"):
@@ -201,7 +206,7 @@ def bench_plain(pt, torch, dev, stream, n_calls=500):
     call_us = e0.elapsed_time(e1) / n_calls * 1e3
     out = {"workload": wl["name"], "us_per_call": call_us, "host_wall_us_per_call": wall_us,
            "value": t.numel() / (call_us * 1e-6), "unit": "flux points/s",
-           "gpu_launches_per_call": 2}   # one geometry: set-up + the tile kernel
+           "gpu_launches_per_call": 1}   # one geometry: the tile kernel
     try:
         g = torch.cuda.CUDAGraph()
         s = torch.cuda.Stream(device=dev)
@@ -265,7 +270,7 @@ def bench_gimenez_zi(pt, torch, dev, stream, K, flush, plan, t, orb, k, ldg, wl,
     err = float((f.double() - f_series.double()).abs().max().item())
     out = {"workload": wl["name"], "grid": "n_in = %d, n_edge = %d" % (n_in, n_edge), "ms_per_call": m,
            "value": n_t * n_v / (m * 1e-3), "unit": "flux points/s", "max_abs_diff_vs_series_fp32": err,
-           "gpu_launches_per_call": 6}
+           "gpu_launches_per_call": 4}   # preparation, product, node values, rows
     return out, {"flux": _host(f[:n_chk, 0]), "n_in": n_in, "n_edge": n_edge, "n_chk": n_chk}
 
 
@@ -961,7 +966,7 @@ def main():
             out_s.copy_(ssr_both, non_blocking=True)
 
         # one step at a time with L2 flushed before each (outside the events),
-        # as the device-side legs: this step's data (pair lists, times,
+        # as the device-side legs: this step's data (rows, records, times,
         # observations) would otherwise stay in L2 from one step to the next
         s_ms = _timed(torch, stream, K, flush, ssr_step)
         s_ms, s_value = whole_job_rate(s_ms, pts_per_step, ws, dev)
@@ -986,45 +991,42 @@ def main():
             stream.wait_event(e_m)
         e2e_ssr["device_only_ms_per_step"] = _timed(torch, stream, K, flush, ssr_dev)
 
-    # roofline of the dominant kernel (the Gimenez series evaluation):
-    # algorithmic work = evaluating the N + 1 truncated series at each
-    # in-transit (time, supersample, vector): one multiply-add per series
-    # coefficient and order, 2 (N + 1) N_J FP32 flops.  The kernel executes
-    # 2 (N + 2) N_J (the shared Chebyshev recurrence on top); the paper's
-    # per-term Jacobi recursion (Sec. 2.1.4: the recursion a + b x, two
-    # products, a sum and the accumulation T_j G_j, 7 flops per (n, j) term)
-    # would spend 7 (N + 1) N_J: reported as a ratio, not as a rate.
+    # roofline of the Gimenez call's longest kernel, the light curves from the
+    # geometries' rows of polynomials: its floor is the traffic it cannot do
+    # without, the flux cube written once and the times, records and rows read
+    # once (the arithmetic, FLOPS_PER_EVAL per in-transit supersample, takes a
+    # quarter of that time at the FP32 peak).  The series itself is summed
+    # once per geometry, for the rows, not per point: the paper's per-term
+    # recursion (Sec. 2.1.4) at every in-transit supersample would take
+    # 7 (N + 1) N_J operations each, reported as a ratio.
     peaks, peak_src = _peaks()
     sm_max = float(peaks.get("sm_max_mhz", 2070.0))
     n_sm = torch.cuda.get_device_properties(dev).multi_processor_count
     fp32_peak_tflops = n_sm * 128 * 2 * sm_max * 1e6 / 1e12
     g_mean_ms = float(np.mean(g_ms))
     k_mean_ms = float(np.mean(k_ms))
-    flops = 2.0 * (N_LD + 1) * n_j * n_intr
-    exec_flops = 2.0 * (N_LD + 2) * n_j * n_intr
+    flops = float(FLOPS_PER_EVAL) * n_intr
     paper_flops = 7.0 * (N_LD + 1) * n_j * n_intr
-    achieved = flops / (k_mean_ms * 1e-3) / 1e12
+    algo_bytes = 4.0 * n_t * n_v + 8.0 * n_t + 96.0 * n_v
+    hbm_gbs = float(peaks.get("hbm_gbs", 6800.0))
+    achieved = algo_bytes / (k_mean_ms * 1e-3) / 1e9
     traffic = None
-    if TRAFFIC["n_j"] == n_j and (n_t, n_ss) == (50000, 10):
-        traffic = TRAFFIC["per_vector_bytes"] * n_v
-    roofline = {"bound": "alu", "kernel": "gim_cheb_kernel (CUDA events recorded around its launch inside pt_gimenez)",
-                "achieved": achieved, "peak": fp32_peak_tflops, "unit": "TFLOP/s", "frac": achieved / fp32_peak_tflops,
+    if (TRAFFIC["n_t"], TRAFFIC["n_v"], TRAFFIC["n_ss"]) == (n_t, n_v, n_ss):
+        traffic = TRAFFIC["bytes"]
+    roofline = {"bound": "hbm", "kernel": "lc_rows_kernel (CUDA events recorded around its launch inside pt_gimenez)",
+                "achieved": achieved, "peak": hbm_gbs, "unit": "GB/s", "frac": achieved / hbm_gbs,
                 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) from the ncu
-                # capture of this kernel, per vector (times, pair lists, records and coefficient rows
-                # all grow with the vectors); null unless the capture was taken at this depth
-                "traffic": traffic,
-                "traffic_source": "ncu capture of this kernel at n_j = %d, scaled per vector" % TRAFFIC["n_j"],
-                "peak_source": "FP32 lanes %d SM x 128 x 2 flop x %.0f MHz (%s sm_max_mhz); of %s"
-                               % (n_sm, sm_max, peak_src, peak_src),
-                "algorithmic_flops_per_launch": flops, "in_transit_evaluations": n_intr,
+                # capture of this kernel; null unless the sizes are the capture's
+                "traffic": traffic, "traffic_source": "ncu capture of this kernel at these sizes",
+                "peak_source": peak_src,
+                "algorithmic_bytes_per_launch": algo_bytes, "in_transit_evaluations": n_intr,
                 "kernel_ms": k_mean_ms, "call_ms": g_mean_ms,
-                "call_frac": flops / (g_mean_ms * 1e-3) / 1e12 / fp32_peak_tflops,
-                "executed_flops_per_launch": exec_flops,
-                "executed_frac": exec_flops / (k_mean_ms * 1e-3) / 1e12 / fp32_peak_tflops,
+                "algorithmic_flops_per_launch": flops, "fp32_peak_tflops": fp32_peak_tflops,
+                "fp32_frac": flops / (k_mean_ms * 1e-3) / 1e12 / fp32_peak_tflops,
                 "paper_recursion_flops_ratio": paper_flops / flops}
 
     extra = {}
-    launches = 10 * K   # MA: set-up, window, scan, pairs; Gimenez: table, coefficients, set-up, window, scan, series
+    launches = 5 * K   # MA: preparation, rows; Gimenez: preparation, product, rows
     if not args.no_extra:
         extra["plain"], legs["plain"] = bench_plain(pt, torch, dev, stream)
         extra["ma_interp"], legs["ma_interp"] = bench_ma_interp(pt, torch, dev, stream, K, flush, t, orb, k, ld, wl, fm)

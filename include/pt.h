@@ -410,7 +410,7 @@ int pt_sur_model_error(pt_sur_model model, int *err_host);
  * to a multiple of 256 bytes,
  *   96 n_geom + 8 n_t + 4 n_v n_b ceil(n_t / 256)
  * (n_geom = n_v, or n_v n_b with k_per_band); this is less than
- * pt_ma_quad_work_bytes(), which sizes pt_ma_quad's pair lists.  A problem
+ * pt_ma_quad_work_bytes(), which sizes pt_ma_quad's row tables as well.  A problem
  * above the limit is rejected with PT_ERR_WORKSPACE (see
  * pt_last_error_string()): for one passband that is about n_t > 375,000 at
  * 200 vectors, or n_t > 173,000 at 1,000.

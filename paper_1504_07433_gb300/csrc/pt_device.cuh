@@ -248,7 +248,7 @@ __device__ __forceinline__ void sincos_near0(float h, float *s, float *c)
 // one-instruction square root (an argument below 2^-126, a separation under
 // 1e-19, gives 0): about one ulp more in z.  ROT takes sin and cos of dE/2 at the solution
 // from the last step's values (below) instead of a second series; the
-// per-supersample loops of the pair-list kernels gain from it, while in the
+// supersample loop of the row kernel gains from it, while in the
 // batched and tile kernels the extra live values cost more than the series.
 template <bool FAST = false, bool ROT = false>
 __device__ __forceinline__ float orbit_z(const GeomRec &r, float dt, int max_iter, bool *bad, float *warm = nullptr)

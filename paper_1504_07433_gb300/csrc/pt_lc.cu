@@ -1,22 +1,18 @@
 // pt_lc.cu -- light-curve kernels and their C ABI (include/pt.h).
 //
 // Kernels of the fused light-curve path (Secs. 2.1, 2.2, 3.2, 3.4):
-//   setup_kernel        per geometry: conjunction anchor, double-float t0/P and
-//                       a conservative transit window; per time: double-float split.
-//   gim_window_kernel   window test of every (time, geometry) pair; the pairs in
-//                       the window go to per-geometry lists, all others get flux 1
-//                       (its leading CTAs also build the Gimenez tables).
-//   gim_scan_kernel     work items of 128 listed pairs per geometry.
-//   ma_pairs_kernel     Mandel-Agol: per item, the in-transit supersamples packed
-//                       into one dense list, evaluated, summed per pair in
-//                       supersample order, limb darkening per passband, stores.
-//   gim_cheb_coef_kernel, gim_cheb_kernel
-//                       Gimenez: the series in a Chebyshev basis (coefficients
-//                       per geometry, then the evaluation over the dense lists).
-//   gim_zi_table_kernel, gim_zi_kernel
-//                       Gimenez interpolated in z (Sec. 3.3).
-//   ma_lc_kernel        the tile kernel (256 times x 8 geometries per CTA) of the
-//                       interpolated and allocation-free Mandel-Agol calls.
+//   row_prep_kernel     per geometry: conjunction anchor, double-float t0/P and
+//                       a conservative transit window; per time: double-float
+//                       split; per geometry and passband: the Mandel-Agol row
+//                       of polynomials (pt_device.cuh), the caller's table at
+//                       the geometry's k, or the weighted Gimenez factors.
+//   product_kernel      Gimenez: the rows as one FP32 product (pt_gim.cuh).
+//   zi_rows_kernel      Gimenez interpolated in z (Sec. 3.3): the node values.
+//   lc_rows_kernel      the light curves from the rows (pt_rows.cuh).
+//   setup_kernel, ma_lc_kernel
+//                       records and the tile kernel (256 times x 8 geometries
+//                       per CTA, exact terms per point) of the Mandel-Agol calls
+//                       with few geometries or points and without a work buffer.
 //   ssr_part_kernel / ssr_reduce_kernel
 //                       residual sums in a fixed order.
 // Every sum is formed in a fixed order, so results are bitwise reproducible.
@@ -86,7 +82,6 @@ struct SetupArgs {
     const float *a, *inc, *e, *w, *k;
     int n_v, n_b, k_per_band, n_geom;
     GeomRec *rec;
-    int *cnt;            // per-geometry list counters to zero, or null
     float half_exp;
     int n_gblocks;
 };
@@ -103,10 +98,7 @@ __global__ void setup_kernel(SetupArgs s)
     pt::chain_begin();
     if ((int)blockIdx.x < s.n_gblocks) {
         int g = blockIdx.x * blockDim.x + threadIdx.x;
-        if (g < s.n_geom) {
-            make_geom(s, g, &s.rec[g]);
-            if (s.cnt) s.cnt[g] = 0;
-        }
+        if (g < s.n_geom) make_geom(s, g, &s.rec[g]);
     } else {
         int i = (blockIdx.x - s.n_gblocks) * blockDim.x + threadIdx.x;
         if (i < s.n_t) {
@@ -1073,32 +1065,15 @@ static void fill_setup(SetupArgs *sa, const double *t, int n_t, const pt_orbit *
     sa->k_per_band = k_per_band;
     sa->n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
     sa->rec = rec;
-    sa->cnt = nullptr;
     sa->half_exp = (float)(0.5 * t_exp);
     sa->n_gblocks = 0;
 }
 
 static int launch_setup(const double *t, int n_t, const pt_orbit *orb, const float *k, int k_per_band, int n_b,
-                        double t_exp, GeomRec *rec, float2 *tsplit, int *cnt, cudaStream_t s)
+                        double t_exp, GeomRec *rec, float2 *tsplit, cudaStream_t s)
 {
     SetupArgs sa;
-    sa.t = t;
-    sa.n_t = n_t;
-    sa.tsplit = tsplit;
-    sa.t0 = orb->t0;
-    sa.P = orb->P;
-    sa.a = orb->a;
-    sa.inc = orb->inc;
-    sa.e = orb->e;
-    sa.w = orb->w;
-    sa.k = k;
-    sa.n_v = orb->n_v;
-    sa.n_b = n_b;
-    sa.k_per_band = k_per_band;
-    sa.n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
-    sa.rec = rec;
-    sa.cnt = cnt;
-    sa.half_exp = (float)(0.5 * t_exp);
+    fill_setup(&sa, t, n_t, orb, k, k_per_band, n_b, t_exp, rec, tsplit);
     const int bs = 64;
     sa.n_gblocks = (sa.n_geom + bs - 1) / bs;
     int n_tblocks = (n_t + bs - 1) / bs;
@@ -1220,7 +1195,7 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     if (own) {
         fill_setup(&A.set, t, n_t, orb, k, k_per_band, n_b, t_exp, rec, tsplit);
     } else {
-        st = launch_setup(t, n_t, orb, k, k_per_band, n_b, t_exp, rec, tsplit, nullptr, s);
+        st = launch_setup(t, n_t, orb, k, k_per_band, n_b, t_exp, rec, tsplit, s);
         if (st) return st;
     }
     A.tsplit = tsplit;

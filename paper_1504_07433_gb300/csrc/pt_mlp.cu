@@ -103,7 +103,7 @@ __global__ void datagen_kernel(uint64_t seed, size_t offset, size_t n, float k_l
 // gradients (biases, W1, W4) are column sums over the tile.
 // The host takes the smallest RM whose tiles fit one per SM: 16,384 samples
 // are 147 tiles of 112.  Measured at 16,384 samples: 83 us for the tiles (ncu),
-// 26 us for the weight gradients, a whole step with Adam 118 us; before, with
+// 26 us for the weight gradients, a whole step with Adam 116 us; before, with
 // one kernel per product, separate activations and one thread per small
 // gradient, 468 us.
 // ---------------------------------------------------------------------------
