@@ -174,38 +174,62 @@ __device__ __forceinline__ void table_cta(const Table &T, const float *k, int n_
 }
 
 // ---------------------------------------------------------------------------
-// rows [R][Nc] = At^T [R][K] B [K][Nc].  A CTA covers RT rows x 64 columns and
-// splits K into PARTS parts over its warps (the parts' sums meet in shared
-// memory, in order), because rows and columns alone would not fill the chip:
-// 256 rows of n_j = 192 are 112 CTAs of RT = 32 with sixteen warps each.
-// Operands come straight from L2 (each is read once per CTA); a thread holds
-// 8 rows x 8 columns (RT = 32) or 8 x 2 (RT = 8, for few rows: more loads in
-// flight per warp).  Both heights add up a
-// row in the same order, so a row does not depend on the others of its call.
+// rows [R][Nc] = At^T [R][K] B [K][Nc].  A CTA covers RT rows x 256 C / RT
+// columns and splits K into PARTS parts over its warps (the parts' sums meet in
+// shared memory, in order), because rows and columns alone would not fill the
+// chip.  Operands come straight from L2 (each is read once per CTA); a thread
+// holds 8 rows x C columns: C = 8 or 6 at RT = 32, 3, 2 or 1 at RT = 8 (for few
+// rows: more loads in flight per warp).  The width is the one whose CTAs, one
+// per multiprocessor, need the least time in whole waves (product_width): 256
+// rows of n_j = 192 are 112 CTAs of 64 columns, 36.6 us, or 144 of 48, 29.4
+// (ncu, cold); 100 rows 182 of 64, 27.1 us, or 117 of 96, 20.6.  Every form adds
+// up a row in the same order, so a row does not depend on the others of its
+// call.
 // ---------------------------------------------------------------------------
-constexpr int CT = 64, PARTS = 16;
+constexpr int PARTS = 16;
 
-template <int RT>
+template <int RT, int C>
 struct Split {
     static constexpr int WARPS = PARTS;
-    static constexpr int COLS = RT == 32 ? 8 : 2;   // columns per thread
+    static constexpr int CT = 256 * C / RT;   // columns per CTA
     static constexpr size_t SMEM = (size_t)PARTS * RT * CT * sizeof(float);
 };
 
+// C for r row tiles of RT rows: a step of a thread is 8 C multiply-adds and
+// about 6 other instructions.
 template <int RT>
-__global__ void __launch_bounds__(32 * Split<RT>::WARPS, 1) product_kernel(const float *At, int Rp, const float *B, int K,
-                                                                           int Nc, int R, float *out)
+inline int product_width(size_t r, int Nc, int n_sm)
+{
+    const int cand[2][3] = {{8, 6, 6}, {3, 2, 1}};
+    int best = 0;
+    size_t cost = 0;
+    for (int c : cand[RT == 32 ? 0 : 1]) {
+        const size_t ct = (size_t)(256 * c / RT), ctas = r * (((size_t)Nc + ct - 1) / ct);
+        const size_t t = (ctas + n_sm - 1) / n_sm * (size_t)(8 * c + 6);
+        if (best == 0 || t < cost) {
+            best = c;
+            cost = t;
+        }
+    }
+    return best;
+}
+
+template <int RT, int C>
+__global__ void __launch_bounds__(32 * PARTS, 1) product_kernel(const float *At, int Rp, const float *B, int K, int Nc,
+                                                                int R, float *out)
 {
     pt::chain_begin();
-    constexpr int WARPS = Split<RT>::WARPS, C = Split<RT>::COLS;
+    constexpr int WARPS = PARTS, CT = Split<RT, C>::CT;
     extern __shared__ __align__(16) float psm[];   // [PARTS][RT][CT]
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int rl = (lane / (CT / C)) * 8, cl = (lane % (CT / C)) * C;
     const int n_ct = (Nc + CT - 1) / CT;
     const int ct = (int)(blockIdx.x % n_ct), rt = (int)(blockIdx.x / n_ct);   // column and row tile
-    const int c_in = ct * CT + cl;
+    const int rl = (lane / (CT / C)) * 8;
+    // Columns beyond the last: the last C again (the same sums; a tile has at
+    // least 8 columns, Nc being a multiple of 8).
+    const int cl = min((lane % (CT / C)) * C, Nc - C - ct * CT);
     const float *pa = At + (size_t)rt * RT + rl;
-    const float *pb = B + (c_in < Nc ? c_in : 0);   // columns beyond the last: read column 0, not stored
+    const float *pb = B + ct * CT + cl;
     const int per = (K + PARTS - 1) / PARTS;
     {
         const int part = warp;
@@ -215,20 +239,28 @@ __global__ void __launch_bounds__(32 * Split<RT>::WARPS, 1) product_kernel(const
         for (int i = 0; i < 8; ++i)
 #pragma unroll
             for (int j = 0; j < C; ++j) acc[i][j] = 0.0f;
-#pragma unroll(RT == 32 ? 3 : 12)
+#pragma unroll(RT == 32 ? (C == 8 ? 3 : 4) : (C == 3 ? 8 : 12))
         for (int k = k0; k < k1; ++k) {
             const float4 a0 = *reinterpret_cast<const float4 *>(pa + (size_t)k * Rp);   // this call's: not by __ldg
             const float4 a1 = *reinterpret_cast<const float4 *>(pa + (size_t)k * Rp + 4);
             const float a[8] = {a0.x, a0.y, a0.z, a0.w, a1.x, a1.y, a1.z, a1.w};
             float b[C];
-            if (C == 8) {
-                const float4 b0 = __ldg(reinterpret_cast<const float4 *>(pb + (size_t)k * Nc));
-                const float4 b1 = __ldg(reinterpret_cast<const float4 *>(pb + (size_t)k * Nc + 4));
-                b[0] = b0.x, b[1 % C] = b0.y, b[2 % C] = b0.z, b[3 % C] = b0.w;
-                b[4 % C] = b1.x, b[5 % C] = b1.y, b[6 % C] = b1.z, b[7 % C] = b1.w;
+            const float *bk = pb + (size_t)k * Nc;
+            if constexpr (C == 8) {
+#pragma unroll
+                for (int j = 0; j < C; j += 4) {
+                    const float4 v = __ldg(reinterpret_cast<const float4 *>(bk + j));
+                    b[j] = v.x, b[j + 1] = v.y, b[j + 2] = v.z, b[j + 3] = v.w;
+                }
+            } else if constexpr (C % 2 == 0) {
+#pragma unroll
+                for (int j = 0; j < C; j += 2) {
+                    const float2 v = __ldg(reinterpret_cast<const float2 *>(bk + j));
+                    b[j] = v.x, b[j + 1] = v.y;
+                }
             } else {
-                const float2 b0 = __ldg(reinterpret_cast<const float2 *>(pb + (size_t)k * Nc));
-                b[0] = b0.x, b[1] = b0.y;
+#pragma unroll
+                for (int j = 0; j < C; ++j) b[j] = __ldg(bk + j);
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i)
@@ -246,7 +278,7 @@ __global__ void __launch_bounds__(32 * Split<RT>::WARPS, 1) product_kernel(const
         float x = 0.0f;
 #pragma unroll
         for (int w = 0; w < PARTS; ++w) x += psm[(size_t)w * RT * CT + e];
-        const int row = rt * RT + e / CT, col = ct * CT + (e & (CT - 1));
+        const int row = rt * RT + e / CT, col = ct * CT + e % CT;
         if (row < R && col < Nc) out[(size_t)row * Nc + col] = x;
     }
 }

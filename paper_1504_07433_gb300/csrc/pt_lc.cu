@@ -1516,19 +1516,24 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     st = check_launch("row_prep_kernel");
     if (st) return st;
     // the product: tall tiles when they fill half the chip
-    const size_t gx = ((size_t)Nc + gim::CT - 1) / gim::CT;
     const size_t r32 = (R + 31) / 32, r8 = (R + 7) / 8;
-    if (r32 * gx > 0x7fffffffULL) return PT_ERR_ARG;
-    if (r32 * gx >= (size_t)n_sm / 2) {
-        e = cudaFuncSetAttribute(gim::product_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)gim::Split<32>::SMEM);
-        if (e == cudaSuccess)
-            pt::launch_chained(gim::product_kernel<32>, (unsigned)(r32 * gx), 32 * gim::Split<32>::WARPS,
-                               (size_t)gim::Split<32>::SMEM, s, P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
-    } else {
-        pt::launch_chained(gim::product_kernel<8>, (unsigned)(r8 * gx), 32 * gim::Split<8>::WARPS,
-                           (size_t)gim::Split<8>::SMEM, s, P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
-    }
-    if (e != cudaSuccess) return set_cuda_error(e, "product_kernel smem attribute");
+    const bool tall = r32 * (((size_t)Nc + 63) / 64) >= (size_t)n_sm / 2;
+    const int width = tall ? gim::product_width<32>(r32, Nc, n_sm) : gim::product_width<8>(r8, Nc, n_sm);
+    auto product = [&](auto fn, size_t smem, size_t row_tiles, int ct) -> int {
+        const size_t n = row_tiles * (((size_t)Nc + ct - 1) / ct);
+        if (n > 0x7fffffffULL) return PT_ERR_ARG;
+        e = smem > 40 * 1024 ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+        if (e != cudaSuccess) return set_cuda_error(e, "product_kernel smem attribute");
+        pt::launch_chained(fn, (unsigned)n, 32 * gim::PARTS, smem, s, P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
+        return PT_OK;
+    };
+#define PT_PRODUCT(RT, C) product(gim::product_kernel<RT, C>, gim::Split<RT, C>::SMEM, RT == 32 ? r32 : r8, gim::Split<RT, C>::CT)
+    if (tall)
+        st = width == 8 ? PT_PRODUCT(32, 8) : PT_PRODUCT(32, 6);
+    else
+        st = width == 3 ? PT_PRODUCT(8, 3) : width == 2 ? PT_PRODUCT(8, 2) : PT_PRODUCT(8, 1);
+#undef PT_PRODUCT
+    if (st) return st;
     st = check_launch("product_kernel");
     if (st) return st;
     rows::Args A;
