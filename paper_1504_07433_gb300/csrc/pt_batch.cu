@@ -668,6 +668,8 @@ BatchFn batch_fn(const pt_batch_plan_s &p, int tt)
     return tt == 128 ? batch_fn_t<128>(p.mode, ss, out) : batch_fn_t<256>(p.mode, ss, out);
 }
 
+static_assert((size_t)BG * pt::MT_ROW * sizeof(float) <= INTERP_SMEM, "one shared-memory limit for all modes");
+
 size_t dyn_smem(const pt_batch_plan_s &p, int n_z)
 {
     if (p.mode == M_ROWS) return (size_t)BG * pt::MT_ROW * sizeof(float);
@@ -774,7 +776,8 @@ int configure(pt_batch_plan_s &p, int tt, int n_slices, int n_z)
 {
     const BatchFn fn = batch_fn(p, tt);
     const size_t smem = dyn_smem(p, n_z);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    // (INTERP_SMEM covers every mode's size, and is the same for every plan)
+    cudaError_t e = pt::allow_smem(fn, INTERP_SMEM);
     int per_sm = 0;
     if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, tt, smem);
     if (e != cudaSuccess) return berr(e, "batch_kernel occupancy");

@@ -1142,6 +1142,18 @@ __device__ __forceinline__ void chain_begin()
     chain_wait();
 }
 
+// Opt-in to `bytes` of dynamic shared memory.  The limit belongs to the function
+// (on the current device), not to the launch, and every host thread sets the same
+// one: a caller passes a constant of the kernel, the most that any of its launches
+// asks for, never this launch's own size (a thread with a smaller launch would
+// otherwise lower the limit between another's setting and its launch, which is
+// then refused).  It costs well under a microsecond.
+template <typename F>
+inline cudaError_t allow_smem(F fn, size_t bytes)
+{
+    return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
 template <typename... P, typename... A>
 inline cudaError_t launch_chained(void (*fn)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
 {

@@ -712,6 +712,13 @@ RowLayout row_layout(int n_t, int n_v, int n_b, int k_per_band, int n_terms, siz
 // points read it.
 constexpr long long ROWS_MIN_POINTS = 512;
 
+// Dynamic shared memory: launches up to the default limit (48 KB, less room for a
+// kernel's static arrays) need no opt-in.  The row kernel's and the preparation's
+// size varies from call to call, so they opt in to one limit that covers all
+// their calls (pt::allow_smem): the row kernel's 16 KB of lists, 96 KB of rows and 32 KB
+// of residuals, the preparation's 2 x 16 chains of 512 steps (134 KB).
+constexpr int DEFAULT_SMEM = 40 * 1024, VARIABLE_SMEM_MAX = 160 * 1024;
+
 // Tile of the row kernel: geometries x blocks of 256 times.  As many
 // geometries as 48 KB of rows hold (so that four CTAs fit an SM), the rest of
 // the 32 bits in blocks of times (which spreads the staging of the rows over
@@ -748,8 +755,9 @@ int launch_rows(int model, rows::Args &A, int n_sm, cudaStream_t s)
     default: PT_ROWS_FN(rows::R_INTERP); break;
     }
 #undef PT_ROWS_FN
-    if (smem > 40 * 1024) {   // beyond the default limit less the static arrays
-        cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (smem > DEFAULT_SMEM) {
+        if (smem > VARIABLE_SMEM_MAX) return pt_internal::set_error(PT_ERR_ARG, "lc_rows_kernel", "tile too large");
+        cudaError_t e = pt::allow_smem(fn, VARIABLE_SMEM_MAX);
         if (e != cudaSuccess) return set_cuda_error(e, "lc_rows_kernel smem attribute");
     }
     // geometries along x, time tiles along y, in as many launches as y takes
@@ -1509,8 +1517,8 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     if (blocks > 0x7fffffffLL || R > 0x7fffffffULL - 32) return PT_ERR_ARG;
     const size_t tsm = gim::table_smem(plan->n_j, P.nr);
     cudaError_t e = cudaSuccess;
-    if (tsm > 40 * 1024)
-        e = cudaFuncSetAttribute(row_prep_kernel<rows::R_GIM>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tsm);
+    if (tsm > VARIABLE_SMEM_MAX) return pt_internal::set_error(PT_ERR_ARG, "row_prep_kernel", "series too long");
+    if (tsm > DEFAULT_SMEM) e = pt::allow_smem(row_prep_kernel<rows::R_GIM>, VARIABLE_SMEM_MAX);
     if (e != cudaSuccess) return set_cuda_error(e, "row_prep_kernel smem attribute");
     row_prep_kernel<rows::R_GIM><<<(unsigned)blocks, ROW_THREADS, tsm, s>>>(P);
     st = check_launch("row_prep_kernel");
@@ -1522,7 +1530,7 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     auto product = [&](auto fn, size_t smem, size_t row_tiles, int ct) -> int {
         const size_t n = row_tiles * (((size_t)Nc + ct - 1) / ct);
         if (n > 0x7fffffffULL) return PT_ERR_ARG;
-        e = smem > 40 * 1024 ? cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) : cudaSuccess;
+        e = smem > DEFAULT_SMEM ? pt::allow_smem(fn, smem) : cudaSuccess;   // (a constant of the instantiation)
         if (e != cudaSuccess) return set_cuda_error(e, "product_kernel smem attribute");
         pt::launch_chained(fn, (unsigned)n, 32 * gim::PARTS, smem, s, P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
         return PT_OK;
