@@ -235,9 +235,8 @@ struct LcArgs {
     const float2 *tsplit;
     int n_t;
     const GeomRec *rec;
-    int n_geom;
-    const float *ld;     // [rows][n_ld]
-    int n_ld;            // 2 (MA) or N (Gimenez)
+    int n_geom, g0;      // geometries of the call, first one of this launch
+    const float *ld;     // [rows][2]
     int n_b, k_per_band, n_bpg;
     int n_ss;
     float t_exp;
@@ -284,13 +283,14 @@ __device__ __forceinline__ void phase_a(const LcArgs &A, GeomRec *srec, float (*
             ts.x = (float)x;
             ts.y = (float)(x - (double)ts.x);
         }
-        if (tl < VT && (int)blockIdx.y * VT + tl < A.n_geom) make_geom(A.set, blockIdx.y * VT + tl, &srec[tl]);
+        if (tl < VT && A.g0 + (int)blockIdx.y * VT + tl < A.n_geom)
+            make_geom(A.set, A.g0 + blockIdx.y * VT + tl, &srec[tl]);
     } else {
         if (tv) ts = A.tsplit[t];
         // stage the geometry records (6 float4 each)
         for (int i = tl; i < VT * 6; i += TT) {
             int vl = i / 6, c = i % 6;
-            int g = blockIdx.y * VT + vl;
+            int g = A.g0 + blockIdx.y * VT + vl;
             if (g < A.n_geom)
                 reinterpret_cast<float4 *>(&srec[vl])[c] = reinterpret_cast<const float4 *>(&A.rec[g])[c];
         }
@@ -299,7 +299,7 @@ __device__ __forceinline__ void phase_a(const LcArgs &A, GeomRec *srec, float (*
     __syncthreads();
 #pragma unroll 1
     for (int vl = 0; vl < VT; ++vl) {
-        int g = blockIdx.y * VT + vl;
+        int g = A.g0 + blockIdx.y * VT + vl;
         bool valid = tv && g < A.n_geom;
         float dt = 0.0f;
         bool inw = false;
@@ -392,7 +392,7 @@ __global__ void __launch_bounds__(TT) ma_lc_kernel(LcArgs A)
     const bool tv = t < A.n_t;
 #pragma unroll 1
     for (int vl = 0; vl < VT_MA; ++vl) {
-        int g = blockIdx.y * VT_MA + vl;
+        int g = A.g0 + blockIdx.y * VT_MA + vl;
         if (g >= A.n_geom) break;
         bool inw = tv && sflag[vl][tl];
         float l0 = 0.0f, l1 = 0.0f, l2 = 0.0f;
@@ -1196,7 +1196,7 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     float *part = (float *)(wb + L.part);
     const int n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
     const int n_tiles = (n_t + TT - 1) / TT, gy = (n_geom + VT_MA - 1) / VT_MA;
-    if (gy > 65535) return PT_ERR_ARG;
+    if ((n_geom + 31) / 32 > 65535) return PT_ERR_ARG;   // as the row path
     const bool own = (long long)n_tiles * gy <= MA_OWN_MAX_BLOCKS;
     LcArgs A;
     memset(&A, 0, sizeof(A));
@@ -1211,7 +1211,6 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     A.rec = rec;
     A.n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
     A.ld = ld;
-    A.n_ld = 2;
     A.n_b = n_b;
     A.k_per_band = k_per_band;
     A.n_bpg = k_per_band ? 1 : n_b;
@@ -1224,7 +1223,6 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     A.ssr_part = ssr ? part : nullptr;
     A.n_tiles = n_tiles;
     A.n_bad = n_bad;
-    dim3 grid(A.n_tiles, gy);
     void (*fn)(LcArgs);
     if (tab) {
         A.mtab = tab->d_tab;
@@ -1238,15 +1236,21 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     } else {
         fn = own ? ma_lc_kernel<false, true> : ma_lc_kernel<false, false>;
     }
-    if (own)
-        fn<<<grid, TT, 0, s>>>(A);
-    else
-        pt::launch_chained(fn, grid, TT, 0, s, A);
-    st = check_launch("ma_lc_kernel");
-    if (st) return st;
+    // time tiles along x, geometries along y, in as many launches as y takes
+    for (int y0 = 0; y0 < gy; y0 += 65535) {
+        const dim3 grid(A.n_tiles, std::min(65535, gy - y0));
+        A.g0 = y0 * VT_MA;
+        if (own)
+            fn<<<grid, TT, 0, s>>>(A);
+        else
+            pt::launch_chained(fn, grid, TT, 0, s, A);
+        st = check_launch("ma_lc_kernel");
+        if (st) return st;
+    }
     if (ssr) {
         int rows = orb->n_v * n_b;
-        pt::launch_chained(ssr_reduce_kernel, (rows * 32 + 255) / 256, 256, 0, s, part, rows, A.n_tiles, ssr);
+        pt::launch_chained(ssr_reduce_kernel, (unsigned)(((size_t)rows * 32 + 255) / 256), 256, 0, s, part, rows, A.n_tiles,
+                           ssr);
         st = check_launch("ssr_reduce_kernel");
     }
     return st;
