@@ -436,8 +436,9 @@ int pt_ma_quad_noalloc(const double *t_dev, int n_t, const pt_orbit *orb, const 
  * coefficients N (Eq. ld_general; alpha_0..alpha_N are evaluated) and series
  * depth n_j: the recursion coefficients of G_j(nu+2, 1; x), the A_{n,j} of
  * Eq. (gimemez_a), and the series' functions of z as piecewise polynomials
- * (4 (N+1) n_j 8 n_int bytes, n_int about (2 n_j + N)/3.75: 5.9 MB at N = 8,
- * n_j = 192), in device memory allocated by pt_gim_plan_create and released by
+ * (4 (N+1) n_j 8 n_int bytes, n_int about (2 n_j + N)/H, H = 1 at
+ * n_j = 2, 2.8 at 64 and 3.75 from 192 on: 5.9 MB at N = 8, n_j = 192; they follow
+ * the series to 8e-9 up to k = 0.3, 3e-8 at 0.5, 6e-7 near k = 1), in device memory allocated by pt_gim_plan_create and released by
  * pt_gim_plan_destroy.  1 <= N <= 16, 2 <= n_j <= 512.
  * A plan may be used from any stream and from several host threads: its
  * tables are read-only after creation, and a call runs on its own stream only.

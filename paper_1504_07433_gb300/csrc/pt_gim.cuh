@@ -14,10 +14,15 @@
 // a product of [rows] x [(N+1) n_j] with [(N+1) n_j] x [8 n_int], and every
 // (time, supersample) then costs one look-up instead of the (N+1) n_j
 // multiply-adds of the series.  The truncated series is kept as it is: the
-// polynomials follow it to a few 1e-9 of the flux (measured in 64 bits over
-// k = 0.05 .. 0.4, n_j = 16 .. 192), below the FP32 rounding of the flux, and
-// the sums are well conditioned (sum of magnitudes below four times the
-// result), where the Chebyshev form used before cancelled by 10^2 to 10^3.
+// polynomials follow its alpha_n to (largest error over z, n = 0, 1, N, in 64
+// bits, N = 1 .. 16, n_j = 2 .. 512)
+//   k      0.05   0.1    0.2    0.3    0.5    0.7    1      1.5    3
+//          2e-9   3e-9   6e-9   8e-9   3e-8   7e-8   6e-7   1e-7   1e-7
+// (near k = 1 the inner contact lies at c = 0 and the terms do not fall off
+// there), below the FP32 rounding of the flux up to k = 0.5, and the sums are
+// well conditioned (at k <= 0.4 the sum of magnitudes is below four times the
+// result), where the Chebyshev form used before cancelled by 10^2 to 10^3 and
+// was off by about 1e-6 near k = 1.
 // The product is FP32 on the FMA pipe: rows and sums stay 32-bit.
 #pragma once
 
@@ -34,12 +39,15 @@ constexpr int Q = rows::GIM_DEG;   // coefficients per interval
 constexpr int GPC = 16;            // geometries per table CTA
 
 // Intervals of a row: W = 2 n_j + N + 4 bounds the frequency of the terms in
-// arccos c; H of it per half interval.  The amplitude at that frequency (the
-// last terms of the series) falls with n_j, so long series take wider
-// intervals: the error left is 3e-9 at n_j = 16 and 192 alike.
+// arccos c; H of it per half interval.  A degree-7 fit leaves H^8 of the last
+// terms' amplitude, and that falls with n_j, so longer series take wider
+// intervals.  H grows such that the error at k = 0.3 stays between 1e-9 and
+// 8e-9 from n_j = 24 on (shorter series: less), and not beyond 3.75: there
+// the product below is already the wider rows' cost, and the error at k >= 0.7
+// would pass 1e-7.
 inline int intervals(int N, int n_j)
 {
-    const double H = n_j >= 96 ? 3.75 : 2.76;
+    const double H = fmin(2.76 * pow(n_j / 64.0, 0.28), 3.75);
     return (int)((2.0 * n_j + N + 4.0) / H) + 2;
 }
 inline float row_scale(int n_int) { return ((float)n_int - 0.5f) * (1.0f - 2e-6f); }
