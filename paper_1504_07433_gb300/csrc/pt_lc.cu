@@ -5,8 +5,8 @@
 //                       a conservative transit window; per time: double-float
 //                       split; per geometry and passband: the Mandel-Agol row
 //                       of polynomials (pt_device.cuh), the caller's table at
-//                       the geometry's k, or the weighted Gimenez factors.
-//   product_kernel      Gimenez: the rows as one FP32 product (pt_gim.cuh).
+//                       the geometry's k, or the Gimenez factors and weights.
+//   product_kernel      Gimenez: the rows as FP32 products (pt_gim.cuh).
 //   zi_rows_kernel      Gimenez interpolated in z (Sec. 3.3): the node values.
 //   lc_rows_kernel      the light curves from the rows (pt_rows.cuh).
 //   setup_kernel, ma_lc_kernel
@@ -130,7 +130,7 @@ struct RowPrep {
     const float4 *mtab;
     int mn_k, mn_z;
     float mk_lo, mk_hi, minv_dk;
-    // R_GIM: the weighted T_{n,j} (pt_gim.cuh)
+    // R_GIM: the T_{n,j} and the passbands' weights (pt_gim.cuh)
     gim::Table gim;
 };
 
@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(ROW_THREADS) row_prep_kernel(RowPrep P)
         return;
     }
     if (MODEL == rows::R_GIM) {
-        gim::table_cta(P.gim, s.k, s.n_geom, P.nr, P.terms, P.n_bpg, P.ld, blk % P.gim.NP1, blk / P.gim.NP1);
+        gim::table_cta(P.gim, s.k, s.n_geom, P.n_bpg, P.ld, blk % P.gim.NP1, blk / P.gim.NP1);
         return;
     }
     const int first = blk * ROW_GEOM;
@@ -877,20 +877,24 @@ namespace {
 
 constexpr int ZI_MAX_VALUES = 16384;   // (n_in + n_edge)(N + 1) per geometry
 
-// The row layout, then the weighted T and (interpolated in z) the node rows.
+// The row layout, then T, the passbands' weights and (interpolated in z) the
+// node rows.
 struct GimLayout {
     RowLayout row;
-    size_t At, zi, total;
+    size_t At, W, zi, total;
 };
 
 GimLayout gim_layout(const pt_gim_plan_s *p, int n_t, int n_v, int n_b, int k_per_band, int n_zi)
 {
     GimLayout L;
     L.row = row_layout(n_t, n_v, n_b, k_per_band, p->N + 1, (size_t)gim::Q * p->n_int);
-    const size_t R = (k_per_band ? (size_t)n_v * n_b : (size_t)n_v) * rows_per_geom(k_per_band ? 1 : n_b, p->N + 1);
+    const size_t n_geom = k_per_band ? (size_t)n_v * n_b : (size_t)n_v;
+    const size_t R = n_geom * rows_per_geom(k_per_band ? 1 : n_b, p->N + 1);
     size_t off = L.row.total;
     L.At = off;
-    off += align256((R + 31) / 32 * 32 * (size_t)(p->N + 1) * p->n_j * sizeof(float));
+    off += align256((n_geom + 31) / 32 * 32 * (size_t)(p->N + 1) * p->n_j * sizeof(float));
+    L.W = off;
+    off += align256((size_t)n_v * n_b * (p->N + 1) * sizeof(float));
     L.zi = off;
     off += align256(R * (((size_t)n_zi + 3) & ~(size_t)3) * sizeof(float));
     L.total = off;
@@ -1474,8 +1478,8 @@ size_t pt_gimenez_work_bytes(pt_gim_plan plan, int n_t, int n_v, int n_b, int k_
 }  // extern "C"
 
 // pt_gimenez (n_in == 0: the series' rows) and pt_gimenez_zi (the rows on z
-// nodes): preparation with the weighted T_{n,j}, the product that forms the
-// rows, (the nodes,) the row kernel.
+// nodes): preparation with the T_{n,j}, the products that form the rows, (the
+// nodes,) the row kernel.
 static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t, int n_t, const pt_orbit *orb,
                         const float *k, int k_per_band, const float *ld, int n_b, int n_ss, double t_exp,
                         int max_iter, const float *y, const float *wt, float *flux, float *ssr, void *work,
@@ -1488,7 +1492,7 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     int st = lc_common_check(t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, flux, ssr, work);
     if (st) return st;
     if (n_t == 0 || orb->n_v == 0) return PT_OK;
-    const int NP1 = plan->N + 1, K = NP1 * plan->n_j, Nc = gim::Q * plan->n_int;
+    const int NP1 = plan->N + 1, Nc = gim::Q * plan->n_int;
     const GimLayout L = gim_layout(plan, n_t, orb->n_v, n_b, k_per_band, zi ? n_in + n_edge : 0);
     if (work_bytes < L.total) return PT_ERR_WORKSPACE;
     const int n_geom = k_per_band ? orb->n_v * n_b : orb->n_v;
@@ -1516,10 +1520,11 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     P.gim.NP1 = NP1;
     P.gim.n_j = plan->n_j;
     P.gim.At = (float *)(wb + L.At);
-    P.gim.Rp = (int)((R + 31) / 32 * 32);
+    P.gim.Gp = (n_geom + 31) / 32 * 32;
+    P.gim.W = (float *)(wb + L.W);
     const long long blocks = (long long)P.s.n_gblocks + P.n_tblocks + (long long)NP1 * ((n_geom + gim::GPC - 1) / gim::GPC);
     if (blocks > 0x7fffffffLL || R > 0x7fffffffULL - 32) return PT_ERR_ARG;
-    const size_t tsm = gim::table_smem(plan->n_j, P.nr);
+    const size_t tsm = gim::table_smem(plan->n_j);
     cudaError_t e = cudaSuccess;
     if (tsm > VARIABLE_SMEM_MAX) return pt_internal::set_error(PT_ERR_ARG, "row_prep_kernel", "series too long");
     if (tsm > DEFAULT_SMEM) e = pt::allow_smem(row_prep_kernel<rows::R_GIM>, VARIABLE_SMEM_MAX);
@@ -1527,23 +1532,46 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     row_prep_kernel<rows::R_GIM><<<(unsigned)blocks, ROW_THREADS, tsm, s>>>(P);
     st = check_launch("row_prep_kernel");
     if (st) return st;
-    // the product: tall tiles when they fill half the chip
-    const size_t r32 = (R + 31) / 32, r8 = (R + 7) / 8;
-    const bool tall = r32 * (((size_t)Nc + 63) / 64) >= (size_t)n_sm / 2;
-    const int width = tall ? gim::product_width<32>(r32, Nc, n_sm) : gim::product_width<8>(r8, Nc, n_sm);
-    auto product = [&](auto fn, size_t smem, size_t row_tiles, int ct) -> int {
-        const size_t n = row_tiles * (((size_t)Nc + ct - 1) / ct);
+    gim::Product pr;
+    memset(&pr, 0, sizeof(pr));
+    pr.At = P.gim.At;
+    pr.Gp = P.gim.Gp;
+    pr.G = n_geom;
+    pr.B = plan->d_B;
+    pr.n_j = plan->n_j;
+    pr.NP1 = NP1;
+    pr.per = gim::chain_len(NP1, plan->n_j);
+    pr.chains = gim::chains(NP1, plan->n_j);
+    pr.Nc = Nc;
+    pr.W = P.terms ? nullptr : P.gim.W;
+    pr.nr = P.nr;
+    pr.out = P.rows;
+    const gim::Form form = gim::product_form((size_t)n_geom, Nc, gim::tall_fits(NP1, plan->n_j, P.terms || P.nr == 1), n_sm);
+    pr.spread = form.spread;
+    auto product = [&](auto fn, auto shape) -> int {
+        using S = decltype(shape);
+        const size_t n = ((size_t)n_geom + form.rt - 1) / form.rt * (((size_t)Nc + S::CT - 1) / S::CT);
         if (n > 0x7fffffffULL) return PT_ERR_ARG;
-        e = smem > DEFAULT_SMEM ? pt::allow_smem(fn, smem) : cudaSuccess;   // (a constant of the instantiation)
+        const int warps = NP1 * (pr.spread ? pr.chains : 1);
+        const size_t smem = ((size_t)warps * S::warp_floats(pr.spread || pr.chains == 1) +
+                             (pr.W ? (size_t)form.rt * pr.nr * NP1 : 0)) * sizeof(float);
+        if (smem > S::SMEM_MAX) return pt_internal::set_error(PT_ERR_ARG, "product_kernel", "too many orders");
+        e = smem > DEFAULT_SMEM ? pt::allow_smem(fn, S::SMEM_MAX) : cudaSuccess;
         if (e != cudaSuccess) return set_cuda_error(e, "product_kernel smem attribute");
-        pt::launch_chained(fn, (unsigned)n, 32 * gim::PARTS, smem, s, P.gim.At, P.gim.Rp, plan->d_B, K, Nc, (int)R, P.rows);
+        pt::launch_chained(fn, (unsigned)n, 32 * warps, smem, s, pr);
         return PT_OK;
     };
-#define PT_PRODUCT(RT, C) product(gim::product_kernel<RT, C>, gim::Split<RT, C>::SMEM, RT == 32 ? r32 : r8, gim::Split<RT, C>::CT)
-    if (tall)
-        st = width == 8 ? PT_PRODUCT(32, 8) : PT_PRODUCT(32, 6);
+#define PT_PRODUCT(RT, C) product(gim::product_kernel<RT, C>, gim::Shape<RT, C>())
+    if (form.rt == gim::TALL) {
+        const size_t n = ((size_t)n_geom + gim::TALL - 1) / gim::TALL * (((size_t)Nc + gim::TALL - 1) / gim::TALL);
+        if (n > 0x7fffffffULL) return PT_ERR_ARG;
+        e = pt::allow_smem(gim::product_tall_kernel, gim::TALL_SMEM);
+        if (e != cudaSuccess) return set_cuda_error(e, "product_tall_kernel smem attribute");
+        pt::launch_chained(gim::product_tall_kernel, (unsigned)n, 256, gim::TALL_SMEM, s, pr);
+    } else if (form.rt == 32)
+        st = form.c == 6 ? PT_PRODUCT(32, 6) : PT_PRODUCT(32, 4);
     else
-        st = width == 3 ? PT_PRODUCT(8, 3) : width == 2 ? PT_PRODUCT(8, 2) : PT_PRODUCT(8, 1);
+        st = form.c == 2 ? PT_PRODUCT(8, 2) : PT_PRODUCT(8, 1);
 #undef PT_PRODUCT
     if (st) return st;
     st = check_launch("product_kernel");
@@ -1567,6 +1595,7 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     A.t_exp = (float)t_exp;
     A.max_iter = max_iter;
     A.scale = gim::row_scale(plan->n_int);
+    A.wts = P.gim.W;
     const bool fused_ssr = ssr && !P.terms;
     float *part = (float *)(wb + L.row.part);
     A.flux = flux ? flux : (P.terms ? (float *)(wb + L.row.fscr) : nullptr);

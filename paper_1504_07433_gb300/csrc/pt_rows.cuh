@@ -55,6 +55,7 @@ struct Args {
     int row_len;            // floats, a multiple of 4
     int nr;                 // rows per geometry
     int terms;              // rows hold the model's terms, combined per passband with its weights
+    const float *wts;       // these weights, [n_geom n_bpg][nr] (Gimenez)
     int n_bpg, n_b, k_per_band;
     const float *ld;
     int N;                  // coefficients per passband (2, or the general law's)
@@ -415,15 +416,9 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
                         pt::ma_weights(ld[0], ld[1], &we, &wd, &wn);
 #pragma unroll
                         for (int u = 0; u < NRT; ++u) w[u] = u == 0 ? we : (u == 1 ? wd : (u == 2 ? wn : 0.0f));
-                    } else {   // C_0 = (1 - sum u)/D, C_n = u_n/D, D = 1 - sum n u_n/(n+2)   (Sec. 2.1.3)
-                        float su = 0.0f, sd = 0.0f;
-                        for (int n = 1; n <= A.N; ++n) {
-                            su += ld[n - 1];
-                            sd += (float)n * ld[n - 1] / (float)(n + 2);
-                        }
+                    } else {
 #pragma unroll
-                        for (int u = 0; u < NRT; ++u)
-                            w[u] = r0 + u > A.N ? 0.0f : (r0 + u == 0 ? 1.0f - su : ld[max(r0 + u - 1, 0)]) / (1.0f - sd);
+                        for (int u = 0; u < NRT; ++u) w[u] = r0 + u < A.nr ? A.wts[(row0 + bb) * A.nr + r0 + u] : 0.0f;
                     }
                     float *fp = A.flux + (row0 + bb) * A.n_t + t;
                     float dep = r0 == 0 ? 0.0f : *fp;
