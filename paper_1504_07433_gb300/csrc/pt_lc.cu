@@ -126,6 +126,7 @@ struct RowPrep {
     float *rows;      // [n_geom][nr][row_len]
     int row_len, nr, terms, n_bpg;
     const float *ld;
+    float *wts;       // terms: the passbands' weights [n_geom n_bpg][3] (R_GIM: in gim)
     // R_INTERP: the caller's table
     const float4 *mtab;
     int mn_k, mn_z;
@@ -156,6 +157,15 @@ __global__ void __launch_bounds__(ROW_THREADS) row_prep_kernel(RowPrep P)
         // one warp per CTA: the records' FP64 operations share one slow pipe per SM
         const int g = blk * 32 + tid;
         if (tid < 32 && g < s.n_geom) make_geom(s, g, &s.rec[g]);
+        if (P.wts && tid >= 32) {
+            // beside them, the weights of the geometries' passbands
+            const long long n = (long long)min(32, s.n_geom - blk * 32) * P.n_bpg;
+            for (long long i = tid - 32; i < n; i += ROW_THREADS - 32) {
+                const size_t row = (size_t)blk * 32 * P.n_bpg + i;
+                float *w = P.wts + 3 * row;
+                pt::ma_weights(P.ld[2 * row], P.ld[2 * row + 1], w, w + 1, w + 2);
+            }
+        }
         return;
     }
     blk -= s.n_gblocks;
@@ -678,7 +688,7 @@ WorkLayout work_layout(int n_t, int n_v, int n_b, int k_per_band)
 // and, when many passbands share a geometry and only residuals are wanted, a
 // flux scratch.
 struct RowLayout {
-    size_t rec, tsplit, rows, part, fscr, total;
+    size_t rec, tsplit, rows, part, wts, fscr, total;
 };
 
 // rows of a geometry: one per passband, or the model's terms when more
@@ -701,6 +711,8 @@ RowLayout row_layout(int n_t, int n_v, int n_b, int k_per_band, int n_terms, siz
     off += align256(n_geom * rows_per_geom(n_bpg, n_terms) * row_len * sizeof(float));
     L.part = off;   // per tile, or per chunk of a flux row
     off += align256((size_t)n_v * n_b * n_tiles * sizeof(float));
+    L.wts = off;    // Mandel-Agol (the Gimenez weights follow the layout)
+    if (row_terms(n_bpg)) off += align256((size_t)n_v * n_b * 3 * sizeof(float));
     L.fscr = off;
     if (row_terms(n_bpg)) off += align256((size_t)n_v * n_b * n_t * sizeof(float));
     L.total = off;
@@ -743,11 +755,10 @@ int launch_rows(int model, rows::Args &A, int n_sm, cudaStream_t s)
     A.flux_vec = A.flux && A.n_t % 4 == 0 && ((uintptr_t)A.flux & 15u) == 0;
     A.n_tiles = (A.n_t + (rows::TB << log_kt) - 1) / (rows::TB << log_kt);
     const int smem = rows::smem_layout(vt, log_kt, A.nr, A.row_len, staged, A.ssr_part ? A.nr : 0).total;
-    const bool one = A.nr == 1;
     void (*fn)(rows::Args) = nullptr;
 #define PT_ROWS_FN(M)                                                                                               \
-    fn = staged ? (one ? rows::lc_rows_kernel<M, 1, true> : rows::lc_rows_kernel<M, 4, true>)                       \
-                : rows::lc_rows_kernel<M, 4, false>
+    fn = A.nr == 1 ? rows::lc_rows_kernel<M, 1, true>                                                               \
+         : A.nr <= 4 ? rows::lc_rows_kernel<M, 4, true> : rows::lc_rows_kernel<M, 9, true>
     switch (model) {
     case rows::R_MA: PT_ROWS_FN(rows::R_MA); break;
     case rows::R_GIM: PT_ROWS_FN(rows::R_GIM); break;
@@ -755,6 +766,8 @@ int launch_rows(int model, rows::Args &A, int n_sm, cudaStream_t s)
     default: PT_ROWS_FN(rows::R_INTERP); break;
     }
 #undef PT_ROWS_FN
+    // (the other models' rows are at most 64 KB)
+    if (!staged) fn = model == rows::R_GIM ? rows::lc_rows_kernel<rows::R_GIM, 9, false> : rows::lc_rows_kernel<rows::R_ZI, 9, false>;
     if (smem > DEFAULT_SMEM) {
         if (smem > VARIABLE_SMEM_MAX) return pt_internal::set_error(PT_ERR_ARG, "lc_rows_kernel", "tile too large");
         cudaError_t e = pt::allow_smem(fn, VARIABLE_SMEM_MAX);
@@ -1124,6 +1137,7 @@ static int ma_quad_rows(const pt_ma_table_s *tab, const double *t, int n_t, cons
     P.terms = row_terms(n_bpg);
     P.n_bpg = n_bpg;
     P.ld = ld;
+    P.wts = P.terms ? (float *)(wb + L.wts) : nullptr;
     if (tab) {
         P.mtab = tab->d_tab;
         P.mn_k = tab->n_k;
@@ -1154,7 +1168,7 @@ static int ma_quad_rows(const pt_ma_table_s *tab, const double *t, int n_t, cons
     A.n_b = n_b;
     A.k_per_band = k_per_band;
     A.ld = ld;
-    A.N = 2;
+    A.wts = P.wts;
     A.n_ss = n_ss;
     A.t_exp = (float)t_exp;
     A.max_iter = max_iter;
@@ -1589,8 +1603,6 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     A.n_bpg = n_bpg;
     A.n_b = n_b;
     A.k_per_band = k_per_band;
-    A.ld = ld;
-    A.N = plan->N;
     A.n_ss = n_ss;
     A.t_exp = (float)t_exp;
     A.max_iter = max_iter;

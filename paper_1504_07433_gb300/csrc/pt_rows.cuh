@@ -13,7 +13,9 @@
 //   - each lane takes a listed pair (the lists end to end, so that lanes stay
 //     full), reduces its time in double-float (a pair beyond the exact window
 //     keeps depth 0), solves the orbit at its supersamples and reads the
-//     pair's rows there; mean, flux, residual;
+//     pair's rows there, up to NRT of them at once (1, 4 or 9: the orbit is
+//     solved once for all of a geometry's rows but the 10 to 17 of a high-order
+//     Gimenez law with many passbands); mean, flux, residual;
 //   - residual sums: each thread adds up its own times, in order.
 // The place of a pair in its list is not determined, but no value depends on
 // it, so results are reproducible bit by bit.
@@ -55,10 +57,9 @@ struct Args {
     int row_len;            // floats, a multiple of 4
     int nr;                 // rows per geometry
     int terms;              // rows hold the model's terms, combined per passband with its weights
-    const float *wts;       // these weights, [n_geom n_bpg][nr] (Gimenez)
+    const float *wts;       // these weights, [n_geom n_bpg][nr]
     int n_bpg, n_b, k_per_band;
-    const float *ld;
-    int N;                  // coefficients per passband (2, or the general law's)
+    const float *ld;        // [n_geom n_bpg][2], R_MA
     int n_ss;
     float t_exp;
     int max_iter;
@@ -355,44 +356,11 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
         const bool series = pt::fg_valid(r, o.E1, x0);
         const pt::FgSeries fg = pt::fg_series(o.E1, o.esin);
         if (series && bad0) nbad += n_ss;
-        float mean[NRT];
-#pragma unroll 1
-        for (int r0 = 0; r0 < A.nr; r0 += NRT) {
-#pragma unroll
-            for (int u = 0; u < NRT; ++u) mean[u] = 0.0f;
-            const unsigned lbase = sbase + (unsigned)((vl * A.nr + r0) * A.row_len) * 4u;
-            const float *grow = A.rows + ((size_t)(g0 + vl) * A.nr + r0) * A.row_len;
-            // one supersample's depth (or terms)
-            auto add = [&](float z) {
-                if (MODEL == R_MA && q.w == 0.0f) {
-                    const float3 te = exact_terms(q.x, z);
-#pragma unroll
-                    for (int u = 0; u < NRT; ++u) {
-                        if (r0 + u >= A.nr) break;
-                        if (A.terms) {
-                            mean[u] += u == 0 ? te.x : (u == 1 ? te.y : te.z);   // (three rows: r0 = 0)
-                        } else {
-                            float we, wd, wn;
-                            const float *ld = A.ld + 2 * (row0 + r0 + u);
-                            pt::ma_weights(ld[0], ld[1], &we, &wd, &wn);
-                            mean[u] += we * te.x + wd * te.y + wn * te.z;
-                        }
-                    }
-                } else {
-                    float off_t;
-                    const unsigned pos = find<MODEL>(A, q, z, &off_t);
-#pragma unroll
-                    for (int u = 0; u < NRT; ++u) {
-                        if (r0 + u >= A.nr) break;
-                        mean[u] += eval<MODEL, SMEM>(lbase + (unsigned)(u * A.row_len) * 4u, grow + u * A.row_len, q, z,
-                                                     pos, off_t);
-                    }
-                }
-            };
+        // f(z) at every supersample
+        auto each_z = [&](auto f, bool count_bad) {
             if (series) {
 #pragma unroll 1
-                for (int s = 0; s < n_ss; ++s)
-                    add(pt::fg_z(o, fg, cosi, x0 + (float)s * dx));
+                for (int s = 0; s < n_ss; ++s) f(pt::fg_z(o, fg, cosi, x0 + (float)s * dx));
             } else {
                 // (exposures too long a part of the period for the series)
                 float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
@@ -401,30 +369,79 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
                     bool bad = false;
                     const float off = A.t_exp * (((float)s + 0.5f) * inv_nss - 0.5f);
                     const float z = pt::orbit_z<true, true>(r, dt + off, A.max_iter, &bad, warm);
-                    if (bad && r0 == 0) ++nbad;
-                    add(z);
+                    if (bad && count_bad) ++nbad;
+                    f(z);
                 }
             }
+        };
+        // a row's depth
+        auto emit = [&](int row, float dep) {
+            if (A.flux) A.flux[(row0 + row) * A.n_t + t] = 1.0f - dep;
+            if (n_ssr) {
+                const int band = sband[vl] + (A.k_per_band ? 0 : row);
+                // y - f with f = 1 - depth not rounded in between
+                const float res = (A.y[(size_t)band * A.n_t + t] - 1.0f) + dep;
+                const int p = ((code >> 8) << log_vt) + vl;
+                sval[((row << (log_vt + log_kt)) + p) * TB + (code & (TB - 1))] =
+                    (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * res * res;
+            }
+        };
+        // the exact terms, for a geometry without a table: once for all passbands
+        const bool exact = MODEL == R_MA && q.w == 0.0f;
+        float3 te = make_float3(0.0f, 0.0f, 0.0f);
+        if (exact) {
+            each_z([&](float z) {
+                const float3 x = exact_terms(q.x, z);
+                te.x += x.x;
+                te.y += x.y;
+                te.z += x.z;
+            }, true);
+            if (!A.terms) {
+                for (int row = 0; row < A.nr; ++row) {
+                    float we, wd, wn;
+                    const float *ld = A.ld + 2 * (row0 + row);
+                    pt::ma_weights(ld[0], ld[1], &we, &wd, &wn);
+                    emit(row, (we * te.x + wd * te.y + wn * te.z) * inv_nss);
+                }
+                continue;
+            }
+        }
+        float mean[NRT];
+#pragma unroll 1
+        for (int r0 = 0; r0 < A.nr; r0 += NRT) {
+            if (exact) {   // (three rows)
+#pragma unroll
+                for (int u = 0; u < NRT; ++u) mean[u] = u == 0 ? te.x : (u == 1 ? te.y : (u == 2 ? te.z : 0.0f));
+            } else {
+#pragma unroll
+                for (int u = 0; u < NRT; ++u) mean[u] = 0.0f;
+                const unsigned lbase = sbase + (unsigned)((vl * A.nr + r0) * A.row_len) * 4u;
+                const float *grow = A.rows + ((size_t)(g0 + vl) * A.nr + r0) * A.row_len;
+                each_z([&](float z) {
+                    float off_t;
+                    const unsigned pos = find<MODEL>(A, q, z, &off_t);
+#pragma unroll
+                    for (int u = 0; u < NRT; ++u) {
+                        if (r0 + u >= A.nr) break;
+                        mean[u] += eval<MODEL, SMEM>(lbase + (unsigned)(u * A.row_len) * 4u, grow + u * A.row_len, q, z,
+                                                     pos, off_t);
+                    }
+                }, r0 == 0);
+            }
+#pragma unroll
+            for (int u = 0; u < NRT; ++u) mean[u] = __fmul_rn(mean[u], inv_nss);
             if (A.terms) {
                 // the terms' share of every passband's depth; the flux holds the
                 // depth so far (this lane's alone) until the last rows
-                for (int bb = 0; bb < A.n_bpg; ++bb) {
-                    const float *ld = A.ld + (row0 + bb) * A.N;
-                    float w[NRT];
-                    if (MODEL == R_MA || MODEL == R_INTERP) {
-                        float we, wd, wn;
-                        pt::ma_weights(ld[0], ld[1], &we, &wd, &wn);
-#pragma unroll
-                        for (int u = 0; u < NRT; ++u) w[u] = u == 0 ? we : (u == 1 ? wd : (u == 2 ? wn : 0.0f));
-                    } else {
-#pragma unroll
-                        for (int u = 0; u < NRT; ++u) w[u] = r0 + u < A.nr ? A.wts[(row0 + bb) * A.nr + r0 + u] : 0.0f;
-                    }
-                    float *fp = A.flux + (row0 + bb) * A.n_t + t;
+                const float *w = A.wts + row0 * A.nr + r0;
+                float *fp = A.flux + row0 * A.n_t + t;
+                for (int bb = 0; bb < A.n_bpg; ++bb, w += A.nr, fp += A.n_t) {
                     float dep = r0 == 0 ? 0.0f : *fp;
 #pragma unroll
-                    for (int u = 0; u < NRT; ++u)
-                        if (r0 + u < A.nr) dep += w[u] * (mean[u] * inv_nss);
+                    for (int u = 0; u < NRT; ++u) {
+                        if (r0 + u >= A.nr) break;
+                        dep += w[u] * mean[u];
+                    }
                     *fp = r0 + NRT >= A.nr ? 1.0f - dep : dep;
                 }
                 continue;
@@ -432,16 +449,7 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
 #pragma unroll
             for (int u = 0; u < NRT; ++u) {
                 if (r0 + u >= A.nr) break;
-                const float dep = __fmul_rn(mean[u], inv_nss);
-                if (A.flux) A.flux[(row0 + r0 + u) * A.n_t + t] = 1.0f - dep;
-                if (n_ssr) {
-                    const int band = sband[vl] + (A.k_per_band ? 0 : r0 + u);
-                    // y - f with f = 1 - depth not rounded in between
-                    const float res = (A.y[(size_t)band * A.n_t + t] - 1.0f) + dep;
-                    const int p = ((code >> 8) << log_vt) + vl;
-                    sval[(((r0 + u) << (log_vt + log_kt)) + p) * TB + (code & (TB - 1))] =
-                        (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * res * res;
-                }
+                emit(r0 + u, mean[u]);
             }
         }
     }
