@@ -33,3 +33,26 @@ def test_short_series_of_many_vectors(n_v, n_t):
     ref, _ = oracle.lc_ma(wl["t"], o, f32(wl["k"])[pick], f32(wl["ld"])[pick])
     assert (ref < 1).sum() > 50
     assert np.abs(f1.cpu().numpy() - ref).max() <= 1e-6
+
+
+@pytest.mark.gpu
+def test_passbands_with_their_own_radius_ratios():
+    """The second launch starts inside a vector's passbands (524,280 is no
+    multiple of 7): its passbands keep their own data."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import paper_1504_07433_gb300 as pt
+    n_v, n_b, n_t = 75000, 7, 20
+    rng = np.random.default_rng(7)
+    wl = W.long_cadence(n_v=n_v, n_t=n_t, n_ss=1, cadence=0.01)
+    wl["orbit"]["t0"] = rng.uniform(0.0, 0.01 * n_t, n_v)
+    wl["k"] = wl["k"][:, None] * rng.uniform(0.9, 1.1, (n_v, n_b))
+    wl["ld"] = np.repeat(wl["ld"][:, :1], n_b, axis=1)
+    t, orb, k, ld = gpu_inputs(wl)
+    y = torch.as_tensor(rng.normal(1.0, 1e-3, (n_b, n_t)).astype(np.float32), device="cuda")
+    flux, ssr = pt.ma_quad(t, orb, k, ld, y=y, want_ssr=True)
+    lo = 524280 // n_b - 10
+    part = {x: None if v is None else v[lo:lo + 40].contiguous() for x, v in orb.items()}
+    f1, s1 = pt.ma_quad(t, part, k[lo:lo + 40].contiguous(), ld[lo:lo + 40].contiguous(), y=y, want_ssr=True)
+    assert torch.equal(flux[lo:lo + 40], f1) and torch.equal(ssr[lo:lo + 40], s1)
