@@ -819,6 +819,20 @@ size_t row_len_max(int n_t)
     return m > (size_t)pt::MT_ROW ? m : (size_t)pt::MT_ROW;
 }
 
+// Building a row and staging it costs its length.  Where many geometries fill the
+// chip with it, a light curve has to read a long row often, from four points
+// (times x supersamples) per node on (50,000 vectors x 3,000 times, half of them
+// in transit, from 1,024 nodes: 1,572 us against 1,294 by the tile kernel; from 256
+// nodes 1,061 against 1,265, and x 600 times 254 against 304).  Up to 8 M nodes in
+// all, the rows' cost is hidden (5,000 vectors x 3,000 times from 1,024 nodes: 120
+// us against 127).
+bool interp_use_rows(int n_t, int n_v, int n_b, int k_per_band, int n_ss, size_t row_len)
+{
+    const size_t n_geom = k_per_band ? (size_t)n_v * n_b : (size_t)n_v;
+    return row_len <= row_len_max(n_t) &&
+           (row_len <= 512 || 4 * row_len <= (size_t)n_t * n_ss || n_geom * row_len <= (size_t)8 << 20);
+}
+
 }  // namespace
 
 struct pt_ma_table_s {
@@ -1202,7 +1216,8 @@ static int ma_quad_impl(const pt_ma_table_s *tab, const double *t, int n_t, cons
     int st = lc_common_check(t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, flux, ssr, work);
     if (st) return st;
     if (n_t == 0 || orb->n_v == 0) return PT_OK;
-    if (use_rows && ma_use_rows(n_t, orb->n_v, n_b, k_per_band, n_ss) && (!tab || interp_row_len(tab->n_z) <= row_len_max(n_t)))
+    if (use_rows && ma_use_rows(n_t, orb->n_v, n_b, k_per_band, n_ss) &&
+        (!tab || interp_use_rows(n_t, orb->n_v, n_b, k_per_band, n_ss, interp_row_len(tab->n_z))))
         return ma_quad_rows(tab, t, n_t, orb, k, k_per_band, ld, n_b, n_ss, t_exp, max_iter, y, wt, flux, ssr, work,
                             work_bytes, n_bad, stream);
     WorkLayout L = work_layout(n_t, orb->n_v, n_b, k_per_band);
