@@ -433,17 +433,26 @@ __global__ void __launch_bounds__(TT) ma_lc_kernel(LcArgs A)
     if (tl == 0 && sbad && A.n_bad) atomicAdd(A.n_bad, sbad);
 }
 
-__global__ void ssr_reduce_kernel(const float *part, int rows, int n_tiles, float *ssr)
+// One warp per row.  The sum's rounding errors are carried along (two-sums), so
+// that the partials' own rounding is all that is left; an infinite sum, whose
+// errors are NaN, is itself.
+__global__ void ssr_reduce_kernel(const float *part, int rows, int n_part, float *ssr)
 {
     pt::chain_begin();
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int lane = threadIdx.x & 31;
     if (warp >= rows) return;
-    float s = 0.0f;
-    for (int i = lane; i < n_tiles; i += 32) s += part[(size_t)warp * n_tiles + i];
+    float h = 0.0f, l = 0.0f;
+    auto add = [&](float v, float vl) {
+        const float s = h + v, bb = s - h;
+        l = (l + vl) + ((h - (s - bb)) + (v - bb));
+        h = s;
+    };
+    for (int i = lane; i < n_part; i += 32) add(part[(size_t)warp * n_part + i], 0.0f);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (lane == 0) ssr[warp] = s;
+    for (int o = 16; o > 0; o >>= 1) add(__shfl_xor_sync(0xffffffffu, h, o), __shfl_xor_sync(0xffffffffu, l, o));
+    const float s = h + l;
+    if (lane == 0) ssr[warp] = s == s ? s : h;
 }
 
 // ssr[row] = sum_t wt (y - flux)^2 over one flux row, in a fixed order;
@@ -754,6 +763,7 @@ int launch_rows(int model, rows::Args &A, int n_sm, cudaStream_t s)
     A.log_kt = log_kt;
     A.flux_vec = A.flux && A.n_t % 4 == 0 && ((uintptr_t)A.flux & 15u) == 0;
     A.n_tiles = (A.n_t + (rows::TB << log_kt) - 1) / (rows::TB << log_kt);
+    A.n_blk = (A.n_t + rows::TB - 1) / rows::TB;
     const int smem = rows::smem_layout(vt, log_kt, A.nr, A.row_len, staged, A.ssr_part ? A.nr : 0).total;
     void (*fn)(rows::Args) = nullptr;
 #define PT_ROWS_FN(M)                                                                                               \
@@ -1201,7 +1211,7 @@ static int ma_quad_rows(const pt_ma_table_s *tab, const double *t, int n_t, cons
     if (st || !ssr) return st;
     const int n_rows = orb->n_v * n_b;
     if (!fused_ssr) return launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)n_rows, part, ssr, s);
-    pt::launch_chained(ssr_reduce_kernel, (unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s, part, n_rows, A.n_tiles,
+    pt::launch_chained(ssr_reduce_kernel, (unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s, part, n_rows, A.n_blk,
                        ssr);
     return check_launch("ssr_reduce_kernel");
 }
@@ -1660,7 +1670,7 @@ static int gimenez_impl(pt_gim_plan plan, int n_in, int n_edge, const double *t,
     if (!ssr) return PT_OK;
     const int n_rows = orb->n_v * n_b;
     if (!fused_ssr) return launch_ssr_rows(A.flux, y, wt, n_t, n_b, (size_t)n_rows, part, ssr, s);
-    pt::launch_chained(ssr_reduce_kernel, (unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s, part, n_rows, A.n_tiles,
+    pt::launch_chained(ssr_reduce_kernel, (unsigned)(((size_t)n_rows * 32 + 255) / 256), 256, 0, s, part, n_rows, A.n_blk,
                        ssr);
     return check_launch("ssr_reduce_kernel");
 }

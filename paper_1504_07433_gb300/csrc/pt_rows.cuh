@@ -16,7 +16,8 @@
 //     pair's rows there, up to NRT of them at once (1, 4 or 9: the orbit is
 //     solved once for all of a geometry's rows but the 10 to 17 of a high-order
 //     Gimenez law with many passbands); mean, flux, residual;
-//   - residual sums: each thread adds up its own times, in order.
+//   - residual sums per block of 256 times, in an order fixed by n_t alone: a
+//     vector's sum does not depend on the other vectors of its call.
 // The place of a pair in its list is not determined, but no value depends on
 // it, so results are reproducible bit by bit.
 // The rows and what a look-up does are the model's:
@@ -64,8 +65,9 @@ struct Args {
     float t_exp;
     int max_iter;
     float *flux;            // [n_geom n_bpg][n_t] or null
-    float *ssr_part;        // [n_geom n_bpg][n_tiles] or null (needs !terms)
+    float *ssr_part;        // [n_geom n_bpg][n_blk] or null (needs !terms)
     int n_tiles, tile0;
+    int n_blk;              // blocks of TB times
     const float *y, *wt;
     int *n_bad;
     int log_vt, log_kt;
@@ -190,7 +192,7 @@ __host__ __device__ inline Smem smem_layout(int vt, int log_kt, int nr, int row_
     s.sval = off;
     off += n_ssr * pairs * 4;
     s.sred = off;
-    off += NW * vt * n_ssr * 4;
+    off += NW * (vt << log_kt) * n_ssr * 4;
     s.total = off;
     return s;
 }
@@ -207,6 +209,7 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
     __shared__ int scnt[MAX_BITS];       // pairs of each geometry
     __shared__ int soff[MAX_BITS + 1];   // ... before each geometry, lists end to end
     __shared__ float swmax[NW];
+    __shared__ bool sexact;              // R_MA: a geometry without a table
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int log_vt = A.log_vt, vt = 1 << log_vt, log_kt = A.log_kt, kt = 1 << log_kt;
     const int tile = A.tile0 + blockIdx.y;
@@ -230,6 +233,7 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
         asm volatile("cp.async.commit_group;" ::: "memory");
     }
     if (tid < MAX_BITS) scnt[tid] = 0;
+    if (tid == 0) sexact = false;
     // the tile's largest |t_h| (non-negative floats order like their bits)
     float am = 0.0f;
     for (int k = 0; k < kt; ++k) {
@@ -255,6 +259,7 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
         else if (!(m < 0.25f)) half = INFINITY;
         stest[tid] = make_float4(r.invP, -(r.t0h + mid) * r.invP, half, 0.0f);
         sgeo[tid] = look_up_constants<MODEL>(A, r.k);
+        if (MODEL == R_MA && sgeo[tid].w == 0.0f) sexact = true;
         sband[tid] = A.k_per_band ? (g0 + tid) % A.n_b : 0;
     }
     // every flux of the tile is 1 until its pair is evaluated
@@ -334,20 +339,52 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
                            (MODEL == R_MA || MODEL == R_GIM ? 32u * pt::MT_BITS0 : 0u);
     float *sval = reinterpret_cast<float *>(dsm + L.sval);   // [n_ssr][kt vt][TB]
     int nbad = 0;
-    for (int e = tid; e < nq; e += TB) {
-        int vl = 0;   // the last geometry with soff <= e
+    auto geometry_of = [&](int e) {   // the last geometry with soff <= e
+        int vl = 0;
         for (int o = vt >> 1; o > 0; o >>= 1)
             if (soff[vl + o] <= e) vl += o;
-        const int code = list[vl * cap + (e - soff[vl])];
+        return vl;
+    };
+    // a row's depth at the time with this code
+    auto emit = [&](int vl, int code, int row, float dep) {
         const int t = tb + code;
+        if (A.flux) A.flux[((size_t)(g0 + vl) * A.n_bpg + row) * A.n_t + t] = 1.0f - dep;
+        if (n_ssr) {
+            const int band = sband[vl] + (A.k_per_band ? 0 : row);
+            // y - f with f = 1 - depth not rounded in between
+            const float res = (A.y[(size_t)band * A.n_t + t] - 1.0f) + dep;
+            const int p = ((code >> 8) << log_vt) + vl;
+            sval[((row << (log_vt + log_kt)) + p) * TB + (code & (TB - 1))] =
+                (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * res * res;
+        }
+    };
+    // f(z) at the supersamples of a pair's exposure (none beyond the window).
+    // Kepler's equation once, at mid-exposure; the supersamples from the f and g
+    // series at offsets x0 + s dx of mean anomaly, or, where the exposure is too
+    // long a part of the period for them, by Newton's method each.
+#define PT_EACH_Z(COUNT, F)                                                                                         \
+    if (series) {                                                                                                   \
+        _Pragma("unroll 1") for (int s = 0; s < n_ss; ++s) F(pt::fg_z(o, fg, cosi, x0 + (float)s * dx));            \
+    } else {                                                                                                        \
+        float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f}; /* Kepler warm start (none yet) */          \
+        _Pragma("unroll 1") for (int s = 0; s < n_ss; ++s)                                                          \
+        {                                                                                                           \
+            bool bad = false;                                                                                       \
+            const float off = A.t_exp * (((float)s + 0.5f) * inv_nss - 0.5f);                                       \
+            const float z = pt::orbit_z<true, true>(r, dt + off, A.max_iter, &bad, warm);                           \
+            if (bad && (COUNT)) ++nbad;                                                                             \
+            F(z);                                                                                                   \
+        }                                                                                                           \
+    }
+    for (int e = tid; e < nq; e += TB) {
+        const int vl = geometry_of(e), code = list[vl * cap + (e - soff[vl])], t = tb + code;
         const GeomRec &r = srec[vl];
         const float4 q = sgeo[vl];
+        if (MODEL == R_MA && q.w == 0.0f) continue;   // without a table: below
         const float2 ts = A.tsplit[t];
         const float dt = pt::reduce_time(ts.x, ts.y, r);
         const int n_ss = dt >= r.win_lo && dt <= r.win_hi ? A.n_ss : 0;
         const size_t row0 = (size_t)(g0 + vl) * A.n_bpg;
-        // Kepler's equation once, at mid-exposure; the supersamples from the
-        // f and g series at offsets x0 + s dx of mean anomaly
         pt::OrbitState o;
         bool bad0 = false;
         pt::orbit_state(r, dt, A.max_iter, &bad0, &o);
@@ -356,81 +393,26 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
         const bool series = pt::fg_valid(r, o.E1, x0);
         const pt::FgSeries fg = pt::fg_series(o.E1, o.esin);
         if (series && bad0) nbad += n_ss;
-        // f(z) at every supersample
-        auto each_z = [&](auto f, bool count_bad) {
-            if (series) {
-#pragma unroll 1
-                for (int s = 0; s < n_ss; ++s) f(pt::fg_z(o, fg, cosi, x0 + (float)s * dx));
-            } else {
-                // (exposures too long a part of the period for the series)
-                float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
-#pragma unroll 1
-                for (int s = 0; s < n_ss; ++s) {
-                    bool bad = false;
-                    const float off = A.t_exp * (((float)s + 0.5f) * inv_nss - 0.5f);
-                    const float z = pt::orbit_z<true, true>(r, dt + off, A.max_iter, &bad, warm);
-                    if (bad && count_bad) ++nbad;
-                    f(z);
-                }
-            }
-        };
-        // a row's depth
-        auto emit = [&](int row, float dep) {
-            if (A.flux) A.flux[(row0 + row) * A.n_t + t] = 1.0f - dep;
-            if (n_ssr) {
-                const int band = sband[vl] + (A.k_per_band ? 0 : row);
-                // y - f with f = 1 - depth not rounded in between
-                const float res = (A.y[(size_t)band * A.n_t + t] - 1.0f) + dep;
-                const int p = ((code >> 8) << log_vt) + vl;
-                sval[((row << (log_vt + log_kt)) + p) * TB + (code & (TB - 1))] =
-                    (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * res * res;
-            }
-        };
-        // the exact terms, for a geometry without a table: once for all passbands
-        const bool exact = MODEL == R_MA && q.w == 0.0f;
-        float3 te = make_float3(0.0f, 0.0f, 0.0f);
-        if (exact) {
-            each_z([&](float z) {
-                const float3 x = exact_terms(q.x, z);
-                te.x += x.x;
-                te.y += x.y;
-                te.z += x.z;
-            }, true);
-            if (!A.terms) {
-                for (int row = 0; row < A.nr; ++row) {
-                    float we, wd, wn;
-                    const float *ld = A.ld + 2 * (row0 + row);
-                    pt::ma_weights(ld[0], ld[1], &we, &wd, &wn);
-                    emit(row, (we * te.x + wd * te.y + wn * te.z) * inv_nss);
-                }
-                continue;
-            }
-        }
         float mean[NRT];
 #pragma unroll 1
         for (int r0 = 0; r0 < A.nr; r0 += NRT) {
-            if (exact) {   // (three rows)
 #pragma unroll
-                for (int u = 0; u < NRT; ++u) mean[u] = u == 0 ? te.x : (u == 1 ? te.y : (u == 2 ? te.z : 0.0f));
-            } else {
+            for (int u = 0; u < NRT; ++u) mean[u] = 0.0f;
+            const unsigned lbase = sbase + (unsigned)((vl * A.nr + r0) * A.row_len) * 4u;
+            const float *grow = A.rows + ((size_t)(g0 + vl) * A.nr + r0) * A.row_len;
+            auto add = [&](float z) {
+                float off_t;
+                const unsigned pos = find<MODEL>(A, q, z, &off_t);
 #pragma unroll
-                for (int u = 0; u < NRT; ++u) mean[u] = 0.0f;
-                const unsigned lbase = sbase + (unsigned)((vl * A.nr + r0) * A.row_len) * 4u;
-                const float *grow = A.rows + ((size_t)(g0 + vl) * A.nr + r0) * A.row_len;
-                each_z([&](float z) {
-                    float off_t;
-                    const unsigned pos = find<MODEL>(A, q, z, &off_t);
-#pragma unroll
-                    for (int u = 0; u < NRT; ++u) {
-                        if (r0 + u >= A.nr) break;
-                        mean[u] += eval<MODEL, SMEM>(lbase + (unsigned)(u * A.row_len) * 4u, grow + u * A.row_len, q, z,
-                                                     pos, off_t);
-                    }
-                }, r0 == 0);
-            }
-#pragma unroll
-            for (int u = 0; u < NRT; ++u) mean[u] = __fmul_rn(mean[u], inv_nss);
+                for (int u = 0; u < NRT; ++u) {
+                    if (r0 + u >= A.nr) break;
+                    mean[u] += eval<MODEL, SMEM>(lbase + (unsigned)(u * A.row_len) * 4u, grow + u * A.row_len, q, z, pos, off_t);
+                }
+            };
+            PT_EACH_Z(r0 == 0, add)
             if (A.terms) {
+#pragma unroll
+                for (int u = 0; u < NRT; ++u) mean[u] = __fmul_rn(mean[u], inv_nss);
                 // the terms' share of every passband's depth; the flux holds the
                 // depth so far (this lane's alone) until the last rows
                 const float *w = A.wts + row0 * A.nr + r0;
@@ -449,50 +431,110 @@ __global__ void __launch_bounds__(TB, 4) lc_rows_kernel(Args A)
 #pragma unroll
             for (int u = 0; u < NRT; ++u) {
                 if (r0 + u >= A.nr) break;
-                emit(r0 + u, mean[u]);
+                emit(vl, code, r0 + u, __fmul_rn(mean[u], inv_nss));
             }
         }
     }
+    if (MODEL == R_MA && sexact) {
+        // the pairs of geometries without a table: the exact terms, once for all
+        // of a geometry's passbands
+        for (int e = tid; e < nq; e += TB) {
+            const int vl = geometry_of(e), code = list[vl * cap + (e - soff[vl])];
+            if (sgeo[vl].w != 0.0f) continue;
+            const GeomRec &r = srec[vl];
+            const float2 ts = A.tsplit[tb + code];
+            const float dt = pt::reduce_time(ts.x, ts.y, r);
+            const int n_ss = dt >= r.win_lo && dt <= r.win_hi ? A.n_ss : 0;
+            pt::OrbitState o;
+            bool bad0 = false;
+            pt::orbit_state(r, dt, A.max_iter, &bad0, &o);
+            const float cosi = r.cosi, dx = A.n_ss > 1 ? r.nang * A.t_exp * inv_nss : 0.0f;
+            const float x0 = -0.5f * (float)(A.n_ss - 1) * dx;
+            const bool series = pt::fg_valid(r, o.E1, x0);
+            const pt::FgSeries fg = pt::fg_series(o.E1, o.esin);
+            if (series && bad0) nbad += n_ss;
+            float3 te = make_float3(0.0f, 0.0f, 0.0f);
+            auto add = [&](float z) {
+                const float3 x = exact_terms(r.k, z);
+                te.x += x.x;
+                te.y += x.y;
+                te.z += x.z;
+            };
+            PT_EACH_Z(true, add)
+            for (int row = 0; row < A.n_bpg; ++row) {
+                const size_t at = (size_t)(g0 + vl) * A.n_bpg + row;
+                float we, wd, wn;
+                if (A.terms) we = A.wts[3 * at], wd = A.wts[3 * at + 1], wn = A.wts[3 * at + 2];
+                else pt::ma_weights(A.ld[2 * at], A.ld[2 * at + 1], &we, &wd, &wn);
+                emit(vl, code, row, (we * te.x + wd * te.y + wn * te.z) * inv_nss);
+            }
+        }
+    }
+#undef PT_EACH_Z
     if (nbad && A.n_bad) atomicAdd(A.n_bad, nbad);
     if (!n_ssr) return;
     __syncthreads();
-    // residual sums per geometry and passband: every thread's own times, from
-    // the evaluated pairs or with the flux at 1
-    float *sred = reinterpret_cast<float *>(dsm + L.sred);     // [NW][vt][n_ssr]
-    for (int bb = 0; bb < n_ssr; ++bb) {
-        float r1 = 0.0f;
-        int band_of = -1;
-        for (int vl = 0; vl < ng; ++vl) {
-            const int band = sband[vl] + (A.k_per_band ? 0 : bb);
-            float x = 0.0f;
-            for (int k = 0; k < kt; ++k) {
-                const int p = (k << log_vt) + vl;
-                if ((bits >> p) & 1u) {
-                    x += sval[((bb << (log_vt + log_kt)) + p) * TB + tid];
-                    continue;
-                }
-                const int t = tb + k * TB + tid;
-                if (kt > 1 || band != band_of) {
-                    r1 = 0.0f;
-                    if (t < A.n_t) {
-                        const float r = A.y[(size_t)band * A.n_t + t] - 1.0f;
-                        r1 = (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * r * r;
-                    }
-                    band_of = band;
-                }
-                x += r1;
+    // residual sums per geometry, passband and block of 256 times (the same sums
+    // whatever the tile's shape): every thread's own time, from the evaluated
+    // pair or with the flux at 1, then the warp's tree.  Eight sums or more go
+    // through the tree eight together: at its first three levels each half of the
+    // lanes keeps half of them, 9 shuffles in place of 40 (20,000 vectors x 4,000
+    // times 461 -> 394 us a call; a lone sum would take 2 us longer that way).
+    float *sred = reinterpret_cast<float *>(dsm + L.sred);     // [NW][n_sum]
+    const int log_p = log_vt + log_kt, n_pair = 1 << log_p;    // pair p: block p / vt, geometry p % vt
+    const int n_sum = n_ssr << log_p;                          // sum i: passband i / n_pair, pair i % n_pair
+    float r1 = 0.0f;
+    int k_of = -1, band_of = -1;
+    auto value = [&](int i) {
+        const int p = i & (n_pair - 1), vl = p & (vt - 1), k = p >> log_vt;
+        if (vl >= ng) return 0.0f;
+        if ((bits >> p) & 1u) return sval[i * TB + tid];
+        const int band = sband[vl] + (A.k_per_band ? 0 : i >> log_p);
+        if (k != k_of || band != band_of) {
+            const int t = tb + k * TB + tid;
+            r1 = 0.0f;
+            if (t < A.n_t) {
+                const float r = A.y[(size_t)band * A.n_t + t] - 1.0f;
+                r1 = (A.wt ? A.wt[(size_t)band * A.n_t + t] : 1.0f) * r * r;
             }
+            k_of = k;
+            band_of = band;
+        }
+        return r1;
+    };
+    if (n_sum < 8) {
+        for (int i = 0; i < n_sum; ++i) {
+            float x = value(i);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-            if (lane == 0) sred[(warp * vt + vl) * n_ssr + bb] = x;
+            if (lane == 0) sred[warp * n_sum + i] = x;
+        }
+    } else {
+        const bool hi16 = lane & 16, hi8 = lane & 8, hi4 = lane & 4;
+        for (int i0 = 0; i0 < n_sum; i0 += 8) {
+            float v[8], x4[4], x2[2];
+#pragma unroll
+            for (int u = 0; u < 8; ++u) v[u] = i0 + u < n_sum ? value(i0 + u) : 0.0f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                x4[i] = (hi16 ? v[4 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, hi16 ? v[i] : v[4 + i], 16);
+#pragma unroll
+            for (int i = 0; i < 2; ++i)
+                x2[i] = (hi8 ? x4[2 + i] : x4[i]) + __shfl_xor_sync(0xffffffffu, hi8 ? x4[i] : x4[2 + i], 8);
+            float x = (hi4 ? x2[1] : x2[0]) + __shfl_xor_sync(0xffffffffu, hi4 ? x2[0] : x2[1], 4);
+            x += __shfl_xor_sync(0xffffffffu, x, 2);
+            x += __shfl_xor_sync(0xffffffffu, x, 1);
+            const int i = i0 + (lane >> 4) * 4 + (hi8 ? 2 : 0) + (hi4 ? 1 : 0);
+            if ((lane & 3) == 0 && i < n_sum) sred[warp * n_sum + i] = x;
         }
     }
     __syncthreads();
-    for (int i = tid; i < ng * n_ssr; i += TB) {
-        const int vl = i / n_ssr, bb = i - vl * n_ssr;
+    for (int i = tid; i < n_sum; i += TB) {
+        const int p = i & (n_pair - 1), vl = p & (vt - 1), blk = tile * kt + (p >> log_vt);
+        if (vl >= ng || blk >= A.n_blk) continue;
         float x = 0.0f;
-        for (int w = 0; w < NW; ++w) x += sred[(w * vt + vl) * n_ssr + bb];
-        A.ssr_part[((size_t)(g0 + vl) * A.n_bpg + bb) * A.n_tiles + tile] = x;
+        for (int w = 0; w < NW; ++w) x += sred[w * n_sum + i];
+        A.ssr_part[((size_t)(g0 + vl) * A.n_bpg + (i >> log_p)) * A.n_blk + blk] = x;
     }
 }
 
