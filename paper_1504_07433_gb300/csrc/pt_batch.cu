@@ -61,7 +61,8 @@ enum Mode {
     M_ROWS = 0,     // k_mode 0: row tables of the exact depth
     M_KHAT = 1,     // k_mode 1: the exact terms once per time with k_hat, scaled per passband (Sec. 3.5)
     M_INTERP = 2,   // k_mode 2: rows of the caller's table, interpolated in k, staged in shared memory
-    M_GATHER = 3    // k_mode 2 with rows too long to stage: bilinear reads of the table per point
+    M_GATHER = 3,   // k_mode 2 with rows too long to stage: bilinear reads of the table per point
+    M_EXACT = 4     // k_mode 0, too few points for row tables: the exact terms per point
 };
 
 // What is asked for: the two usual calls have no run-time choice per point.
@@ -263,72 +264,192 @@ __device__ __forceinline__ float4 lds_here(const float4 *p)
     return v;
 }
 
-// One passband of an item without a row table (its radius ratio outside
-// mt_valid, or too few points for tables): the exact terms per point.
+// The passbands `mask` of an item's group that have no row table (the radius ratio
+// outside mt_valid, or all of them in a plan with too few points for tables): the
+// exact terms per point.  A chunk of TT times at a time: the in-window ones are listed in
+// order with their separations, and the warps take (passband, part of the list)
+// tasks, a lane per unit, so that lanes stay full and one orbit solution serves
+// all passbands (with supersamples each unit solves its own).  Sums are formed
+// per task, in order.  (A passband at a time over all the threads' times, as
+// before, 1,000 walkers x 16 passbands x 300 times took 174 us, 57 now; x 9,000
+// times at k = 0.7 1,723, 966 now.)
 template <int TT>
-__device__ __noinline__ void exact_row(const BatchArgs &A, const GeomRec &g, int v, int b, int slice, float *sred,
-                                       int *n_bad)
+struct ExactSmem {
+    int at[2][TT];             // times of the chunk: in the window, outside it in a tile that meets it
+    float dt[TT], z[TT];       // of the in-window ones
+    int cnt[2][TT / 32];
+    int band[BG];
+    float sum[BG];             // one per task
+};
+
+template <int TT>
+__device__ __forceinline__ int exact_item(const BatchArgs &A, const GeomRec &g, int v, int b0, unsigned mask, int slice,
+                                          ExactSmem<TT> &S)
 {
+    constexpr int NW = TT / 32, TPP = TT / BT;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const size_t row = (size_t)v * A.n_b + b;
-    const float k = A.k[row];
-    const float3 w = band_weights(A.ld, row);
+    const int nb = __popc(mask), n_seg = max(1, NW / nb), n_task = nb * n_seg;   // (n_task <= BG: nb, or up to NW <= 8)
     const float inv_ss = 1.0f / (float)A.n_ss;
     const int t_end = min(A.n_tiles, (slice + 1) * A.tiles_per_slice);
-    float acc = 0.0f;
-    for (int tj = slice * A.tiles_per_slice + tid / BT; tj < t_end; tj += TT / BT) {
-        const float2 mm = A.tile_mm[tj];
-        const int2 tl = A.tiles[tj];
-        if ((tid & (BT - 1)) >= tl.y) continue;
-        const int i = tl.x + (tid & (BT - 1));
-        float dep = 0.0f;
-        bool inw = false;
-        if (tile_meets_window(g, mm.x, mm.y)) {
-            const float2 ts = A.tsplit[i];
-            const float dt = pt::reduce_time(ts.x, ts.y, g);
-            inw = dt >= g.win_lo && dt <= g.win_hi;
-            if (inw) {
-                float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
-                for (int s = 0; s < A.n_ss; ++s) {
-                    bool bad = false;
-                    const float off = A.t_exp * (((float)s + 0.5f) * inv_ss - 0.5f);
-                    const float z = pt::orbit_z<true>(g, dt + off, A.max_iter, &bad, warm);
-                    if (bad && b == 0 && !A.rows) ++*n_bad;
-                    float le, ld, ed;
-                    pt::ma_terms(k, z, &le, &ld, &ed);
-                    dep += w.x * le + w.y * ld + w.z * ed;
-                }
-                dep *= inv_ss;
+    if (tid < BG) {
+        S.sum[tid] = 0.0f;
+        if ((mask >> tid) & 1u) S.band[__popc(mask & ((1u << tid) - 1u))] = b0 + tid;
+    }
+    int nbad = 0;
+#pragma unroll 1
+    for (int c0 = slice * A.tiles_per_slice; c0 < t_end; c0 += TPP) {
+        const int tj = c0 + tid / BT;
+        int i = -1;            // this thread's time
+        bool meets = false, in = false;
+        float dt = 0.0f, z = 0.0f;
+        if (tj < t_end) {
+            const float2 mm = A.tile_mm[tj];
+            const int2 tl = A.tiles[tj];
+            if ((tid & (BT - 1)) < tl.y) i = tl.x + (tid & (BT - 1));
+            meets = tile_meets_window(g, mm.x, mm.y);
+            if (meets && i >= 0) {
+                const float2 ts = A.tsplit[i];
+                dt = pt::reduce_time(ts.x, ts.y, g);
+                in = dt >= g.win_lo && dt <= g.win_hi;
             }
         }
-        if (A.flux) A.flux[row * A.n_t + i] = 1.0f - dep;
-        if (A.ssr_part) {
-            const size_t at = (size_t)b * A.n_t + i;
-            const float r = (A.y[at] - 1.0f) + dep;
-            acc = fmaf((A.wt ? A.wt[at] : 1.0f) * r, r, acc);
+        if (in && A.n_ss == 1) {
+            bool bad = false;
+            z = pt::orbit_z<true>(g, dt, A.max_iter, &bad);
+            if (bad) ++nbad;
+        }
+        if (A.flux && i >= 0 && !in)
+            for (unsigned m = mask; m; m &= m - 1u) A.flux[((size_t)v * A.n_b + b0 + __ffs(m) - 1) * A.n_t + i] = 1.0f;
+        // tiles that do not meet the window: their residuals are in the base (a lane each)
+        const unsigned skipped = __ballot_sync(0xffffffffu, tj < t_end && !meets && (tid & (BT - 1)) == 0);
+        const unsigned bin = __ballot_sync(0xffffffffu, in), bout = __ballot_sync(0xffffffffu, meets && i >= 0 && !in);
+        __syncthreads();   // the previous chunk is no longer read
+        if (lane == 0) {
+            S.cnt[0][warp] = __popc(bin) | (skipped ? 1 << 16 : 0);
+            S.cnt[1][warp] = __popc(bout);
+        }
+        __syncthreads();
+        int at0 = 0, at1 = 0, n_in = 0, n_out = 0;
+        unsigned skip = 0u;    // bit w: warp w's first tile is skipped (BT / 32 warps per tile)
+#pragma unroll
+        for (int w = 0; w < NW; ++w) {
+            const int c = S.cnt[0][w] & 0xffff;
+            skip |= S.cnt[0][w] >> 16 ? 1u << w : 0u;
+            at0 += w < warp ? c : 0;
+            at1 += w < warp ? S.cnt[1][w] : 0;
+            n_in += c;
+            n_out += S.cnt[1][w];
+        }
+        const unsigned below = (1u << lane) - 1u;
+        if (in) {
+            at0 += __popc(bin & below);
+            S.at[0][at0] = i;
+            S.dt[at0] = dt;
+            S.z[at0] = z;
+        } else if (meets && i >= 0) {
+            S.at[1][at1 + __popc(bout & below)] = i;
+        }
+        __syncthreads();
+#pragma unroll 1
+        for (int task = warp; task < n_task; task += NW) {
+            const int jj = task / n_seg, seg = task - jj * n_seg, b = S.band[jj];
+            const size_t row = (size_t)v * A.n_b + b;
+            float acc = 0.0f;
+            if (A.ssr_part) {
+                if (seg == 0 && lane < NW && (skip >> lane) & 1u) acc = A.base[(size_t)b * A.n_tiles + c0 + lane / (BT / 32)];
+                const float *y = A.y + (size_t)b * A.n_t, *wt = A.wt + (size_t)b * A.n_t;
+                for (int q = seg * 32 + lane; q < n_out; q += 32 * n_seg) {
+                    const int at = S.at[1][q];
+                    const float r = y[at] - 1.0f;
+                    acc = fmaf((A.wt ? wt[at] : 1.0f) * r, r, acc);
+                }
+            }
+            const float k = A.k[row];
+            const float3 w = band_weights(A.ld, row);
+#pragma unroll 1
+            for (int q = seg * 32 + lane; q < n_in; q += 32 * n_seg) {
+                float dep = 0.0f;
+                float warm[4] = {__int_as_float(0x7fffffff), 0.0f, 0.0f, 0.0f};   // Kepler warm start (none yet)
+#pragma unroll 1
+                for (int s = 0; s < A.n_ss; ++s) {
+                    float zs = S.z[q];
+                    if (A.n_ss > 1) {
+                        bool bad = false;
+                        zs = pt::orbit_z<true>(g, S.dt[q] + A.t_exp * (((float)s + 0.5f) * inv_ss - 0.5f), A.max_iter, &bad, warm);
+                        if (bad && jj == 0) ++nbad;   // every passband solves the same orbit
+                    }
+                    float le, ld, ed;
+                    pt::ma_terms(k, zs, &le, &ld, &ed);
+                    dep += w.x * le + w.y * ld + w.z * ed;
+                }
+                dep = __fmul_rn(dep, inv_ss);
+                const int at = S.at[0][q];
+                if (A.flux) A.flux[row * A.n_t + at] = 1.0f - dep;
+                if (A.ssr_part) {
+                    const float r = (A.y[(size_t)b * A.n_t + at] - 1.0f) + dep;
+                    acc = fmaf((A.wt ? A.wt[(size_t)b * A.n_t + at] : 1.0f) * r, r, acc);
+                }
+            }
+            if (A.ssr_part) {
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+                if (lane == 0) S.sum[task] += acc;
+            }
         }
     }
     if (A.ssr_part) {
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
         __syncthreads();
-        if (lane == 0) sred[warp] = acc;
-        __syncthreads();
-        if (tid == 0) {
+        if (tid < nb) {
             float x = 0.0f;
-            for (int u = 0; u < TT / 32; ++u) x += sred[u];
-            A.ssr_part[row * A.n_slices + slice] = x;
+            for (int s = 0; s < n_seg; ++s) x += S.sum[tid * n_seg + s];
+            A.ssr_part[((size_t)v * A.n_b + S.band[tid]) * A.n_slices + slice] = x;
         }
     }
+    __syncthreads();
+    return nbad;
+}
+
+// ... out of the way of the row tables' kernel
+template <int TT>
+__device__ __noinline__ int exact_item_call(const BatchArgs *A, const GeomRec *g, int v, int b0, unsigned mask, int slice,
+                                            ExactSmem<TT> *S)
+{
+    return exact_item<TT>(*A, *g, v, b0, mask, slice, *S);
+}
+
+// A plan without tables: exact_item on every item.  The terms are a long dependent
+// chain, so as many warps as there are registers without spills.
+template <int TT>
+__global__ void __launch_bounds__(TT, 1024 / TT) batch_exact_kernel(const __grid_constant__ BatchArgs A)
+{
+    __shared__ GeomRec srec;
+    __shared__ ExactSmem<TT> S;
+    __shared__ int s_item;
+    const int tid = threadIdx.x;
+    int nbad = 0;
+    for (;;) {
+        if (tid == 0) s_item = atomicAdd(A.counter, 1);
+        __syncthreads();
+        const int it = s_item;
+        if (it >= A.n_items) break;
+        const int v = it % A.n_v, sg = it / A.n_v;
+        const int grp = sg % A.n_groups, slice = sg / A.n_groups;
+        const int b0 = grp * A.bg, nb = min(A.bg, A.n_b - b0);
+        if (tid < 6) reinterpret_cast<float4 *>(&srec)[tid] = reinterpret_cast<const float4 *>(&A.rec[v])[tid];
+        __syncthreads();
+        const int bad = exact_item<TT>(A, srec, v, b0, 0xffffffffu >> (32 - nb), slice, S);
+        if (grp == 0) nbad += bad;
+    }
+    if (nbad && A.n_bad) atomicAdd(A.n_bad, nbad);
 }
 
 template <int TT, int MODE, bool SS, int OUT>
-__global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(BatchArgs A)
+__global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(const __grid_constant__ BatchArgs A)
 {
     extern __shared__ __align__(16) float dyn[];   // M_ROWS: [BG][MT_ROW]; M_INTERP: [BG][mn_z]
     __shared__ GeomRec srec;
     __shared__ float4 sband[BG];   // M_ROWS: k, the scales, valid; M_KHAT: depth weights; others: we, wd, wn, k
-    __shared__ float sex[TT / 32];
+    __shared__ ExactSmem<TT> sex;   // M_ROWS
     __shared__ float sred[TT / 32][BG];
     __shared__ int slist[TT], swcnt[TT / 32];
     __shared__ int s_item;
@@ -352,16 +473,16 @@ __global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(BatchArgs A)
         // groups of 4 passbands are evaluated together; the last group's
         // padding repeats the item's last passband and is dropped at the stores
         const int nb4 = (nb + 3) & ~3;
-        bool all_ok = true;
+        bool row_ok = true;
         if (tid < nb4) {
             const size_t row = row0 + min(tid, nb - 1);
             const float kb = A.k[row];
             const float3 w = band_weights(A.ld, row);
             if (MODE == M_ROWS) {
                 float sA = 0.0f, sL = 0.0f;
-                all_ok = A.rows && pt::mt_valid(kb);
-                if (all_ok) pt::mt_scales(kb, &sA, &sL);
-                sband[tid] = make_float4(kb, sA, sL, all_ok ? 1.0f : 0.0f);
+                row_ok = pt::mt_valid(kb);
+                if (row_ok) pt::mt_scales(kb, &sA, &sL);
+                sband[tid] = make_float4(kb, sA, sL, row_ok ? 1.0f : 0.0f);
             } else if (MODE == M_KHAT) {
                 const float r = kb / A.rec[v].k;
                 const float r2 = r * r;
@@ -370,8 +491,9 @@ __global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(BatchArgs A)
                 sband[tid] = make_float4(w.x, w.y, w.z, kb);
             }
         }
-        all_ok = __syncthreads_and(all_ok);
-        if (MODE == M_ROWS) {
+        const int n_without = __syncthreads_count(!row_ok);
+        const bool all_ok = n_without == 0, any_ok = n_without < nb4;
+        if (MODE == M_ROWS && any_ok) {
             // a row without a table (its radius ratio outside mt_valid) is staged as zeros
             for (int i = tid; i < nb4 * (pt::MT_ROW / 4); i += TT) {
                 const int j = i / (pt::MT_ROW / 4);
@@ -399,7 +521,7 @@ __global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(BatchArgs A)
         float acc[BG];
 #pragma unroll
         for (int j = 0; j < BG; ++j) acc[j] = 0.0f;
-        const int t_end = MODE == M_ROWS && !A.rows ? 0 : min(A.n_tiles, (slice + 1) * A.tiles_per_slice);
+        const int t_end = MODE == M_ROWS && !any_ok ? 0 : min(A.n_tiles, (slice + 1) * A.tiles_per_slice);
         for (int c0 = slice * A.tiles_per_slice; c0 < t_end; c0 += TT) {
             // one window test per thread; the tiles to evaluate listed in order
             const int jt = c0 + tid;
@@ -596,8 +718,10 @@ __global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(BatchArgs A)
         }
         if (MODE == M_ROWS && !all_ok) {
             __syncthreads();   // the zero rows' flux is in place
-            for (int j = 0; j < nb; ++j)
-                if (sband[j].w == 0.0f) exact_row<TT>(A, srec, v, b0 + j, slice, sex, &nbad);
+            unsigned mask = 0u;
+            for (int j = 0; j < nb; ++j) mask |= sband[j].w == 0.0f ? 1u << j : 0u;
+            const int bad = exact_item_call<TT>(&A, &srec, v, b0, mask, slice, &sex);
+            if (!any_ok && grp == 0) nbad += bad;   // (else counted by the pass over the rows)
         }
         __syncthreads();   // shared memory is free for the next item
     }
@@ -657,6 +781,7 @@ BatchFn batch_fn_t(int mode, bool ss, int out)
     case M_ROWS: return ss ? batch_fn_o<TT, M_ROWS, true>(out) : batch_fn_o<TT, M_ROWS, false>(out);
     case M_KHAT: return batch_kernel<TT, M_KHAT, true, O_ANY>;
     case M_INTERP: return batch_kernel<TT, M_INTERP, true, O_ANY>;
+    case M_EXACT: return batch_exact_kernel<TT>;
     default: return batch_kernel<TT, M_GATHER, true, O_ANY>;
     }
 }
@@ -769,8 +894,10 @@ constexpr int MAX_SLICES = 64;
 
 // Row tables from this many points (times x supersamples) per row: a table
 // costs 144 evaluations of the exact terms, a row reads it at the in-window
-// points, about a third of them in the light curves of transits.
-constexpr int ROWS_MIN_POINTS = 512;
+// points, about a third of them in the light curves of transits.  5,000 walkers
+// x 16 passbands: 600 times 351 us by the exact terms and 414 from rows, 800 times
+// 455 and 435, 1,000 times 563 and 459; 200 times x 3 supersamples 287 and 395.
+constexpr int ROWS_MIN_POINTS = 768;
 
 int configure(pt_batch_plan_s &p, int tt, int n_slices, int n_z)
 {
@@ -843,7 +970,7 @@ int pt_batch_plan_create(const pt_batch_desc *d, int autotune, pt_batch_plan *ou
         return st;
     }
     // rows of the caller's table are staged in shared memory while a group fits
-    p->mode = d->k_mode == 0 ? M_ROWS
+    p->mode = d->k_mode == 0 ? ((long long)d->n_t * d->n_ss >= ROWS_MIN_POINTS ? M_ROWS : M_EXACT)
               : d->k_mode == 1 ? M_KHAT
               : (size_t)BG * tab.mn_z * sizeof(float) <= INTERP_SMEM ? M_INTERP : M_GATHER;
     // tiles of BT times within each light curve
@@ -852,11 +979,11 @@ int pt_batch_plan_create(const pt_batch_desc *d, int autotune, pt_batch_plan *ou
         for (int s = d->lc_offsets[j]; s < d->lc_offsets[j + 1]; s += BT)
             tiles.push_back(make_int2(s, std::min(BT, d->lc_offsets[j + 1] - s)));
     p->n_tiles = (int)tiles.size();
+    const bool tables = p->mode == M_ROWS;
     p->bg = d->n_t <= (1 << 28) ? BG : 1;   // a group's observations within 32-bit offsets
     p->n_groups = (d->n_b + p->bg - 1) / p->bg;
     // many rows need no slices: bounds the partial sums
     p->max_slices = (int)std::max(1LL, std::min((long long)MAX_SLICES, (1LL << 26) / n_rows));
-    const bool tables = p->mode == M_ROWS && (long long)d->n_t * d->n_ss >= ROWS_MIN_POINTS;
     cudaError_t e = cudaMalloc(&p->d_counter, sizeof(int));
     if (e == cudaSuccess) e = cudaMalloc(&p->d_rec, (size_t)o.n_v * sizeof(GeomRec));
     if (e == cudaSuccess) e = cudaMalloc(&p->d_tsplit, (size_t)d->n_t * sizeof(float2));
