@@ -409,6 +409,26 @@ __device__ __forceinline__ int exact_item(const BatchArgs &A, const GeomRec &g, 
     return nbad;
 }
 
+// The warp's sums of 16 values per lane, value j on lanes 2 j and 2 j + 1: at each
+// level of the tree half the lanes keep half of the values (16 shuffles for 80).
+__device__ __forceinline__ float warp_sums(const float (&v)[BG])
+{
+    static_assert(BG == 16, "a value per pair of lanes");
+    const int lane = threadIdx.x & 31;
+    float a[8], b[4], c[2];
+#pragma unroll
+    for (int i = 0; i < 8; ++i)
+        a[i] = (lane & 16 ? v[8 + i] : v[i]) + __shfl_xor_sync(0xffffffffu, lane & 16 ? v[i] : v[8 + i], 16);
+#pragma unroll
+    for (int i = 0; i < 4; ++i)
+        b[i] = (lane & 8 ? a[4 + i] : a[i]) + __shfl_xor_sync(0xffffffffu, lane & 8 ? a[i] : a[4 + i], 8);
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+        c[i] = (lane & 4 ? b[2 + i] : b[i]) + __shfl_xor_sync(0xffffffffu, lane & 4 ? b[i] : b[2 + i], 4);
+    const float x = (lane & 2 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, lane & 2 ? c[0] : c[1], 2);
+    return x + __shfl_xor_sync(0xffffffffu, x, 1);
+}
+
 // ... out of the way of the row tables' kernel
 template <int TT>
 __device__ __noinline__ int exact_item_call(const BatchArgs *A, const GeomRec *g, int v, int b0, unsigned mask, int slice,
@@ -518,11 +538,12 @@ __global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(const __grid_consta
             }
             __syncthreads();
         }
-        float acc[BG];
-#pragma unroll
-        for (int j = 0; j < BG; ++j) acc[j] = 0.0f;
+        bool first = true;
         const int t_end = MODE == M_ROWS && !any_ok ? 0 : min(A.n_tiles, (slice + 1) * A.tiles_per_slice);
         for (int c0 = slice * A.tiles_per_slice; c0 < t_end; c0 += TT) {
+            float acc[BG];   // residual sums of this chunk: at most BT + 1 terms each
+#pragma unroll
+            for (int j = 0; j < BG; ++j) acc[j] = 0.0f;
             // one window test per thread; the tiles to evaluate listed in order
             const int jt = c0 + tid;
             bool ev = false;
@@ -700,19 +721,21 @@ __global__ void __launch_bounds__(TT, 768 / TT) batch_kernel(const __grid_consta
                     }
                 }
             }
+            if (want_ssr) {
+                // The chunk's sums go to the warp's: carried on in the registers, a
+                // thread's sum would be one chain over the whole slice (4,000 terms
+                // at 1e6 times).
+                const float x = warp_sums(acc);
+                if ((lane & 1) == 0) sred[warp][lane >> 1] = first ? x : sred[warp][lane >> 1] + x;
+                first = false;
+            }
         }
         if (want_ssr) {
-#pragma unroll
-            for (int j = 0; j < BG; ++j) {
-                float x = acc[j];
-#pragma unroll
-                for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-                if (lane == 0) sred[warp][j] = x;
-            }
             __syncthreads();
             if (tid < nb) {
                 float x = 0.0f;
-                for (int w = 0; w < NW; ++w) x += sred[w][tid];
+                if (!first)
+                    for (int w = 0; w < NW; ++w) x += sred[w][tid];
                 if (MODE != M_ROWS || sband[tid].w != 0.0f) A.ssr_part[(row0 + tid) * A.n_slices + slice] = x;
             }
         }
