@@ -278,7 +278,13 @@ int pt_ma_quad_bwd(const double *t_dev, int n_t, const pt_theta *theta, int n_ss
  * CUDA graph.  pt_batch_run() replays that graph on a stream: update the
  * contents of the bound buffers (new walker parameters, new data) between
  * runs.  The plan allocates its own work list and scratch (device memory)
- * at creation and releases them in pt_batch_plan_destroy().
+ * at creation and releases them in pt_batch_plan_destroy(); the row tables take
+ * 768 bytes per (walker, passband), 2 GB at most: the walkers beyond come in
+ * further passes of the same graph.  A plan with fewer than 768 points (times x
+ * supersamples) has no tables and takes the exact terms per point.
+ * pt_batch_plan_info() gives the chosen configuration: *tile, the times a CTA takes
+ * at once (its threads), *ctas_per_sm, *n_items, the work items of a run, and
+ * *tuned_ms, the time measured at creation.
  * ---------------------------------------------------------------------- */
 typedef struct pt_batch_desc {
     const double *t;        /* [n_t] device, concatenated exposure times */

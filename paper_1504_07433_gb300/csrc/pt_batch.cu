@@ -767,6 +767,7 @@ struct pt_batch_plan_s {
     int tt, ctas_per_sm, grid, n_sm;
     int mode;
     int n_tiles, bg, n_groups, n_slices, n_items, max_slices;
+    int v_chunk;           // walkers whose row tables exist at a time
     int2 *d_tiles;
     float2 *d_mm;
     float *d_base;
@@ -843,65 +844,82 @@ int enqueue(pt_batch_plan_s &p, cudaStream_t s)
     const pt_batch_desc &d = p.d;
     cudaError_t e = cudaMemsetAsync(p.d_counter, 0, sizeof(int), s);
     if (e != cudaSuccess) return berr(e, "cudaMemsetAsync");
-    PrepArgs sa;
-    sa.t = d.t;
-    sa.n_t = d.n_t;
-    sa.tsplit = p.d_tsplit;
-    sa.orb = d.orb;
-    sa.k = d.k;
-    sa.ld = d.ld;
-    sa.khat = d.k_mode == 1;
-    sa.n_b = d.n_b;
-    sa.half_exp = (float)(0.5 * d.t_exp);
-    sa.rec = p.d_rec;
-    sa.tiles = p.d_tiles;
-    sa.tile_mm = p.d_mm;
-    sa.base = p.d_base;
-    sa.y = d.y;
-    sa.wt = d.wt;
-    sa.n_tiles = p.n_tiles;
-    sa.rows = p.d_rows;
-    sa.n_gblocks = (d.orb.n_v + 31) / 32;
-    sa.n_tblocks = (p.n_tiles + PREP_TILES - 1) / PREP_TILES;
-    const long long per = (long long)(PREP / 32) * PREP_BASE;
-    sa.n_bblocks = d.ssr ? (int)(((long long)d.n_b * p.n_tiles + per - 1) / per) : 0;
-    const long long blocks = (long long)sa.n_gblocks + sa.n_tblocks + sa.n_bblocks +
-                             (p.d_rows ? ((long long)d.orb.n_v * d.n_b + PREP_ROWS - 1) / PREP_ROWS : 0);
-    batch_prep_kernel<<<(unsigned)blocks, PREP, 0, s>>>(sa);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return berr(e, "batch_prep_kernel");
-    BatchArgs A;
-    int st = table_args(d, &A);
-    if (st) return st;
-    A.tsplit = p.d_tsplit;
-    A.n_t = d.n_t;
-    A.rec = p.d_rec;
-    A.k = d.k;
-    A.ld = d.ld;
-    A.rows = p.d_rows;
-    A.tiles = p.d_tiles;
-    A.tile_mm = p.d_mm;
-    A.base = p.d_base;
-    A.n_tiles = p.n_tiles;
-    A.n_v = d.orb.n_v;
-    A.n_b = d.n_b;
-    A.n_ss = d.n_ss;
-    A.t_exp = (float)d.t_exp;
-    A.max_iter = d.max_iter;
-    A.y = d.y;
-    A.wt = d.wt;
-    A.flux = d.flux;
-    A.ssr_part = d.ssr ? p.d_part : nullptr;
-    A.bg = p.bg;
-    A.n_groups = p.n_groups;
-    A.n_slices = p.n_slices;
-    A.tiles_per_slice = (p.n_tiles + p.n_slices - 1) / p.n_slices;
-    A.n_items = p.n_items;
-    A.counter = p.d_counter;
-    A.n_bad = d.n_bad;
-    batch_fn(p, p.tt)<<<p.grid, p.tt, dyn_smem(p, A.mn_z), s>>>(A);
-    e = cudaGetLastError();
-    if (e != cudaSuccess) return berr(e, "batch_kernel");
+    // walkers [v0, v0 + n): as many as the row tables hold
+    for (int v0 = 0; v0 < d.orb.n_v; v0 += p.v_chunk) {
+        const int n = std::min(p.v_chunk, d.orb.n_v - v0);
+        const size_t r0 = (size_t)v0 * d.n_b;
+        if (v0 > 0) {
+            e = cudaMemsetAsync(p.d_counter, 0, sizeof(int), s);
+            if (e != cudaSuccess) return berr(e, "cudaMemsetAsync");
+        }
+        PrepArgs sa;
+        sa.t = d.t;
+        sa.n_t = d.n_t;
+        sa.tsplit = p.d_tsplit;
+        sa.orb = d.orb;
+        sa.orb.t0 += v0;
+        sa.orb.P += v0;
+        sa.orb.a += v0;
+        sa.orb.inc += v0;
+        if (sa.orb.e) sa.orb.e += v0;
+        if (sa.orb.w) sa.orb.w += v0;
+        sa.orb.n_v = n;
+        sa.k = d.k + r0;
+        sa.ld = d.ld + 2 * r0;
+        sa.khat = d.k_mode == 1;
+        sa.n_b = d.n_b;
+        sa.half_exp = (float)(0.5 * d.t_exp);
+        sa.rec = p.d_rec + v0;
+        sa.tiles = p.d_tiles;
+        sa.tile_mm = p.d_mm;
+        sa.base = p.d_base;
+        sa.y = d.y;
+        sa.wt = d.wt;
+        sa.n_tiles = p.n_tiles;
+        sa.rows = p.d_rows;
+        sa.n_gblocks = (n + 31) / 32;
+        // (the times' share does not depend on the walkers: once)
+        sa.n_tblocks = v0 > 0 ? 0 : (p.n_tiles + PREP_TILES - 1) / PREP_TILES;
+        const long long per = (long long)(PREP / 32) * PREP_BASE;
+        sa.n_bblocks = d.ssr && v0 == 0 ? (int)(((long long)d.n_b * p.n_tiles + per - 1) / per) : 0;
+        const long long blocks = (long long)sa.n_gblocks + sa.n_tblocks + sa.n_bblocks +
+                                 (p.d_rows ? ((long long)n * d.n_b + PREP_ROWS - 1) / PREP_ROWS : 0);
+        batch_prep_kernel<<<(unsigned)blocks, PREP, 0, s>>>(sa);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return berr(e, "batch_prep_kernel");
+        BatchArgs A;
+        int st = table_args(d, &A);
+        if (st) return st;
+        A.tsplit = p.d_tsplit;
+        A.n_t = d.n_t;
+        A.rec = p.d_rec + v0;
+        A.k = d.k + r0;
+        A.ld = d.ld + 2 * r0;
+        A.rows = p.d_rows;
+        A.tiles = p.d_tiles;
+        A.tile_mm = p.d_mm;
+        A.base = p.d_base;
+        A.n_tiles = p.n_tiles;
+        A.n_v = n;
+        A.n_b = d.n_b;
+        A.n_ss = d.n_ss;
+        A.t_exp = (float)d.t_exp;
+        A.max_iter = d.max_iter;
+        A.y = d.y;
+        A.wt = d.wt;
+        A.flux = d.flux ? d.flux + r0 * d.n_t : nullptr;
+        A.ssr_part = d.ssr ? p.d_part + r0 * p.n_slices : nullptr;
+        A.bg = p.bg;
+        A.n_groups = p.n_groups;
+        A.n_slices = p.n_slices;
+        A.tiles_per_slice = (p.n_tiles + p.n_slices - 1) / p.n_slices;
+        A.n_items = n * p.n_groups * p.n_slices;
+        A.counter = p.d_counter;
+        A.n_bad = d.n_bad;
+        batch_fn(p, p.tt)<<<std::min(p.grid, A.n_items), p.tt, dyn_smem(p, A.mn_z), s>>>(A);
+        e = cudaGetLastError();
+        if (e != cudaSuccess) return berr(e, "batch_kernel");
+    }
     if (d.ssr) {
         int rows = d.orb.n_v * d.n_b;
         batch_reduce_kernel<<<(rows + 127) / 128, 128, 0, s>>>(p.d_part, rows, p.n_slices, d.ssr);
@@ -921,6 +939,11 @@ constexpr int MAX_SLICES = 64;
 // x 16 passbands: 600 times 351 us by the exact terms and 414 from rows, 800 times
 // 455 and 435, 1,000 times 563 and 459; 200 times x 3 supersamples 287 and 395.
 constexpr int ROWS_MIN_POINTS = 768;
+
+// A plan's row tables are made for this many bytes of walkers at a time (768 bytes
+// per walker and passband: 100,000 walkers x 256 passbands would be 20 GB).  A chunk
+// still has millions of rows, so the launches between chunks do not show.
+constexpr size_t ROWS_MAX_BYTES = (size_t)2 << 30;
 
 int configure(pt_batch_plan_s &p, int tt, int n_slices, int n_z)
 {
@@ -1014,9 +1037,17 @@ int pt_batch_plan_create(const pt_batch_desc *d, int autotune, pt_batch_plan *ou
     if (e == cudaSuccess) e = cudaMalloc(&p->d_mm, tiles.size() * sizeof(float2));
     if (e == cudaSuccess && d->ssr) e = cudaMalloc(&p->d_base, (size_t)d->n_b * tiles.size() * sizeof(float));
     if (e == cudaSuccess && d->ssr) e = cudaMalloc(&p->d_part, (size_t)n_rows * p->max_slices * sizeof(float));
-    if (e == cudaSuccess && tables) e = cudaMalloc(&p->d_rows, (size_t)n_rows * pt::MT_ROW * sizeof(float));
-    // (the two unused floats per interval are staged with the others)
-    if (e == cudaSuccess && tables) e = cudaMemset(p->d_rows, 0, (size_t)n_rows * pt::MT_ROW * sizeof(float));
+    // row tables of as many walkers as ROWS_MAX_BYTES hold, in equal chunks
+    p->v_chunk = o.n_v;
+    if (tables) {
+        const long long cap = std::max(1LL, (long long)(ROWS_MAX_BYTES / ((size_t)d->n_b * pt::MT_ROW * sizeof(float))));
+        const long long n_chunk = (o.n_v + cap - 1) / cap;
+        p->v_chunk = (int)((o.n_v + n_chunk - 1) / n_chunk);
+        const size_t bytes = (size_t)p->v_chunk * d->n_b * pt::MT_ROW * sizeof(float);
+        if (e == cudaSuccess) e = cudaMalloc(&p->d_rows, bytes);
+        // (the two unused floats per interval are staged with the others)
+        if (e == cudaSuccess) e = cudaMemset(p->d_rows, 0, bytes);
+    }
     if (e == cudaSuccess) e = cudaMemcpy(p->d_tiles, tiles.data(), tiles.size() * sizeof(int2), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         st = berr(e, "pt_batch_plan_create");
