@@ -431,12 +431,17 @@ __device__ __forceinline__ float point_sums(const PointConst &c, float dts, floa
     const float V = c.Vtr + dV;
     if (V <= 0.0f) return 0.0f;
     const float Vi = V * c.ci;
-    const float z = pt::sqrt_a(fmaf(U, U, Vi * Vi));
+    // z and w dF/dz / z: approximate root and reciprocal, each once corrected by its
+    // remainder, for the errors of sqrtf and a division (4,096 vectors x 10,000 times:
+    // 182 us so, 195 with those two, 179 uncorrected).  At z = 0 dF/dz is 0 but for a
+    // row's rounding; z is then 1e-18.
+    const float zz = fmaxf(fmaf(U, U, Vi * Vi), 1e-36f), z0 = pt::sqrt_a(zz), iz = pt::rcp_a(z0);
+    const float z = fmaf(0.5f * fmaf(-z0, z0, zz), iz, z0);
     const LimbTerms l = ROWS ? limb_row(c.base, c.k, c.sA, c.sL, z) : limb_exact(c.lc, c.k, z);
     if (ss1) w *= 2.0f * (yw - l.dep);   // one supersample: w is the point's weight
     const float cE = c.cE + dC, sE = c.sE + dS;
     const float iecE = pt::rcp_a(1.0f - c.ecE * (1.0f - omc) + c.esE * sn);   // 1 - e cos E
-    const float G = w * l.dz * pt::rcp_a(fmaxf(z, 1e-30f));
+    const float wdz = w * l.dz, g0 = wdz * iz, G = fmaf(fmaf(-g0, z, wdz), iz, g0);
     const float GU = G * U, GV = G * V;
     const float GVc = GV * c.ci2, Vp = iecE * (c.Vc * cE - c.Vs * sE);
     const float X = GVc * Vp - GU * (iecE * (c.Uc * sE + c.Us * cE));
