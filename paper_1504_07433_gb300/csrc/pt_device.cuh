@@ -418,9 +418,9 @@ __device__ __forceinline__ FgSeries fg_series(float E1, float esin)
 __device__ __forceinline__ float fg_z(const OrbitState &o, const FgSeries &c, float cosi, float x)
 {
     const float x2 = x * x;
-    const float f = fmaf(fmaf(fmaf(fmaf(c.f5, x, c.f4), x, c.f3), x, c.f2), x2, 1.0f);
+    const float f1 = fmaf(fmaf(fmaf(c.f5, x, c.f4), x, c.f3), x, c.f2) * x2;   // f - 1
     const float g = fmaf(fmaf(fmaf(c.g5, x, c.g4), x, c.g3), x2 * x, x);
-    const float U = fmaf(f, o.U, g * o.Up), V = fmaf(f, o.V, g * o.Vp);
+    const float U = o.U + fmaf(f1, o.U, g * o.Up), V = o.V + fmaf(f1, o.V, g * o.Vp);
     const float Vi = V * cosi;
     return V > 0.0f ? sqrt_a(fmaf(U, U, Vi * Vi)) : PT_ZBEHIND;
 }
