@@ -503,11 +503,14 @@ struct BwdArgs {
 constexpr int TT = 64;   // times per tile
 
 // Blocks of 384 threads for few vectors, where the chip has room and a
-// vector's passes are one chain: 200 vectors x 10,000 times take 20.2 us in
-// them and 29.8 us in blocks of 128, 300 x 2,000 x 3 supersamples 17.5 and
-// 24.2 (400 x 3,000, the other way, 23.8 and 20.0); from 600 vectors on blocks
-// of 128 (800 x 3,000: 46.5 and 24.1 us).
-constexpr int WIDE_MAX_VECTORS = 600;
+// vector's passes are one chain.  Two of them fit on an SM: as many vectors
+// as that take one wave (304 vectors x 3,000 times 16.4 us, in blocks of 128
+// 18.5; x 40,000 49.1 and 83.3; x 30 to 300 the same to 2 us).  Vectors of a
+// second wave pay its start: 400 x 301 18.5 us and 12.4, x 3,000 24.6 and
+// 18.6, so up to 600 vectors they come in wide blocks only where they are long,
+// from about 12,000 points (400 x 10,000 32.8 and 34.9, 599 x 20,000 54.9 and
+// 57.4; 599 x 5,000 x 3 supersamples 50.5 and 49.2, x 10,000 x 3 74.1 and 81.1).
+constexpr int WIDE_PER_SM = 2, WIDE_MAX_VECTORS = 600, WIDE_LONG_POINTS = 12000;
 
 // Rows pay from about 1,280 in-transit points a vector (4,096 vectors, a
 // quarter of the points in transit: 3,000 times 93 us with rows, 82 with the
@@ -884,7 +887,11 @@ int pt_ma_quad_bwd(const double *t, int n_t, const pt_theta *th, int n_ss, doubl
     A.ssr = ssr;
     A.flux = flux;
     A.n_bad = n_bad;
-    if (th->n_v >= WIDE_MAX_VECTORS)
+    int dev = 0, n_sm = 0;
+    e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return pt_internal::set_error(PT_ERR_CUDA, "SM count", cudaGetErrorString(e));
+    if (th->n_v > (n_t * (int64_t)n_ss < WIDE_LONG_POINTS ? WIDE_PER_SM * n_sm : WIDE_MAX_VECTORS - 1))
         pt::launch_chained(n_ss == 1 ? ma_bwd_kernel<128, true> : ma_bwd_kernel<128, false>, th->n_v, 128, 0, s, A);
     else
         pt::launch_chained(n_ss == 1 ? ma_bwd_kernel<384, true> : ma_bwd_kernel<384, false>, th->n_v, 384, 0, s, A);
