@@ -55,44 +55,121 @@ inline int intervals(int N, int n_j)
 inline float row_scale(int n_int) { return ((float)n_int - 0.5f) * (1.0f - 2e-6f); }
 
 // ---------------------------------------------------------------------------
-// Plan: node values of Phi_{n,j}, then coefficients.  rec [N+1][n_j][3]: the
-// recursion of G_j(nu+2, 1; x); all in FP64 (once per plan).
+// Plan: the polynomials' coefficients, from the values of Phi_{n,j} at eight
+// Chebyshev points per interval.  One CTA per order and four intervals: its
+// first warp runs the recursion of G_j(nu+2, 1; x) at the 32 points, one a
+// lane, in double-float arithmetic (a chain of n_j steps; FP64 has a 64th of
+// the FP32 rate here), and the other three turn the previous BJ terms' values into
+// coefficients.  The points are symmetric, so even and odd Chebyshev
+// coefficients come from the sums and differences of four pairs; in powers of
+// x in [-1, 1] they are 4 x 4 products, and t = x / 2 scales them by powers of
+// two.  Only the first interval, t in [0, 1/2], shifts them (x = 4 t - 1).
+// The high powers cancel to about 2^-6 of their terms, which double-float
+// sums leave far below the rounding to FP32 at the end.  The same work in
+// two FP64 passes with the node values in global memory took 83 us at N = 8,
+// n_j = 192 and 454 at N = 16, n_j = 512; here launch and wait take 42 and 155.
 // ---------------------------------------------------------------------------
-__global__ void basis_nodes_kernel(const double *rec, int NP1, int n_j, int n_int, double scale, double *V)
-{
-    const int n_node = Q * n_int;
-    const int id = blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= NP1 * n_node) return;
-    const int n = id / n_node, node = id - n * n_node, i = node / Q, q = node - i * Q;
-    const double xq = cospi((q + 0.5) / Q);
-    const double u = (i == 0 ? 0.25 * (1.0 + xq) : i + 0.5 * xq) / scale;
-    const double c = 1.0 - u * u, x = c * c;
-    const double sn = u * sqrt(2.0 - u * u);   // sqrt(1 - c^2)
-    double pw = 1.0;
-    for (int m = 0; m < n + 4; ++m) pw *= sn;
-    double g = pw, gp = 0.0;
-    for (int j = 0; j < n_j; ++j) {
-        V[((size_t)n * n_j + j) * n_node + node] = g;
-        const double *r = rec + ((size_t)n * n_j + j) * 3;
-        const double gn = (r[0] + r[1] * x) * g + r[2] * gp;
-        gp = g;
-        g = gn;
-    }
-}
+constexpr int BJ = 32;          // terms per step
+constexpr int BASIS_TB = 128;   // threads
 
-// mat [2][Q][Q]: node values -> monomial coefficients (first interval, others)
-__global__ void basis_coef_kernel(const double *V, const double *mat, int K, int n_int, float *B)
+struct Basis {
+    const double *A, *recb;   // uploaded: A_{n,j}; [N+1][n_j][3] recursion of G_j(nu+2, nu+1; x)
+    const float2 *rec;        // uploaded: recursion of G_j(nu+2, 1; x), double-float
+    float4 *coef;             // the same in FP32
+    float2 *dA, *drb;         // A and recb as double-float pairs
+    float *B;                 // [(N+1) n_j][n_int][8]
+    int NP1, n_j, n_int;
+    double scale;
+    double xq[Q];             // the points in [-1, 1]
+    float2 m[2][4][4];        // [parity][power / 2][pair]: pair sums, differences -> powers of x
+};
+
+__global__ void __launch_bounds__(BASIS_TB) basis_kernel(const __grid_constant__ Basis P)
 {
-    const long long id = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (id >= (long long)K * n_int) return;
-    const long long k = id / n_int;
-    const int i = (int)(id - k * n_int);
-    const double *v = V + (k * n_int + i) * Q, *m = mat + (i == 0 ? 0 : Q * Q);
-    for (int c = 0; c < Q; ++c) {
-        double a = 0.0;
-        for (int q = 0; q < Q; ++q) a += m[c * Q + q] * v[q];
-        // the depth is exactly 0 at the contact (u = 0)
-        B[(k * n_int + i) * Q + c] = (i == 0 && c == 0) ? 0.0f : (float)a;
+    extern __shared__ __align__(16) unsigned char bsm[];
+    float2 *srec = reinterpret_cast<float2 *>(bsm);   // [n_j][3]
+    __shared__ float2 sv[2][BJ][32];                  // node values
+    __shared__ float sF[Q][Q];                        // powers of x -> powers of t, first interval
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, n_j = P.n_j;
+    const int n = blockIdx.y, i0 = 4 * blockIdx.x, q = lane & 7, i = min(i0 + (lane >> 3), P.n_int - 1);
+
+    // the other forms of the uploaded tables, a share of them per CTA
+    const int id0 = (blockIdx.y * gridDim.x + blockIdx.x) * BASIS_TB + tid, nth = gridDim.x * gridDim.y * BASIS_TB;
+    for (int at = id0; at < P.NP1 * n_j; at += nth) {
+        const DF a = pt::df_of(P.A[at]);
+        P.dA[at] = make_float2(a.h, a.l);
+        for (int c = 0; c < 3; ++c) {
+            const DF r = pt::df_of(P.recb[3 * at + c]);
+            P.drb[3 * at + c] = make_float2(r.h, r.l);
+        }
+        P.coef[at] = make_float4(P.rec[3 * at].x, P.rec[3 * at + 1].x, P.rec[3 * at + 2].x, 0.0f);
+    }
+    for (int at = tid; at < 3 * n_j; at += BASIS_TB) srec[at] = P.rec[(size_t)n * n_j * 3 + at];
+    if (tid < Q * Q) {   // (4 t - 1)^c by powers r of t: binomial(c, r) 4^r (-1)^(c - r)
+        const int r = tid / Q, c = tid % Q;
+        float bin = r <= c ? 1.0f : 0.0f;
+        for (int m = 1; m <= r && r <= c; ++m) bin = bin * (float)(c - r + m) / (float)m;
+        sF[r][c] = bin * (float)(1 << (2 * r)) * ((c - r) & 1 ? -1.0f : 1.0f);
+    }
+    DF g = {}, gp = {}, x = {};
+    DF M[4];
+    if (warp == 0) {
+        const double xq = P.xq[q], u = (i == 0 ? 0.25 * (1.0 + xq) : i + 0.5 * xq) / P.scale, c = 1.0 - u * u;
+        const double sn = u * sqrt(2.0 - u * u);   // sqrt(1 - c^2)
+        double pw = 1.0;
+        for (int m = 0; m < n + 4; ++m) pw *= sn;
+        x = pt::df_of(c * c);
+        g = pt::df_of(pw);
+    } else {
+        for (int p = 0; p < 4; ++p) {
+            const float2 v = P.m[q >> 2][q & 3][p];
+            M[p] = DF{v.x, v.y};
+        }
+    }
+    const int pw = q < 4 ? 2 * q : 2 * q - 7;   // the power of this lane's coefficient
+    const float two = (float)(1 << pw);
+    __syncthreads();
+    const int n_step = (n_j + BJ - 1) / BJ;
+    for (int st = 0; st <= n_step; ++st) {
+        if (warp == 0 && st < n_step) {
+            const int j1 = min(BJ, n_j - st * BJ);
+            for (int j = 0; j < j1; ++j) {
+                sv[st & 1][j][lane] = make_float2(g.h, g.l);
+                const float2 *r = srec + 3 * (st * BJ + j);
+                const DF al = df_mad(DF{r[1].x, r[1].y}, x, DF{r[0].x, r[0].y});
+                const DF gn = df_mad(al, g, df_mul(DF{r[2].x, r[2].y}, gp));
+                gp = g;
+                g = gn;
+            }
+        }
+        if (warp > 0 && st > 0) {
+            const int j0 = (st - 1) * BJ, j1 = min(BJ, n_j - j0);
+            for (int j = warp - 1; j < j1; j += BASIS_TB / 32 - 1) {
+                const float2 v = sv[(st - 1) & 1][j][lane], o = sv[(st - 1) & 1][j][lane ^ 7];
+                const float sg = q < 4 ? 1.0f : -1.0f;   // lanes 0..3 the pairs' sums, 4..7 differences (pair 7 - q)
+                const DF sd = df_add(DF{o.x, o.y}, DF{sg * v.x, sg * v.y});
+                DF b = {};
+                for (int p = 0; p < 4; ++p) {
+                    const int src = (lane & 24) + (q < 4 ? p : 7 - p);
+                    const DF w = {__shfl_sync(~0u, sd.h, src), __shfl_sync(~0u, sd.l, src)};
+                    b = p == 0 ? df_mul(M[0], w) : df_mad(M[p], w, b);
+                }
+                float out = two * b.h;
+                if (i0 == 0) {
+                    DF a = {};
+                    for (int c = 0; c < Q; ++c) {
+                        const int src = c & 1 ? 4 + c / 2 : c / 2;
+                        const DF w = {__shfl_sync(~0u, b.h, src), __shfl_sync(~0u, b.l, src)};
+                        a = df_mad(DF{sF[pw][c], 0.0f}, w, a);
+                    }
+                    // the depth is exactly 0 at the contact (u = 0)
+                    if (lane < 8) out = pw == 0 ? 0.0f : a.h;
+                }
+                if (i0 + (lane >> 3) < P.n_int)
+                    P.B[(((size_t)n * n_j + j0 + j) * P.n_int + i) * Q + pw] = out;
+            }
+        }
+        __syncthreads();
     }
 }
 

@@ -24,7 +24,9 @@
 #include <string.h>
 
 #include <algorithm>
+#include <memory>
 #include <mutex>
+#include <new>
 
 #include "../../include/pt.h"
 #include "pt_device.cuh"
@@ -870,9 +872,10 @@ bool ma_table_view(pt_ma_table t, const float4 **tab, int *n_k, int *n_z, float 
 
 struct pt_gim_plan_s {
     int N, n_j;
+    void *d_mem;      // the one allocation that holds the tables below
     float4 *d_coef;   // [N+1][n_j]: recursion of G_j(nu+2, 1; x), FP32
-    double *d_A;      // [N+1][n_j]: A_{n,j}, FP64
-    double *d_recb;   // [N+1][n_j][3]: recursion of G_j(nu+2, nu+1; x), FP64
+    const double *d_A;      // [N+1][n_j]: A_{n,j}, FP64
+    const double *d_recb;   // [N+1][n_j][3]: recursion of G_j(nu+2, nu+1; x), FP64
     float2 *d_dA;     // the same A_{n,j} and recursion as double-float pairs
     float2 *d_drb;
     float *d_B;       // [(N+1) n_j][8 n_int]: piecewise polynomials of the series' functions (pt_gim.cuh)
@@ -1383,18 +1386,25 @@ int pt_gim_plan_create(int N, int n_j, pt_gim_plan *out)
 {
     if (!out || N < 1 || N > 16 || n_j < 2 || n_j > 512) return PT_ERR_ARG;
     *out = nullptr;
-    int NP1 = N + 1;
-    size_t cnt = (size_t)NP1 * n_j;
-    float4 *hcoef = new float4[cnt];
-    double *hA = new double[cnt];
-    double *hrb = new double[cnt * 3];
-    double *hrc = new double[cnt * 3];
-    float2 *hdA = new float2[cnt];
-    float2 *hdrb = new float2[cnt * 3];
-    auto df = [](double v) {
-        const float h = (float)v;
-        return make_float2(h, (float)(v - (double)h));
+    const int NP1 = N + 1;
+    const size_t cnt = (size_t)NP1 * n_j;
+    const int n_int = gim::intervals(N, n_j);
+    constexpr int Q = gim::Q;
+    // one allocation: the uploaded tables, then those that the kernel derives
+    size_t total = 0;
+    auto part = [&](size_t bytes) {
+        const size_t at = total;
+        total += (bytes + 255) & ~(size_t)255;
+        return at;
     };
+    const size_t oA = part(cnt * sizeof(double)), orb = part(cnt * 3 * sizeof(double)),
+                 orc = part(cnt * 3 * sizeof(float2)), upload = total, oc = part(cnt * sizeof(float4)),
+                 odA = part(cnt * sizeof(float2)), odrb = part(cnt * 3 * sizeof(float2)),
+                 oB = part(cnt * n_int * Q * sizeof(float));
+    std::unique_ptr<double[]> host(new (std::nothrow) double[upload / sizeof(double)]);
+    if (!host) return pt_internal::set_error(PT_ERR_CUDA, "pt_gim_plan_create", "out of host memory");
+    double *hA = host.get() + oA / sizeof(double), *hrb = host.get() + orb / sizeof(double);
+    float2 *hrc = (float2 *)(host.get() + orc / sizeof(double));
     for (int n = 0; n < NP1; ++n) {
         double nu = 0.5 * (n + 2);
         // A_{n,j} = (-1)^j (2j+nu+2)/nu * prod_{i=1..j} (nu+i)/(i+1)   (Eq. gimemez_a)
@@ -1403,82 +1413,70 @@ int pt_gim_plan_create(int N, int n_j, pt_gim_plan *out)
             const size_t at = (size_t)n * n_j + j;
             if (j > 0) prod *= (nu + j) / (j + 1.0);
             hA[at] = ((j & 1) ? -1.0 : 1.0) * (2.0 * j + nu + 2.0) / nu * prod;
-            hdA[at] = df(hA[at]);
-            jacobi_rec(nu + 2.0, 1.0, j, hrc + 3 * at);
-            hcoef[at] = make_float4((float)hrc[3 * at], (float)hrc[3 * at + 1], (float)hrc[3 * at + 2], 0.0f);
+            double rc[3];
+            jacobi_rec(nu + 2.0, 1.0, j, rc);
+            for (int c = 0; c < 3; ++c) {
+                const float h = (float)rc[c];
+                hrc[3 * at + c] = make_float2(h, (float)(rc[c] - (double)h));
+            }
             jacobi_rec(nu + 2.0, nu + 1.0, j, hrb + 3 * at);
-            for (int c = 0; c < 3; ++c) hdrb[3 * at + c] = df(hrb[3 * at + c]);
         }
     }
-    // node values -> monomials on an interval, by Chebyshev coefficients: the
-    // first interval (t in [0, 1/2]) and the others (t in [-1/2, 1/2])
-    constexpr int Q = gim::Q;
-    double mat[2][Q][Q];
-    for (int kind = 0; kind < 2; ++kind) {
-        const double al = kind == 0 ? 4.0 : 2.0, be = kind == 0 ? -1.0 : 0.0;
-        double T[Q][Q] = {};   // T_k(al t + be) by powers of t
-        T[0][0] = 1.0;
-        T[1][0] = be;
-        T[1][1] = al;
-        for (int k = 2; k < Q; ++k)
-            for (int c = 0; c < Q; ++c)
-                T[k][c] = 2.0 * be * T[k - 1][c] + (c > 0 ? 2.0 * al * T[k - 1][c - 1] : 0.0) - T[k - 2][c];
-        for (int q = 0; q < Q; ++q)
-            for (int c = 0; c < Q; ++c) {
-                double v = 0.0;
-                for (int k = 0; k < Q; ++k) v += (k == 0 ? 1.0 : 2.0) / Q * cos(k * (q + 0.5) * PI_D / Q) * T[k][c];
-                mat[kind][c][q] = v;
-            }
-    }
-    pt_gim_plan p = new pt_gim_plan_s;
-    p->N = N;
-    p->n_j = n_j;
-    p->d_coef = nullptr;
-    p->d_A = nullptr;
-    p->d_recb = nullptr;
-    p->d_dA = p->d_drb = nullptr;
-    p->d_B = nullptr;
-    p->n_int = gim::intervals(N, n_j);
-    p->ev0 = p->ev1 = nullptr;
-    const int n_node = Q * p->n_int;
-    double *d_rc = nullptr, *d_mat = nullptr, *d_V = nullptr;   // while the basis is built
-    cudaError_t e = cudaMalloc(&p->d_coef, cnt * sizeof(float4));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_A, cnt * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_recb, cnt * 3 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_dA, cnt * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_drb, cnt * 3 * sizeof(float2));
-    if (e == cudaSuccess) e = cudaMalloc(&p->d_B, cnt * n_node * sizeof(float));
-    if (e == cudaSuccess) e = cudaMalloc(&d_rc, cnt * 3 * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc(&d_mat, sizeof(mat));
-    if (e == cudaSuccess) e = cudaMalloc(&d_V, cnt * n_node * sizeof(double));
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_coef, hcoef, cnt * sizeof(float4), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_A, hA, cnt * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_recb, hrb, cnt * 3 * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_dA, hdA, cnt * sizeof(float2), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(p->d_drb, hdrb, cnt * 3 * sizeof(float2), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(d_rc, hrc, cnt * 3 * sizeof(double), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMemcpy(d_mat, mat, sizeof(mat), cudaMemcpyHostToDevice);
+    gim::Basis P;
+    // values at the points x_q -> Chebyshev coefficients -> powers of x, for
+    // the sums (even powers) and differences (odd) of the pairs x_q, -x_q
+    double T[Q][Q] = {};   // T_k by powers of x
+    T[0][0] = T[1][1] = 1.0;
+    for (int k = 2; k < Q; ++k)
+        for (int c = 0; c < Q; ++c) T[k][c] = (c > 0 ? 2.0 * T[k - 1][c - 1] : 0.0) - T[k - 2][c];
+    for (int q = 0; q < Q; ++q) P.xq[q] = cos((q + 0.5) * PI_D / Q);
+    for (int c = 0; c < Q; ++c)
+        for (int q = 0; q < Q / 2; ++q) {
+            double v = 0.0;
+            for (int k = 0; k < Q; ++k) v += (k == 0 ? 1.0 : 2.0) / Q * cos(k * (q + 0.5) * PI_D / Q) * T[k][c];
+            const float h = (float)v;
+            P.m[c & 1][c / 2][q] = make_float2(h, (float)(v - (double)h));
+        }
+    unsigned char *d = nullptr;
+    cudaError_t e = cudaMalloc(&d, total);
+    if (e != cudaSuccess) return set_cuda_error(e, "pt_gim_plan_create");
+    e = cudaMemcpy(d, host.get(), upload, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
-        const int n1 = NP1 * n_node;
-        const long long n2 = (long long)cnt * p->n_int;
-        gim::basis_nodes_kernel<<<(n1 + 63) / 64, 64>>>(d_rc, NP1, n_j, p->n_int, (double)gim::row_scale(p->n_int), d_V);
-        gim::basis_coef_kernel<<<(unsigned)((n2 + 127) / 128), 128>>>(d_V, d_mat, (int)cnt, p->n_int, p->d_B);
+        P.A = (const double *)(d + oA);
+        P.recb = (const double *)(d + orb);
+        P.rec = (const float2 *)(d + orc);
+        P.coef = (float4 *)(d + oc);
+        P.dA = (float2 *)(d + odA);
+        P.drb = (float2 *)(d + odrb);
+        P.B = (float *)(d + oB);
+        P.NP1 = NP1;
+        P.n_j = n_j;
+        P.n_int = n_int;
+        P.scale = (double)gim::row_scale(n_int);
+        gim::basis_kernel<<<dim3((n_int + 3) / 4, NP1), gim::BASIS_TB, 3 * n_j * sizeof(float2)>>>(P);
         e = cudaGetLastError();
     }
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
-    cudaFree(d_rc);
-    cudaFree(d_mat);
-    cudaFree(d_V);
-    delete[] hcoef;
-    delete[] hA;
-    delete[] hrb;
-    delete[] hrc;
-    delete[] hdA;
-    delete[] hdrb;
+    if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     if (e != cudaSuccess) {
-        pt_gim_plan_destroy(p);
+        cudaFree(d);
         return set_cuda_error(e, "pt_gim_plan_create");
     }
+    pt_gim_plan p = new (std::nothrow) pt_gim_plan_s;
+    if (!p) {
+        cudaFree(d);
+        return pt_internal::set_error(PT_ERR_CUDA, "pt_gim_plan_create", "out of host memory");
+    }
+    p->N = N;
+    p->n_j = n_j;
+    p->n_int = n_int;
+    p->d_mem = d;
+    p->d_coef = P.coef;
+    p->d_A = P.A;
+    p->d_recb = P.recb;
+    p->d_dA = P.dA;
+    p->d_drb = P.drb;
+    p->d_B = P.B;
+    p->ev0 = p->ev1 = nullptr;
     *out = p;
     return PT_OK;
 }
@@ -1494,12 +1492,7 @@ int pt_gim_plan_time_evaluation(pt_gim_plan p, void *ev_start, void *ev_end)
 int pt_gim_plan_destroy(pt_gim_plan p)
 {
     if (!p) return PT_OK;
-    cudaFree(p->d_coef);
-    cudaFree(p->d_A);
-    cudaFree(p->d_recb);
-    cudaFree(p->d_dA);
-    cudaFree(p->d_drb);
-    cudaFree(p->d_B);
+    cudaFree(p->d_mem);
     delete p;
     return PT_OK;
 }
