@@ -1,12 +1,13 @@
 """Gimenez plans: what creating one costs, and the tables of plans at the
 ends of the accepted orders and depths.
 
-A plan is one allocation, one upload and one kernel.  A small table of the
-Mandel-Agol terms (MATable) is one allocation and one kernel, so twice its time
-stands for what cannot be saved; to that come the host's tables, the upload
-and the kernel (75 us at N = 8, n_j = 192, 250 at N = 16, n_j = 512), allowed about
-twice.  Creation with nine allocations, seven uploads and two FP64 passes took
-390 to 450 us and 930 to 970 where the table took 22 to 100.
+A plan is one allocation, one upload and one kernel.  What the driver takes
+for a block of the plan's size differs by several times between machines, so
+a table of the Mandel-Agol terms (MATable) of as many bytes, one allocation and one kernel, is
+timed beside it.  To that come the host's tables, the upload and the longer
+kernel (75 us at N = 8, n_j = 192, 250 at N = 16, n_j = 512), allowed about twice.
+Creation with nine allocations, seven uploads and two FP64 passes took 330 and
+660 us more than the table.
 
 The light curves' bounds are those of the series' depth test: at k <= 0.7 1e-6,
 up to 1.5 2.5e-6 (rows 9e-8 and 6e-7 in 64 bits, FP32 roundings, sum |C_n| <= 2).
@@ -30,8 +31,8 @@ def _torch():
     return torch
 
 
-@pytest.mark.parametrize("N,n_j,allowed_us", [(8, 192, 150.0), (16, 512, 500.0)])
-def test_creation_time(N, n_j, allowed_us):
+@pytest.mark.parametrize("N,n_j,n_k,n_z,allowed_us", [(8, 192, 128, 2976, 150.0), (16, 512, 2048, 2408, 500.0)])
+def test_creation_time(N, n_j, n_k, n_z, allowed_us):
     torch = _torch()
     import paper_1504_07433_gb300 as pt
     torch.zeros(1, device="cuda")
@@ -47,8 +48,9 @@ def test_creation_time(N, n_j, allowed_us):
             out.append(time.perf_counter() - t0)
         return sorted(out)[12]
 
-    table, plan = median(lambda: pt.MATable(0.05, 0.2, 128, 256)), median(lambda: pt.GimenezPlan(N, n_j))
-    assert plan <= 2.0 * table + 1e-6 * allowed_us, (plan, table)
+    table, plan = median(lambda: pt.MATable(0.05, 0.2, n_k, n_z)), median(lambda: pt.GimenezPlan(N, n_j))
+    print("table %.0f us, plan %.0f us" % (table * 1e6, plan * 1e6))
+    assert plan <= table + 1e-6 * allowed_us, (plan, table)
 
 
 @pytest.mark.parametrize("N,n_j", [(1, 2), (16, 2), (1, 33), (16, 32), (3, 65), (1, 512)])
