@@ -116,7 +116,7 @@ class ClockSampler:
 # (dram__bytes_read.sum + dram__bytes_write.sum) from its ncu capture at the
 # long-cadence workload (50,000 times x 256 vectors x 10 supersamples; null
 # for any other sizes; the 51 MB of fluxes were still in L2 at its end)
-TRAFFIC = {"bytes": 1.56e6, "n_t": 50000, "n_v": 256, "n_ss": 10}
+TRAFFIC = {"bytes": 1.63e6, "n_t": 50000, "n_v": 256, "n_ss": 10}
 # FP32 operations of one in-transit supersample in that kernel: the f and g
 # series (18), the position and its separation (11), the interval and offset
 # of the look-up (10) and a degree-7 polynomial (14)

@@ -176,6 +176,10 @@ int pt_ma_terms(const float *k_dev, const float *z_dev, size_t n, float *lam_e_d
  * (the factoring of Sec. 2.2.2); with k_per_band == 1 every passband has its
  * own radius ratio and is evaluated as its own geometry.
  * At least one of flux_dev and ssr_dev must be non-NULL.
+ * Residual sums are formed in an order fixed by n_t: per 256 times, then over
+ * these blocks.  A vector's flux and sum do not depend on the call's other
+ * vectors, but for the choice between row tables and exact terms (up to four
+ * geometries, and few times, take the latter), which differ by rounding.
  * Accuracy: fluxes within 1e-6 of the FP64 model for k <= 1 (3e-6 above,
  * as for pt_ma_terms).  PT_ERR_DOMAIN for t_exp < 0 or not finite.
  * ---------------------------------------------------------------------- */

@@ -6,7 +6,8 @@
 //                       split; per geometry and passband: the Mandel-Agol row
 //                       of polynomials (pt_device.cuh), the caller's table at
 //                       the geometry's k, or the Gimenez factors and weights.
-//   product_kernel      Gimenez: the rows as FP32 products (pt_gim.cuh).
+//   product_kernel, product_tall_kernel
+//                       Gimenez: the rows as FP32 products (pt_gim.cuh).
 //   zi_rows_kernel      Gimenez interpolated in z (Sec. 3.3): the node values.
 //   lc_rows_kernel      the light curves from the rows (pt_rows.cuh).
 //   setup_kernel, ma_lc_kernel

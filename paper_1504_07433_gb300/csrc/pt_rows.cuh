@@ -30,9 +30,9 @@
 // a scan, and an evaluation kernel per model that solved Kepler's equation for
 // every supersample, packed the in-transit ones and evaluated the terms for
 // each.  50,000 times x 256 eccentric vectors x 10 supersamples: Mandel-Agol
-// 85.4 -> 47.8 us a call, from the caller's table 109 -> 44.1 us; 3,001 times x
-// 800 circular geometries x 3, residual sums: 75.8 -> 39.6 us.  What bounds it:
-// issue (about 65 %), two thirds of the instructions in the window test, the
+// 85.4 -> 45.9 us a call, from the caller's table 109 -> 43.8 us; 3,001 times x
+// 800 circular geometries x 3, residual sums: 75.8 -> 38.9 us.  What bounds it:
+// issue (about 67 %), two thirds of the instructions in the window test, the
 // lists and the stores of a survey's mostly empty pairs.
 #pragma once
 

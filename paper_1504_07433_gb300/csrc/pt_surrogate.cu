@@ -22,9 +22,9 @@
 // What bounds it: the special-function unit (512 operations per point: two
 // hidden layers by tanh, the last by exp and a reciprocal) and the activations'
 // other instructions, not the tensor cores.  2e7 points, 12 % of them served by
-// the network: classify_kernel 433 -> 211 us, sur_kernel 1047 -> 380 us
-// with four groups (664 us with one, 478 with two)
-// (before: one group, the last layer's SiLU by expf and an IEEE division).
+// the network: classify_kernel 433 -> 211 us, sur_kernel 1047 -> 423 us with four
+// groups and the last layer's SiLU by a corrected quotient (before: one group, an
+// IEEE division; with the uncorrected quotient one group took 664 us, two 478, four 373).
 // Every mbarrier wait is bounded; on time-out the kernel records an error,
 // stops issuing work, frees its tensor memory and returns.
 #include <cuda_bf16.h>
