@@ -416,6 +416,7 @@ __device__ __forceinline__ float point_sums(const PointConst &c, float dts, floa
             conv = true;
             break;
         }
+        if (it + 1 >= pt::KEPLER_FREE) dE = pt::kepler_bracket(dE, dM, c.esE, c.nq);
     }
     if (!conv) *bad = true;
     // sin and cos of dE/2 at the solution (as in pt::orbit_z)

@@ -250,6 +250,23 @@ __device__ __forceinline__ void sincos_near0(float h, float *s, float *c)
 // from the last step's values (below) instead of a second series; the
 // supersample loop of the row kernel gains from it, while in the
 // batched and tile kernels the extra live values cost more than the series.
+
+// E = M + e sin E puts dE within e of dM - e sin E_tr.  Far from transit at a high
+// eccentricity Newton's method, from either start, can leap out of that interval and
+// not come back (e = 0.9, exposures of 0.4 d at P = 3 d: 2.6 % of the exposures did
+// not converge from the second-order start, none from a first-order one; over
+// the whole orbit 14 % from the cold start), so from the fourth step on its iterate is
+// brought back into it: then every one converges, in eight steps at most up to e
+// = 0.9 and ten at 0.95.  The steps before are free: over a transit there are one
+// to three.
+constexpr int KEPLER_FREE = 4;
+
+__device__ __forceinline__ float kepler_bracket(float dE, float dM, float esE, float nq)
+{
+    const float e = 1.0001f * nq * rcp_a(1.0f + nq), c = dM - esE;   // nq = e / (1 - e)
+    return fminf(fmaxf(dE, c - e), c + e);
+}
+
 template <bool FAST = false, bool ROT = false>
 __device__ __forceinline__ float orbit_z(const GeomRec &r, float dt, int max_iter, bool *bad, float *warm = nullptr)
 {
@@ -269,8 +286,7 @@ __device__ __forceinline__ float orbit_z(const GeomRec &r, float dt, int max_ite
         dE = dM / (1.0f - r.ecE);
     }
     float sh = 0.0f, ch = 1.0f, dEdM = 1.0f, step = 0.0f, esin = 0.0f;
-    bool conv = false;
-    for (int it = 0; it < max_iter; ++it) {
+    auto newton = [&]() {
         sincos_near0(0.5f * dE, &sh, &ch);
         float sn = 2.0f * sh * ch, omc = 2.0f * sh * sh;
         float F = (dE - r.ecE * sn) + (r.esE * omc - dM);
@@ -284,10 +300,18 @@ __device__ __forceinline__ float orbit_z(const GeomRec &r, float dt, int max_ite
             if (warm) dEdM = __fdividef(1.0f, Fp);
         }
         dE -= step;
-        if (r.nq * step * step <= 6e-8f * fabsf(dE) + 1e-12f) {
-            conv = true;
-            break;
-        }
+        return r.nq * step * step <= 6e-8f * fabsf(dE) + 1e-12f;
+    };
+    // (the bracketed steps in a loop of their own: in one loop their test cost the
+    // batch kernel 1 %; the other way round in orbit_state and the adjoint)
+    bool conv = false;
+    int it = 0;
+#pragma unroll 1
+    for (; it < min(max_iter, KEPLER_FREE) && !conv; ++it) conv = newton();
+#pragma unroll 1
+    for (; it < max_iter && !conv; ++it) {
+        dE = kepler_bracket(dE, dM, r.esE, r.nq);
+        conv = newton();
     }
     if (!conv) *bad = true;
     if (warm) {
@@ -369,6 +393,7 @@ __device__ __forceinline__ void orbit_state(const GeomRec &r, float dt, int max_
             conv = true;
             break;
         }
+        if (it + 1 >= KEPLER_FREE) dE = kepler_bracket(dE, dM, r.esE, r.nq);
     }
     if (!conv) *bad = true;
     const float h = 0.5f * step;
