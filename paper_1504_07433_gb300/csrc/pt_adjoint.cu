@@ -735,7 +735,7 @@ __device__ __forceinline__ void vector_sums(const BwdArgs &A, const VecConst &sc
 // One block per vector.  What bounds it: instruction issue (65% of the cycles;
 // 4,096 vectors x 10,000 times, a quarter in transit: 290 instructions per
 // warp of in-transit points, 9,000 per vector for its constants, row and sums).  Measured
-// there 182 us against 274 when every point took the exact terms (540
+// there 183 us against 274 when every point took the exact terms (540
 // instructions) and the derivative of each parameter by itself; with the exact
 // terms and these sums it is 197.  72 registers: seven blocks per multiprocessor
 // (six took 3% longer, eight the same).

@@ -13,7 +13,7 @@
 //     then read at tens of thousands of separations (all in-window times of
 //     all light curves), so the elliptic integrals have left the per-point
 //     work: at 1,024 walkers x 64 passbands x 81,058 times a call went from
-//     17.5 ms (the terms evaluated per point) to 2.79 ms.
+//     17.5 ms (the terms evaluated per point) to 2.80 ms.
 // batch_kernel: persistent CTAs take (walker, group of BG passbands, slice of
 // the times) items from an atomic counter, ordered so that consecutive items
 // share their observations in L2.  Per item the group's rows are staged in

@@ -303,7 +303,7 @@ __device__ __forceinline__ float orbit_z(const GeomRec &r, float dt, int max_ite
         return r.nq * step * step <= 6e-8f * fabsf(dE) + 1e-12f;
     };
     // (the bracketed steps in a loop of their own: in one loop their test cost the
-    // batch kernel 1 %; the other way round in orbit_state and the adjoint)
+    // batch kernel 1 %, so 0.5 %; the other way round in orbit_state and the adjoint)
     bool conv = false;
     int it = 0;
 #pragma unroll 1
